@@ -137,6 +137,7 @@ int ensure_io(qcd_ctx *c, size_t bytes) {
 }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
+bool aligned32(const void *p) { return ((uintptr_t)p & 31) == 0; }
 
 }  // namespace
 
@@ -301,32 +302,18 @@ int qcd_apply_D(qcd_ctx *c, void *out, const void *in, int prec, int nrhs) {
     const bool dev_in = is_device_ptr(in), dev_out = is_device_ptr(out);
     if ((dev_in && !aligned16(in)) || (dev_out && !aligned16(out)))
         return fail(c, QCD_ERR_ARG, "device spinors must be 16-byte aligned");
-    if ((rc = ensure_io(c, 3 * obytes))) return rc;  // internal in, internal out, staged host in / out
+    // Device spinors are read and written where they are when their alignment allows the kernels'
+    // 32-byte accesses, else through an aligned copy (the input too when the output overlaps it: D
+    // reads a site's neighbours while others are written); host spinors through a staging copy.
+    const bool overlap = (const char *)in < (char *)out + obytes && (char *)out < (const char *)in + bytes;
+    const bool cp_in = !dev_in || overlap || !aligned32(in), cp_out = !dev_out || !aligned32(out);
+    if ((cp_in || cp_out) && (rc = ensure_io(c, (cp_in ? bytes : 0) + (cp_out ? obytes : 0)))) return rc;
     char *io = (char *)c->d_io;
-    const void *din = in;
-    void *dout = dev_out ? out : io + 2 * obytes;
-    if (!dev_in) {
-        QCD_CUDA(c, cudaMemcpyAsync(io + 2 * obytes, in, bytes, cudaMemcpyHostToDevice, c->stream));
-        din = io + 2 * obytes;
-    }
-    if (prec == QCD_F32X2) {
-        float4 *a = (float4 *)io;
-        double2 *b = (double2 *)(io + obytes);
-        if ((rc = spinor32_to_internal(c, a, (const float2 *)din, nrhs))) return rc;
-        if ((rc = dslash_x2(c, b, a, nrhs))) return rc;
-        if ((rc = spinor64_from_internal(c, (double2 *)dout, b, nrhs))) return rc;
-    } else if (prec == QCD_F64) {
-        double2 *a = (double2 *)io, *b = (double2 *)(io + bytes);
-        if ((rc = spinor64_to_internal(c, a, (const double2 *)din, nrhs))) return rc;
-        if ((rc = dslash64(c, b, a, nrhs))) return rc;
-        if ((rc = spinor64_from_internal(c, (double2 *)dout, b, nrhs))) return rc;
-    } else {
-        float4 *a = (float4 *)io, *b = (float4 *)(io + bytes);
-        if ((rc = spinor32_to_internal(c, a, (const float2 *)din, nrhs))) return rc;
-        if ((rc = (prec == QCD_F16 ? dslash16 : prec == QCD_F32_SU3 ? dslash12 : dslash32)(c, b, a, nrhs))) return rc;
-        if ((rc = spinor32_from_internal(c, (float2 *)dout, b, nrhs))) return rc;
-    }
-    if (!dev_out) QCD_CUDA(c, cudaMemcpyAsync(out, dout, obytes, cudaMemcpyDeviceToHost, c->stream));
+    const void *din = cp_in ? io : in;
+    void *dout = cp_out ? io + (cp_in ? bytes : 0) : out;
+    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(io, in, bytes, cudaMemcpyDefault, c->stream));
+    if ((rc = dslash_canonical(c, dout, din, prec, nrhs))) return rc;
+    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, dout, obytes, cudaMemcpyDefault, c->stream));
     if (!dev_in || !dev_out) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     return QCD_OK;
 }

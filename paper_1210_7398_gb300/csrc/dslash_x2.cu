@@ -147,8 +147,8 @@ __device__ __forceinline__ void reconstruct_x2(int a, const CX &w0, const CX &w1
 
 // one hop term: (1 - gamma_mu) U_mu(n) psi(n+mu) forward, (1 + gamma_mu) U_mu(n-mu)^dag psi(n-mu)
 // backward; ulink is the site whose link is used
-template <int MU, bool FWD>
-__device__ __forceinline__ void hop_x2(const float4 *__restrict__ src, const float4 *__restrict__ Ux2, long V,
+template <int MU, bool FWD, typename SP>
+__device__ __forceinline__ void hop_x2(const SP *__restrict__ src, const float4 *__restrict__ Ux2, long V,
                                        long nb, long ulink, float sgn, CX acc[12]) {
     float2 p[12];
     load_spinor(src, V, nb, p);
@@ -218,8 +218,8 @@ __device__ __forceinline__ void herm6_x2(const float4 *__restrict__ F, long V, c
 
 __device__ __forceinline__ double to_f64(float h, float l) { return (double)h + (double)l; }
 
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restrict__ out, const float4 *__restrict__ in,
+template <int MINB, typename SP, typename SO>
+__global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(SO *__restrict__ out, const SP *__restrict__ in,
                                                           const float4 *__restrict__ Ux2,
                                                           const float4 *__restrict__ Fx2, float kh, float kl,
                                                           Geo g, int nrhs) {
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restric
     const long n = sblk * blockDim.x + threadIdx.x;
     if (n >= g.V) return;
     const long V = g.V;
-    const float4 *src = in + (long)rhs * 6 * V;
+    const SP *src = in + (long)rhs * 6 * V;
     int x[4];
     site_coords(g, n, x);
     CX acc[12];
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restric
     herm6_x2(Fx2 + 18 * V + n, V, c1, e1);
     float2 psi[12];
     load_spinor(src, V, n, psi);
-    double2 *dst = out + (long)rhs * 12 * V + n;
+    double2 res[12];
     const float2 kH = splat(kh), kL = splat(kl);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
@@ -276,8 +276,9 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restric
         float2 e;
         const float2 s = two_sum(psi[k], neg2(P), e);
         const float2 lo = sub2(e, add2(E, cr));
-        dst[(long)k * V] = make_double2(to_f64(s.x, lo.x), to_f64(s.y, lo.y));
+        res[k] = make_double2(to_f64(s.x, lo.x), to_f64(s.y, lo.y));
     }
+    store_spinor(out + (long)rhs * 12 * V, V, n, res);
 }
 
 // hi + lo split of FP64 values: hi = fl32(v), lo = fl32(v - hi); |v - hi - lo| <= 2^-48 |v|
@@ -298,7 +299,7 @@ __global__ void k_fields_to_x2(float4 *__restrict__ Ux2, float4 *__restrict__ Fx
 
 }  // namespace
 
-int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) {
+template <typename SO, typename SP> static int launch_x2(qcd_ctx *c, SO *out, const SP *in, int nrhs) {
     Geo g;
     for (int m = 0; m < 4; m++) g.L[m] = c->lat.L[m];
     g.V = c->lat.V;
@@ -317,11 +318,17 @@ int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) {
     const float kl = (float)(c->kappa - (double)kh);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH64, &ev);
-    // three CTAs of 128 threads per SM (168 registers, a few spilled): 12% faster than two
-    // without spills at 24^3x48 and 48^3x96
-    dslash_x2_kernel<3><<<dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, c->stream>>>(out, in, c->Ux2, c->Fx2,
+    // four CTAs of 128 threads per SM (128 registers, some spilled): the instruction fetch that the
+    // long unrolled body stalls on is hidden by more warps.  24^3x48, 4 right-hand sides: 1332 / 1241 /
+    // 1199 / 2131 us with 2 / 3 / 4 / 5
+    dslash_x2_kernel<4, SP, SO><<<dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, c->stream>>>(out, in, c->Ux2, c->Fx2,
                                                                                            kh, kl, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
+}
+
+int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) { return launch_x2(c, out, in, nrhs); }
+int dslash_x2_canonical(qcd_ctx *c, double2 *out, const float2 *in, int nrhs) {
+    return launch_x2(c, (Site64 *)out, (const Site32 *)in, nrhs);
 }
 
 }  // namespace qcd

@@ -234,6 +234,9 @@ int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs);
 int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
 int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
 int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
+// D on the caller's canonical layout [nrhs][V][12] (32-byte aligned), any qcd_apply_D precision
+int dslash_canonical(qcd_ctx *c, void *out, const void *in, int prec, int nrhs);
+int dslash_x2_canonical(qcd_ctx *c, double2 *out, const float2 *in, int nrhs);
 // FP32 D (two right-hand sides per thread when there are several) fused with the inner
 // products of the BiCGStab step that follows: mode 1: red[rhs] = <other, out>, |out|^2; mode 2:
 // <out, other>, |out|^2; mode 0: none.  Right-hand sides inactive in gate (may be null) are
