@@ -180,8 +180,9 @@ int qcd_apply_D(qcd_ctx *ctx, void *out, const void *in, int prec, int nrhs);
  * p->nsweep, p->nsap, p->sap_storage.  All right-hand sides go through one
  * batched application (one grid row of block solves per right-hand side);
  * each result equals, bit for bit, the call with that one alone.  Device
- * scratch grows to 4 nrhs + 1 complex64 fields (7 nrhs + 1 with
- * p->block_solver = 1). */
+ * scratch grows to 2 nrhs complex64 fields (5 nrhs with p->block_solver = 1),
+ * and nrhs more for each of in and out that needs a copy (host memory, off a
+ * 32-byte boundary, overlapping). */
 int qcd_sap_precondition(qcd_ctx *ctx, float *out, const float *in, const qcd_params *p, int nrhs);
 
 /* The paper has no counterpart to this entry point; it serves callers that

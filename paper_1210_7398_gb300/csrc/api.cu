@@ -138,6 +138,9 @@ int ensure_io(qcd_ctx *c, size_t bytes) {
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 bool aligned32(const void *p) { return ((uintptr_t)p & 31) == 0; }
+bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+    return (const char *)a < (const char *)b + nb && (const char *)b < (const char *)a + na;
+}
 
 }  // namespace
 
@@ -305,14 +308,13 @@ int qcd_apply_D(qcd_ctx *c, void *out, const void *in, int prec, int nrhs) {
     // Device spinors are read and written where they are when their alignment allows the kernels'
     // 32-byte accesses, else through an aligned copy (the input too when the output overlaps it: D
     // reads a site's neighbours while others are written); host spinors through a staging copy.
-    const bool overlap = (const char *)in < (char *)out + obytes && (char *)out < (const char *)in + bytes;
-    const bool cp_in = !dev_in || overlap || !aligned32(in), cp_out = !dev_out || !aligned32(out);
+    const bool cp_in = !dev_in || !aligned32(in) || overlap(in, bytes, out, obytes), cp_out = !dev_out || !aligned32(out);
     if ((cp_in || cp_out) && (rc = ensure_io(c, (cp_in ? bytes : 0) + (cp_out ? obytes : 0)))) return rc;
     char *io = (char *)c->d_io;
     const void *din = cp_in ? io : in;
     void *dout = cp_out ? io + (cp_in ? bytes : 0) : out;
     if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(io, in, bytes, cudaMemcpyDefault, c->stream));
-    if ((rc = dslash_canonical(c, dout, din, prec, nrhs))) return rc;
+    if ((rc = dslash(c, dout, din, prec, nrhs))) return rc;
     if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, dout, obytes, cudaMemcpyDefault, c->stream));
     if (!dev_in || !dev_out) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     return QCD_OK;
@@ -326,36 +328,23 @@ int qcd_sap_precondition(qcd_ctx *c, float *out, const float *in, const qcd_para
     if ((rc = check_params(c, p))) return rc;
     if ((rc = sap_prepare(c, p->block, p->subblock, p->sap_storage == QCD_F16))) return rc;
     const long V = c->lat.V;
-    const size_t bytes = 8 * 12 * V;  // one complex64 right-hand side
+    const size_t bytes = 8 * 12 * V * nrhs;
     const bool dev_in = is_device_ptr(in), dev_out = is_device_ptr(out);
     if ((dev_in && !aligned16(in)) || (dev_out && !aligned16(out)))
         return fail(c, QCD_ERR_ARG, "device spinors must be 16-byte aligned");
-    // io: v, x (internal, nrhs each), work (2 or 5 nrhs), staging (1); all right-hand sides go
-    // through one batched SAP application
+    // io: work (2 or 5 nrhs), and copies of the input or output where they are on the host, off a
+    // 32-byte boundary or overlapping
+    const bool cp_in = !dev_in || !aligned32(in) || overlap(in, bytes, out, bytes), cp_out = !dev_out || !aligned32(out);
     const int nw = sap_work_fields(p->block_solver);
-    if ((rc = ensure_io(c, ((2 + nw) * (size_t)nrhs + 1) * bytes))) return rc;
-    char *io = (char *)c->d_io;
-    float4 *v = (float4 *)io, *x = (float4 *)(io + nrhs * bytes), *work = (float4 *)(io + 2 * nrhs * bytes);
-    char *stage = io + (2 + nw) * nrhs * bytes;
-    if (dev_in) {
-        if ((rc = spinor32_to_internal(c, v, (const float2 *)in, nrhs))) return rc;
-    } else {
-        for (int k = 0; k < nrhs; k++) {
-            QCD_CUDA(c, cudaMemcpyAsync(stage, (const char *)in + k * bytes, bytes, cudaMemcpyHostToDevice, c->stream));
-            if ((rc = spinor32_to_internal(c, v + k * 6 * V, (const float2 *)stage, 1))) return rc;
-        }
-    }
+    if ((rc = ensure_io(c, (size_t)(nw + cp_in + cp_out) * bytes))) return rc;
+    float4 *work = (float4 *)c->d_io;
+    char *end = (char *)c->d_io + nw * bytes;
+    const float4 *v = cp_in ? (const float4 *)end : (const float4 *)in;
+    float4 *x = cp_out ? (float4 *)(end + (cp_in ? bytes : 0)) : (float4 *)out;
+    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(end, in, bytes, cudaMemcpyDefault, c->stream));
     if ((rc = sap_apply(c, x, v, work, p->omega, p->nsweep, p->nsap, nrhs, nullptr, p->block_solver))) return rc;
-    if (dev_out) {
-        if ((rc = spinor32_from_internal(c, (float2 *)out, x, nrhs))) return rc;
-    } else {
-        for (int k = 0; k < nrhs; k++) {
-            if ((rc = spinor32_from_internal(c, (float2 *)stage, x + k * 6 * V, 1))) return rc;
-            QCD_CUDA(c, cudaMemcpyAsync((char *)out + k * bytes, stage, bytes, cudaMemcpyDeviceToHost, c->stream));
-            QCD_CUDA(c, cudaStreamSynchronize(c->stream));
-        }
-    }
-    if (!dev_in) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, x, bytes, cudaMemcpyDefault, c->stream));
+    if (!dev_in || !dev_out) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     return QCD_OK;
 }
 
@@ -378,8 +367,11 @@ int qcd_solve(qcd_ctx *c, double *x, const double *b, const qcd_params *p, int n
     const bool dev_x = is_device_ptr(x), dev_b = is_device_ptr(b);
     if ((dev_x && !aligned16(x)) || (dev_b && !aligned16(b)))
         return fail(c, QCD_ERR_ARG, "device spinors must be 16-byte aligned");
+    // x and b are used where they are, or through copies as in the calls above
+    const bool cp_x = !dev_x || !aligned32(x);
+    const bool cp_b = !dev_b || !aligned32(b) || overlap(x, per * nrhs, b, per * nrhs);
     // right-hand sides per group: as asked, or as many as the free device memory holds (the
-    // solver's FP64 and FP32 vectors, the internal copies of x and b, host staging)
+    // solver's FP64 and FP32 vectors and the copies of x and b)
     int g = p->rhs_group > 0 ? std::min(p->rhs_group, nrhs) : nrhs;
     if (p->rhs_group == 0) {
         size_t fr = 0, tot = 0;
@@ -387,8 +379,8 @@ int qcd_solve(qcd_ctx *c, double *x, const double *b, const qcd_params *p, int n
         const size_t held = c->ws64_bytes + c->ws32_bytes + c->d_io_bytes;
         const size_t margin = (size_t)1 << 30;
         const size_t avail = fr + held > margin + tot / 50 ? fr + held - margin - tot / 50 : 0;
-        const size_t need = 16 * 12 * (size_t)V * 11 + 16 * 6 * (size_t)V * (10 + sap_work_fields(p->block_solver)) +
-                            per * (dev_x && dev_b ? 2 : 4);
+        const size_t need = 16 * 12 * (size_t)V * 9 + 16 * 6 * (size_t)V * (10 + sap_work_fields(p->block_solver)) +
+                            per * (cp_x + cp_b);
         g = (int)std::max<size_t>(1, std::min<size_t>((size_t)nrhs, avail / need));
     }
     // learned = 1 falls back to plain SAP when the last evaluation found the correction slower
@@ -404,27 +396,20 @@ int qcd_solve(qcd_ctx *c, double *x, const double *b, const qcd_params *p, int n
     for (int k0 = 0; k0 < nrhs; k0 += g) {
         const int n = std::min(g, nrhs - k0);
         const size_t bytes = per * n;
-        if ((rc = ensure_io(c, 4 * per * g))) return rc;
-        char *io = (char *)c->d_io;
-        double2 *xi = (double2 *)io, *bi = (double2 *)(io + bytes);
-        char *sx = io + 2 * bytes, *sb = io + 3 * bytes;
-        const char *bsrc = (const char *)b + per * k0, *xsrc = (const char *)x + per * k0;
-        if (!dev_b) {
-            QCD_CUDA(c, cudaMemcpyAsync(sb, bsrc, bytes, cudaMemcpyHostToDevice, c->stream));
-            bsrc = sb;
+        if (cp_x + cp_b && (rc = ensure_io(c, (cp_x + cp_b) * per * g))) return rc;
+        char *io = (char *)c->d_io, *xdst = (char *)x + per * k0;
+        const char *bsrc = (const char *)b + per * k0;
+        double2 *xi = cp_x ? (double2 *)io : (double2 *)xdst;
+        if (cp_x) QCD_CUDA(c, cudaMemcpyAsync(xi, xdst, bytes, cudaMemcpyDefault, c->stream));
+        if (cp_b) {
+            char *bi = io + (cp_x ? bytes : 0);
+            QCD_CUDA(c, cudaMemcpyAsync(bi, bsrc, bytes, cudaMemcpyDefault, c->stream));
+            bsrc = bi;
         }
-        if (!dev_x) {
-            QCD_CUDA(c, cudaMemcpyAsync(sx, xsrc, bytes, cudaMemcpyHostToDevice, c->stream));
-            xsrc = sx;
-        }
-        if ((rc = spinor64_to_internal(c, bi, (const double2 *)bsrc, n))) return rc;
-        if ((rc = spinor64_to_internal(c, xi, (const double2 *)xsrc, n))) return rc;
-        const int s = solve(c, xi, bi, &pe, n, &local);
+        const int s = solve(c, xi, (const double2 *)bsrc, &pe, n, &local);
         if (s == QCD_ERR_CUDA || s == QCD_ERR_OOM || s == QCD_ERR_STATE || s == QCD_ERR_ARG) return s;
         if (s != QCD_OK && (status == QCD_OK || s == QCD_ERR_BREAKDOWN)) status = s;
-        char *xdst = dev_x ? (char *)x + per * k0 : sx;
-        if ((rc = spinor64_from_internal(c, (double2 *)xdst, xi, n))) return rc;
-        if (!dev_x) QCD_CUDA(c, cudaMemcpyAsync((char *)x + per * k0, sx, bytes, cudaMemcpyDeviceToHost, c->stream));
+        if (cp_x) QCD_CUDA(c, cudaMemcpyAsync(xdst, xi, bytes, cudaMemcpyDefault, c->stream));
     }
     QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     if (c->prof.on) {
@@ -635,15 +620,16 @@ int qcd_learned_load(qcd_ctx *c, const char *path) {
     return qcd_learned_set_weights(c, w.data(), n);
 }
 
-// stage a complex64 [k][V][12] field (host or device) into the internal plane layout
-static int stage_in32(qcd_ctx *c, float4 *dst, const float *src, int k, char *scratch) {
-    const size_t bytes = 8 * 12 * (size_t)c->lat.V * k;
-    const void *s = src;
-    if (!is_device_ptr(src)) {
-        QCD_CUDA(c, cudaMemcpyAsync(scratch, src, bytes, cudaMemcpyHostToDevice, c->stream));
-        s = scratch;
+// a complex64 field as the kernels can read it: the caller's where it lies on the device on a
+// 32-byte boundary, else copied into scratch
+static int readable(qcd_ctx *c, const float *src, size_t bytes, char *scratch, const float4 **out) {
+    if (is_device_ptr(src) && aligned32(src)) {
+        *out = (const float4 *)src;
+        return QCD_OK;
     }
-    return spinor32_to_internal(c, dst, (const float2 *)s, k);
+    QCD_CUDA(c, cudaMemcpyAsync(scratch, src, bytes, cudaMemcpyDefault, c->stream));
+    *out = (const float4 *)scratch;
+    return QCD_OK;
 }
 
 int qcd_learned_apply(qcd_ctx *c, float *out, const float *in) {
@@ -652,14 +638,14 @@ int qcd_learned_apply(qcd_ctx *c, float *out, const float *in) {
     if (!c->net.ready) return fail(c, QCD_ERR_STATE, "qcd_learned_set_weights must be called first");
     if (!out || !in) return fail(c, QCD_ERR_ARG, "NULL argument");
     const size_t bytes = 8 * 12 * (size_t)c->lat.V;
-    if ((rc = ensure_io(c, 3 * bytes))) return rc;
+    if ((rc = ensure_io(c, 2 * bytes))) return rc;
     char *io = (char *)c->d_io;
-    float4 *x = (float4 *)io, *y = (float4 *)(io + bytes);
-    if ((rc = stage_in32(c, x, in, 1, io + 2 * bytes))) return rc;
+    const float4 *x = nullptr;
+    if ((rc = readable(c, in, bytes, io, &x))) return rc;
+    const bool cp_out = !is_device_ptr(out) || !aligned32(out);
+    float4 *y = cp_out ? (float4 *)(io + bytes) : (float4 *)out;
     if ((rc = learned_forward(c, y, x))) return rc;
-    const bool dev_out = is_device_ptr(out);
-    if ((rc = spinor32_from_internal(c, (float2 *)(dev_out ? (char *)out : io + 2 * bytes), y, 1))) return rc;
-    if (!dev_out) QCD_CUDA(c, cudaMemcpyAsync(out, io + 2 * bytes, bytes, cudaMemcpyDeviceToHost, c->stream));
+    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, y, bytes, cudaMemcpyDefault, c->stream));
     return learned_tc_status(c);  // synchronises
 }
 
@@ -669,16 +655,14 @@ int qcd_learned_loss_grad(qcd_ctx *c, const float *rho, const float *eps, double
     if (!c->net.ready) return fail(c, QCD_ERR_STATE, "qcd_learned_set_weights must be called first");
     if (!rho || !eps) return fail(c, QCD_ERR_ARG, "NULL argument");
     const size_t bytes = 8 * 12 * (size_t)c->lat.V;
-    if ((rc = ensure_io(c, 5 * bytes))) return rc;
+    if ((rc = ensure_io(c, 3 * bytes))) return rc;
     char *io = (char *)c->d_io;
-    float4 *r = (float4 *)io, *e4 = (float4 *)(io + bytes), *y = (float4 *)(io + 2 * bytes);
-    float2 *es = (float2 *)(io + 3 * bytes);
-    if ((rc = stage_in32(c, r, rho, 1, io + 4 * bytes))) return rc;
-    if ((rc = stage_in32(c, e4, eps, 1, io + 4 * bytes))) return rc;
-    if ((rc = plane_to_site(c, es, e4))) return rc;
+    const float4 *r = nullptr, *e = nullptr;
+    if ((rc = readable(c, rho, bytes, io, &r))) return rc;
+    if ((rc = readable(c, eps, bytes, io + bytes, &e))) return rc;
     if ((rc = learned_zero_grad(c))) return rc;
     double l = 0;
-    if ((rc = learned_loss_grad(c, r, es, &l, y))) return rc;
+    if ((rc = learned_loss_grad(c, r, (const float2 *)e, &l, (float4 *)(io + 2 * bytes)))) return rc;
     if (loss) *loss = l;
     if (grad)
         QCD_CUDA(c, cudaMemcpyAsync(grad, c->net.grad, sizeof(float2) * learned_weight_count(),
@@ -701,7 +685,7 @@ int qcd_learned_train(qcd_ctx *c, const float *sources, int npairs, const qcd_pa
     if ((rc = sap_prepare(c, pp.block, pp.subblock, pp.sap_storage == QCD_F16))) return rc;
     const long V = c->lat.V;
     const size_t f32 = 96 * (size_t)V, f64 = 192 * (size_t)V;
-    // pairs: rho (plane FP32) then eps (site FP32), per pair
+    // pairs: rho then eps (FP32), per pair
     const size_t need = 2 * f32 * (size_t)npairs;
     if (c->net.pairs_bytes < need) {
         dev_free(c, c->net.pairs);
@@ -712,33 +696,26 @@ int qcd_learned_train(qcd_ctx *c, const float *sources, int npairs, const qcd_pa
     }
     char *pairs = (char *)c->net.pairs;
     const int chunk = npairs < 16 ? npairs : 16;
-    // chunk buffers: staging, r, x, Dx, SAP work (2), FP64 rhs and solution
+    // chunk buffers: r, x, Dx, SAP work (2), FP64 rhs and solution
     void *tmpb = nullptr;
-    if ((rc = dev_alloc(c, &tmpb, (size_t)chunk * (6 * f32 + 2 * f64)))) return rc;
+    if ((rc = dev_alloc(c, &tmpb, (size_t)chunk * (5 * f32 + 2 * f64)))) return rc;
     struct Free {
         qcd_ctx *c;
         void *p;
         ~Free() { dev_free(c, p); }
     } guard{c, tmpb};
     char *tb = (char *)tmpb;
-    char *stg = tb;
-    float4 *r = (float4 *)(tb + chunk * f32), *x = (float4 *)(tb + 2 * chunk * f32);
-    float4 *dx = (float4 *)(tb + 3 * chunk * f32), *work = (float4 *)(tb + 4 * chunk * f32);
-    double2 *b64 = (double2 *)(tb + 6 * chunk * f32), *x64 = (double2 *)(tb + 6 * chunk * f32 + chunk * f64);
+    float4 *r = (float4 *)tb, *x = (float4 *)(tb + chunk * f32);
+    float4 *dx = (float4 *)(tb + 2 * chunk * f32), *work = (float4 *)(tb + 3 * chunk * f32);
+    double2 *b64 = (double2 *)(tb + 5 * chunk * f32), *x64 = (double2 *)(tb + 5 * chunk * f32 + chunk * f64);
     qcd_params ps = pp;
     ps.tol = 1e-9;
-    const bool dev_src = is_device_ptr(sources);
     for (int k0 = 0; k0 < npairs; k0 += chunk) {
         const int k = std::min(chunk, npairs - k0);
-        const float *src = sources + (size_t)k0 * 24 * V;
-        if (!dev_src) {
-            QCD_CUDA(c, cudaMemcpyAsync(stg, src, (size_t)k * f32, cudaMemcpyHostToDevice, c->stream));
-            src = (const float *)stg;
-        }
-        if ((rc = spinor32_to_internal(c, r, (const float2 *)src, k))) return rc;
+        QCD_CUDA(c, cudaMemcpyAsync(r, sources + (size_t)k0 * 24 * V, (size_t)k * f32, cudaMemcpyDefault, c->stream));
         if ((rc = sap_apply(c, x, r, work, pp.omega, pp.nsweep, pp.nsap, k))) return rc;
         if ((rc = dslash32(c, dx, x, k))) return rc;
-        if ((rc = sub_plane(c, dx, r, dx, k))) return rc;  // rho = r - D M_SAP r
+        if ((rc = sub_spinors(c, dx, r, dx, k))) return rc;  // rho = r - D M_SAP r
         for (int j = 0; j < k; j++)
             QCD_CUDA(c, cudaMemcpyAsync(pairs + (size_t)(k0 + j) * 2 * f32, (char *)dx + j * f32, f32,
                                         cudaMemcpyDeviceToDevice, c->stream));
@@ -751,7 +728,8 @@ int qcd_learned_train(qcd_ctx *c, const float *sources, int npairs, const qcd_pa
         if (s != QCD_OK) return s == QCD_ERR_NOCONV || s == QCD_ERR_BREAKDOWN ? fail(c, s, "training pairs: solve failed") : s;
         if ((rc = spinor64_to_32(c, x, x64, k))) return rc;
         for (int j = 0; j < k; j++)
-            if ((rc = plane_to_site(c, (float2 *)(pairs + (size_t)(k0 + j) * 2 * f32 + f32), x + j * 6 * V))) return rc;
+            QCD_CUDA(c, cudaMemcpyAsync(pairs + (size_t)(k0 + j) * 2 * f32 + f32, x + j * 6 * V, f32,
+                                        cudaMemcpyDeviceToDevice, c->stream));
     }
     // training
     float4 *ybuf = dx;
@@ -847,11 +825,7 @@ int qcd_bench_dslash(qcd_ctx *c, int prec, int nrhs, int iters) {
         QCD_CUDA(c, cudaMemsetAsync(c->bench_in, 0x3c, bytes, c->stream));
     }
     for (int i = 0; i < iters; i++) {
-        if (prec == QCD_F64) rc = dslash64(c, (double2 *)c->bench_out, (const double2 *)c->bench_in, nrhs);
-        else if (prec == QCD_F32X2) rc = dslash_x2(c, (double2 *)c->bench_out, (const float4 *)c->bench_in, nrhs);
-        else if (prec == QCD_F16) rc = dslash16(c, (float4 *)c->bench_out, (const float4 *)c->bench_in, nrhs);
-        else if (prec == QCD_F32_SU3) rc = dslash12(c, (float4 *)c->bench_out, (const float4 *)c->bench_in, nrhs);
-        else rc = dslash32(c, (float4 *)c->bench_out, (const float4 *)c->bench_in, nrhs);
+        rc = dslash(c, c->bench_out, c->bench_in, prec, nrhs);
         if (rc) return rc;
     }
     return QCD_OK;

@@ -10,7 +10,6 @@
 // threads are consecutive, so neighbour re-reads hit L1/L2 and the HBM traffic
 // stays close to one read of each field (768 B/site in FP32).
 #include <algorithm>
-#include <type_traits>
 
 #include "fields.cuh"
 #include "qcd_internal.h"
@@ -78,8 +77,8 @@ __global__ void __launch_bounds__(128, MINB) dslash_kernel(SP *__restrict__ out,
     const int rhs = (int)(blockIdx.x - sblk * nrhs);
     const long n = sblk * blockDim.x + threadIdx.x;
     if (n >= g.V) return;
-    constexpr int PLANES = sizeof(C) * 12 / sizeof(SP);
-    const SP *src = in + (long)rhs * PLANES * g.V;
+    constexpr int PARTS = sizeof(C) * 12 / sizeof(SP);
+    const SP *src = in + (long)rhs * PARTS * g.V;
     int x[4];
     site_coords(g, n, x);
     C acc[12];
@@ -89,25 +88,25 @@ __global__ void __launch_bounds__(128, MINB) dslash_kernel(SP *__restrict__ out,
     const R tsgn_f = (x[3] == g.L[3] - 1) ? (R)g.bc_t : (R)1;
     const R tsgn_b = (x[3] == 0) ? (R)g.bc_t : (R)1;
     // mu = 0
-    { long m = nbr_fwd<0>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, n, 0, u); hop_term<0, true>(psi, u, (R)1, acc); }
-    { long m = nbr_bwd<0>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, m, 0, u); hop_term<0, false>(psi, u, (R)1, acc); }
-    { long m = nbr_fwd<1>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, n, 1, u); hop_term<1, true>(psi, u, (R)1, acc); }
-    { long m = nbr_bwd<1>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, m, 1, u); hop_term<1, false>(psi, u, (R)1, acc); }
-    { long m = nbr_fwd<2>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, n, 2, u); hop_term<2, true>(psi, u, (R)1, acc); }
-    { long m = nbr_bwd<2>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, m, 2, u); hop_term<2, false>(psi, u, (R)1, acc); }
-    { long m = nbr_fwd<3>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, n, 3, u); hop_term<3, true>(psi, u, tsgn_f, acc); }
-    { long m = nbr_bwd<3>(g, n, x); load_spinor(src, g.V, m, psi); load_link(U, g.V, m, 3, u); hop_term<3, false>(psi, u, tsgn_b, acc); }
+    { long m = nbr_fwd<0>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, n, 0, u); hop_term<0, true>(psi, u, (R)1, acc); }
+    { long m = nbr_bwd<0>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, m, 0, u); hop_term<0, false>(psi, u, (R)1, acc); }
+    { long m = nbr_fwd<1>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, n, 1, u); hop_term<1, true>(psi, u, (R)1, acc); }
+    { long m = nbr_bwd<1>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, m, 1, u); hop_term<1, false>(psi, u, (R)1, acc); }
+    { long m = nbr_fwd<2>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, n, 2, u); hop_term<2, true>(psi, u, (R)1, acc); }
+    { long m = nbr_bwd<2>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, m, 2, u); hop_term<2, false>(psi, u, (R)1, acc); }
+    { long m = nbr_fwd<3>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, n, 3, u); hop_term<3, true>(psi, u, tsgn_f, acc); }
+    { long m = nbr_bwd<3>(g, n, x); load_spinor(src, m, psi); load_link(U, g.V, m, 3, u); hop_term<3, false>(psi, u, tsgn_b, acc); }
     R f[72];
     load_clover(F, g.V, n, f);
     C fa[12];
     clover_mul<R, C>(f, acc, fa);
-    load_spinor(src, g.V, n, psi);
+    load_spinor(src, n, psi);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
         psi[k].x = fma(-kappa, fa[k].x, psi[k].x);
         psi[k].y = fma(-kappa, fa[k].y, psi[k].y);
     }
-    store_spinor(out + (long)rhs * PLANES * g.V, g.V, n, psi);
+    store_spinor(out + (long)rhs * PARTS * g.V, n, psi);
 }
 
 template <int NR, int MODE, typename R, typename SP, typename LK, typename CL>
@@ -175,8 +174,8 @@ __device__ __forceinline__ void dslash_site(SP *__restrict__ out, const SP *__re
                                             const Geo &g, long n, int r0, const bool act[NR],
                                             const SP *__restrict__ other, float part[NR][3]) {
     using C = typename CT<R>::C;
-    constexpr int PLANES = sizeof(C) * 12 / sizeof(SP);
-    const SP *src = in + (long)r0 * PLANES * g.V;
+    constexpr int PARTS = sizeof(C) * 12 / sizeof(SP);
+    const SP *src = in + (long)r0 * PARTS * g.V;
     bool any = false;
 #pragma unroll
     for (int r = 0; r < NR; r++) any |= act[r];
@@ -196,7 +195,7 @@ __device__ __forceinline__ void dslash_site(SP *__restrict__ out, const SP *__re
         const long m = FWD ? nbr_fwd<MU>(g, n, x) : nbr_bwd<MU>(g, n, x);               \
         load_link(U, g.V, FWD ? n : m, MU, u);                                           \
         _Pragma("unroll") for (int r = 0; r < NR; r++) if (act[r]) {                     \
-            load_spinor(src + (long)r * PLANES * g.V, g.V, m, psi);                      \
+            load_spinor(src + (long)r * PARTS * g.V, m, psi);                      \
             hop_term<MU, FWD>(psi, u, SGN, acc[r]);                                      \
         }                                                                               \
     }
@@ -216,16 +215,16 @@ __device__ __forceinline__ void dslash_site(SP *__restrict__ out, const SP *__re
         if (act[r]) {
             C fa[12];
             clover_mul<R, C>(f, acc[r], fa);
-            load_spinor(src + (long)r * PLANES * g.V, g.V, n, psi);
+            load_spinor(src + (long)r * PARTS * g.V, n, psi);
 #pragma unroll
             for (int k = 0; k < 12; k++) {
                 psi[k].x = fma(-kappa, fa[k].x, psi[k].x);
                 psi[k].y = fma(-kappa, fa[k].y, psi[k].y);
             }
-            store_spinor(out + (long)(r0 + r) * PLANES * g.V, g.V, n, psi);
+            store_spinor(out + (long)(r0 + r) * PARTS * g.V, n, psi);
             if constexpr (MODE != 0) {
                 C o[12];
-                load_spinor(other + (long)(r0 + r) * PLANES * g.V, g.V, n, o);
+                load_spinor(other + (long)(r0 + r) * PARTS * g.V, n, o);
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
                     const C a = MODE == 1 ? o[k] : psi[k], b = MODE == 1 ? psi[k] : o[k];
@@ -271,26 +270,15 @@ static Geo geo_of(const qcd_ctx *c) {
     return g;
 }
 
-// SP: the plane layout's element (float4, double2; the solver's vectors) or the caller's canonical
-// layout (Site32, Site64).  In the canonical layout a lane reads its site as whole 32-byte sectors,
-// fewer and wider loads than the planes', so each form runs best with fewer blocks and more
-// registers than on planes.  Measured, canonical (us; CTAs of 128 threads per SM): FP32, 48^3x96,
-// one right-hand side: 1567 / 1468 / 1405 / 1446 / 1491 with 7 / 6 / 5 / 4 / 3; 24^3x48, two-row links,
-// 12 right-hand sides: 673 / 656 / 625 / 708 with 6 / 5 / 4 / 3; FP16 fields, 4: 211 / 212 / 208 / 229.
-template <typename SP> constexpr int blocks_per_sm(int planes, int canonical) {
-    return std::is_same<SP, Site32>::value ? canonical : planes;
-}
-
-template <typename SP> static int launch64(qcd_ctx *c, SP *out, const SP *in, int nrhs) {
+int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs) {
     Geo g = geo_of(c);
     dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH64, &ev);
-    dslash_kernel<3, double, SP, double2, double2><<<grid, 128, 0, c->stream>>>(out, in, c->U64, c->F64, c->kappa, g,
-                                                                                nrhs);
+    dslash_kernel<3, double, double2, double2, double2><<<grid, 128, 0, c->stream>>>(out, in, c->U64, c->F64,
+                                                                                     c->kappa, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
 }
-int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs) { return launch64(c, out, in, nrhs); }
 
 // the links as their first two rows (Table 1's SU(3) 12-real form), made on first use after each
 // field change
@@ -323,29 +311,27 @@ static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, co
     if (rc) return rc;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
-    dslash_kernel_nr<7, 1, float, float4, float4, float4, MODE><<<dim3(nblk * nrhs), 128, 0, c->stream>>>(
+    dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE><<<dim3(nblk * nrhs), 128, 0, c->stream>>>(
         out, in, c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate);
     rc = prof_end(c, QCD_K_DSLASH32, ev);
     if (rc || !MODE) return rc;
     return reduce_tiles(c, part, nblk, nrhs, red);
 }
 
-template <typename SP> static int launch32(qcd_ctx *c, SP *out, const SP *in, int nrhs) {
+int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     Geo g = geo_of(c);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<blocks_per_sm<SP>(7, 5), float, SP, float2, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
+        dslash_kernel<5, float, float4, float2, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
             out, in, c->U32, c->F32, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * ((nrhs + 1) / 2)));
-        dslash_kernel_nr<4, 2, float, SP, float2, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U32, c->F32,
+        dslash_kernel_nr<4, 2, float, float4, float2, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U32, c->F32,
                                                                                  (float)c->kappa, g, nrhs);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
-int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) { return launch32(c, out, in, nrhs); }
-
 int dslash32_dot(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, int mode, double *red,
                  const BicgScalars *gate) {
     if (mode == 1) return dslash32_tile<1>(c, out, in, nrhs, other, red, gate);
@@ -353,7 +339,7 @@ int dslash32_dot(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const floa
     return dslash32_tile<0>(c, out, in, nrhs, nullptr, nullptr, gate);
 }
 
-template <typename SP> static int launch16(qcd_ctx *c, SP *out, const SP *in, int nrhs) {
+int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     Geo g = geo_of(c);
     if (!c->U16) {
         int rc = dev_alloc(c, (void **)&c->U16, sizeof(__half2) * 36 * g.V);
@@ -368,49 +354,39 @@ template <typename SP> static int launch16(qcd_ctx *c, SP *out, const SP *in, in
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<blocks_per_sm<SP>(7, 4), float, SP, __half2, uint2><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
+        dslash_kernel<4, float, float4, __half2, uint2><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
             out, in, c->U16, c->F16, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
-        dslash_kernel_nr<blocks_per_sm<SP>(7, 4), 1, float, SP, __half2, uint2><<<grid, 128, 0, c->stream>>>(out, in, c->U16, c->F16,
+        dslash_kernel_nr<4, 1, float, float4, __half2, uint2><<<grid, 128, 0, c->stream>>>(out, in, c->U16, c->F16,
                                                                                      (float)c->kappa, g, nrhs);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
 
-int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) { return launch16(c, out, in, nrhs); }
-
-template <typename SP> static int launch12(qcd_ctx *c, SP *out, const SP *in, int nrhs) {
+int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     Geo g = geo_of(c);
     if (int rc = ensure_u12(c, g)) return rc;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<blocks_per_sm<SP>(7, 4), float, SP, float4, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
+        dslash_kernel<4, float, float4, float4, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
             out, in, c->U12, c->F32, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
-        dslash_kernel_nr<blocks_per_sm<SP>(7, 4), 1, float, SP, float4, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U12, c->F32,
+        dslash_kernel_nr<4, 1, float, float4, float4, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U12, c->F32,
                                                                                      (float)c->kappa, g, nrhs);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
 
-int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) { return launch12(c, out, in, nrhs); }
-
-// D straight from the caller's input to the caller's output.  The conversions to and from the plane
-// layout that this replaces moved 384 bytes per site and right-hand side in FP32, twice what D's own
-// spinors need: 48^3x96, one right-hand side 2035 -> 1405 us; 24^3x48, 12 right-hand sides 1200 -> 673 us;
-// 8^3x16, where three launches became one, 14.3 -> 6.2 us.
-int dslash_canonical(qcd_ctx *c, void *out, const void *in, int prec, int nrhs) {
-    Site32 *o = (Site32 *)out;
-    const Site32 *i = (const Site32 *)in;
+int dslash(qcd_ctx *c, void *out, const void *in, int prec, int nrhs) {
     switch (prec) {
-        case QCD_F64: return launch64(c, (Site64 *)out, (const Site64 *)in, nrhs);
-        case QCD_F32: return launch32(c, o, i, nrhs);
-        case QCD_F16: return launch16(c, o, i, nrhs);
-        case QCD_F32_SU3: return launch12(c, o, i, nrhs);
-        default: return dslash_x2_canonical(c, (double2 *)out, (const float2 *)in, nrhs);
+        case QCD_F64: return dslash64(c, (double2 *)out, (const double2 *)in, nrhs);
+        case QCD_F32: return dslash32(c, (float4 *)out, (const float4 *)in, nrhs);
+        case QCD_F16: return dslash16(c, (float4 *)out, (const float4 *)in, nrhs);
+        case QCD_F32_SU3: return dslash12(c, (float4 *)out, (const float4 *)in, nrhs);
+        default: return dslash_x2(c, (double2 *)out, (const float4 *)in, nrhs);
     }
 }
 

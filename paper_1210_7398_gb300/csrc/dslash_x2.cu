@@ -12,8 +12,7 @@
 // 1e-13 of the FP64 D in norm, and all of it runs on the FP32 pipe as packed FP32x2 instructions
 // (real and imaginary part in one).  The FP64 output is formed once per component at the end.
 //
-// Layout: input FP32 spinors [nrhs][6][V] float4, output FP64 [nrhs][12][V] double2 (the internal
-// layouts); links [4][9][V] and clover [36][V] as float4 (hi of two reals, lo of the same two), made
+// Layout: input FP32 spinors [nrhs][V][6] float4, output FP64 [nrhs][V][12] double2; links [4][9][V] and clover [36][V] as float4 (hi of two reals, lo of the same two), made
 // from the FP64 fields on first use after each field change.  One thread per (site, right-hand
 // side), the right-hand side fastest over the grid as in the other D kernels.
 #include "fields.cuh"
@@ -147,11 +146,11 @@ __device__ __forceinline__ void reconstruct_x2(int a, const CX &w0, const CX &w1
 
 // one hop term: (1 - gamma_mu) U_mu(n) psi(n+mu) forward, (1 + gamma_mu) U_mu(n-mu)^dag psi(n-mu)
 // backward; ulink is the site whose link is used
-template <int MU, bool FWD, typename SP>
-__device__ __forceinline__ void hop_x2(const SP *__restrict__ src, const float4 *__restrict__ Ux2, long V,
+template <int MU, bool FWD>
+__device__ __forceinline__ void hop_x2(const float4 *__restrict__ src, const float4 *__restrict__ Ux2, long V,
                                        long nb, long ulink, float sgn, CX acc[12]) {
     float2 p[12];
-    load_spinor(src, V, nb, p);
+    load_spinor(src, nb, p);
     CX h[6];
     project_x2<MU, FWD>(p, sgn, h);
     float2 hr[6], hlr[6];
@@ -218,8 +217,8 @@ __device__ __forceinline__ void herm6_x2(const float4 *__restrict__ F, long V, c
 
 __device__ __forceinline__ double to_f64(float h, float l) { return (double)h + (double)l; }
 
-template <int MINB, typename SP, typename SO>
-__global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(SO *__restrict__ out, const SP *__restrict__ in,
+template <int MINB>
+__global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restrict__ out, const float4 *__restrict__ in,
                                                           const float4 *__restrict__ Ux2,
                                                           const float4 *__restrict__ Fx2, float kh, float kl,
                                                           Geo g, int nrhs) {
@@ -231,7 +230,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(SO *__restrict__ o
     const long n = sblk * blockDim.x + threadIdx.x;
     if (n >= g.V) return;
     const long V = g.V;
-    const SP *src = in + (long)rhs * 6 * V;
+    const float4 *src = in + (long)rhs * 6 * V;
     int x[4];
     site_coords(g, n, x);
     CX acc[12];
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(SO *__restrict__ o
     herm6_x2(Fx2 + n, V, c0, e0);
     herm6_x2(Fx2 + 18 * V + n, V, c1, e1);
     float2 psi[12];
-    load_spinor(src, V, n, psi);
+    load_spinor(src, n, psi);
     double2 res[12];
     const float2 kH = splat(kh), kL = splat(kl);
 #pragma unroll
@@ -278,7 +277,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(SO *__restrict__ o
         const float2 lo = sub2(e, add2(E, cr));
         res[k] = make_double2(to_f64(s.x, lo.x), to_f64(s.y, lo.y));
     }
-    store_spinor(out + (long)rhs * 12 * V, V, n, res);
+    store_spinor(out + (long)rhs * 12 * V, n, res);
 }
 
 // hi + lo split of FP64 values: hi = fl32(v), lo = fl32(v - hi); |v - hi - lo| <= 2^-48 |v|
@@ -299,7 +298,7 @@ __global__ void k_fields_to_x2(float4 *__restrict__ Ux2, float4 *__restrict__ Fx
 
 }  // namespace
 
-template <typename SO, typename SP> static int launch_x2(qcd_ctx *c, SO *out, const SP *in, int nrhs) {
+int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) {
     Geo g;
     for (int m = 0; m < 4; m++) g.L[m] = c->lat.L[m];
     g.V = c->lat.V;
@@ -321,14 +320,9 @@ template <typename SO, typename SP> static int launch_x2(qcd_ctx *c, SO *out, co
     // four CTAs of 128 threads per SM (128 registers, some spilled): the instruction fetch that the
     // long unrolled body stalls on is hidden by more warps.  24^3x48, 4 right-hand sides: 1332 / 1241 /
     // 1199 / 2131 us with 2 / 3 / 4 / 5
-    dslash_x2_kernel<4, SP, SO><<<dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, c->stream>>>(out, in, c->Ux2, c->Fx2,
+    dslash_x2_kernel<4><<<dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, c->stream>>>(out, in, c->Ux2, c->Fx2,
                                                                                            kh, kl, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
-}
-
-int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) { return launch_x2(c, out, in, nrhs); }
-int dslash_x2_canonical(qcd_ctx *c, double2 *out, const float2 *in, int nrhs) {
-    return launch_x2(c, (Site64 *)out, (const Site32 *)in, nrhs);
 }
 
 }  // namespace qcd

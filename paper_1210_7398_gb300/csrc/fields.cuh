@@ -50,44 +50,11 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(
 
 // ---- loads / stores in the internal layouts ---------------------------------
 
-__device__ __forceinline__ void load_spinor(const float4 *__restrict__ p, long V, long n, float2 s[12]) {
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        float4 v = __ldg(p + k * V + n);
-        s[2 * k] = make_float2(v.x, v.y);
-        s[2 * k + 1] = make_float2(v.z, v.w);
-    }
-}
-__device__ __forceinline__ void load_spinor(const double2 *__restrict__ p, long V, long n, double2 s[12]) {
-#pragma unroll
-    for (int k = 0; k < 12; k++) s[k] = __ldg(p + k * V + n);
-}
-// coherent loads (data written earlier by the same kernel)
-__device__ __forceinline__ void load_spinor_rw(const float4 *p, long V, long n, float2 s[12]) {
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        float4 v = p[k * V + n];
-        s[2 * k] = make_float2(v.x, v.y);
-        s[2 * k + 1] = make_float2(v.z, v.w);
-    }
-}
-__device__ __forceinline__ void store_spinor(float4 *p, long V, long n, const float2 s[12]) {
-#pragma unroll
-    for (int k = 0; k < 6; k++) p[k * V + n] = make_float4(s[2 * k].x, s[2 * k].y, s[2 * k + 1].x, s[2 * k + 1].y);
-}
-__device__ __forceinline__ void store_spinor(double2 *p, long V, long n, const double2 s[12]) {
-#pragma unroll
-    for (int k = 0; k < 12; k++) p[k * V + n] = s[k];
-}
-
-// Spinors in the caller's canonical layout [rhs][V][12] complex: one site's components are
-// contiguous (96 or 192 bytes), read and written as 32-byte vectors (the base 32-byte aligned).
-// The element types have the size of the plane layouts' (16 bytes), so a right-hand side's offset is
-// counted alike in both.
-struct alignas(16) Site32 { float2 c[2]; };
-struct alignas(16) Site64 { double2 c; };
-__device__ __forceinline__ void load_spinor(const Site32 *__restrict__ p, long, long n, float2 s[12]) {
-    const Site32 *q = p + 6 * n;
+// Spinors lie site by site, [rhs][V][12] complex (the caller's layout): one site's 96 (FP32) or 192
+// (FP64) bytes are read and written as 32-byte vectors, whole sectors for any set of sites a warp
+// takes, in half the instructions of 16-byte accesses.  Every spinor base is 32-byte aligned.
+__device__ __forceinline__ void load_spinor(const float4 *__restrict__ p, long n, float2 s[12]) {
+    const float4 *q = p + 6 * n;
 #pragma unroll
     for (int k = 0; k < 3; k++)
         asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -95,8 +62,27 @@ __device__ __forceinline__ void load_spinor(const Site32 *__restrict__ p, long, 
               "=f"(s[4 * k + 2].y), "=f"(s[4 * k + 3].x), "=f"(s[4 * k + 3].y)
             : "l"(q + 2 * k));
 }
-__device__ __forceinline__ void store_spinor(Site32 *p, long, long n, const float2 s[12]) {
-    Site32 *q = p + 6 * n;
+__device__ __forceinline__ void load_spinor(const double2 *__restrict__ p, long n, double2 s[12]) {
+    const double2 *q = p + 12 * n;
+#pragma unroll
+    for (int k = 0; k < 6; k++)
+        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
+            : "=d"(s[2 * k].x), "=d"(s[2 * k].y), "=d"(s[2 * k + 1].x), "=d"(s[2 * k + 1].y)
+            : "l"(q + 2 * k));
+}
+// coherent loads (data written earlier by the same kernel)
+__device__ __forceinline__ void load_spinor_rw(const float4 *p, long n, float2 s[12]) {
+    const float4 *q = p + 6 * n;
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(s[4 * k].x), "=f"(s[4 * k].y), "=f"(s[4 * k + 1].x), "=f"(s[4 * k + 1].y),
+                       "=f"(s[4 * k + 2].x), "=f"(s[4 * k + 2].y), "=f"(s[4 * k + 3].x), "=f"(s[4 * k + 3].y)
+                     : "l"(q + 2 * k)
+                     : "memory");
+}
+__device__ __forceinline__ void store_spinor(float4 *p, long n, const float2 s[12]) {
+    float4 *q = p + 6 * n;
 #pragma unroll
     for (int k = 0; k < 3; k++)
         asm volatile("st.global.v8.f32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"f"(s[4 * k].x), "f"(s[4 * k].y),
@@ -104,16 +90,8 @@ __device__ __forceinline__ void store_spinor(Site32 *p, long, long n, const floa
                      "f"(s[4 * k + 3].x), "f"(s[4 * k + 3].y), "l"(q + 2 * k)
                      : "memory");
 }
-__device__ __forceinline__ void load_spinor(const Site64 *__restrict__ p, long, long n, double2 s[12]) {
-    const Site64 *q = p + 12 * n;
-#pragma unroll
-    for (int k = 0; k < 6; k++)
-        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-            : "=d"(s[2 * k].x), "=d"(s[2 * k].y), "=d"(s[2 * k + 1].x), "=d"(s[2 * k + 1].y)
-            : "l"(q + 2 * k));
-}
-__device__ __forceinline__ void store_spinor(Site64 *p, long, long n, const double2 s[12]) {
-    Site64 *q = p + 12 * n;
+__device__ __forceinline__ void store_spinor(double2 *p, long n, const double2 s[12]) {
+    double2 *q = p + 12 * n;
 #pragma unroll
     for (int k = 0; k < 6; k++)
         asm volatile("st.global.v4.f64 [%4], {%0,%1,%2,%3};" ::"d"(s[2 * k].x), "d"(s[2 * k].y), "d"(s[2 * k + 1].x),

@@ -27,24 +27,17 @@ namespace qcd {
 namespace {
 
 // activation formats
-enum { PLANE32 = 0, SITE16 = 1, SITE32 = 2 };
+enum { SITE16 = 1, SITE32 = 2 };
 
 template <int FMT> __device__ __forceinline__ float2 act_ld(const void *base, long V, int ch, long n, int k) {
-    if constexpr (FMT == PLANE32) {
-        const float4 *p = static_cast<const float4 *>(base) + (long)ch * 6 * V + (long)(k >> 1) * V + n;
-        const float4 v = *p;
-        return (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-    } else if constexpr (FMT == SITE16) {
+    if constexpr (FMT == SITE16) {
         return __bfloat1622float2(static_cast<const __nv_bfloat162 *>(base)[((long)ch * V + n) * 12 + k]);
     } else {
         return static_cast<const float2 *>(base)[((long)ch * V + n) * 12 + k];
     }
 }
 template <int FMT> __device__ __forceinline__ void act_st(void *base, long V, int ch, long n, int k, float2 v) {
-    if constexpr (FMT == PLANE32) {
-        float2 *p = reinterpret_cast<float2 *>(static_cast<float4 *>(base) + (long)ch * 6 * V + (long)(k >> 1) * V + n);
-        p[k & 1] = v;
-    } else if constexpr (FMT == SITE16) {
+    if constexpr (FMT == SITE16) {
         static_cast<__nv_bfloat162 *>(base)[((long)ch * V + n) * 12 + k] = __float22bfloat162_rn(v);
     } else {
         static_cast<float2 *>(base)[((long)ch * V + n) * 12 + k] = v;
@@ -204,27 +197,18 @@ __device__ __forceinline__ void layer_issue(unsigned char *smem, const int *nbt,
     float2 *L = reinterpret_cast<float2 *>(X + S::x_bytes);
     __nv_bfloat16 *B = reinterpret_cast<__nv_bfloat16 *>(X + S::x_bytes + S::l_bytes);
     const int *nb = nbt + d * kLayerSites;
-    if constexpr (FIN == PLANE32) {
-        static_assert(CIN == 1, "plane layout holds one channel");
-        for (int i = tid; i < kLayerSites * 6; i += nth) {
-            const int st = i % kLayerSites, p = i / kLayerSites;
-            const int m = nb[st];
-            cp_async16z(X + st * XS + p * 16, static_cast<const float4 *>(x) + (long)p * V + (m < 0 ? 0 : m), m >= 0);
-        }
-    } else {
-        // thread -> (site, 16-byte chunk) fixed, channels strided: no index arithmetic in the loop
-        constexpr int CH16 = 12 * S::XC / 16;  // 16-byte chunks per site and channel
-        constexpr int PAIRS = kLayerSites * CH16;
-        static_assert(kLayerWarps * 32 % PAIRS == 0 || PAIRS % (kLayerWarps * 32) == 0, "even split");
-        for (int pr = tid; pr < PAIRS; pr += nth) {
-            const int st = pr / CH16, k = pr - st * CH16;
-            const int m = nb[st];
-            const unsigned char *src = static_cast<const unsigned char *>(x) + ((long)(m < 0 ? 0 : m) * 12) * S::XC + k * 16;
-            unsigned char *dst = X + st * XS + k * 16;
-            const long sstride = (long)V * 12 * S::XC;
+    // thread -> (site, 16-byte chunk) fixed, channels strided: no index arithmetic in the loop
+    constexpr int CH16 = 12 * S::XC / 16;  // 16-byte chunks per site and channel
+    constexpr int PAIRS = kLayerSites * CH16;
+    static_assert(kLayerWarps * 32 % PAIRS == 0 || PAIRS % (kLayerWarps * 32) == 0, "even split");
+    for (int pr = tid; pr < PAIRS; pr += nth) {
+        const int st = pr / CH16, k = pr - st * CH16;
+        const int m = nb[st];
+        const unsigned char *src = static_cast<const unsigned char *>(x) + ((long)(m < 0 ? 0 : m) * 12) * S::XC + k * 16;
+        unsigned char *dst = X + st * XS + k * 16;
+        const long sstride = (long)V * 12 * S::XC;
 #pragma unroll
-            for (int ch = 0; ch < CIN; ch++) cp_async16z(dst + ch * CH16 * 16, src + ch * sstride, m >= 0);
-        }
+        for (int ch = 0; ch < CIN; ch++) cp_async16z(dst + ch * CH16 * 16, src + ch * sstride, m >= 0);
     }
     if (d > 0) {
         const int mu = (d - 1) >> 1;
@@ -614,17 +598,17 @@ __global__ void k_wgrad_finish(float2 *__restrict__ grad, const float *__restric
     grad[i].y += 2.f * (ri - ir);
 }
 
-// r = a - b (plane layout FP32, 6 float4 per site); r may be b (each element is read and
+// r = a - b (FP32, 6 float4 per site); r may be b (each element is read and
 // written by one thread)
-__global__ void k_sub_plane(float4 *r, const float4 *a, const float4 *b, long n,
+__global__ void k_sub_spinors(float4 *r, const float4 *a, const float4 *b, long n,
                             const BicgScalars *__restrict__ gate = nullptr) {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= n || (gate && !gate->active)) return;
     const float4 x = a[i], y = b[i];
     r[i] = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
 }
-// x += y (plane layout FP32)
-__global__ void k_add_plane(float4 *__restrict__ x, const float4 *__restrict__ y, long n,
+// x += y (FP32)
+__global__ void k_add_spinors(float4 *__restrict__ x, const float4 *__restrict__ y, long n,
                             const BicgScalars *__restrict__ gate = nullptr) {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= n || (gate && !gate->active)) return;
@@ -632,8 +616,8 @@ __global__ void k_add_plane(float4 *__restrict__ x, const float4 *__restrict__ y
     x[i] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
-// loss += |y - eps|^2 / en2 over one pair; g = (y - eps) / en2 (site layout, FP32)
-__global__ void k_loss(float2 *__restrict__ g, double *__restrict__ loss, const float4 *__restrict__ y,
+// loss += |y - eps|^2 / en2 over one pair; g = (y - eps) / en2 (FP32)
+__global__ void k_loss(float2 *__restrict__ g, double *__restrict__ loss, const float2 *__restrict__ y,
                        const float2 *__restrict__ eps, const double *__restrict__ en2, long V) {
     __shared__ double sh[256];
     const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -642,8 +626,7 @@ __global__ void k_loss(float2 *__restrict__ g, double *__restrict__ loss, const 
         const float inv = (float)(1.0 / *en2);
 #pragma unroll
         for (int k = 0; k < 12; k++) {
-            const float4 v = y[(long)(k >> 1) * V + n];
-            const float2 yk = (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+            const float2 yk = y[n * 12 + k];
             const float2 e = eps[n * 12 + k];
             const float2 r = make_float2(yk.x - e.x, yk.y - e.y);
             acc += ((double)r.x * r.x + (double)r.y * r.y) * inv;
@@ -659,7 +642,7 @@ __global__ void k_loss(float2 *__restrict__ g, double *__restrict__ loss, const 
     if (threadIdx.x == 0) atomicAdd(loss, sh[0]);
 }
 
-// |eps|^2 of one pair (site layout)
+// |eps|^2 of one pair 
 __global__ void k_norm2(double *__restrict__ out, const float2 *__restrict__ e, long n) {
     __shared__ double sh[256];
     double acc = 0;
@@ -683,18 +666,6 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
     m[i] = b1 * m[i] + (1.f - b1) * gi;
     v[i] = b2 * v[i] + (1.f - b2) * gi * gi;
     w[i] -= lr * (m[i] / c1) / (sqrtf(v[i] / c2) + eps);
-}
-
-// plane-layout FP32 spinor -> site layout FP32
-__global__ void k_plane_to_site(float2 *__restrict__ out, const float4 *__restrict__ in, long V) {
-    const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (n >= V) return;
-#pragma unroll
-    for (int p = 0; p < 6; p++) {
-        const float4 v = in[(long)p * V + n];
-        out[n * 12 + 2 * p] = make_float2(v.x, v.y);
-        out[n * 12 + 2 * p + 1] = make_float2(v.z, v.w);
-    }
 }
 
 Geo geo(const qcd_ctx *c) {
@@ -864,19 +835,19 @@ int learned_get_weights(qcd_ctx *c, float2 *w_host) {
     return QCD_OK;
 }
 
-// y = N(x) for one right-hand side in the FP32 plane layout (layers 1 -> 8 -> 8 -> 1); with
+// y = N(x) for one right-hand side in FP32 (layers 1 -> 8 -> 8 -> 1); with
 // gate, every kernel returns at once while that right-hand side is inactive
 int learned_forward(qcd_ctx *c, float4 *y, const float4 *x, const BicgScalars *gate) {
     Learned &L = c->net;
     if (!L.ready) return fail(c, QCD_ERR_STATE, "no learned weights set");
     int rc = ensure_net(c);
     if (rc) return rc;
-    if ((rc = launch_layer<1, 8, PLANE32, SITE16>(c, L.a1, x, L.B + layer_boff(0, false), gate))) return rc;
+    if ((rc = launch_layer<1, 8, SITE32, SITE16>(c, L.a1, x, L.B + layer_boff(0, false), gate))) return rc;
     if ((rc = learned_layer_tc(c, L.a2, L.a1, L.B + layer_boff(1, false), false, gate))) return rc;
-    return launch_layer_wfirst<8, SITE16, PLANE32>(c, y, L.a2, L.B + layer_boff(2, false), gate);
+    return launch_layer_wfirst<8, SITE16, SITE32>(c, y, L.a2, L.B + layer_boff(2, false), gate);
 }
 
-// loss of one pair (rho: plane layout FP32, eps: site layout FP32) and, with accumulate,
+// loss of one pair (FP32) and, with accumulate,
 // its gradient added to the running sum in L.grad (real pairs, 2 (Re, Im) of dL/dW*)
 int learned_loss_grad(qcd_ctx *c, const float4 *rho, const float2 *eps, double *loss_out, float4 *ybuf) {
     Learned &L = c->net;
@@ -889,7 +860,7 @@ int learned_loss_grad(qcd_ctx *c, const float4 *rho, const float2 *eps, double *
     k_norm2<<<256, 256, 0, c->stream>>>(L.scal + 1, eps, 12 * V);
     if ((rc = prof_end(c, QCD_K_LEARNED, ev))) return rc;
     prof_begin(c, QCD_K_LEARNED, &ev);
-    k_loss<<<(unsigned)((V + 255) / 256), 256, 0, c->stream>>>(L.g3, L.scal, ybuf, eps, L.scal + 1, V);
+    k_loss<<<(unsigned)((V + 255) / 256), 256, 0, c->stream>>>(L.g3, L.scal, (const float2 *)ybuf, eps, L.scal + 1, V);
     if ((rc = prof_end(c, QCD_K_LEARNED, ev))) return rc;
     // backward: layer 3 (8 -> 1), layer 2 (8 -> 8), layer 1 (1 -> 8)
     auto wgrad_layer = [&](int l, auto launcher) -> int {
@@ -907,7 +878,7 @@ int learned_loss_grad(qcd_ctx *c, const float4 *rho, const float2 *eps, double *
     if ((rc = launch_layer<1, 8, SITE32, SITE32>(c, L.g2, L.g3, L.B + layer_boff(2, true)))) return rc;
     if ((rc = wgrad_layer(1, [&]() { return launch_wgrad<8, 8, SITE16>(c, L.P, L.a1, L.g2); }))) return rc;
     if ((rc = learned_layer_tc(c, L.g1, L.g2, L.B + layer_boff(1, true), true))) return rc;
-    if ((rc = wgrad_layer(0, [&]() { return launch_wgrad<1, 8, PLANE32>(c, L.P, rho, L.g1); }))) return rc;
+    if ((rc = wgrad_layer(0, [&]() { return launch_wgrad<1, 8, SITE32>(c, L.P, rho, L.g1); }))) return rc;
     if (loss_out) {
         double h = 0;
         QCD_CUDA(c, cudaMemcpyAsync(&h, L.scal, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -937,7 +908,7 @@ int learned_zero_grad(qcd_ctx *c) {
     return QCD_OK;
 }
 
-// out = out + N(v - D out) for nrhs right-hand sides (plane layout): the learned correction
+// out = out + N(v - D out) for nrhs right-hand sides: the learned correction
 // applied after SAP; w1, w2: two scratch spinors of nrhs fields each
 int learned_correct(qcd_ctx *c, float4 *out, const float4 *v, float4 *w1, float4 *w2, int nrhs,
                     const BicgScalars *gate) {
@@ -948,30 +919,23 @@ int learned_correct(qcd_ctx *c, float4 *out, const float4 *v, float4 *w1, float4
         const BicgScalars *gk = gate ? gate + k : nullptr;
         cudaEvent_t ev;
         prof_begin(c, QCD_K_LEARNED, &ev);
-        k_sub_plane<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(w1 + k * n4, v + k * n4, w1 + k * n4, n4,
+        k_sub_spinors<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(w1 + k * n4, v + k * n4, w1 + k * n4, n4,
                                                                          gk);
         if ((rc = prof_end(c, QCD_K_LEARNED, ev))) return rc;
         if ((rc = learned_forward(c, w2, w1 + k * n4, gk))) return rc;
         prof_begin(c, QCD_K_LEARNED, &ev);
-        k_add_plane<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(out + k * n4, w2, n4, gk);
+        k_add_spinors<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(out + k * n4, w2, n4, gk);
         if ((rc = prof_end(c, QCD_K_LEARNED, ev))) return rc;
     }
     return QCD_OK;
 }
 
-int sub_plane(qcd_ctx *c, float4 *r, const float4 *a, const float4 *b, int nrhs) {
+int sub_spinors(qcd_ctx *c, float4 *r, const float4 *a, const float4 *b, int nrhs) {
     const long n4 = 6 * c->lat.V * nrhs;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_LEARNED, &ev);
-    k_sub_plane<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(r, a, b, n4);
+    k_sub_spinors<<<(unsigned)((n4 + 255) / 256), 256, 0, c->stream>>>(r, a, b, n4);
     return prof_end(c, QCD_K_LEARNED, ev);
-}
-
-int plane_to_site(qcd_ctx *c, float2 *out, const float4 *in) {
-    cudaEvent_t ev;
-    prof_begin(c, QCD_K_OTHER, &ev);
-    k_plane_to_site<<<(unsigned)((c->lat.V + 255) / 256), 256, 0, c->stream>>>(out, in, c->lat.V);
-    return prof_end(c, QCD_K_OTHER, ev);
 }
 
 }  // namespace qcd

@@ -146,8 +146,15 @@ extern "C" int qcd_sap_precondition_noalloc(qcd_ctx *c, float *out, const float 
             plan = h.plan;
         }
     }
-    if ((rc = spinor32_to_internal(c, v, reinterpret_cast<const float2 *>(in), 1))) return rc;
-    if ((rc = sap_apply_plan(c, plan, x, v, work, p->omega, p->nsweep, p->nsap))) return rc;
-    if ((rc = spinor32_from_internal(c, reinterpret_cast<float2 *>(out), x, 1))) return rc;
+    // spinors off a 32-byte boundary (and overlapping ones) go through the scratch
+    const size_t bytes = sizeof(float4) * 6 * (size_t)c->lat.V;
+    const bool cp_in = ((uintptr_t)in & 31) || ((const char *)in < (char *)out + bytes && (char *)out < (const char *)in + bytes);
+    const bool cp_out = ((uintptr_t)out & 31) != 0;
+    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(v, in, bytes, cudaMemcpyDeviceToDevice, c->stream));
+    float4 *dst = cp_out ? x : reinterpret_cast<float4 *>(out);
+    if ((rc = sap_apply_plan(c, plan, dst, cp_in ? v : reinterpret_cast<const float4 *>(in), work, p->omega, p->nsweep,
+                             p->nsap)))
+        return rc;
+    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, x, bytes, cudaMemcpyDeviceToDevice, c->stream));
     return QCD_OK;
 }

@@ -2,14 +2,16 @@
 //
 // Internal field layouts (all in device memory, V sites, site order as the
 // canonical lexicographic order n = x + Lx*(y + Ly*(z + Lz*t))):
-//   FP64 spinor   [nrhs][12][V] double2   plane k = spin*3 + colour
-//   FP32 spinor   [nrhs][6][V]  float4    plane p holds components 2p, 2p+1
+//   FP64 spinor   [nrhs][V][12] double2   component k = spin*3 + colour
+//   FP32 spinor   [nrhs][V][6]  float4    float4 p holds components 2p, 2p+1
+// (the caller's layout, so no call converts spinors; 32-byte aligned bases)
 //   FP64 links    [4][9][V]     double2   plane mu*9 + a*3 + b
 //   FP32 links    [4][9][V]     float2
 //   FP64 clover   [36][V]       double2   chiral blocks of F/2, packed (see clover.cu)
 //   FP32 clover   [18][V]       float4    the same 72 reals per site
-// Each plane is contiguous over sites, so a warp of consecutive sites reads
-// one contiguous segment per plane (coalesced 16-byte or 8-byte loads).
+// Each link and clover plane is contiguous over sites, so a warp of consecutive sites reads one
+// contiguous segment per plane (coalesced 16-byte or 8-byte loads); a spinor's site is contiguous
+// (whole 32-byte sectors for any set of sites: neighbours, blocks).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -97,7 +99,7 @@ struct Learned {
     void *act = nullptr;     // one allocation for the buffers below
     void *a1 = nullptr, *a2 = nullptr;   // hidden activations (BF16, 8 channels)
     float2 *g1 = nullptr, *g2 = nullptr, *g3 = nullptr, *tmp = nullptr;
-    float4 *pairs = nullptr;  // training pairs: rho (plane FP32) then eps (site FP32) per pair
+    float4 *pairs = nullptr;  // training pairs: rho then eps (FP32) per pair
     size_t pairs_bytes = 0;
 };
 
@@ -212,11 +214,7 @@ int dev_alloc(qcd_ctx *c, void **p, size_t bytes);
 void dev_free(qcd_ctx *c, void *p);
 
 // ---- kernels (launchers return QCD_OK or an error) ----------------------------
-// layout conversion (layout.cu)
-int spinor64_to_internal(qcd_ctx *c, double2 *dst, const double2 *canon, int nrhs);
-int spinor64_from_internal(qcd_ctx *c, double2 *canon, const double2 *src, int nrhs);
-int spinor32_to_internal(qcd_ctx *c, float4 *dst, const float2 *canon, int nrhs);
-int spinor32_from_internal(qcd_ctx *c, float2 *canon, const float4 *src, int nrhs);
+// links to the internal layout, spinor precision conversion (layout.cu)
 int spinor64_to_32(qcd_ctx *c, float4 *dst, const double2 *src, int nrhs);
 int spinor32_to_64(qcd_ctx *c, double2 *dst, const float4 *src, int nrhs);
 int links_to_internal(qcd_ctx *c, const double2 *canon);
@@ -227,16 +225,15 @@ int build_clover(qcd_ctx *c, double kappa, double csw);
 // operator D (dslash.cu)
 struct BicgScalars;
 int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs);
-// D in pair-of-FP32 arithmetic: FP32 input (internal layout), FP64 output (internal layout)
 // makes the two-row link copy the inner solver's D reads (before any graph capture of it)
 int dslash32_prepare(qcd_ctx *c);
+// D in pair-of-FP32 arithmetic: FP32 input, FP64 output
 int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs);
 int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
 int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
 int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs);
-// D on the caller's canonical layout [nrhs][V][12] (32-byte aligned), any qcd_apply_D precision
-int dslash_canonical(qcd_ctx *c, void *out, const void *in, int prec, int nrhs);
-int dslash_x2_canonical(qcd_ctx *c, double2 *out, const float2 *in, int nrhs);
+// D in any qcd_apply_D precision
+int dslash(qcd_ctx *c, void *out, const void *in, int prec, int nrhs);
 // FP32 D (two right-hand sides per thread when there are several) fused with the inner
 // products of the BiCGStab step that follows: mode 1: red[rhs] = <other, out>, |out|^2; mode 2:
 // <out, other>, |out|^2; mode 0: none.  Right-hand sides inactive in gate (may be null) are
@@ -259,7 +256,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &pla
 int sap_prepare(qcd_ctx *c, const int b[4], const int s[4], bool half);
 // drops the cached plan (it is rebuilt on next use)
 void sap_invalidate(qcd_ctx *c);
-// x = M_SAP v (FP32 internal layout, nrhs right-hand sides); right-hand sides inactive in gate
+// x = M_SAP v (FP32, nrhs right-hand sides); right-hand sides inactive in gate
 // (may be null) are skipped.  block_solver 0: ll-SSOR block inverses (nsweep sweeps), work = 2 nrhs
 // spinors; 1: even-odd minimal-residual block inverses (nsweep steps), work = 5 nrhs spinors
 struct BicgScalars;
@@ -362,9 +359,9 @@ long learned_weight_count();
 int learned_set_weights(qcd_ctx *c, const float2 *w, bool on_device);
 int learned_get_weights(qcd_ctx *c, float2 *w_host);
 int learned_sync_B(qcd_ctx *c);
-// y = N(x), one right-hand side, plane layout FP32
+// y = N(x), one right-hand side, FP32
 int learned_forward(qcd_ctx *c, float4 *y, const float4 *x, const BicgScalars *gate = nullptr);
-// loss of one pair (rho plane layout, eps site layout FP32); gradient added to net.grad
+// loss of one pair (FP32); gradient added to net.grad
 int learned_loss_grad(qcd_ctx *c, const float4 *rho, const float2 *eps, double *loss, float4 *ybuf);
 int learned_zero_grad(qcd_ctx *c);
 int learned_adam(qcd_ctx *c, float lr);
@@ -379,11 +376,10 @@ int learned_layer_tc(qcd_ctx *c, void *y, const void *x, const __nv_bfloat16 *Bt
 // QCD_ERR_TIMEOUT (and the flag cleared) if a tensor-core layer gave up a wait since the last
 // check; synchronises the stream
 int learned_tc_status(qcd_ctx *c);
-int sub_plane(qcd_ctx *c, float4 *r, const float4 *a, const float4 *b, int nrhs);
-int plane_to_site(qcd_ctx *c, float2 *out, const float4 *in);
+int sub_spinors(qcd_ctx *c, float4 *r, const float4 *a, const float4 *b, int nrhs);
 
 // solver (solver.cu)
-// x, b: internal FP64 layout, nrhs right-hand sides
+// x (iterated in place) and b: FP64, nrhs right-hand sides
 int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrhs, qcd_stats *st);
 
 }  // namespace qcd

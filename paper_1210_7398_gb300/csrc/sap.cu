@@ -55,7 +55,7 @@ __device__ __forceinline__ void masked_hops(const float4 *src, const float2 *__r
         const bool fin = yl[MU] + 1 < bg.b[MU];                                                         \
         if (fin == INB) {                                                                               \
             long m = nbr_fwd<MU>(g, n, x);                                                              \
-            if (COHERENT) load_spinor_rw(src, g.V, m, psi); else load_spinor(src, g.V, m, psi);         \
+            if (COHERENT) load_spinor_rw(src, m, psi); else load_spinor(src, m, psi);         \
             load_link(U, g.V, n, MU, u);                                                                \
             const float sg = (MU == 3 && x[3] == g.L[3] - 1) ? (float)g.bc_t : 1.0f;                    \
             hop_term<MU, true>(psi, u, sg, acc);                                                        \
@@ -63,7 +63,7 @@ __device__ __forceinline__ void masked_hops(const float4 *src, const float2 *__r
         const bool bin = yl[MU] > 0;                                                                    \
         if (bin == INB) {                                                                               \
             long m = nbr_bwd<MU>(g, n, x);                                                              \
-            if (COHERENT) load_spinor_rw(src, g.V, m, psi); else load_spinor(src, g.V, m, psi);         \
+            if (COHERENT) load_spinor_rw(src, m, psi); else load_spinor(src, m, psi);         \
             load_link(U, g.V, m, MU, u);                                                                \
             const float sg = (MU == 3 && x[3] == 0) ? (float)g.bc_t : 1.0f;                             \
             hop_term<MU, false>(psi, u, sg, acc);                                                       \
@@ -212,8 +212,8 @@ __global__ void k_sap_records(float *__restrict__ rec, const float2 *__restrict_
 }
 
 struct SsorArgs {
-    float4 *y;                 // out: the block solutions, plane layout
-    const float4 *f;           // source (the SAP residual), plane layout
+    float4 *y;                 // out: the block solutions
+    const float4 *f;           // source (the SAP residual)
     const float4 *rec;         // per-site records of this colour's blocks
     float kappa, omega;
     int nsweep;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(32 * MAXW) k_ssor_warp(SsorArgs a) {
             const int sl = i / 6, q = i - 6 * sl;
             const int off = a.own_off[rank * a.slab_vol + sl];
             if (off < 0) continue;
-            const float4 v = a.f[(long)q * a.V + n0 + off];
+            const float4 v = a.f[(n0 + off) * 6 + q];
             m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
         for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(32 * MAXW) k_ssor_warp(SsorArgs a) {
 #pragma unroll
                 for (int q = lane; q < L::stage_chunks; q += 32) {
                     if (q < L::chunks) cp_async16(dst + 4 * q, src + q);
-                    else cp_async16(dst + 4 * q, a.f + (long)(q - L::chunks) * a.V + n0 + e.y);
+                    else cp_async16(dst + 4 * q, a.f + (n0 + e.y) * 6 + (q - L::chunks));
                 }
             }
             if (++kiss == 2 * nch) kiss = 0;
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(32 * MAXW) k_ssor_warp(SsorArgs a) {
         } else {
             v = ys4[i];
         }
-        a.y[(long)q * a.V + n] = v;
+        a.y[n * 6 + q] = v;
     }
 }
 
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(256) k_ssor_oct(SsorArgs a) {
             const int sl = i / 6, q = i - 6 * sl;
             const int off = a.own_off[rank * a.slab_vol + sl];
             if (off < 0) continue;
-            const float4 v = a.f[(long)q * a.V + n0 + off];
+            const float4 v = a.f[(n0 + off) * 6 + q];
             m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
         for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256) k_ssor_oct(SsorArgs a) {
                     const int2 e = csite[base + s4 + i];
                     float *dst = stage + (s4 + i) * L::stage;
                     if (p < L::chunks) cp_async16(dst + 4 * p, rec + (size_t)e.x * L::chunks + p);
-                    else cp_async16(dst + 4 * p, a.f + (long)(p - L::chunks) * a.V + n0 + e.y);
+                    else cp_async16(dst + 4 * p, a.f + (n0 + e.y) * 6 + (p - L::chunks));
                 }
             }
             if (++kiss == 2 * nch) kiss = 0;
@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(256) k_ssor_oct(SsorArgs a) {
         } else {
             v = ys4[i];
         }
-        a.y[(long)q * a.V + n] = v;
+        a.y[n * 6 + q] = v;
     }
 }
 
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(kTsMaxThreads) k_ssor_soa(SsorArgs a) {
                 float2 fa[12];
                 clover_mul<float, float2>(fc, acc, fa);
                 float2 fv[12], yo[12];
-                load_spinor(a.f, a.V, n0 + e.y, fv);
+                load_spinor(a.f, n0 + e.y, fv);
                 ld_y(yl, yo);
                 float4 *yp = reinterpret_cast<float4 *>(ys + yl * kTsY);
 #pragma unroll
@@ -876,7 +876,7 @@ __global__ void __launch_bounds__(kTsMaxThreads) k_ssor_soa(SsorArgs a) {
         }
     for (int i = threadIdx.x; i < vol * 6; i += blockDim.x) {
         const int yl = i / 6, q = i - 6 * yl;
-        a.y[(long)q * a.V + n0 + a.site_off[yl]] = reinterpret_cast<const float4 *>(ys + yl * kTsY)[q];
+        a.y[(n0 + a.site_off[yl]) * 6 + q] = reinterpret_cast<const float4 *>(ys + yl * kTsY)[q];
     }
 }
 
@@ -936,25 +936,25 @@ __global__ void __launch_bounds__(128) k_sap_hop(float4 *__restrict__ r, float4 
     for (int q = 0; q < 12; q++) acc[q] = make_float2(0.f, 0.f);
     if (col == colour) {
         float2 yv[12], xv[12];
-        load_spinor(y, g.V, n, yv);
-        load_spinor_rw(x, g.V, n, xv);
+        load_spinor(y, n, yv);
+        load_spinor_rw(x, n, xv);
 #pragma unroll
         for (int q = 0; q < 12; q++) { xv[q].x += yv[q].x; xv[q].y += yv[q].y; }
-        store_spinor(x, g.V, n, xv);
+        store_spinor(x, n, xv);
         if (!upd_in) return;
         masked_hops<true, false>(y, U, g, n, xc, yl, bg, acc);
         float fc[72];
         load_clover(F, g.V, n, fc);
         float2 fa[12], rv[12];
         clover_mul<float, float2>(fc, acc, fa);
-        load_spinor_rw(r, g.V, n, rv);
+        load_spinor_rw(r, n, rv);
 #pragma unroll
         for (int q = 0; q < 12; q++) {
             // r -= y - kappa F H_BB y
             rv[q].x = rv[q].x - yv[q].x + kappa * fa[q].x;
             rv[q].y = rv[q].y - yv[q].y + kappa * fa[q].y;
         }
-        store_spinor(r, g.V, n, rv);
+        store_spinor(r, n, rv);
     } else {
         if (!upd_cross) return;
         bool face = false;
@@ -965,13 +965,13 @@ __global__ void __launch_bounds__(128) k_sap_hop(float4 *__restrict__ r, float4 
         load_clover(F, g.V, n, fc);
         float2 fa[12], rv[12];
         clover_mul<float, float2>(fc, acc, fa);
-        load_spinor_rw(r, g.V, n, rv);
+        load_spinor_rw(r, n, rv);
 #pragma unroll
         for (int q = 0; q < 12; q++) {
             rv[q].x = fmaf(kappa, fa[q].x, rv[q].x);
             rv[q].y = fmaf(kappa, fa[q].y, rv[q].y);
         }
-        store_spinor(r, g.V, n, rv);
+        store_spinor(r, n, rv);
     }
 }
 
@@ -1037,15 +1037,15 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
         if (odd(yl)) continue;
         float2 h[12], v[12];
         block_FH<false>(f, U, F, g, n, xc, yl, bg, h);
-        load_spinor(f, g.V, n, v);
+        load_spinor(f, n, v);
 #pragma unroll
         for (int q = 0; q < 12; q++) {
             v[q].x = fmaf(kappa, h[q].x, v[q].x);
             v[q].y = fmaf(kappa, h[q].y, v[q].y);
             h[q] = zero;
         }
-        store_spinor(R, g.V, n, v);
-        store_spinor(y, g.V, n, h);
+        store_spinor(R, n, v);
+        store_spinor(y, n, h);
     }
     __syncthreads();
     const float k2 = kappa * kappa;
@@ -1057,7 +1057,7 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
             if (!odd(yl)) continue;
             float2 h[12];
             block_FH<true>(R, U, F, g, n, xc, yl, bg, h);
-            store_spinor(T, g.V, n, h);
+            store_spinor(T, n, h);
         }
         __syncthreads();
         // p = r - kappa^2 F_e H_eo t on the even sites, with <p, r> and <p, p>
@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
             if (odd(yl)) continue;
             float2 h[12], rv[12];
             block_FH<true>(T, U, F, g, n, xc, yl, bg, h);
-            load_spinor_rw(R, g.V, n, rv);
+            load_spinor_rw(R, n, rv);
 #pragma unroll
             for (int q = 0; q < 12; q++) {
                 const float2 pv = make_float2(fmaf(-k2, h[q].x, rv[q].x), fmaf(-k2, h[q].y, rv[q].y));
@@ -1077,7 +1077,7 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
                 pp = fmaf(pv.x, pv.x, fmaf(pv.y, pv.y, pp));
                 h[q] = pv;
             }
-            store_spinor(P, g.V, n, h);
+            store_spinor(P, n, h);
         }
         double a0 = pr_re, a1 = pr_im, a2 = pp;
         for (int sft = 16; sft > 0; sft >>= 1) {
@@ -1109,16 +1109,16 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
             const long n = site(i, xc, yl);
             if (odd(yl)) continue;
             float2 xv[12], rv[12], pv[12];
-            load_spinor_rw(y, g.V, n, xv);
-            load_spinor_rw(R, g.V, n, rv);
-            load_spinor_rw(P, g.V, n, pv);
+            load_spinor_rw(y, n, xv);
+            load_spinor_rw(R, n, rv);
+            load_spinor_rw(P, n, pv);
 #pragma unroll
             for (int q = 0; q < 12; q++) {
                 xv[q] = cfma(al, rv[q], xv[q]);
                 rv[q] = cfma(make_float2(-al.x, -al.y), pv[q], rv[q]);
             }
-            store_spinor(y, g.V, n, xv);
-            store_spinor(R, g.V, n, rv);
+            store_spinor(y, n, xv);
+            store_spinor(R, n, rv);
         }
         __syncthreads();
     }
@@ -1129,13 +1129,13 @@ __global__ void __launch_bounds__(kEoThreads) k_block_eo_mr(float4 *y, const flo
         if (!odd(yl)) continue;
         float2 h[12], v[12];
         block_FH<true>(y, U, F, g, n, xc, yl, bg, h);
-        load_spinor(f, g.V, n, v);
+        load_spinor(f, n, v);
 #pragma unroll
         for (int q = 0; q < 12; q++) {
             v[q].x = fmaf(kappa, h[q].x, v[q].x);
             v[q].y = fmaf(kappa, h[q].y, v[q].y);
         }
-        store_spinor(y, g.V, n, v);
+        store_spinor(y, n, v);
     }
 }
 

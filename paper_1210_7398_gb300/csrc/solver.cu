@@ -34,9 +34,10 @@ namespace {
 struct Ws {
     int nrhs;
     long V;
-    // FP64 internal vectors [nrhs][12][V]
-    double2 *b, *x, *r, *rh, *p, *v, *s, *t, *ph, *sh, *tmp;
-    // FP32 internal vectors [nrhs][6][V]
+    // FP64 vectors [nrhs][V][12]; b and x are the caller's
+    const double2 *b;
+    double2 *x, *r, *rh, *p, *v, *s, *t, *ph, *sh, *tmp;
+    // FP32 vectors [nrhs][V][6]
     float4 *q, *y, *ir, *irh, *ip, *iv, *is, *it, *ipt, *ist, *sapw;
     BicgScalars *So, *Si;  // outer, inner scalars (device)
     BicgScalars *hSo, *hSi;  // pinned host mirrors
@@ -244,7 +245,7 @@ int ensure(qcd_ctx *c, void **ptr, size_t *have, size_t need) {
 int workspace(qcd_ctx *c, int nrhs, int block_solver, Ws *w) {
     const long V = c->lat.V;
     const size_t b64 = sizeof(double2) * 12 * V * nrhs, b32 = sizeof(float4) * 6 * V * nrhs;
-    TRY(ensure(c, &c->ws64, &c->ws64_bytes, 11 * b64));
+    TRY(ensure(c, &c->ws64, &c->ws64_bytes, 9 * b64));
     TRY(ensure(c, &c->ws32, &c->ws32_bytes, (10 + sap_work_fields(block_solver)) * b32));
     if (c->red_rhs < nrhs) {
         dev_free(c, c->d_red);
@@ -275,8 +276,8 @@ int workspace(qcd_ctx *c, int nrhs, int block_solver, Ws *w) {
     w->nrhs = nrhs;
     w->V = V;
     double2 *base = (double2 *)c->ws64;
-    double2 **v64[] = {&w->b, &w->x, &w->r, &w->rh, &w->p, &w->v, &w->s, &w->t, &w->ph, &w->sh, &w->tmp};
-    for (int k = 0; k < 11; k++) *v64[k] = base + (size_t)k * 12 * V * nrhs;
+    double2 **v64[] = {&w->r, &w->rh, &w->p, &w->v, &w->s, &w->t, &w->ph, &w->sh, &w->tmp};
+    for (int k = 0; k < 9; k++) *v64[k] = base + (size_t)k * 12 * V * nrhs;
     float4 *b32p = (float4 *)c->ws32;
     float4 **v32[] = {&w->q, &w->y, &w->ir, &w->irh, &w->ip, &w->iv, &w->is, &w->it, &w->ipt, &w->ist, &w->sapw};
     for (int k = 0; k < 11; k++) *v32[k] = b32p + (size_t)k * 6 * V * nrhs;  // sapw spans the SAP work fields
@@ -308,8 +309,8 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
         }
     } guard{gp};
 
-    TRY(blas_copy(c, w.b, b, b64));
-    TRY(blas_copy(c, w.x, x, b64));
+    w.b = b;
+    w.x = x;
     // |b|^2 and |x0|^2 per rhs
     TRY(reduce64(c, RED_NORM, w.b, nullptr, n, R, w.red, nullptr));
     std::vector<double> bn2(R), h(6 * R);
@@ -473,7 +474,6 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
         for (int k = 0; k < R; k++) w.hmask[k] = status[k] != QCD_OK ? 1 : 0;
         TRY(true_residual(w.hmask, &any_masked));
     }
-    TRY(blas_copy(c, x, w.x, b64));
     int worst = QCD_OK;
     for (int k = 0; k < R; k++)
         if (status[k] != QCD_OK) worst = (worst == QCD_OK || status[k] == QCD_ERR_BREAKDOWN) ? status[k] : worst;

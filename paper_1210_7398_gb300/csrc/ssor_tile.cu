@@ -227,7 +227,7 @@ template <bool HALF> __device__ __forceinline__ void clover_rec(const uint4 *rec
 }
 
 struct TileArgs {
-    float4 *x;                 // M_SAP v being accumulated, plane layout [nrhs][6][V]
+    float4 *x;                 // M_SAP v being accumulated, [nrhs][V][6]
     float4 *r;                 // SAP residual (this colour's sites read and rewritten)
     float4 *y;                 // block solutions: this colour's sites written, the other colour's read
     const float4 *v;           // the SAP input (read in the first cycle)
@@ -261,7 +261,7 @@ struct TileArgs {
 };
 
 // the other colour's block solution at site mm, in the neighbouring block of rank nrank among its
-// colour, for one right-hand side: FP32 in the lattice layout, or (FP16 storage) the FP16 record
+// colour, for one right-hand side: FP32 in the lattice, or (FP16 storage) the FP16 record
 // times its block's scale
 template <bool HALF>
 __device__ __forceinline__ void load_y_other(const TileArgs &a, int rhs, long mm, int nrank, float2 psi[12]) {
@@ -275,7 +275,7 @@ __device__ __forceinline__ void load_y_other(const TileArgs &a, int rhs, long mm
             psi[4 * k + 2] = cscale(h2f(v.z), sc); psi[4 * k + 3] = cscale(h2f(v.w), sc);
         }
     } else {
-        load_spinor(a.y + (size_t)rhs * 6 * a.V, a.V, mm, psi);
+        load_spinor(a.y + (size_t)rhs * 6 * a.V, mm, psi);
     }
 }
 
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
     }
     const int r_me = tid % R;  // every item this thread takes has right-hand side r_me (T % R == 0)
     const bool me_active = act_s[r_me] != 0;
-    const size_t roff = (size_t)(rhs0 + r_me) * 6 * a.V + n0;
+    const size_t roff = ((size_t)(rhs0 + r_me) * a.V + n0) * 6;
     float4 *rr = a.r + roff;  // this right-hand side's residual, from the block origin
     const int *org = a.origin + 4 * blk;
 
@@ -386,15 +386,15 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
             }
             {
                 float2 base[12];
-                if (a.first) load_spinor(a.v + roff, a.V, pa.x, base);
-                else load_spinor_rw(rr, a.V, pa.x, base);
+                if (a.first) load_spinor(a.v + roff, pa.x, base);
+                else load_spinor_rw(rr, pa.x, base);
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
                     f[k].x = fmaf(a.kappa, f[k].x, base[k].x);
                     f[k].y = fmaf(a.kappa, f[k].y, base[k].y);
                 }
             }
-            store_spinor(rr, a.V, pa.x, f);
+            store_spinor(rr, pa.x, f);
             if constexpr (HALF) {
 #pragma unroll
                 for (int k = 0; k < 12; k++) m = fmaxf(m, fmaxf(fabsf(f[k].x), fabsf(f[k].y)));
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
             for (int i = tid; i < a.vol * R; i += T) {
                 const int4 pa = __ldg(a.pos + 2 * (i / R));
                 float2 f[12];
-                load_spinor_rw(rr, a.V, pa.x, f);
+                load_spinor_rw(rr, pa.x, f);
 #pragma unroll
                 for (int k = 0; k < 12; k++) f[k] = cscale(f[k], inv_scale);
                 st_y<true>(fs + pa.y * a.stride + r_me * L::y_words, f);
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
         block_FH(pos, pa, pb, fa);
         float2 fv[12];
         if constexpr (HALF) ld_y<true>(fs + pa.y * a.stride + r_me * L::y_words, fv);
-        else load_spinor_rw(rr, a.V, pa.x, fv);
+        else load_spinor_rw(rr, pa.x, fv);
         float *yp = ys + pa.y * a.stride + r_me * L::y_words;
         float2 yo[12];
         ld_y<HALF>(yp, yo);
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
                 block_FH(pos, pa, pb, f);  // F H_BB y, then f - y + kappa F H_BB y
                 {
                     float2 base[12];
-                    load_spinor_rw(rr, a.V, pa.x, base);
+                    load_spinor_rw(rr, pa.x, base);
 #pragma unroll
                     for (int k = 0; k < 12; k++) {
                         if constexpr (HALF) f[k] = cscale(f[k], my_scale);
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
                     if constexpr (HALF) yv[k] = cscale(yv[k], my_scale);
                     f[k] = csub(f[k], yv[k]);
                 }
-                store_spinor(rr, a.V, pa.x, f);
+                store_spinor(rr, pa.x, f);
             }
             float2 yv[12];
             ld_y<HALF>(ys + pa.y * a.stride + r_me * L::y_words, yv);
@@ -524,13 +524,13 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
                 for (int k = 0; k < 12; k++) yv[k] = cscale(yv[k], my_scale);
             }
             if (a.first) {
-                store_spinor(xr, a.V, pa.x, yv);
+                store_spinor(xr, pa.x, yv);
             } else {
                 float2 xv[12];
-                load_spinor_rw(xr, a.V, pa.x, xv);
+                load_spinor_rw(xr, pa.x, xv);
 #pragma unroll
                 for (int k = 0; k < 12; k++) xv[k] = cadd(xv[k], yv[k]);
-                store_spinor(xr, a.V, pa.x, xv);
+                store_spinor(xr, pa.x, xv);
             }
             if (a.store_y) {
                 if constexpr (HALF) {
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
                     dst[1] = src[1];
                     dst[2] = src[2];
                 } else {
-                    store_spinor(yo4, a.V, pa.x, yv);
+                    store_spinor(yo4, pa.x, yv);
                 }
             }
         }

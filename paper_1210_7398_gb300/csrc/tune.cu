@@ -170,22 +170,17 @@ extern "C" int qcd_autotune(qcd_ctx *c, const double *b, int nrhs, const qcd_par
     }
     const long V = c->lat.V;
     const size_t bytes = sizeof(double2) * 12 * V * nrhs;
-    // right-hand sides in the internal layout, solution buffer
+    // right-hand sides, solution buffer
     void *buf = nullptr;
-    int rc = dev_alloc(c, &buf, 3 * bytes);
+    int rc = dev_alloc(c, &buf, 2 * bytes);
     if (rc) return rc;
     struct Free {
         qcd_ctx *c;
         void *p;
         ~Free() { dev_free(c, p); }
     } guard{c, buf};
-    double2 *bi = (double2 *)buf, *xi = bi + 12 * V * nrhs, *stage = xi + 12 * V * nrhs;
-    cudaPointerAttributes at;
-    const bool on_dev = cudaPointerGetAttributes(&at, b) == cudaSuccess &&
-                        (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
-    cudaGetLastError();
-    QCD_CUDA(c, cudaMemcpyAsync(stage, b, bytes, on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
-    if ((rc = spinor64_to_internal(c, bi, stage, nrhs))) return rc;
+    double2 *bi = (double2 *)buf, *xi = bi + 12 * V * nrhs;
+    QCD_CUDA(c, cudaMemcpyAsync(bi, b, bytes, cudaMemcpyDefault, c->stream));
     const bool old_prof = c->prof.on;
     c->prof.on = false;
 

@@ -99,6 +99,42 @@ def test_dslash_alignment_and_overlap(prec, dims, nrhs):
     s.close()
 
 
+@pytest.mark.parametrize("ctas,block_solver", [(-2, 0), (0, 0), (-1, 0), (0, 1)])
+def test_sap_and_solve_alignment_and_overlap(ctas, block_solver):
+    """M_SAP and the solve on spinors off a 32-byte boundary, in place, and with x over b: these take
+    the copies and equal the direct calls bit for bit."""
+    dims, block, sub = (4, 6, 4, 8), (2, 3, 2, 4), (1, 3, 1, 2)
+    s, U, F = make_solver(dims, 0.12, seed=1000)
+    prm = q.make_params(0.12, CSW, block, sub, omega=1.1, nsweep=2, nsap=2, sap_ctas=ctas, block_solver=block_solver)
+    psi = qi.gaussian_spinor(dims, seed=2000, nrhs=3)
+
+    def shifted(t):
+        skip = 16 // t.element_size()
+        skip = max(skip, 1)
+        buf = torch.empty(t.numel() + skip, dtype=t.dtype, device="cuda")[skip:].view(t.shape).copy_(t)
+        assert buf.data_ptr() % 32 == 16
+        return buf
+
+    v = torch.from_numpy(psi).cuda().to(torch.complex64)
+    out = torch.empty_like(v)
+    s.sap_precondition(out, v, prm, 3)
+    outs, inplace = shifted(torch.zeros_like(v)), v.clone()
+    s.sap_precondition(outs, shifted(v), prm, 3)
+    s.sap_precondition(inplace, inplace, prm, 3)
+    torch.cuda.synchronize()
+    assert torch.equal(out, outs) and torch.equal(out, inplace)
+    b = torch.from_numpy(psi).cuda()
+    x, xs, xb = torch.zeros_like(b), shifted(torch.zeros_like(b)), b.clone()
+    s.solve(x, b, prm, 3)
+    s.solve(xs, shifted(b), prm, 3)
+    assert torch.equal(x, xs)
+    s.solve(xb, xb, prm, 3)  # start vector and source in one buffer
+    x0 = b.clone()
+    s.solve(x0, b, prm, 3)
+    assert torch.equal(xb, x0)
+    s.close()
+
+
 @pytest.mark.parametrize("dims,bc_t", [((4, 4, 4, 4), 1), ((6, 4, 4, 6), -1), ((8, 8, 8, 16), 1),
                                        ((2, 6, 4, 2), -1)])
 def test_dslash_pair_fp32_vs_oracle(dims, bc_t):
