@@ -620,17 +620,8 @@ int qcd_learned_load(qcd_ctx *c, const char *path) {
     return qcd_learned_set_weights(c, w.data(), n);
 }
 
-// a complex64 field as the kernels can read it: the caller's where it lies on the device on a
-// 32-byte boundary, else copied into scratch
-static int readable(qcd_ctx *c, const float *src, size_t bytes, char *scratch, const float4 **out) {
-    if (is_device_ptr(src) && aligned32(src)) {
-        *out = (const float4 *)src;
-        return QCD_OK;
-    }
-    QCD_CUDA(c, cudaMemcpyAsync(scratch, src, bytes, cudaMemcpyDefault, c->stream));
-    *out = (const float4 *)scratch;
-    return QCD_OK;
-}
+// whether the kernels can use a complex64 field where it is: on the device, on a 32-byte boundary
+static bool usable(const float *p) { return is_device_ptr(p) && aligned32(p); }
 
 int qcd_learned_apply(qcd_ctx *c, float *out, const float *in) {
     int rc = ready(c);
@@ -638,12 +629,12 @@ int qcd_learned_apply(qcd_ctx *c, float *out, const float *in) {
     if (!c->net.ready) return fail(c, QCD_ERR_STATE, "qcd_learned_set_weights must be called first");
     if (!out || !in) return fail(c, QCD_ERR_ARG, "NULL argument");
     const size_t bytes = 8 * 12 * (size_t)c->lat.V;
-    if ((rc = ensure_io(c, 2 * bytes))) return rc;
+    const bool cp_in = !usable(in), cp_out = !usable(out);
+    if (cp_in + cp_out && (rc = ensure_io(c, (cp_in + cp_out) * bytes))) return rc;
     char *io = (char *)c->d_io;
-    const float4 *x = nullptr;
-    if ((rc = readable(c, in, bytes, io, &x))) return rc;
-    const bool cp_out = !is_device_ptr(out) || !aligned32(out);
-    float4 *y = cp_out ? (float4 *)(io + bytes) : (float4 *)out;
+    const float4 *x = (const float4 *)(cp_in ? io : (const char *)in);
+    float4 *y = (float4 *)(cp_out ? io + cp_in * bytes : (char *)out);
+    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(io, in, bytes, cudaMemcpyDefault, c->stream));
     if ((rc = learned_forward(c, y, x))) return rc;
     if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, y, bytes, cudaMemcpyDefault, c->stream));
     return learned_tc_status(c);  // synchronises
@@ -655,14 +646,16 @@ int qcd_learned_loss_grad(qcd_ctx *c, const float *rho, const float *eps, double
     if (!c->net.ready) return fail(c, QCD_ERR_STATE, "qcd_learned_set_weights must be called first");
     if (!rho || !eps) return fail(c, QCD_ERR_ARG, "NULL argument");
     const size_t bytes = 8 * 12 * (size_t)c->lat.V;
-    if ((rc = ensure_io(c, 3 * bytes))) return rc;
+    const bool cp_r = !usable(rho), cp_e = !usable(eps);
+    if (cp_r + cp_e && (rc = ensure_io(c, (cp_r + cp_e) * bytes))) return rc;
     char *io = (char *)c->d_io;
-    const float4 *r = nullptr, *e = nullptr;
-    if ((rc = readable(c, rho, bytes, io, &r))) return rc;
-    if ((rc = readable(c, eps, bytes, io + bytes, &e))) return rc;
+    const float4 *r = (const float4 *)(cp_r ? io : (const char *)rho);
+    const float2 *e = (const float2 *)(cp_e ? io + cp_r * bytes : (const char *)eps);
+    if (cp_r) QCD_CUDA(c, cudaMemcpyAsync(io, rho, bytes, cudaMemcpyDefault, c->stream));
+    if (cp_e) QCD_CUDA(c, cudaMemcpyAsync(io + cp_r * bytes, eps, bytes, cudaMemcpyDefault, c->stream));
     if ((rc = learned_zero_grad(c))) return rc;
     double l = 0;
-    if ((rc = learned_loss_grad(c, r, (const float2 *)e, &l, (float4 *)(io + 2 * bytes)))) return rc;
+    if ((rc = learned_loss_grad(c, r, e, &l, (float4 *)c->net.tmp))) return rc;
     if (loss) *loss = l;
     if (grad)
         QCD_CUDA(c, cudaMemcpyAsync(grad, c->net.grad, sizeof(float2) * learned_weight_count(),

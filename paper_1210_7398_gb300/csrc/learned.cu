@@ -6,16 +6,16 @@
 // T on colour and site, a layer is, per direction, a dense contraction over
 // (input channel, spin) for every (site, colour) row: a GEMM with M = 3V rows,
 // K = 9 x Cin x 4 complex, N = Cout x 4 complex.  It runs on the tensor cores
-// in BF16 with FP32 accumulation (mma.sync m16n8k16): per direction a CTA
-// stages the neighbour inputs and links of 64 sites in shared memory with
-// coalesced loads, transports them into the BF16 A tile, loads that
-// direction's weights as a real 2x2-block matrix (the B tile), multiplies,
-// and moves to the next direction with the accumulators in registers.  The data gradient is the same kernel with the adjoint
-// weights (T_d^dag = T_{opposite d} and W commutes with T); the weight
-// gradient is sum over rows of A^T G, computed the same way with the
-// reduction over rows.
+// in BF16 with FP32 accumulation (here mma.sync m16n8k16, the 8 -> 8 layer in
+// learned_tc.cu on tcgen05), the weights as real 2x2-block matrices.  A layer
+// with one input channel transports that in all directions at once (K = 72);
+// the one with one output channel applies the weights first and transports
+// the output.  The data gradient is the same with the adjoint weights
+// (T_d^dag = T_{opposite d} and W commutes with T); the weight gradient is a
+// product with the reduction over the rows.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -29,13 +29,6 @@ namespace {
 // activation formats
 enum { SITE16 = 1, SITE32 = 2 };
 
-template <int FMT> __device__ __forceinline__ float2 act_ld(const void *base, long V, int ch, long n, int k) {
-    if constexpr (FMT == SITE16) {
-        return __bfloat1622float2(static_cast<const __nv_bfloat162 *>(base)[((long)ch * V + n) * 12 + k]);
-    } else {
-        return static_cast<const float2 *>(base)[((long)ch * V + n) * 12 + k];
-    }
-}
 template <int FMT> __device__ __forceinline__ void act_st(void *base, long V, int ch, long n, int k, float2 v) {
     if constexpr (FMT == SITE16) {
         static_cast<__nv_bfloat162 *>(base)[((long)ch * V + n) * 12 + k] = __float22bfloat162_rn(v);
@@ -56,54 +49,6 @@ __device__ __forceinline__ void mma_bf16(float c[4], uint32_t a0, uint32_t a1, u
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// Row (n, a) of the transported inputs of direction d: z[c'][beta] = sum_b W_d[a][b] x_{c'}(m)[beta][b]
-// with W = 1 (d = 0), U_mu(n) and m = n + mu (forward), U_mu(n - mu)^dag and m = n - mu (backward),
-// times the boundary sign; written as CIN x 4 complex into the BF16 row `dst` (2 values each).
-template <int CIN, int FMT>
-__device__ __forceinline__ void transport_row(const void *x, const float2 *__restrict__ U, const Geo &g, int d,
-                                              long n, int a, __nv_bfloat16 *dst) {
-    long m = n;
-    float2 w[3];
-    if (d == 0) {
-        w[0] = w[1] = w[2] = make_float2(0.f, 0.f);
-        w[a] = make_float2(1.f, 0.f);
-    } else {
-        const int mu = (d - 1) >> 1;
-        const bool fwd = ((d - 1) & 1) == 0;
-        int xc[4];
-        site_coords(g, n, xc);
-        long stride = 1;
-        for (int q = 0; q < mu; q++) stride *= g.L[q];
-        float sgn = 1.f;
-        if (fwd) {
-            m = (xc[mu] == g.L[mu] - 1) ? n - stride * (g.L[mu] - 1) : n + stride;
-            if (mu == 3 && xc[3] == g.L[3] - 1) sgn = (float)g.bc_t;
-        } else {
-            m = (xc[mu] == 0) ? n + stride * (g.L[mu] - 1) : n - stride;
-            if (mu == 3 && xc[3] == 0) sgn = (float)g.bc_t;
-        }
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            // forward: row a of U_mu(n); backward: row a of U_mu(m)^dag = conj(column a of U_mu(m))
-            float2 u = fwd ? __ldg(U + (long)(mu * 9 + a * 3 + b) * g.V + n) : __ldg(U + (long)(mu * 9 + b * 3 + a) * g.V + m);
-            if (!fwd) u.y = -u.y;
-            w[b] = cscale(u, sgn);
-        }
-    }
-#pragma unroll
-    for (int ch = 0; ch < CIN; ch++) {
-        uint32_t packed[4];
-#pragma unroll
-        for (int be = 0; be < 4; be++) {
-            float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int b = 0; b < 3; b++) acc = cfma(w[b], act_ld<FMT>(x, g.V, ch, m, be * 3 + b), acc);
-            packed[be] = pack_bf16(acc.x, acc.y);
-        }
-        *reinterpret_cast<uint4 *>(dst + ch * 8) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    }
 }
 
 constexpr int kLayerSites = 64;                 // sites per CTA tile of the layer kernel
@@ -292,93 +237,163 @@ __device__ __forceinline__ void transport_item(const unsigned char *xs, const fl
     }
 }
 
-// y = layer(x): CIN -> COUT channels.  Bt: [9][N][KDP] BF16, N = COUT*8, KDP = max(16, CIN*8).
-// A CTA owns 64 sites (192 rows, one 16-row MMA tile per warp).  Per direction: the neighbour
-// inputs (all channels), their links and the direction's weights are staged with cp.async one
-// direction ahead; one thread per (site, channel pair) applies the 3x3 colour transport to the
-// four spins and writes the BF16 A rows; the warps then accumulate A B into registers, with
-// fragments read by ldmatrix.
-template <int CIN, int COUT, int FIN, int FOUT>
-__global__ void __launch_bounds__(kLayerWarps * 32, FIN == SITE32 ? 1 : 2) k_layer(void *y, const void *x, const float2 *__restrict__ U,
-                                                               const __nv_bfloat16 *__restrict__ Bt, Geo g,
-                                                               const BicgScalars *__restrict__ gate = nullptr) {
-    if (gate && !gate->active) return;  // a right-hand side that has left the iteration
-    using S = LayerSmem<CIN, COUT, FIN>;
-    constexpr int KDP = S::KDP, N = S::N, AS = S::AS, NT = N / 8, XS = S::XS;
-    constexpr int NTH = kLayerWarps * 32;
-    constexpr int CPI = 1;                            // channels per transport item
-    constexpr int ITEMS = kLayerSites * (CIN / CPI);  // transport items per direction
-    static_assert(CIN % CPI == 0, "whole channel groups");
-    extern __shared__ __align__(16) unsigned char ly_smem[];
-    __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16 *>(ly_smem + 2 * S::stage);
-    int *nbt = reinterpret_cast<int *>(ly_smem + 2 * S::stage + S::a_bytes);  // [9][64] neighbour, -1 past the end
-    float *sgt = reinterpret_cast<float *>(nbt + 9 * kLayerSites);            // [9][64] boundary sign
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
-    const int n0 = blockIdx.x * kLayerSites;
-
-    layer_neighbours(nbt, sgt, g, n0, tid);
-    __syncthreads();
-    auto issue = [&](int d) { layer_issue<CIN, COUT, FIN>(ly_smem, nbt, x, U, Bt, g, n0, d, tid, NTH); };
-
-    // KDP > CIN*8 (one input channel): the upper K half of A stays zero
-    if constexpr (KDP > CIN * 8) {
-        for (int i = tid; i < kLayerRows; i += NTH)
-            *reinterpret_cast<uint4 *>(A + i * AS + CIN * 8) = make_uint4(0, 0, 0, 0);
-    }
-    float acc[NT][4];
+// rows 3 st + a (colour a) of a 12-component site: four spins as BF16 pairs, 16 bytes per row
+__device__ __forceinline__ void put_rows(__nv_bfloat16 *row0, int stride, const float2 v[12]) {
 #pragma unroll
-    for (int j = 0; j < NT; j++) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+    for (int a = 0; a < 3; a++)
+        *reinterpret_cast<uint4 *>(row0 + a * stride) =
+            make_uint4(pack_bf16(v[a].x, v[a].y), pack_bf16(v[3 + a].x, v[3 + a].y), pack_bf16(v[6 + a].x, v[6 + a].y),
+                       pack_bf16(v[9 + a].x, v[9 + a].y));
+}
 
-    issue(0);
-#pragma unroll 1
-    for (int d = 0; d < 9; d++) {
-        cp_wait<0>();
-        __syncthreads();  // stage d visible; every warp is done with the previous A and stage
-        if (d + 1 < 9) issue(d + 1);
-        const unsigned char *X = ly_smem + (d & 1) * S::stage;
-        const float2 *L = reinterpret_cast<const float2 *>(X + S::x_bytes);
-        const __nv_bfloat16 *B = reinterpret_cast<const __nv_bfloat16 *>(X + S::x_bytes + S::l_bytes);
-        // transport: A[3 st + a][8 ch + 2 be (+1)] = sum_b W[a][b] x_ch(m)[be][b], W = 1, U_mu(n) or
-        // U_mu(n - mu)^dag, times the boundary sign (time direction only)
-        for (int it = tid; it < ITEMS; it += NTH) {
-            const int st = it / (CIN / CPI), cg = (it % (CIN / CPI)) * CPI;
-            const float sg = sgt[d * kLayerSites + st];
-            if (d == 0) transport_item<CIN, CPI, FIN, 0>(X + st * XS, L + st * 9, sg, A + st * 3 * AS, cg, AS);
-            else if (d < 7 && (d & 1)) transport_item<CIN, CPI, FIN, 1>(X + st * XS, L + st * 9, sg, A + st * 3 * AS, cg, AS);
-            else if (d < 7) transport_item<CIN, CPI, FIN, 2>(X + st * XS, L + st * 9, sg, A + st * 3 * AS, cg, AS);
-            else if (d & 1) transport_item<CIN, CPI, FIN, 3>(X + st * XS, L + st * 9, sg, A + st * 3 * AS, cg, AS);
-            else transport_item<CIN, CPI, FIN, 4>(X + st * XS, L + st * 9, sg, A + st * 3 * AS, cg, AS);
+// One thread's share of a one-channel field (FP32) of a 64-site tile, transported in every direction:
+// thread (st, grp) takes site st and direction grp + 1 (or its opposite, FLIP), and one float4 of the tile's
+// own sites for the identity.  The A rows it makes hold the nine directions' four spins side by side,
+// 72 columns of a row of kSingleCols BF16 (80 multiplied, the last 8 zero; 88: no ldmatrix bank conflicts).
+constexpr int kTileThreads = 512;
+constexpr int kSingleCols = 88;
+template <bool FLIP> struct SingleField {
+    float2 x[12], u[9];
+    float4 own;
+    float sg;
+    int st, mu, d, Lm, stride, V;
+    bool fwd;
+    __device__ __forceinline__ SingleField(const Geo &g, int tid) {
+        const int grp = tid >> 6;
+        st = tid & (kLayerSites - 1);
+        mu = grp >> 1;
+        d = grp + 1;
+        fwd = ((grp & 1) == 0) != FLIP;
+        Lm = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+        stride = mu == 0 ? 1 : mu == 1 ? g.L[0] : mu == 2 ? g.L[0] * g.L[1] : g.L[0] * g.L[1] * g.L[2];
+        V = (int)g.V;
+    }
+    // the loads of a tile; n: the site (0 past the end of the lattice, where `in` is false)
+    __device__ __forceinline__ void load(const Geo &g, const float4 *__restrict__ S, const float2 *__restrict__ U, int tile,
+                                         int tid, int &n, bool &in) {
+        n = tile * kLayerSites + st;
+        in = n < V;
+        if (!in) n = 0;
+        int r = n, xm = 0, xt = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = q < 3 ? r % g.L[q] : r;
+            if (q < 3) r /= g.L[q];
+            if (q == mu) xm = c;
+            if (q == 3) xt = c;
+        }
+        const int m = fwd ? (xm == Lm - 1 ? n - stride * (Lm - 1) : n + stride)
+                          : (xm == 0 ? n + stride * (Lm - 1) : n - stride);
+        sg = !in ? 0.f : (mu == 3 && xt == (fwd ? Lm - 1 : 0)) ? (float)g.bc_t : 1.f;
+        load_spinor(S, m, x);
+        const int ls = fwd ? n : m;
+#pragma unroll
+        for (int e = 0; e < 9; e++) u[e] = __ldg(U + (long)(mu * 9 + e) * V + ls);
+        const long o = (long)tile * kLayerSites * 6 + tid;
+        own = tid < kLayerSites * 6 && o < (long)V * 6 ? __ldg(S + o) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __device__ __forceinline__ void put(__nv_bfloat16 *Ss, int tid) const {
+        float2 z[12];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            float2 w[3];  // row a of the transport
+#pragma unroll
+            for (int b = 0; b < 3; b++) {
+                w[b] = fwd ? u[a * 3 + b] : make_float2(u[b * 3 + a].x, -u[b * 3 + a].y);
+                w[b] = cscale(w[b], sg);
+            }
+#pragma unroll
+            for (int be = 0; be < 4; be++) {
+                float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int b = 0; b < 3; b++) t = cfma(w[b], x[be * 3 + b], t);
+                z[be * 3 + a] = t;
+            }
+        }
+        put_rows(Ss + 3 * st * kSingleCols + d * 8, kSingleCols, z);
+        if (tid < kLayerSites * 6) {
+            const int os = tid / 6, k0 = 2 * (tid % 6), k1 = k0 + 1;
+            *reinterpret_cast<uint32_t *>(Ss + (3 * os + k0 % 3) * kSingleCols + 2 * (k0 / 3)) = pack_bf16(own.x, own.y);
+            *reinterpret_cast<uint32_t *>(Ss + (3 * os + k1 % 3) * kSingleCols + 2 * (k1 / 3)) = pack_bf16(own.z, own.w);
+        }
+    }
+    // the zero columns 72 ... 79 of `rows` rows
+    static __device__ __forceinline__ void pad(__nv_bfloat16 *Ss, int rows, int tid) {
+        for (int i = tid; i < rows; i += kTileThreads)
+            *reinterpret_cast<uint4 *>(Ss + i * kSingleCols + 72) = make_uint4(0, 0, 0, 0);
+    }
+};
+
+// y = layer(x) for one input channel, 1 -> 8.  With one channel to transport, all nine directions'
+// A columns of a 64-site tile are made at once, and the layer is one product of 192 rows x 80 by 80 x 64;
+// the weights stay in registers as fragments, the next tile's fields are loaded while this one is
+// multiplied, and the output leaves through shared memory in whole lines.  Bound by the loads' latency
+// at 16 warps per SM.  24^3x48: 0.19 (BF16 out) and 0.23 ms (FP32 out), against 0.57 and 0.60 ms with
+// one direction after the other.
+template <int FOUT>
+__global__ void __launch_bounds__(kTileThreads, 1) k_layer_single(void *y, const float4 *__restrict__ x,
+                                                                  const float2 *__restrict__ U,
+                                                                  const __nv_bfloat16 *__restrict__ Bt, Geo g, int ntiles,
+                                                                  const BicgScalars *__restrict__ gate) {
+    if (gate && !gate->active) return;  // a right-hand side that has left the iteration
+    extern __shared__ __align__(16) unsigned char l1_smem[];
+    __nv_bfloat16 *Sb = reinterpret_cast<__nv_bfloat16 *>(l1_smem);  // two A tiles
+    constexpr int OW = FOUT == SITE16 ? 1 : 2;                       // 4-byte words of one complex output
+    uint32_t *out = reinterpret_cast<uint32_t *>(l1_smem + 2 * kLayerRows * kSingleCols * sizeof(__nv_bfloat16));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+    SingleField<false> f(g, tid);
+    SingleField<false>::pad(Sb, 2 * kLayerRows, tid);
+    // warp: three 16-row tiles from mt0 on, two output channels; the weights' fragments
+    const int mt0 = 3 * (warp >> 2), c0 = 2 * (warp & 3);
+    uint32_t bw[5][2][2];
+#pragma unroll
+    for (int q = 0; q < 5; q++)
+#pragma unroll
+        for (int j = 0; j < 2; j++)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {  // rows k = 16 q + 8 h + 2 tq (+1) = direction 2 q + h, column (c0 + j) 8 + gq
+                const int d = 2 * q + h;
+                bw[q][j][h] = d < 9 ? *reinterpret_cast<const uint32_t *>(Bt + ((long)d * 64 + (c0 + j) * 8 + gq) * 16 + 2 * tq) : 0u;
+            }
+    int n;
+    bool in;
+    if ((int)blockIdx.x < ntiles) f.load(g, x, U, blockIdx.x, tid, n, in);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        __nv_bfloat16 *Ss = Sb + buf * kLayerRows * kSingleCols;
+        f.put(Ss, tid);
+        if (tile + (int)gridDim.x < ntiles) f.load(g, x, U, tile + gridDim.x, tid, n, in);
+        __syncthreads();  // the A tile is whole; the previous tile's output has left
+        float acc[3][2][4];
+#pragma unroll
+        for (int t = 0; t < 3; t++) {
+#pragma unroll
+            for (int j = 0; j < 2; j++) acc[t][j][0] = acc[t][j][1] = acc[t][j][2] = acc[t][j][3] = 0.f;
+#pragma unroll
+            for (int q = 0; q < 5; q++) {
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4(Ss + ((mt0 + t) * 16 + (lane & 15)) * kSingleCols + q * 16 + (lane >> 4) * 8, a0, a1, a2, a3);
+                mma_bf16(acc[t][0], a0, a1, a2, a3, bw[q][0][0], bw[q][0][1]);
+                mma_bf16(acc[t][1], a0, a1, a2, a3, bw[q][1][0], bw[q][1][1]);
+            }
+            // (row, column pair) -> [channel][site][spin 3 + colour], spin tq
+#pragma unroll
+            for (int j = 0; j < 2; j++)
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int r = (mt0 + t) * 16 + gq + 8 * h;
+                    uint32_t *o = out + ((c0 + j) * kLayerSites * 12 + (r / 3) * 12 + tq * 3 + r % 3) * OW;
+                    if constexpr (FOUT == SITE16) *o = pack_bf16(acc[t][j][2 * h], acc[t][j][2 * h + 1]);
+                    else *reinterpret_cast<float2 *>(o) = make_float2(acc[t][j][2 * h], acc[t][j][2 * h + 1]);
+                }
         }
         __syncthreads();
-        const int r0 = warp * 16;
-#pragma unroll
-        for (int k0 = 0; k0 < KDP; k0 += 16) {
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4(A + (r0 + (lane & 15)) * AS + k0 + (lane >> 4) * 8, a0, a1, a2, a3);
-#pragma unroll
-            for (int j = 0; j + 1 < NT; j += 2) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4(B + (j * 8 + (lane >> 4) * 8 + (lane & 7)) * AS + k0 + ((lane >> 3) & 1) * 8, b0, b1, b2, b3);
-                mma_bf16(acc[j], a0, a1, a2, a3, b0, b1);
-                mma_bf16(acc[j + 1], a0, a1, a2, a3, b2, b3);
-            }
-            if constexpr (NT % 2 == 1) {
-                uint32_t b0, b1;
-                ldsm_x2(B + ((NT - 1) * 8 + (lane & 7)) * AS + k0 + ((lane >> 3) & 1) * 8, b0, b1);
-                mma_bf16(acc[NT - 1], a0, a1, a2, a3, b0, b1);
-            }
-        }
-    }
-    // epilogue: accumulator (row, column pair) -> output channel, spin, colour (complex)
-#pragma unroll
-    for (int j = 0; j < NT; j++) {
-        const int col = j * 8 + 2 * tq;  // even: the (re, im) pair of one complex output
-        const int c = col / 8, al = (col % 8) / 2;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int r = warp * 16 + gq + 8 * h;
-            const long n = (long)n0 + r / 3;
-            if (n < g.V) act_st<FOUT>(y, g.V, c, n, al * 3 + r % 3, make_float2(acc[j][2 * h], acc[j][2 * h + 1]));
+        constexpr int W16 = 3 * OW;  // 16-byte words per site and channel
+        for (int i = tid; i < 8 * kLayerSites * W16; i += kTileThreads) {
+            const int c = i / (kLayerSites * W16), r = i % (kLayerSites * W16);
+            const long at = ((long)c * g.V + (long)tile * kLayerSites) * W16 + r;
+            if ((long)tile * kLayerSites + r / W16 < g.V)
+                static_cast<uint4 *>(y)[at] = reinterpret_cast<const uint4 *>(out)[i];
         }
     }
 }
@@ -477,80 +492,197 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 2) k_layer_wfirst(void *y, c
     }
 }
 
-// P[d][k][j] += sum over rows of A_d[row][k] G[row][j]  (real; A from x, G from the output gradient)
-template <int CIN, int COUT, int FIN>
-__global__ void __launch_bounds__(kLayerWarps * 32) k_wgrad(float *__restrict__ P, const void *x,
-                                                            const float2 *__restrict__ G,
-                                                            const float2 *__restrict__ U, Geo g, int ntiles) {
-    constexpr int KD = CIN * 8, KDP = KD < 16 ? 16 : KD, N = COUT * 8, NM = KDP / 16, NT = N / 8;
-    constexpr int NW = kLayerWarps, PAIRS = NM * NT, PW = (PAIRS + NW - 1) / NW;  // (m-tile, n-tile) pairs per warp
-    constexpr int AS = KDP + 8, RS = kLayerRows + 8;
-    // dynamic shared memory: A [rows][AS] as built, At [KDP][RS] transposed for the MMA, Gt [N][RS]
-    extern __shared__ __align__(16) unsigned char wg_smem[];
-    auto A = reinterpret_cast<__nv_bfloat16(*)[AS]>(wg_smem);
-    auto At = reinterpret_cast<__nv_bfloat16(*)[RS]>(wg_smem + sizeof(__nv_bfloat16) * kLayerRows * AS);
-    auto Gt = reinterpret_cast<__nv_bfloat16(*)[RS]>(wg_smem + sizeof(__nv_bfloat16) * (kLayerRows * AS + KDP * RS));
+// The weight gradient: P[d][k][j] += sum over rows (site, colour) of A_d[row][k] G[row][j] (real; A_d the
+// transported inputs, G the output gradient), of which k_wgrad_finish takes conj(A) G.  Both operands lie
+// in shared memory row by row as BF16 and meet in mma.sync with the reduction over the rows, their
+// fragments transposed by ldmatrix; a persistent CTA keeps all nine directions' sums in registers
+// over its tiles of 64 sites.
+__device__ __forceinline__ void ldsm_x4_t(const void *p, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(sa)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm_x2_t(const void *p, uint32_t &r0, uint32_t &r1) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(sa) : "memory");
+}
+// The layers with one channel on one side.  Only that side is transported: with T_d^dag = T_e, e the
+// opposite direction, sum_n conj(T_d x)(n) G(n) = sum_m conj(x(m)) (T_e G)(m).  S: the one-channel field
+// (FP32), transported in all nine directions into 72 columns; H: the eight-channel field, 64 columns, as
+// it is.  FLIP = false: S is the layer's input, P[d][16][64]; true: S is the output gradient,
+// P[d][64][8], column group d transported by T_e.  The next tile's fields are loaded while this one is
+// multiplied.  Bound by those loads' latency at 16 warps per SM.  24^3x48: 0.23 (one input channel) and
+// 0.21 ms (one output channel), against 2.5 and 3.2 ms with the operands gathered and transposed anew
+// for each direction and, for the latter, all eight inputs transported.
+constexpr int kWgHS = 72;  // BF16 per row of H: no ldmatrix bank conflicts
+constexpr int kWgTile = kLayerRows * (kSingleCols + kWgHS);
+template <bool FLIP, int FH>
+__global__ void __launch_bounds__(kTileThreads, 1) k_wgrad_single(float *__restrict__ P, const float4 *__restrict__ S,
+                                                                  const void *__restrict__ H,
+                                                                  const float2 *__restrict__ U, Geo g, int ntiles) {
+    extern __shared__ __align__(16) __nv_bfloat16 ws_smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
-    for (int i = tid; i < kLayerRows * AS; i += NW * 32) (&A[0][0])[i] = __float2bfloat16(0.f);
-    for (int d = 0; d < 9; d++) {
-        float acc[PW][4];
+    const int st = tid & (kLayerSites - 1), ch = tid >> 6;
+    SingleField<FLIP> f(g, tid);
+    SingleField<FLIP>::pad(ws_smem, kLayerRows, tid);
+    SingleField<FLIP>::pad(ws_smem + kWgTile, kLayerRows, tid);
+    float2 hv[12];
+    uint4 hw[3];
+    auto load = [&](int tile) {
+        int n;
+        bool in;
+        f.load(g, S, U, tile, tid, n, in);
+        if constexpr (FH == SITE16) {
+            const uint4 *q = reinterpret_cast<const uint4 *>(H) + ((long)ch * g.V + n) * 3;
 #pragma unroll
-        for (int q = 0; q < PW; q++) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            const long n0 = (long)tile * kLayerSites;
-            __syncthreads();
-            if (tid < kLayerRows) {
-                const int r = tid;
-                const long n = n0 + r / 3;
-                if (n < g.V) {
-                    transport_row<CIN, FIN>(x, U, g, d, n, r % 3, &A[r][0]);
-                } else {
-                    for (int k = 0; k < KD; k++) A[r][k] = __float2bfloat16(0.f);
-                }
-                // output gradient row (n, a): COUT x 4 complex
-                for (int c = 0; c < COUT; c++)
+            for (int t = 0; t < 3; t++) hw[t] = in ? __ldg(q + t) : make_uint4(0, 0, 0, 0);
+        } else {
+            load_spinor(static_cast<const float4 *>(H) + (long)ch * g.V * 6, n, hv);
+            if (!in)
 #pragma unroll
-                    for (int al = 0; al < 4; al++) {
-                        const float2 v = n < g.V ? G[((long)c * g.V + n) * 12 + al * 3 + r % 3] : make_float2(0.f, 0.f);
-                        Gt[(c * 4 + al) * 2][r] = __float2bfloat16(v.x);
-                        Gt[(c * 4 + al) * 2 + 1][r] = __float2bfloat16(v.y);
-                    }
-            }
-            __syncthreads();
-            for (int i = tid; i < kLayerRows * KDP; i += NW * 32) {
-                const int r = i % kLayerRows, k = i / kLayerRows;
-                At[k][r] = A[r][k];
-            }
-            __syncthreads();
-#pragma unroll
-            for (int r0 = 0; r0 < kLayerRows; r0 += 16) {
-#pragma unroll
-                for (int q = 0; q < PW; q++) {
-                    const int pr = warp + NW * q;
-                    if (pr >= PAIRS) break;
-                    const int m0 = (pr / NT) * 16, j0 = (pr % NT) * 8;
-                    const uint32_t a0 = *reinterpret_cast<const uint32_t *>(&At[m0 + gq][r0 + 2 * tq]);
-                    const uint32_t a1 = *reinterpret_cast<const uint32_t *>(&At[m0 + gq + 8][r0 + 2 * tq]);
-                    const uint32_t a2 = *reinterpret_cast<const uint32_t *>(&At[m0 + gq][r0 + 2 * tq + 8]);
-                    const uint32_t a3 = *reinterpret_cast<const uint32_t *>(&At[m0 + gq + 8][r0 + 2 * tq + 8]);
-                    const uint32_t b0 = *reinterpret_cast<const uint32_t *>(&Gt[j0 + gq][r0 + 2 * tq]);
-                    const uint32_t b1 = *reinterpret_cast<const uint32_t *>(&Gt[j0 + gq][r0 + 2 * tq + 8]);
-                    mma_bf16(acc[q], a0, a1, a2, a3, b0, b1);
-                }
-            }
+                for (int k = 0; k < 12; k++) hv[k] = make_float2(0.f, 0.f);
         }
+    };
+    float acc[5][4];
 #pragma unroll
-        for (int q = 0; q < PW; q++) {
-            const int pr = warp + NW * q;
-            if (pr >= PAIRS) break;
-            const int m0 = (pr / NT) * 16, j0 = (pr % NT) * 8;
-            float *Pd = P + (long)d * KDP * N;
-            atomicAdd(&Pd[(m0 + gq) * N + j0 + 2 * tq], acc[q][0]);
-            atomicAdd(&Pd[(m0 + gq) * N + j0 + 2 * tq + 1], acc[q][1]);
-            atomicAdd(&Pd[(m0 + gq + 8) * N + j0 + 2 * tq], acc[q][2]);
-            atomicAdd(&Pd[(m0 + gq + 8) * N + j0 + 2 * tq + 1], acc[q][3]);
+    for (int q = 0; q < 5; q++) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
+    if ((int)blockIdx.x < ntiles) load(blockIdx.x);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        __nv_bfloat16 *Ss = ws_smem + buf * kWgTile, *Hs = Ss + kLayerRows * kSingleCols;
+        f.put(Ss, tid);
+        if constexpr (FH == SITE16) {
+            const uint32_t w[12] = {hw[0].x, hw[0].y, hw[0].z, hw[0].w, hw[1].x, hw[1].y,
+                                    hw[1].z, hw[1].w, hw[2].x, hw[2].y, hw[2].z, hw[2].w};
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                *reinterpret_cast<uint4 *>(Hs + (3 * st + a) * kWgHS + ch * 8) = make_uint4(w[a], w[3 + a], w[6 + a], w[9 + a]);
+        } else {
+            put_rows(Hs + 3 * st * kWgHS + ch * 8, kWgHS, hv);
+        }
+        if (tile + (int)gridDim.x < ntiles) load(tile + gridDim.x);
+        __syncthreads();  // this buffer is whole; the other one's products are done
+        // warp: eight H columns, half of the rows
+        const int n0 = (warp & 7) * 8, rb = (warp >> 3) * (kLayerRows / 2);
+#pragma unroll
+        for (int r0 = rb; r0 < rb + kLayerRows / 2; r0 += 16) {
+            uint32_t b0, b1;
+            ldsm_x2_t(Hs + (r0 + (lane & 15)) * kWgHS + n0, b0, b1);
+#pragma unroll
+            for (int q = 0; q < 5; q++) {
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4_t(Ss + (r0 + (lane & 7) + (lane >> 4) * 8) * kSingleCols + q * 16 + ((lane >> 3) & 1) * 8, a0, a1, a2, a3);
+                mma_bf16(acc[q], a0, a1, a2, a3, b0, b1);
+            }
         }
     }
+#pragma unroll
+    for (int q = 0; q < 5; q++)
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int row = q * 16 + gq + 8 * (e >> 1), h = (warp & 7) * 8 + 2 * tq + (e & 1);
+            if (row < 72)
+                atomicAdd(FLIP ? &P[(row >> 3) * 512 + h * 8 + (row & 7)] : &P[(row >> 3) * 1024 + (row & 7) * 64 + h], acc[q][e]);
+        }
+}
+
+// The 8 -> 8 layer: per direction the neighbour inputs and links of a tile are staged with cp.async one
+// direction ahead, one thread per (site, channel) transports them into the A rows, and each warp
+// multiplies a 16 x 16 piece of P_d.  G is staged once for all nine directions.  24^3x48: 1.5 ms, against
+// 4.2 ms with G gathered and both operands transposed in shared memory for every direction.
+struct Wg88 {
+    static constexpr int XS = 8 * 48 + 16, AS = 72;  // bytes per staged site, BF16 per A or G row
+    static constexpr size_t x_bytes = (size_t)kLayerSites * XS, l_bytes = (size_t)kLayerSites * 9 * sizeof(float2);
+    static constexpr size_t stage = x_bytes + l_bytes, a_bytes = (size_t)kLayerRows * AS * sizeof(__nv_bfloat16);
+    static constexpr size_t total = 2 * stage + 2 * a_bytes + (size_t)9 * kLayerSites * (sizeof(int) + sizeof(float));
+};
+__global__ void __launch_bounds__(kTileThreads, 1) k_wgrad88(float *__restrict__ P, const void *__restrict__ x,
+                                                           const float4 *__restrict__ G, const float2 *__restrict__ U,
+                                                           Geo g, int ntiles) {
+    extern __shared__ __align__(16) unsigned char wg_smem[];
+    __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16 *>(wg_smem + 2 * Wg88::stage), *Gs = A + kLayerRows * Wg88::AS;
+    int *nbt = reinterpret_cast<int *>(wg_smem + 2 * Wg88::stage + 2 * Wg88::a_bytes);
+    float *sgt = reinterpret_cast<float *>(nbt + 9 * kLayerSites);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+    const int V = (int)g.V, st = tid >> 3, ch = tid & 7;
+    const int m0 = (warp & 3) * 16, j0 = (warp >> 2) * 16;
+    float acc[9][2][4];
+#pragma unroll
+    for (int d = 0; d < 9; d++)
+#pragma unroll
+        for (int q = 0; q < 2; q++) acc[d][q][0] = acc[d][q][1] = acc[d][q][2] = acc[d][q][3] = 0.f;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int n0 = tile * kLayerSites;
+        auto issue = [&](int d) {
+            unsigned char *X = wg_smem + (d & 1) * Wg88::stage;
+            float2 *L = reinterpret_cast<float2 *>(X + Wg88::x_bytes);
+            const int *nb = nbt + d * kLayerSites;
+#pragma unroll
+            for (int q = 0; q < 3; q++) {  // 64 sites x 8 channels x 3 words of 16 bytes, sites fastest
+                const int i = tid + q * kTileThreads, c = i / (3 * kLayerSites), r = i % (3 * kLayerSites), s = r / 3, k = r % 3;
+                const int m = nb[s];
+                cp_async16z(X + s * Wg88::XS + c * 48 + k * 16,
+                            static_cast<const unsigned char *>(x) + ((long)c * V + (m < 0 ? 0 : m)) * 48 + k * 16, m >= 0);
+            }
+            if (d > 0) {
+                const int mu = (d - 1) >> 1;
+                const bool fwd = ((d - 1) & 1) == 0;
+                for (int i = tid; i < kLayerSites * 9; i += kTileThreads) {
+                    const int s = i % kLayerSites, e = i / kLayerSites;
+                    const int m = nb[s], ls = fwd ? n0 + s : m;
+                    cp_async8z(L + s * 9 + e, U + (long)(mu * 9 + e) * V + (m < 0 ? 0 : ls), m >= 0);
+                }
+            }
+            cp_commit();
+        };
+        __syncthreads();  // the previous tile's tables and operands are done with
+        layer_neighbours(nbt, sgt, g, n0, tid);
+        float2 gv[12];
+        {
+            const int n = n0 + st;
+            load_spinor(G + (long)ch * V * 6, n < V ? n : 0, gv);
+            if (n >= V)
+#pragma unroll
+                for (int k = 0; k < 12; k++) gv[k] = make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        issue(0);
+        put_rows(Gs + 3 * st * Wg88::AS + ch * 8, Wg88::AS, gv);
+#pragma unroll
+        for (int d = 0; d < 9; d++) {
+            cp_wait<0>();
+            __syncthreads();  // stage d visible; the products of direction d - 1 are done
+            if (d + 1 < 9) issue(d + 1);
+            const unsigned char *X = wg_smem + (d & 1) * Wg88::stage;
+            const float2 *L = reinterpret_cast<const float2 *>(X + Wg88::x_bytes);
+            constexpr int kind[9] = {0, 1, 2, 1, 2, 1, 2, 3, 4};
+            const float sg = sgt[d * kLayerSites + st];
+            __nv_bfloat16 *row = A + 3 * st * Wg88::AS;
+            if (kind[d] == 0) transport_item<8, 1, SITE16, 0>(X + st * Wg88::XS, L + st * 9, sg, row, ch, Wg88::AS);
+            else if (kind[d] == 1) transport_item<8, 1, SITE16, 1>(X + st * Wg88::XS, L + st * 9, sg, row, ch, Wg88::AS);
+            else if (kind[d] == 2) transport_item<8, 1, SITE16, 2>(X + st * Wg88::XS, L + st * 9, sg, row, ch, Wg88::AS);
+            else if (kind[d] == 3) transport_item<8, 1, SITE16, 3>(X + st * Wg88::XS, L + st * 9, sg, row, ch, Wg88::AS);
+            else transport_item<8, 1, SITE16, 4>(X + st * Wg88::XS, L + st * 9, sg, row, ch, Wg88::AS);
+            __syncthreads();
+#pragma unroll 4
+            for (int r0 = 0; r0 < kLayerRows; r0 += 16) {
+                uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
+                ldsm_x4_t(A + (r0 + (lane & 7) + (lane >> 4) * 8) * Wg88::AS + m0 + ((lane >> 3) & 1) * 8, a0, a1, a2, a3);
+                ldsm_x4_t(Gs + (r0 + (lane & 15)) * Wg88::AS + j0 + (lane >> 4) * 8, b0, b1, b2, b3);
+                mma_bf16(acc[d][0], a0, a1, a2, a3, b0, b1);
+                mma_bf16(acc[d][1], a0, a1, a2, a3, b2, b3);
+            }
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 9; d++)
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                atomicAdd(&P[d * 4096 + (m0 + gq + 8 * (e >> 1)) * 64 + j0 + q * 8 + 2 * tq + (e & 1)], acc[d][q][e]);
 }
 
 // B matrices (BF16, [9][N][KDP]) of a layer from its complex weights W [9][cout][cin][4][4];
@@ -676,22 +808,29 @@ Geo geo(const qcd_ctx *c) {
     return g;
 }
 
-template <int CIN, int COUT, int FIN, int FOUT>
-int launch_layer(qcd_ctx *c, void *y, const void *x, const __nv_bfloat16 *Bt, const BicgScalars *gate = nullptr) {
-    constexpr size_t smem = LayerSmem<CIN, COUT, FIN>::total;
+// CTAs of a persistent kernel: one per SM (fewer tiles: one each)
+int tile_grid(const qcd_ctx *c, int tiles) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
+        cudaGetLastError();
+        sms = 1;
+    }
+    return std::min(tiles, std::max(1, sms));
+}
+template <int FOUT>
+int launch_layer_single(qcd_ctx *c, void *y, const float4 *x, const __nv_bfloat16 *Bt, const BicgScalars *gate = nullptr) {
+    constexpr size_t smem = 2 * kLayerRows * kSingleCols * sizeof(__nv_bfloat16) + 8 * kLayerSites * (FOUT == SITE16 ? 48 : 96);
     static std::atomic<unsigned long long> attr{0};
     static std::mutex attr_mu;
     if (int arc = once_per_device(attr, attr_mu, c->device, [&]() -> int {
-            QCD_CUDA(c, cudaFuncSetAttribute(k_layer<CIN, COUT, FIN, FOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem));
+            QCD_CUDA(c, cudaFuncSetAttribute(k_layer_single<FOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             return QCD_OK;
         }))
         return arc;
-    const long tiles = (c->lat.V + kLayerSites - 1) / kLayerSites;
+    const int tiles = (int)((c->lat.V + kLayerSites - 1) / kLayerSites);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_LEARNED, &ev);
-    k_layer<CIN, COUT, FIN, FOUT><<<(unsigned)tiles, kLayerWarps * 32, smem, c->stream>>>(y, x, c->U32, Bt, geo(c),
-                                                                                       gate);
+    k_layer_single<FOUT><<<tile_grid(c, tiles), kTileThreads, smem, c->stream>>>(y, x, c->U32, Bt, geo(c), tiles, gate);
     return prof_end(c, QCD_K_LEARNED, ev);
 }
 
@@ -715,22 +854,34 @@ int launch_layer_wfirst(qcd_ctx *c, void *y, const void *x, const __nv_bfloat16 
     return prof_end(c, QCD_K_LEARNED, ev);
 }
 
-template <int CIN, int COUT, int FIN>
-int launch_wgrad(qcd_ctx *c, float *P, const void *x, const float2 *G) {
-    constexpr int KD = CIN * 8, KDP = KD < 16 ? 16 : KD, N = COUT * 8;
-    constexpr size_t smem = sizeof(__nv_bfloat16) * ((size_t)kLayerRows * (KDP + 8) + (size_t)(KDP + N) * (kLayerRows + 8));
+// P zeroed by the caller
+template <bool FLIP, int FH> int launch_wgrad_single(qcd_ctx *c, float *P, const float4 *S, const void *H) {
+    constexpr size_t smem = 2 * kWgTile * sizeof(__nv_bfloat16);
     static std::atomic<unsigned long long> attr{0};
     static std::mutex attr_mu;
     if (int arc = once_per_device(attr, attr_mu, c->device, [&]() -> int {
-            QCD_CUDA(c, cudaFuncSetAttribute(k_wgrad<CIN, COUT, FIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            QCD_CUDA(c, cudaFuncSetAttribute(k_wgrad_single<FLIP, FH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             return QCD_OK;
         }))
         return arc;
     const int tiles = (int)((c->lat.V + kLayerSites - 1) / kLayerSites);
-    const int grid = tiles < 304 ? tiles : 304;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_LEARNED, &ev);
-    k_wgrad<CIN, COUT, FIN><<<grid, kLayerWarps * 32, smem, c->stream>>>(P, x, G, c->U32, geo(c), tiles);
+    k_wgrad_single<FLIP, FH><<<tile_grid(c, tiles), kTileThreads, smem, c->stream>>>(P, S, H, c->U32, geo(c), tiles);
+    return prof_end(c, QCD_K_LEARNED, ev);
+}
+int launch_wgrad88(qcd_ctx *c, float *P, const void *x, const float4 *G) {
+    static std::atomic<unsigned long long> attr{0};
+    static std::mutex attr_mu;
+    if (int arc = once_per_device(attr, attr_mu, c->device, [&]() -> int {
+            QCD_CUDA(c, cudaFuncSetAttribute(k_wgrad88, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wg88::total));
+            return QCD_OK;
+        }))
+        return arc;
+    const int tiles = (int)((c->lat.V + kLayerSites - 1) / kLayerSites);
+    cudaEvent_t ev;
+    prof_begin(c, QCD_K_LEARNED, &ev);
+    k_wgrad88<<<tile_grid(c, tiles), kTileThreads, Wg88::total, c->stream>>>(P, x, G, c->U32, geo(c), tiles);
     return prof_end(c, QCD_K_LEARNED, ev);
 }
 
@@ -842,7 +993,7 @@ int learned_forward(qcd_ctx *c, float4 *y, const float4 *x, const BicgScalars *g
     if (!L.ready) return fail(c, QCD_ERR_STATE, "no learned weights set");
     int rc = ensure_net(c);
     if (rc) return rc;
-    if ((rc = launch_layer<1, 8, SITE32, SITE16>(c, L.a1, x, L.B + layer_boff(0, false), gate))) return rc;
+    if ((rc = launch_layer_single<SITE16>(c, L.a1, x, L.B + layer_boff(0, false), gate))) return rc;
     if ((rc = learned_layer_tc(c, L.a2, L.a1, L.B + layer_boff(1, false), false, gate))) return rc;
     return launch_layer_wfirst<8, SITE16, SITE32>(c, y, L.a2, L.B + layer_boff(2, false), gate);
 }
@@ -874,11 +1025,11 @@ int learned_loss_grad(qcd_ctx *c, const float4 *rho, const float2 *eps, double *
                                                                             kLearnedChans[l], kLearnedChans[l + 1]);
         return prof_end(c, QCD_K_LEARNED, e2);
     };
-    if ((rc = wgrad_layer(2, [&]() { return launch_wgrad<8, 1, SITE16>(c, L.P, L.a2, L.g3); }))) return rc;
-    if ((rc = launch_layer<1, 8, SITE32, SITE32>(c, L.g2, L.g3, L.B + layer_boff(2, true)))) return rc;
-    if ((rc = wgrad_layer(1, [&]() { return launch_wgrad<8, 8, SITE16>(c, L.P, L.a1, L.g2); }))) return rc;
+    if ((rc = wgrad_layer(2, [&]() { return launch_wgrad_single<true, SITE16>(c, L.P, (const float4 *)L.g3, L.a2); }))) return rc;
+    if ((rc = launch_layer_single<SITE32>(c, L.g2, (const float4 *)L.g3, L.B + layer_boff(2, true)))) return rc;
+    if ((rc = wgrad_layer(1, [&]() { return launch_wgrad88(c, L.P, L.a1, (const float4 *)L.g2); }))) return rc;
     if ((rc = learned_layer_tc(c, L.g1, L.g2, L.B + layer_boff(1, true), true))) return rc;
-    if ((rc = wgrad_layer(0, [&]() { return launch_wgrad<1, 8, SITE32>(c, L.P, rho, L.g1); }))) return rc;
+    if ((rc = wgrad_layer(0, [&]() { return launch_wgrad_single<false, SITE32>(c, L.P, rho, L.g1); }))) return rc;
     if (loss_out) {
         double h = 0;
         QCD_CUDA(c, cudaMemcpyAsync(&h, L.scal, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

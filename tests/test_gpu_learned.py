@@ -93,6 +93,31 @@ def test_loss_and_gradient_vs_oracle():
     s.close()
 
 
+@pytest.mark.parametrize("dims,bc_t", [((3, 5, 2, 7), -1),      # one site more than three 64-site tiles, odd extents
+                                       ((2, 2, 2, 4), 1),       # half a tile, forward = backward neighbour
+                                       ((10, 11, 9, 12), -1)])  # more tiles than SMs: the persistent loop
+def test_forward_and_gradient_ragged(dims, bc_t):
+    """Tiles that the volume does not fill, the time boundary sign, several tiles per CTA; every layer's
+    weight gradient by itself."""
+    s, U = setup(dims)
+    s.set_boundary(bc_t)
+    W = q.learned_init_weights(21, scale_last=0.5)
+    q.qcd_learned_set_weights(s.ctx, W)
+    rho, eps = qi.gaussian_spinor(dims, seed=22), qi.gaussian_spinor(dims, seed=23)
+    out = np.empty((qi.volume(dims), 4, 3), dtype=np.complex64)
+    q.qcd_learned_apply(s.ctx, out, rho[0].astype(np.complex64))
+    ref = oracle.learned_forward(dims, U, CH, W.astype(np.complex128), rho, bc_t)[0]
+    assert rel_norm(out.astype(np.complex128), ref) <= 2e-2
+    loss, grad = q.qcd_learned_loss_grad(s.ctx, rho[0].astype(np.complex64), eps[0].astype(np.complex64))
+    rloss, rgrad = oracle.learned_loss_grad(dims, U, CH, W.astype(np.complex128), rho, eps, bc_t)
+    assert abs(loss - rloss) <= 2e-2 * rloss
+    n1, n2 = 2 * 9 * 8 * 16, 2 * 9 * 64 * 16
+    rgrad = rgrad.ravel()
+    for a, b in ((0, n1), (n1, n1 + n2), (n1 + n2, len(grad))):
+        assert rel_norm(grad[a:b].astype(np.float64), rgrad[a:b]) <= 5e-2
+    s.close()
+
+
 def test_training_reduces_loss_and_solver_converges():
     dims = (8, 8, 8, 8)
     s, U = setup(dims)
