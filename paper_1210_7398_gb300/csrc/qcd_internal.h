@@ -73,9 +73,12 @@ struct SapPlan {
     int *d_own_off = nullptr;
     int *d_pos = nullptr;
     int *d_origin_site[2] = {nullptr, nullptr};
-    std::vector<int4> h_tile_pos;   // tile form: [vol][2] per level position (offset, slots, site)
+    std::vector<int4> h_tile_pos;   // tile form: [2][vol][2] per pass, level position and lane of a pair
     int4 *d_tile_pos = nullptr;
-    int *d_lev_ptr = nullptr;       // tile form: [nsteps + 1] level boundaries (h_step_ptr)
+    std::vector<int> h_tile_site;   // tile form: [vol] block-local site of a level position, [vol] its coordinates
+    int *d_tile_site = nullptr;
+    std::vector<int4> h_tile_item;  // tile form: [4][nsteps] the levels' positions and warps, R = 1, 2, 4, 8
+    int4 *d_tile_item = nullptr;
     int tile_zslots = 1;            // tile form: zero slots after the vol site slots
     float *d_rec = nullptr;         // per-site records (links, clover, neighbour codes), V x 912 bytes
     long rec_version = -1;          // field version the records were built from
@@ -280,7 +283,7 @@ size_t sap_record_bytes(const SapPlan &plan);
 int sap_build_records(qcd_ctx *c, SapPlan &plan, float *rec);
 
 // RHS-tiled thread form of the SAP cycle (ssor_tile.cu): one CTA per (block, tile of up to
-// kTileMaxRhs right-hand sides), one thread per site update, the block spinors of the tile in
+// kTileMaxRhs right-hand sides), two lanes per site update, the block spinors of the tile in
 // shared memory; per-site records of kTileRecordBytes (FP32) / kTileRecordBytesHalf (FP16)
 constexpr int kTileMaxThreads = 256;
 constexpr int kTileMinBlocks = 2;  // resident CTAs per SM the register allocation is made for (128 registers)
@@ -297,6 +300,8 @@ size_t tile_smem_bytes(const SapPlan &p, int R);
 // tile form: h_tile_pos from the level schedule, the positions of a level ordered against
 // shared-memory bank conflicts (needs h_step_site, h_step_ptr, h_site_off, b, vol, half)
 void tile_make_positions(SapPlan &p);
+// tile form: h_tile_item, how the items of the levels are dealt to the warps (needs h_step_ptr)
+void tile_level_table(SapPlan &p);
 // the host check of h_tile_pos that the tile kernel relies on for in-bounds shared memory
 bool tile_positions_valid(const SapPlan &p);
 int tile_build_records(qcd_ctx *c, const SapPlan &p, void *rec);

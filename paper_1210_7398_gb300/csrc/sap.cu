@@ -1390,6 +1390,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
             tile_make_positions(np);
             if (tile_positions_valid(np) && tile_smem_bytes(np, 1) <= kTileSmemLimit) {
                 np.tile = true;
+                tile_level_table(np);
                 np.nwarps = 0;
                 np.smem_bytes = tile_smem_bytes(np, 1);
                 make_flags(np);
@@ -1453,7 +1454,8 @@ size_t sap_table_bytes(const SapPlan &p) {
            up16(sizeof(int) * p.h_chunk_ptr.size()) + up16(sizeof(int2) * p.h_chunk_site.size()) +
            up16(sizeof(int) * p.h_site_off.size()) + up16(p.h_flags.size()) + up16(sizeof(int) * p.h_own.size()) +
            up16(sizeof(int) * p.h_own_off.size()) + up16(sizeof(int) * p.h_pos.size()) +
-           up16(sizeof(int4) * p.h_tile_pos.size()) + (p.tile ? up16(sizeof(int) * p.h_step_ptr.size()) : 0);
+           up16(sizeof(int4) * p.h_tile_pos.size()) +
+           (p.tile ? up16(sizeof(int) * p.h_tile_site.size()) + up16(sizeof(int4) * p.h_tile_item.size()) : 0);
 }
 
 // Copies every table of the plan into one device region (sap_table_bytes long) on the
@@ -1484,10 +1486,11 @@ int sap_upload_tables(qcd_ctx *c, SapPlan &p, void *region) {
     p.d_own_off = (int *)put(p.h_own_off.data(), sizeof(int) * p.h_own_off.size());
     p.d_pos = p.h_pos.empty() ? nullptr : (int *)put(p.h_pos.data(), sizeof(int) * p.h_pos.size());
     p.d_tile_pos = p.tile ? (int4 *)put(p.h_tile_pos.data(), sizeof(int4) * p.h_tile_pos.size()) : nullptr;
-    p.d_lev_ptr = p.tile ? (int *)put(p.h_step_ptr.data(), sizeof(int) * p.h_step_ptr.size()) : nullptr;
+    p.d_tile_site = p.tile ? (int *)put(p.h_tile_site.data(), sizeof(int) * p.h_tile_site.size()) : nullptr;
+    p.d_tile_item = p.tile ? (int4 *)put(p.h_tile_item.data(), sizeof(int4) * p.h_tile_item.size()) : nullptr;
     if (!p.d_origin[0] || !p.d_origin[1] || !p.d_origin_site[0] || !p.d_origin_site[1] || !p.d_chunk_ptr ||
         !p.d_chunk_site || !p.d_site_off || !p.d_flags || !p.d_own || !p.d_own_off || (p.thread && !p.d_pos) ||
-        (p.tile && (!p.d_tile_pos || !p.d_lev_ptr)))
+        (p.tile && (!p.d_tile_pos || !p.d_tile_site || !p.d_tile_item)))
         return cuda_fail(c, cudaGetLastError(), "cudaMemcpyAsync(SAP tables)");
     // the host vectors may be released only once the copies have consumed them
     QCD_CUDA(c, cudaStreamSynchronize(c->stream));

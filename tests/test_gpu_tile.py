@@ -76,6 +76,65 @@ def test_tile_sap_vs_oracle(case):
     s.close()
 
 
+EDGE_CASES = [
+    # dims, block, subblock, omega, nsweep, nsap: one level (a block of one site), two levels, volumes that no
+    # warp item or bank class divides, more levels than warps, one sweep, and three
+    ((4, 4, 4, 4), (1, 1, 1, 1), (1, 1, 1, 1), 1.2, 2, 2),
+    ((4, 4, 4, 4), (2, 1, 1, 1), (1, 1, 1, 1), 1.2, 2, 2),
+    ((6, 4, 6, 10), (3, 2, 3, 5), (3, 2, 3, 5), 1.1, 1, 1),
+    ((6, 10, 2, 14), (3, 5, 1, 7), (1, 5, 1, 7), 0.9, 3, 2),
+    ((12, 4, 4, 8), (6, 2, 2, 4), (2, 2, 1, 2), 1.3, 2, 1),
+]
+
+
+@pytest.mark.parametrize("st", ["f32", "f16"])
+@pytest.mark.parametrize("case", EDGE_CASES, ids=lambda c: "x".join(map(str, c[0])) + "_b" + "x".join(map(str, c[1])))
+def test_tile_edges_vs_oracle(case, st):
+    """Antiperiodic in t, three right-hand sides (one tile of two and one half empty), against the oracle
+    to the tolerances of the cases above."""
+    dims, b, sb, omega, nsweep, nsap = case
+    kappa = 0.12
+    U = qi.gauge_field(dims, 0.3, seed=1003)
+    s = q.Solver(dims)
+    s.set_boundary(-1)
+    s.load_gauge(torch.from_numpy(U).cuda())
+    s.build_clover(kappa, CSW)
+    _, F = oracle.clover(dims, U, CSW, kappa)
+    v = qi.gaussian_spinor(dims, seed=2003, nrhs=3)
+    v[1] *= 1e-6  # scales apart: each right-hand side has its own
+    prm = q.make_params(kappa, CSW, b, sb, omega=omega, nsweep=nsweep, nsap=nsap, sap_storage=storage(st), sap_ctas=-2,
+                        bc_t=-1)
+    vin = torch.from_numpy(v.astype(np.complex64)).cuda()
+    out = torch.empty_like(vin)
+    s.sap_precondition(out, vin, prm, nrhs=3)
+    torch.cuda.synchronize()
+    for k in range(3):
+        ref = oracle.sap(dims, U, F, kappa, b, sb, omega, nsweep, nsap, v[k], -1)
+        assert rel_norm(out[k].cpu().numpy().astype(np.complex128), ref) <= (1e-5 if st == "f32" else SAP_F16_TOL)
+    s.close()
+
+
+@pytest.mark.parametrize("st", ["f32", "f16"])
+def test_tile_uncached_sums_equal_cached(st):
+    """With 3^3 x 6 blocks in natural order (12 levels) on 24^4, seven CTAs share an SM for one right-hand
+    side and not every hop sum has a place in tensor memory; four right-hand sides leave room for
+    all.  The sums formed anew equal those kept, bit for bit."""
+    dims, b, kappa = (24, 24, 24, 24), (3, 3, 3, 6), 0.12
+    s = q.Solver(dims)
+    s.load_gauge(qi.gauge_field(dims, 0.3, seed=1004, device="cuda"))
+    s.build_clover(kappa, CSW)
+    v = qi.gaussian_spinor_torch(dims, 2004, 4, "cuda").to(torch.complex64).contiguous()
+    prm = q.make_params(kappa, CSW, b, b, omega=1.2, nsweep=2, nsap=2, sap_storage=storage(st), sap_ctas=-2)
+    out = torch.empty_like(v)
+    s.sap_precondition(out, v, prm, nrhs=4)
+    one = torch.empty_like(v[:1])
+    for k in (0, 3):
+        s.sap_precondition(one, v[k:k + 1].contiguous(), prm)
+        torch.cuda.synchronize()
+        assert torch.equal(one[0], out[k])
+    s.close()
+
+
 def test_tile_falls_back_where_the_block_does_not_fit():
     """A 6^3 x 12 block's FP32 spinor (249 KB) exceeds a CTA's shared memory: sap_ctas = -2 then
     runs the automatic cluster form, bit for bit."""
