@@ -202,7 +202,7 @@ int qcd_sap_precondition(qcd_ctx *ctx, float *out, const float *in, const qcd_pa
  * qcd_sap_precondition.  It calls no cudaMalloc, cudaFree or allocating
  * library routine: its scratch (four FP32 spinor fields, the per-site SSOR
  * records and the ll-schedule tables) is one fixed __device__ array of about
- * 68.3 MB that every GPU loading the library holds until the process exits.
+ * 66.4 MB that every GPU loading the library holds until the process exits.
  * Lattices above 41,472 sites (12^3 x 24) are rejected with QCD_ERR_ARG.  The
  * first call on a device looks up the array's device address
  * (cudaGetSymbolAddress), so make that first call before any stream capture.
@@ -248,28 +248,24 @@ int qcd_solve_multi(int n, qcd_ctx *const *ctxs, double *const *x, const double 
 int qcd_set_graphs(qcd_ctx *ctx, int on);
 
 /* Tuning knob of the SAP block kernel; results do not depend on it.  The
- * block solve has two forms.  The warp form runs 32 lanes (or 8, see
- * qcd_set_sap_form) per site update over
- * a cluster of C CTAs per block (C <= 16, each CTA owning an equal share of
- * every dependency level of the sweep and keeping its sites' spinors in its
- * shared memory, which must fit).  The thread form (FP32 storage, blocks whose
- * spinor fits one CTA) runs one thread per site update with the block's links
- * and clover field stored per block in level order.  min_ctas >= 1: the warp
- * form with the smallest such C >= min_ctas.  0 (default): the warp form with
- * the largest C in {1, 2, 4, 8} for which one colour's clusters still fit the
- * SM count (at least the smallest C that fits).  -1: the thread form where it
- * fits, else as 0.  More CTAs per block spread a level's sites over more SMs
- * at the price of more cluster barriers. */
+ * block solve has three forms.  The cluster form runs four lanes per site
+ * update over a cluster of C CTAs per block (C <= 16, each CTA owning an equal
+ * share of every dependency level of the sweep and keeping its sites' spinors
+ * in its shared memory, which must fit).  The thread form (FP32 storage, blocks
+ * whose spinor fits one CTA) runs one thread per site update with the block's
+ * links and clover field stored per block in level order.  The tile form
+ * (blocks whose spinor fits one CTA) runs two lanes per site update and several
+ * right-hand sides of a block in one CTA.  min_ctas >= 1: the cluster form with
+ * the smallest such C >= min_ctas.  0 (default): the cluster form with the
+ * largest C in {1, 2, 4, 8} for which one colour's clusters still fit the SM
+ * count (at least the smallest C that fits).  -1: the thread form where it fits,
+ * -2: the tile form where it fits, else as 0.  More CTAs per block spread a
+ * level's sites over more SMs at the price of more cluster barriers. */
 int qcd_set_sap_ctas(qcd_ctx *ctx, int min_ctas);
 
-/* Second tuning knob of the warp form above: lanes per site update.  form = 1:
- * 32 lanes (lane = hop direction and colour row, one update per warp); 2: 8
- * lanes (lane = hop direction, four updates per warp: about two thirds of the
- * issued instructions, but a quarter of the warps to hide latency); 0 (default):
- * per launch, the 8-lane form where the grid keeps at least 16 of its warps
- * resident per SM (many small blocks, several right-hand sides), else 32.
- * Both perform the same rounding steps in the same order: results are
- * identical bit for bit.  QCD_ERR_ARG outside 0..2. */
+/* Kept for callers that chose between 32 and 8 lanes per site update of the
+ * cluster form; it has one form now, so every value gives the same launches and
+ * the same bits.  QCD_ERR_ARG outside 0..2. */
 int qcd_set_sap_form(qcd_ctx *ctx, int form);
 
 /* Diagnostic, host only (needs no GPU and no context): the schedule of the
@@ -281,7 +277,9 @@ int qcd_set_sap_form(qcd_ctx *ctx, int form);
  * level of its in-block neighbours earlier in the ll order); each CTA of the
  * block's cluster owns some sites of every level; each level is cut into
  * chunks (timeline steps of the forward pass; the backward pass runs them in
- * reverse, step 2 nchunks - 1 - c for chunk c), and a barrier flag before a
+ * reverse, step 2 nchunks - 1 - c for chunk c; the cluster form runs consecutive
+ * chunks of a level as one step, with the flags of the same rule for its steps),
+ * and a barrier flag before a
  * step orders the steps that exchange data (1: CTA barrier, 2: cluster
  * barrier).  meta[8] receives: sites per block, levels, CTAs per block (C),
  * chunks, most sites of one CTA in one chunk, most sites one CTA owns,

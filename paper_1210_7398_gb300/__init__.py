@@ -253,7 +253,7 @@ def qcd_sap_plan_tables(dims, block, subblock, sap_ctas: int = 0, half: bool = F
 
 
 def qcd_set_sap_form(ctx, form: int):
-    """0: lanes per SSOR site update chosen per launch; 1: 32; 2: 8 (identical results)."""
+    """Kept for callers: the cluster form has one form; 0, 1 and 2 give the same launches."""
     return _check(ctx, load_library().qcd_set_sap_form(ctx, int(form)))
 
 

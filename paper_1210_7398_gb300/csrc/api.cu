@@ -493,8 +493,7 @@ int qcd_set_sap_form(qcd_ctx *c, int form) {
     int rc = ready(c);
     if (rc) return rc;
     if (form < 0 || form > 2) return fail(c, QCD_ERR_ARG, "form must lie in 0..2");
-    c->sap_form = form;
-    return QCD_OK;
+    return QCD_OK;  // the cluster form has one form
 }
 
 int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half, int sms,
@@ -510,6 +509,7 @@ int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subbloc
     c.sms_override = sms;
     SapPlan p;
     if (sap_plan_host(&c, block, subblock, p, sap_ctas, half != 0) != QCD_OK) return QCD_ERR_ARG;
+    sap_plan_flags(p);
     const int vals[8] = {p.vol, p.nsteps, p.C, p.nchunks, p.nslot, p.slab_vol, p.tile ? 2 : p.thread ? 1 : 0,
                          (int)p.smem_bytes};
     for (int k = 0; k < 8; k++) meta[k] = vals[k];

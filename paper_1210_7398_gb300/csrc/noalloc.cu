@@ -37,7 +37,7 @@ constexpr long kNoAllocMaxSites = 41472;
 constexpr size_t kSpinorBytes = sizeof(float4) * 6 * (size_t)kNoAllocMaxSites;  // one FP32 spinor field
 constexpr size_t kRecordBytes = kSapRecordBytesPerSite * (size_t)kNoAllocMaxSites;  // per-site SSOR records
 constexpr size_t kTableBytes = 64 * (size_t)kNoAllocMaxSites;                    // ll schedule, block tables
-constexpr size_t kScratchBytes = 4 * kSpinorBytes + kRecordBytes + kTableBytes;  // about 68.3 MB
+constexpr size_t kScratchBytes = 4 * kSpinorBytes + kRecordBytes + kTableBytes;  // about 66.4 MB
 
 static __device__ __align__(256) unsigned char g_sap_scratch[kScratchBytes];
 

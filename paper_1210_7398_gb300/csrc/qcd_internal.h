@@ -59,10 +59,15 @@ struct SapPlan {
     size_t smem_bytes = 0;
     std::vector<int> h_chunk_ptr;   // [C][nchunks + 1], offsets into h_chunk_site
     std::vector<int> h_chunk_site;  // block-local site indices, CTA-major
-    std::vector<unsigned char> h_flags;  // [2 * nchunks]
+    std::vector<unsigned char> h_flags;  // [2 * nchunks], thread form
     std::vector<int> h_site_off;    // [vol] global index offset of a block-local site from its block origin
     std::vector<int> h_own;         // [vol] (owning CTA << 24) | index in that CTA's slab of y
     std::vector<int> h_own_off;     // [C][slab_vol] global offset of each owned site, -1 past the last
+    std::vector<int> h_quad;        // cluster form: [vol][4 lanes][4] neighbour codes in the order of h_chunk_site
+    std::vector<int> h_run_ptr;     // cluster form: [C][nrun + 1] steps of the kernel, offsets into h_chunk_site
+    std::vector<unsigned char> h_run_flags;  // cluster form: [2 * nrun] barrier before a step
+    int nrun = 0, form = 0;  // steps; which instance of the kernel
+    int ypitch = 0;                 // cluster form: words from spinor to spinor in a CTA's slab
     std::vector<int> h_pos;         // thread form: [vol] level position of each block-local site
     std::vector<int> h_origin_site[2];  // [nblk[c]] global index of each block origin
     int *d_chunk_ptr = nullptr;
@@ -71,6 +76,9 @@ struct SapPlan {
     int *d_site_off = nullptr;
     int *d_own = nullptr;
     int *d_own_off = nullptr;
+    int4 *d_quad = nullptr;
+    int *d_run_ptr = nullptr;
+    unsigned char *d_run_flags = nullptr;
     int *d_pos = nullptr;
     int *d_origin_site[2] = {nullptr, nullptr};
     std::vector<int4> h_tile_pos;   // tile form: [2][vol][2] per pass, level position and lane of a pair
@@ -154,7 +162,6 @@ struct qcd_ctx {
     int sap_min_ctas = 0;    // lower bound on the CTAs (cluster size) per SAP block; 0: fill the SMs
     int sap_ctas_user = 0;   // the qcd_set_sap_ctas setting, which params with sap_ctas = 0 use
     int sms_override = 0;    // SM count the SAP plan is made for (0: ask the device); diagnostics
-    int sap_form = 0;        // SSOR lanes per site update: 0 by occupancy, 1 warp form (32), 2 octet form (8)
     int inject_breakdown = 0;  // test hook: outer iterations still to start from rho = 0 (a host-made breakdown)
     bool tc_skip_commit = false;  // test hook: the tensor-core layer issues no MMA or commit (its waits run out)
 
@@ -252,6 +259,8 @@ void use_sap_ctas(qcd_ctx *c, int sap_ctas);
 // block decomposition valid for the lattice (L % block == 0, L / block even and >= 2,
 // block % subblock == 0)
 bool sap_geometry_ok(const qcd_ctx *c, const int b[4], const int s[4]);
+// the barrier flags of the plan's chunks (sap_plan_host makes those its kernel runs with)
+void sap_plan_flags(SapPlan &plan);
 // host part of a plan (tables in h_*; device pointers left null); QCD_ERR_ARG on bad geometry
 int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &plan, int min_ctas = 1,
                   bool half = false);
@@ -278,7 +287,7 @@ size_t sap_table_bytes(const SapPlan &plan);
 int sap_upload_tables(qcd_ctx *c, SapPlan &plan, void *region);
 // bytes of one per-site SSOR record (links, clover rows, neighbour codes), of all records of a
 // plan, and building them into rec (plan.d_rec is set to rec)
-constexpr size_t kSapRecordBytesPerSite = 1200;
+constexpr size_t kSapRecordBytesPerSite = 1152;
 size_t sap_record_bytes(const SapPlan &plan);
 int sap_build_records(qcd_ctx *c, SapPlan &plan, float *rec);
 

@@ -16,16 +16,11 @@
 // level after level gives exactly the sequential result.  Each CTA owns an
 // equal share of every level (dealt round-robin); barriers (CTA or cluster)
 // are placed only where data flows (the paper's OpenMP barriers between
-// dependent sites).  Each site update is done by one warp: lane (d, c) takes
-// hop direction d = 2 mu + (backward) and colour row c, the 8 directions are
-// summed with butterfly shuffles, and 24 lanes apply the chiral clover rows
-// (k_ssor_warp); or by 8 lanes, one per direction, four sites per warp
-// (k_ssor_oct: the same rounding steps, chosen per launch where many CTAs fill
-// the SMs).
+// dependent sites).  Four lanes share a site update (k_ssor_quad).
 // Each CTA keeps its sites' spinors in shared memory (neighbours owned by peer
-// CTAs are read through distributed shared memory); records and source of the
-// sites of the next two chunks are staged with cp.async while the current one
-// computes.
+// CTAs are read through distributed shared memory); a lane's part of the next
+// site's record and source is loaded into registers while the CTA is on its
+// way through the barrier.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
@@ -79,41 +74,59 @@ __device__ __forceinline__ void masked_hops(const float4 *src, const float2 *__r
 
 namespace cg = cooperative_groups;
 
-constexpr int kRing = 3;           // staging depth (timeline steps in flight)
-constexpr int kMaxSlots = 32;      // sites (one warp each) per CTA per timeline step
+constexpr int kMaxSlots = 32;      // most sites of one CTA in one chunk of the plan
+// Most sites of one CTA in one step of the kernel (consecutive chunks of a level run together): clusters;
+// one CTA per block and per SM; one CTA per block, several per SM.  Sites beyond the warps of a step start
+// another step without a barrier, but wait for their records then.  Measured, 6^3x12 blocks: 24^3x48 FP16,
+// C = 1: 24 sites 6190 us, 48 4122, 64 3342, 96 2919; 12^3x24 FP32, C = 8 (52 sites in the widest level):
+// 24 sites 1633 us, 32 1487, 64 1258, and 8^4 blocks FP16: 32 sites 297 us, 48 273, 64 250, 96 327.  Where
+// CTAs share an SM the others fill the gaps: 24^3x48, 4^4 blocks FP16: 8 sites 2761 us, 16 1967, 32 2147.
+constexpr int kMaxRun = 64;
+constexpr int kMaxRunAlone = 96;
+constexpr int kMaxRunShared = 16;
 constexpr int kMaxCluster = 16;    // CTAs per SAP block (clusters above 8 need the non-portable size)
 constexpr size_t kSmemLimit = 200 * 1024;
-constexpr size_t kSmemPerSm = 228 * 1024;  // shared memory of one SM (GB300)
+// shared memory a plan sets aside per site of a chunk, beside the slab, when it chooses the CTAs per block
+constexpr size_t kSlotBytes = 3984, kSlotBytesHalf = 2256;
+constexpr size_t kCtaSmemLimit = 227 * 1024;  // dynamic shared memory of one CTA (GB300)
 
-// Per-site record of the SSOR kernel, in 4-byte words.  W_d for d = 2 mu + (backward):
-// U_mu(n) forward, U_mu(n - mu)^dag backward, 3x3 row-major complex (zero when the hop leaves
-// the block); then the two chiral blocks of F/2 as full 6x6 complex rows; then ints: global
-// site, offset (words) of the site's spinor in its owner CTA's slab of y, and per direction
-// the neighbour code (owner CTA << 24) | offset (words) of the neighbour's spinor in that
-// CTA's slab, or -1 when the hop leaves the block.  FP32 storage keeps complex numbers as
-// float2 (2 words), FP16 storage as half2 (1 word) with the spinors a CTA owns scaled by one
-// FP32 factor per CTA.
+// Per-site record of the SSOR kernel (k_ssor_quad), in 4-byte words: what its four lanes read, 36 complex
+// numbers each (2 words in FP32 storage, 1 word, a half2, in FP16).  Lane j has W_d of directions j and
+// j + 4 (d = 2 mu + (backward)): U_mu(n) forward, U_mu(n - mu)^dag backward, 3x3 row-major, zero when the
+// hop leaves the block; then the rows 3 (j & 1) .. 3 (j & 1) + 2 of chiral block j >> 1 of F/2, six numbers
+// each.  Load q of a lane holds its numbers 4 q .. 4 q + 3, and the four lanes' loads lie side by side.
+// FP16: the spinors a CTA owns are scaled by one FP32 factor per CTA.
 template <bool HALF> struct Rec {
     static constexpr int cw = HALF ? 1 : 2;        // words per complex
-    static constexpr int W = 0, F = 72 * cw;       // colour matrices, clover rows
-    static constexpr int site = 144 * cw, yoff = site + 1, nbr = site + 2;
-    static constexpr int words = site + 12;        // 300 (FP32) or 156 (FP16)
-    static constexpr int chunks = words / 4;
-    static constexpr int stage = words + 24;       // + the site's FP32 source spinor
-    static constexpr int stage_chunks = stage / 4;
+    static constexpr int load_words = 4 * cw;      // one lane's load
+    static constexpr int words = 4 * 36 * cw;      // 288 (FP32) or 144 (FP16)
     static constexpr int ywords = 12 * cw;         // words of one site's spinor in shared memory
+    // word of number e of lane j
+    __host__ __device__ static constexpr int at(int j, int e) { return ((e >> 2) * 4 + j) * load_words + (e & 3) * cw; }
 };
 static_assert(Rec<false>::words * 4 == kSapRecordBytesPerSite, "record size");
-static_assert(Rec<true>::words % 4 == 0 && Rec<false>::words % 4 == 0, "records are 16-byte chunks");
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
+// one lane's part of a record, as stored
+template <bool HALF> struct QuadRecord {
+    uint32_t r[HALF ? 36 : 72];
+    __device__ __forceinline__ void load(const float *p) {  // p: the lane's first load
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            const float *s = p + q * 4 * Rec<HALF>::load_words;
+            if constexpr (HALF)
+                asm("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(r[4 * q]), "=r"(r[4 * q + 1]), "=r"(r[4 * q + 2]), "=r"(r[4 * q + 3]) : "l"(s));
+            else
+                asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=r"(r[8 * q]), "=r"(r[8 * q + 1]), "=r"(r[8 * q + 2]), "=r"(r[8 * q + 3]), "=r"(r[8 * q + 4]),
+                               "=r"(r[8 * q + 5]), "=r"(r[8 * q + 6]), "=r"(r[8 * q + 7]) : "l"(s));
+        }
+    }
+    __device__ __forceinline__ float2 at(int e) const {
+        if constexpr (HALF) return __half22float2(*reinterpret_cast<const __half2 *>(&r[e]));
+        else return make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+    }
+};
 
 // complex load / store in the storage format (w points at the number's first word)
 template <bool HALF> __device__ __forceinline__ float2 ld_c(const float *w) {
@@ -132,15 +145,24 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t a) {
     asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(a) : "memory");
     return v;
 }
-template <bool HALF> __device__ __forceinline__ float2 ld_cl_c(uint32_t a) {
-    if constexpr (HALF) {
-        uint32_t w;
-        asm volatile("ld.shared::cluster.b32 %0, [%1];\n" : "=r"(w) : "r"(a) : "memory");
-        return __half22float2(*reinterpret_cast<const __half2 *>(&w));
-    } else {
-        float2 v;
-        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-        return v;
+// a spinor in the storage format at a shared-window address (CL: of any CTA of the cluster)
+template <bool HALF, bool CL> __device__ __forceinline__ void ld_spinor_smem(uint32_t a, float2 q[12]) {
+#pragma unroll
+    for (int i = 0; i < (HALF ? 3 : 6); i++) {
+        uint32_t w[4];
+        if constexpr (CL)
+            asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(a + 16u * i) : "memory");
+        else
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(a + 16u * i) : "memory");
+        if constexpr (HALF) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) q[4 * i + k] = __half22float2(*reinterpret_cast<const __half2 *>(&w[k]));
+        } else {
+            q[2 * i] = make_float2(__uint_as_float(w[0]), __uint_as_float(w[1]));
+            q[2 * i + 1] = make_float2(__uint_as_float(w[2]), __uint_as_float(w[3]));
+        }
     }
 }
 template <bool HALF> __device__ __forceinline__ void st_c(float *w, float2 v) {
@@ -148,15 +170,16 @@ template <bool HALF> __device__ __forceinline__ void st_c(float *w, float2 v) {
     else *reinterpret_cast<float2 *>(w) = v;
 }
 
-// Builds the per-site records of every block (blocks of colour 0 first).
+// Builds the per-site records of every block (blocks of colour 0 first), each block's in the order of
+// the CTAs' chunk lists: position i % vol holds block-local site list[i % vol].x.
 template <bool HALF>
 __global__ void k_sap_records(float *__restrict__ rec, const float2 *__restrict__ U, const float4 *__restrict__ F,
-                              Geo g, BlockGeo bg, const int *__restrict__ own, const int *__restrict__ org0,
+                              Geo g, BlockGeo bg, const int2 *__restrict__ list, const int *__restrict__ org0,
                               const int *__restrict__ org1, int nblk0, long total) {
     using L = Rec<HALF>;
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const int gb = (int)(i / bg.vol), yl = (int)(i % bg.vol);
+    const int gb = (int)(i / bg.vol), yl = list[i % bg.vol].x;
     const int *o = gb < nblk0 ? org0 + 4 * gb : org1 + 4 * (gb - nblk0);
     int y[4], r = yl;
     for (int m = 0; m < 4; m++) { y[m] = r % bg.b[m]; r /= bg.b[m]; }
@@ -164,32 +187,21 @@ __global__ void k_sap_records(float *__restrict__ rec, const float2 *__restrict_
     long n = 0;
     for (int m = 0; m < 4; m++) n += gs[m] * (o[m] + y[m]);
     float *R = rec + i * L::words;
-    int *Ri = reinterpret_cast<int *>(R);
-    const int bs[4] = {1, bg.b[0], bg.b[0] * bg.b[1], bg.b[0] * bg.b[1] * bg.b[2]};
     for (int d = 0; d < 8; d++) {
-        const int mu = d >> 1;
+        const int mu = d >> 1, e0 = d < 4 ? 0 : 9;
         const bool fwd = (d & 1) == 0;
         const int ym = y[mu] + (fwd ? 1 : -1);
-        float *W = R + L::W + d * 9 * L::cw;
-        if (ym < 0 || ym >= bg.b[mu]) {
-            for (int k = 0; k < 9; k++) st_c<HALF>(W + k * L::cw, make_float2(0.f, 0.f));
-            Ri[L::nbr + d] = -1;
-            continue;
-        }
+        const bool leaves = ym < 0 || ym >= bg.b[mu];
         const long src = fwd ? n : n - gs[mu];
         for (int a = 0; a < 3; a++)
             for (int bb = 0; bb < 3; bb++) {
-                float2 u;
-                if (fwd) {
-                    u = U[(long)(mu * 9 + a * 3 + bb) * g.V + src];
-                } else {
-                    u = U[(long)(mu * 9 + bb * 3 + a) * g.V + src];
-                    u.y = -u.y;
+                float2 u = make_float2(0.f, 0.f);
+                if (!leaves) {
+                    u = U[(long)(mu * 9 + (fwd ? a * 3 + bb : bb * 3 + a)) * g.V + src];
+                    if (!fwd) u.y = -u.y;
                 }
-                st_c<HALF>(W + (a * 3 + bb) * L::cw, u);
+                st_c<HALF>(R + L::at(d & 3, e0 + a * 3 + bb), u);
             }
-        const int nb = yl + (fwd ? bs[mu] : -bs[mu]);
-        Ri[L::nbr + d] = (own[nb] & ~0xffffff) | ((own[nb] & 0xffffff) * L::ywords);
     }
     float fp[72];
     for (int k = 0; k < 18; k++) {
@@ -204,11 +216,13 @@ __global__ void k_sap_records(float *__restrict__ rec, const float2 *__restrict_
                 if (ii == j) e = make_float2(fp[36 * ch + ii], 0.f);
                 else if (j < ii) { const int q = 36 * ch + 6 + 2 * (ii * (ii - 1) / 2 + j); e = make_float2(fp[q], fp[q + 1]); }
                 else { const int q = 36 * ch + 6 + 2 * (j * (j - 1) / 2 + ii); e = make_float2(fp[q], -fp[q + 1]); }
-                st_c<HALF>(R + L::F + (36 * ch + 6 * ii + j) * L::cw, e);
+                st_c<HALF>(R + L::at(2 * ch + ii / 3, 18 + 6 * (ii % 3) + j), e);
             }
-    Ri[L::site] = (int)n;
-    Ri[L::yoff] = (own[yl] & 0xffffff) * L::ywords;
-    for (int k = L::nbr + 8; k < L::words; k++) Ri[k] = 0;
+}
+
+enum { kFormShared, kFormAlone, kFormCluster };  // several CTAs per SM, one CTA per SM, clusters
+constexpr int quad_threads(bool half, int form) {
+    return form == kFormShared ? 4 * kMaxRunShared : form == kFormCluster && half ? 4 * kMaxRun : 4 * kMaxRunAlone;
 }
 
 struct SsorArgs {
@@ -218,104 +232,83 @@ struct SsorArgs {
     float kappa, omega;
     int nsweep;
     long V;
-    int vol, C, slab_vol, nchunks, nslot;
-    const int *chunk_ptr;      // [C][nchunks + 1]
-    const int2 *chunk_site;    // (block-local site, global offset from the block origin)
-    const int *site_off;       // [vol] global offset of a block-local site from the block origin
+    int vol, C, slab_vol, nchunks, ypitch;  // nchunks: steps; ypitch: words from one spinor to the next in the slab
+    const int *chunk_ptr;      // [C][nchunks + 1] the steps, as offsets into the CTA-major list of sites
+    const int4 *quad;          // [vol][4] per site of the CTA-major list and lane j: where the neighbours in
+                               // directions j and j + 4 lie ((owner CTA << 24) | word in its slab, the zero
+                               // spinor when the hop leaves the block), the site's own word in the slab, and
+                               // its global offset from the block origin
+    const int2 *chunk_site;    // thread form: (block-local site, global offset from the block origin)
+    const int *site_off;       // thread form: [vol] global offset of a block-local site from the block origin
     const int *own_off;        // [C][slab_vol] global offset of each site a CTA owns, -1 past the last
-    const unsigned char *flags;  // [2 * nchunks] cluster barrier before a timeline step
+    const unsigned char *flags;  // [2 * nchunks] CTA (1) or cluster (2) barrier before a timeline step
     const int *origin_site;    // [blocks of this colour] global index of the block origin
     const BicgScalars *gate;   // blockIdx.y = right-hand side; skipped when inactive (null: all)
     int gb0;                   // thread form: index of this colour's first block in the SoA records
     int b[4];                  // thread form: block extents
 };
 
-// K3: y = A_BB f on every block of one colour; blockIdx.x / C enumerates blocks.  MAXW: the
-// most warps per CTA the instance is launched with (32 leaves each thread 64 registers)
-template <bool HALF, int MAXW, bool CL>
-__global__ void __launch_bounds__(32 * MAXW) k_ssor_warp(SsorArgs a) {
+// K3: y = A_BB f on every block of one colour; blockIdx.x / C enumerates blocks, blockIdx.y is the
+// right-hand side.  Four lanes share a site update: lane j forms the hops of directions j and j + 4
+// (d = 2 mu + (backward)), the four partial sums meet in a reduce-scatter that leaves lane j with
+// spin j, and lane j applies the three clover rows that give spin j (its chirality's, then the sum or
+// difference with the other's).
+//
+// Bound by the chain of levels: about 1.4 us a step in a cluster of 8 with 6^3x12 blocks, 0.6 us of it the
+// barrier, the rest one update's latency.  Eight lanes per update shorten no step (the instructions were
+// never the chain's longest part) and issue a quarter more per site; a warp per update, with its records
+// staged in shared memory, was bound by instruction issue (about 450 per site, 100 here).  Loads wait for
+// the arrival at the barrier: issued before it, they delay its release (1313 us instead of 1192).
+// 12^3x24, 6^3x12 blocks, 3^3x6 sub-blocks, FP32, 4 sweeps, 4 cycles: 2010 -> 1192 us; 24^3x48, FP16, 2
+// sweeps, 4 right-hand sides: 6^3x12 blocks 6098 -> 2749, 4^4 blocks 3619 -> 1880 (before: a warp per update,
+// or an octet of lanes where many CTAs shared an SM).
+template <bool HALF, int FORM>
+__global__ void __launch_bounds__(quad_threads(HALF, FORM), FORM == kFormShared && HALF ? 8 : 0) k_ssor_quad(SsorArgs a) {
+    constexpr bool CL = FORM == kFormCluster;
     using L = Rec<HALF>;
     extern __shared__ __align__(16) float sm[];
-    // one right-hand side per blockIdx.y (the whole cluster shares it, so the early exit is uniform)
+    // the whole cluster shares a right-hand side, so the early exit is uniform
     if (a.gate && !a.gate[blockIdx.y].active) return;
     a.f += (size_t)blockIdx.y * 6 * a.V;
     a.y += (size_t)blockIdx.y * 6 * a.V;
     const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
     const int nch = a.nchunks;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    int lane;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const int j = lane & 3, grp = lane >> 2;
     const int *cptr_g = a.chunk_ptr + rank * (nch + 1);
-    const int tab0 = cptr_g[0], ntab = cptr_g[nch] - tab0;
-    // shared memory: [y slab | scale | staging ring | chunk pointers | chunk sites | per-warp scratch];
-    // the slab and the scale sit at the same offsets in every CTA of the cluster (peers read them)
-    float *ys = sm;                                                    // [slab_vol][ywords]
-    float *yscale = ys + (size_t)a.slab_vol * L::ywords;               // [4]
-    float *ring = yscale + 4;                                          // [kRing][nslot][stage]
-    int *cptr = reinterpret_cast<int *>(ring + (size_t)kRing * a.nslot * L::stage);      // [nch + 1]
-    int2 *csite = reinterpret_cast<int2 *>(cptr + ((nch + 1 + 3) & ~3));                  // [ntab]
-    float2 *scr0 = reinterpret_cast<float2 *>(csite + ((ntab + 1) & ~1));                 // [nw][12]
-    float2 *scr = scr0 + warp * 12;
+    // shared memory: [y slab, then a zero spinor | scales of the cluster's CTAs | chunk pointers];
+    // the slab sits at the same offset in every CTA of the cluster (peers read it)
+    float *ys = sm;
+    float *yscale = ys + (size_t)(a.slab_vol + 1) * a.ypitch;              // [kMaxCluster] + own, being formed
+    int *cptr = reinterpret_cast<int *>(yscale + kMaxCluster + 4);         // [nch + 1], from the CTA-major list
     const uint32_t ys_u32 = (uint32_t)__cvta_generic_to_shared(ys);
-    const uint32_t scale_u32 = (uint32_t)__cvta_generic_to_shared(yscale);
     const int blk = blockIdx.x / a.C;
     const long n0 = a.origin_site[blk];
-    const float4 *rec = a.rec + (size_t)blk * a.vol * L::chunks;
+    const float *rec = reinterpret_cast<const float *>(a.rec) + (size_t)blk * a.vol * L::words + j * L::load_words;
+    const float2 *f2 = reinterpret_cast<const float2 *>(a.f) + n0 * 12 + j * 3;
 
-    // ---- lane constants of the hop phase: direction d = 2 mu + (backward), colour row c ----
-    const int d = lane >> 2, c = lane & 3;
-    // half-spinor h0 = psi[pa] + za psi[pb], h1 = psi[pc] + zc psi[pd] (spin rows) and the
-    // reconstruction acc[s] += al[s] w0 + be[s] w1, for (1 -+ gamma_mu) in the Dirac representation
-    int pa = 0, pb = 3, pc = 1, pd = 2;
-    float2 za = make_float2(0.f, 1.f), zc = make_float2(0.f, 1.f);
-    float2 al[4] = {make_float2(1.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    float2 be[4] = {make_float2(0.f, 0.f), make_float2(1.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    switch (d) {
-        case 0: al[3] = make_float2(0.f, -1.f); be[2] = make_float2(0.f, -1.f); break;
-        case 1: za = zc = make_float2(0.f, -1.f); al[3] = make_float2(0.f, 1.f); be[2] = make_float2(0.f, 1.f); break;
-        case 2: za = make_float2(1.f, 0.f); zc = make_float2(-1.f, 0.f); al[3] = make_float2(1.f, 0.f);
-                be[2] = make_float2(-1.f, 0.f); break;
-        case 3: za = make_float2(-1.f, 0.f); zc = make_float2(1.f, 0.f); al[3] = make_float2(-1.f, 0.f);
-                be[2] = make_float2(1.f, 0.f); break;
-        case 4: pb = 2; pd = 3; za = make_float2(0.f, 1.f); zc = make_float2(0.f, -1.f);
-                al[2] = make_float2(0.f, -1.f); be[3] = make_float2(0.f, 1.f); break;
-        case 5: pb = 2; pd = 3; za = make_float2(0.f, -1.f); zc = make_float2(0.f, 1.f);
-                al[2] = make_float2(0.f, 1.f); be[3] = make_float2(0.f, -1.f); break;
-        case 6: pa = pb = 2; pc = pd = 3; za = zc = make_float2(1.f, 0.f);
-                al[0] = make_float2(0.f, 0.f); be[1] = make_float2(0.f, 0.f);
-                al[2] = make_float2(1.f, 0.f); be[3] = make_float2(1.f, 0.f); break;
-        default: pa = pb = 0; pc = pd = 1; za = zc = make_float2(1.f, 0.f); break;
-    }
-    // the four spin contributions a lane forms, in the order the reduce-scatter consumes them:
-    // e0 = spin 2 b4 + b3 (kept), e1 = its pair-mate, f0 / f1 = the spins of the other pair sent
-    // to lane ^ 16; each is (al w0 or be w1) for one non-zero factor in {+-1, +-i}, or zero
-    float2 rm[4];
-    bool rw1[4];
-    {
-        const int hb4 = (lane >> 4) & 1, hb3 = (lane >> 3) & 1;
-        const int sp[4] = {2 * hb4 + hb3, 2 * hb4 + 1 - hb3, 2 * (1 - hb4) + hb3, 2 * (1 - hb4) + 1 - hb3};
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            float2 av = al[0], bv = be[0];
-#pragma unroll
-            for (int t = 1; t < 4; t++)
-                if (sp[j] == t) {
-                    av = al[t];
-                    bv = be[t];
-                }
-            rw1[j] = bv.x != 0.f || bv.y != 0.f;
-            rm[j] = rw1[j] ? bv : av;
-        }
-    }
-    // ---- lane constants of the clover phase: lane (s, c), s = lane >> 3, holds spin s ----
-    const int so = lane >> 3;
-    const int fch = so >> 1, fk = (so & 1) * 3 + (c < 3 ? c : 0);
-    const int frow = L::F + (36 * fch + 6 * fk) * L::cw;  // this lane's row of the chiral block
-    const bool owner = c < 3 && (lane & 4) == 0;         // one lane per (spin, colour) stores
+    // lane constants: half-spinors h0 = psi_a + za psi_b, h1 = psi_c + zc psi_d of directions j (x or y:
+    // psi_0, psi_3, psi_1, psi_2) and j + 4 (z: psi_0, psi_2, psi_1, psi_3; t: 2 psi_2, 2 psi_3 forward,
+    // 2 psi_0, 2 psi_1 backward), and the factors that rebuild the spins from w = W_d h, in the Dirac
+    // representation
+    const bool bwd = (j & 1) != 0, up = (j & 2) != 0;
+    const float sg = bwd ? -1.f : 1.f;
+    const float2 za = up ? make_float2(sg, 0.f) : make_float2(0.f, sg);      // direction j
+    const float2 zc = up ? make_float2(-sg, 0.f) : make_float2(0.f, sg);
+    const float2 f3a = up ? make_float2(sg, 0.f) : make_float2(0.f, -sg);    // spin 3 gets f3a w0
+    const float2 f2a = up ? make_float2(-sg, 0.f) : make_float2(0.f, -sg);   // spin 2 gets f2a w1
+    const float2 zA = up ? make_float2(1.f, 0.f) : make_float2(0.f, sg);     // direction j + 4
+    const float2 zC = up ? make_float2(1.f, 0.f) : make_float2(0.f, -sg);
+    const float f0b = up && !bwd ? 0.f : 1.f;                                // spins 0 and 1: f0b w0, f0b w1
+    const float2 f2b = up ? make_float2(bwd ? 0.f : 1.f, 0.f) : make_float2(0.f, -sg);  // spin 2: f2b w0
+    const float2 f3b = up ? make_float2(bwd ? 0.f : 1.f, 0.f) : make_float2(0.f, sg);   // spin 3: f3b w1
 
-    // ---- set-up: zero this CTA's slab of y, copy its chunk tables, FP16: the slab's scale ----
-    float4 *ys4 = reinterpret_cast<float4 *>(ys);
-    for (int i = threadIdx.x; i < a.slab_vol * L::ywords / 4; i += blockDim.x) ys4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = threadIdx.x; i <= nch; i += blockDim.x) cptr[i] = cptr_g[i] - tab0;
-    for (int i = threadIdx.x; i < ntab; i += blockDim.x) csite[i] = a.chunk_site[tab0 + i];
+    // ---- set-up: zero this CTA's slab of y, copy its chunk pointers, FP16: the slab's scale ----
+    const int nz = (a.slab_vol + 1) * a.ypitch / 4;
+    for (int i = threadIdx.x; i < nz; i += blockDim.x) reinterpret_cast<float4 *>(ys)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i <= nch; i += blockDim.x) cptr[i] = cptr_g[i];
     float inv_scale = 1.f, my_scale = 1.f;
     if constexpr (HALF) {
         // scale = largest |component| of the source on this slab (the block solve is O(1) in it)
@@ -328,454 +321,227 @@ __global__ void __launch_bounds__(32 * MAXW) k_ssor_warp(SsorArgs a) {
             m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
         for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (threadIdx.x == 0) yscale[0] = 0.f;
+        if (threadIdx.x == 0) yscale[kMaxCluster] = 0.f;
         __syncthreads();
-        if (lane == 0) atomicMax(reinterpret_cast<int *>(yscale), __float_as_int(m));  // m >= 0: int order = float order
+        if (lane == 0) atomicMax(reinterpret_cast<int *>(yscale + kMaxCluster), __float_as_int(m));  // m >= 0: int order = float order
         __syncthreads();
-        my_scale = yscale[0] > 0.f ? yscale[0] : 1.f;
+        my_scale = yscale[kMaxCluster] > 0.f ? yscale[kMaxCluster] : 1.f;
         inv_scale = 1.f / my_scale;
-        __syncthreads();
-        if (threadIdx.x == 0) yscale[0] = my_scale;
     }
-    __syncthreads();
-
-    const int T = a.nsweep * 2 * nch;
-    int kiss = 0, tiss = 0;  // sweep position and ring slot of the next staging
-    // stage the records and sources of the sites of the next timeline step
-    auto issue = [&](int t) {
-        if (t < T) {
-            const int ch = kiss < nch ? kiss : 2 * nch - 1 - kiss;
-            const int base = cptr[ch], cnt = cptr[ch + 1] - base;
-            float *stage = ring + (size_t)tiss * a.nslot * L::stage;
-            for (int slot = warp; slot < cnt; slot += nw) {
-                const int2 e = csite[base + slot];
-                float *dst = stage + slot * L::stage;
-                const float4 *src = rec + (size_t)e.x * L::chunks;
-#pragma unroll
-                for (int q = lane; q < L::stage_chunks; q += 32) {
-                    if (q < L::chunks) cp_async16(dst + 4 * q, src + q);
-                    else cp_async16(dst + 4 * q, a.f + (n0 + e.y) * 6 + (q - L::chunks));
-                }
-            }
-            if (++kiss == 2 * nch) kiss = 0;
-            if (++tiss == kRing) tiss = 0;
-        }
-        cp_async_commit();
-    };
-    // one SSOR site update by the whole warp
-    auto update = [&](const float *sd) {
-        const int *sdi = reinterpret_cast<const int *>(sd);
-        float2 e[4];  // e0, e1, f0, f1 (see the lane constants)
-#pragma unroll
-        for (int j = 0; j < 4; j++) e[j] = make_float2(0.f, 0.f);
-        const int code = sdi[L::nbr + d];
-        if (c < 3 && code >= 0) {
-            const int sl = code >> 24;
-            float sc = my_scale;
-            const float *W = sd + L::W + (d * 9 + c * 3) * L::cw;
-            float2 w0 = make_float2(0.f, 0.f), w1 = make_float2(0.f, 0.f);
-            // the neighbour spinor: a shared-window address (mapped to the owning CTA when it is
-            // remote), read with ld.shared::cluster; a CTA without a cluster reads its own shared memory
-            uint32_t ad = ys_u32 + 4u * (uint32_t)(code & 0xffffff);
-            if constexpr (CL) {
-                if (sl != rank) {
-                    ad = mapa_u32(ad, sl);
-                    if constexpr (HALF) sc = ld_cluster_f32(mapa_u32(scale_u32, sl));
-                }
-            }
-            auto nq = [&](int k) -> float2 {  // complex k of the neighbour spinor
-                if constexpr (CL) return ld_cl_c<HALF>(ad + 4u * (uint32_t)(k * L::cw));
-                else return ld_c<HALF>(ys + (code & 0xffffff) + k * L::cw);
-            };
-#pragma unroll
-            for (int cc = 0; cc < 3; cc++) {
-                const float2 qa = nq(pa * 3 + cc), qb = nq(pb * 3 + cc), qc = nq(pc * 3 + cc), qd = nq(pd * 3 + cc);
-                const float2 u = ld_c<HALF>(W + cc * L::cw);
-                w0 = cfma(u, cfma(za, qb, qa), w0);
-                w1 = cfma(u, cfma(zc, qd, qc), w1);
-            }
-            if constexpr (HALF) { w0 = cscale(w0, sc); w1 = cscale(w1, sc); }
-#pragma unroll
-            for (int j = 0; j < 4; j++) e[j] = cmul(rm[j], rw1[j] ? w1 : w0);
-        }
-        // reduce-scatter over the 8 directions (lane bits 4, 3, 2): the pair of the other b4 goes to
-        // lane ^ 16, the pair-mate to lane ^ 8, then the two halves of the direction sum meet
-        e[0].x += __shfl_xor_sync(0xffffffffu, e[2].x, 16);
-        e[0].y += __shfl_xor_sync(0xffffffffu, e[2].y, 16);
-        e[1].x += __shfl_xor_sync(0xffffffffu, e[3].x, 16);
-        e[1].y += __shfl_xor_sync(0xffffffffu, e[3].y, 16);
-        float2 A = e[0];
-        A.x += __shfl_xor_sync(0xffffffffu, e[1].x, 8);
-        A.y += __shfl_xor_sync(0xffffffffu, e[1].y, 8);
-        A.x += __shfl_xor_sync(0xffffffffu, A.x, 4);
-        A.y += __shfl_xor_sync(0xffffffffu, A.y, 4);
-        // lane (s, c) holds spin s, colour c of the hop sum; its chiral component (chirality s >> 1)
-        float2 P;
-        P.x = __shfl_xor_sync(0xffffffffu, A.x, 16);
-        P.y = __shfl_xor_sync(0xffffffffu, A.y, 16);
-        const float2 cv = so < 2 ? csub(A, P) : cadd(P, A);
-        if (owner) scr[fch * 6 + (so & 1) * 3 + c] = cv;
-        __syncwarp();
-        // row fk of the chiral clover block fch against the block's 6 components
-        const float4 *cvv = reinterpret_cast<const float4 *>(scr + fch * 6);
-        float2 eta = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-            const float4 x = cvv[q];
-            eta = cfma(ld_c<HALF>(sd + frow + (2 * q) * L::cw), make_float2(x.x, x.y), eta);
-            eta = cfma(ld_c<HALF>(sd + frow + (2 * q + 1) * L::cw), make_float2(x.z, x.w), eta);
-        }
-        __syncwarp();  // the scratch may be rewritten by this warp's next site
-        float2 Q;
-        Q.x = __shfl_xor_sync(0xffffffffu, eta.x, 16);
-        Q.y = __shfl_xor_sync(0xffffffffu, eta.y, 16);
-        // upper spins (s < 2): eta0 + eta1; lower: eta1 - eta0
-        const float2 out = so < 2 ? cadd(eta, Q) : csub(eta, Q);
-        if (owner) {
-            float *yp = ys + sdi[L::yoff] + (so * 3 + c) * L::cw;
-            const float2 fv = *reinterpret_cast<const float2 *>(sd + L::words + (so * 3 + c) * 2);
-            float2 yo = ld_c<HALF>(yp);
-            if constexpr (HALF) yo = cscale(yo, my_scale);
-            float2 t;
-            t.x = fmaf(a.kappa, out.x, fv.x);
-            t.y = fmaf(a.kappa, out.y, fv.y);
-            float2 yn;
-            yn.x = fmaf(a.omega, t.x - yo.x, yo.x);
-            yn.y = fmaf(a.omega, t.y - yo.y, yo.y);
-            if constexpr (HALF) yn = cscale(yn, inv_scale);
-            st_c<HALF>(yp, yn);
-        }
-    };
-
-    issue(0);
-    issue(1);
     if (CL) cg::this_cluster().sync();
     else __syncthreads();
-    int k = 0, tring = 0;  // sweep position and ring slot of the current step
-    for (int t = 0; t < T; t++) {
-        issue(t + 2);
-        cp_async_wait<2>();
-        __syncwarp();
+    if constexpr (HALF) {
+        if (threadIdx.x < a.C) {
+            const uint32_t s_u32 = (uint32_t)__cvta_generic_to_shared(yscale + kMaxCluster);
+            float v = my_scale;
+            if (CL && (int)threadIdx.x != rank) {
+                v = ld_cluster_f32(mapa_u32(s_u32, threadIdx.x));
+                v = v > 0.f ? v : 1.f;
+            }
+            yscale[threadIdx.x] = v;
+        }
+        __syncthreads();
+    }
+
+    const int T = a.nsweep * 2 * nch;
+    const int slot = warp * 8 + grp;
+    // this lane's site of the chunk at sweep position k: its index in the CTA-major list (the last site of
+    // the chunk for the lanes past it, whose results are dropped), -1 for a warp past the chunk
+    auto position = [&](int k, bool &mine) -> int {
         const int ch = k < nch ? k : 2 * nch - 1 - k;
         const int base = cptr[ch], cnt = cptr[ch + 1] - base;
-        const float *stage = ring + (size_t)tring * a.nslot * L::stage;
-        for (int slot = warp; slot < cnt; slot += nw) update(stage + slot * L::stage);
-        if (++k == 2 * nch) k = 0;
-        if (++tring == kRing) tring = 0;
-        if (t + 1 < T) {
-            const unsigned char f = a.flags[k];
-            if (CL && f == 2) cg::this_cluster().sync();
-            else if (f == 1) __syncthreads();
-        }
-    }
-    cp_async_wait<0>();
-    // no CTA may leave (or overwrite) its slab while a peer can still read it
-    if (CL) cg::this_cluster().sync();
-    else __syncthreads();
-    for (int i = threadIdx.x; i < a.slab_vol * 6; i += blockDim.x) {
-        const int sl = i / 6, q = i - 6 * sl;
-        const int off = a.own_off[rank * a.slab_vol + sl];
-        if (off < 0) continue;
-        const long n = n0 + off;
-        float4 v;
-        if constexpr (HALF) {
-            const float2 lo = cscale(ld_c<true>(ys + sl * 12 + 2 * q), my_scale);
-            const float2 hi = cscale(ld_c<true>(ys + sl * 12 + 2 * q + 1), my_scale);
-            v = make_float4(lo.x, lo.y, hi.x, hi.y);
-        } else {
-            v = ys4[i];
-        }
-        a.y[n * 6 + q] = v;
-    }
-}
-
-// K3, octet form: the same ll wavefront, chunks, staging and barriers as k_ssor_warp, but one
-// site update per 8 lanes (lane = hop direction d = 2 mu + (backward)) and four sites per warp.
-// A lane forms its direction's whole projected hop (3 colours, 4 spins), the 8 directions meet
-// in a three-step reduce-scatter, every lane gathers the sum, and each chirality's 4 lanes apply
-// 1 or 2 rows of its 6x6 block.  The arithmetic per site is the warp form's, rounding step by
-// rounding step, spread over 8 lanes instead of 32: about two thirds of the issued instructions
-// per update (no idle colour lanes, fewer shuffles per site), but a quarter of the warps to hide
-// each lane's longer dependency chains.
-template <bool HALF, bool CL>
-__global__ void __launch_bounds__(256) k_ssor_oct(SsorArgs a) {
-    using L = Rec<HALF>;
-    extern __shared__ __align__(16) float sm[];
-    if (a.gate && !a.gate[blockIdx.y].active) return;  // uniform over the cluster
-    a.f += (size_t)blockIdx.y * 6 * a.V;
-    a.y += (size_t)blockIdx.y * 6 * a.V;
-    const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
-    const int nch = a.nchunks;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int grp = lane >> 3, d = lane & 7;             // site slot in the warp, direction
-    const unsigned gm = 0xffu << (lane & 24);            // the 8 lanes of this site
-    const int *cptr_g = a.chunk_ptr + rank * (nch + 1);
-    const int tab0 = cptr_g[0], ntab = cptr_g[nch] - tab0;
-    // shared memory as in k_ssor_warp: [y slab | scale | staging ring | chunk pointers | chunk sites]
-    float *ys = sm;
-    float *yscale = ys + (size_t)a.slab_vol * L::ywords;
-    float *ring = yscale + 4;
-    int *cptr = reinterpret_cast<int *>(ring + (size_t)kRing * a.nslot * L::stage);
-    int2 *csite = reinterpret_cast<int2 *>(cptr + ((nch + 1 + 3) & ~3));
-    const uint32_t ys_u32 = (uint32_t)__cvta_generic_to_shared(ys);
-    const uint32_t scale_u32 = (uint32_t)__cvta_generic_to_shared(yscale);
-    const int blk = blockIdx.x / a.C;
-    const long n0 = a.origin_site[blk];
-    const float4 *rec = a.rec + (size_t)blk * a.vol * L::chunks;
-
-    // ---- direction constants: half-spinors h0 = psi[pa] + za psi[pb], h1 = psi[pc] + zc psi[pd],
-    // w = W_d h, and spin s of the hop gets fs[s] (w1 if u1[s], else w0), (1 -+ gamma_mu) in the
-    // Dirac representation ----
-    int pa = 0, pb = 3, pc = 1, pd = 2;
-    float2 za = make_float2(0.f, 1.f), zc = make_float2(0.f, 1.f);
-    float2 al[4] = {make_float2(1.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    float2 be[4] = {make_float2(0.f, 0.f), make_float2(1.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    switch (d) {
-        case 0: al[3] = make_float2(0.f, -1.f); be[2] = make_float2(0.f, -1.f); break;
-        case 1: za = zc = make_float2(0.f, -1.f); al[3] = make_float2(0.f, 1.f); be[2] = make_float2(0.f, 1.f); break;
-        case 2: za = make_float2(1.f, 0.f); zc = make_float2(-1.f, 0.f); al[3] = make_float2(1.f, 0.f);
-                be[2] = make_float2(-1.f, 0.f); break;
-        case 3: za = make_float2(-1.f, 0.f); zc = make_float2(1.f, 0.f); al[3] = make_float2(-1.f, 0.f);
-                be[2] = make_float2(1.f, 0.f); break;
-        case 4: pb = 2; pd = 3; za = make_float2(0.f, 1.f); zc = make_float2(0.f, -1.f);
-                al[2] = make_float2(0.f, -1.f); be[3] = make_float2(0.f, 1.f); break;
-        case 5: pb = 2; pd = 3; za = make_float2(0.f, -1.f); zc = make_float2(0.f, 1.f);
-                al[2] = make_float2(0.f, 1.f); be[3] = make_float2(0.f, -1.f); break;
-        case 6: pa = pb = 2; pc = pd = 3; za = zc = make_float2(1.f, 0.f);
-                al[0] = make_float2(0.f, 0.f); be[1] = make_float2(0.f, 0.f);
-                al[2] = make_float2(1.f, 0.f); be[3] = make_float2(1.f, 0.f); break;
-        default: pa = pb = 0; pc = pd = 1; za = zc = make_float2(1.f, 0.f); break;
-    }
-    float2 fs[4];
-    bool u1[4];
-#pragma unroll
-    for (int s = 0; s < 4; s++) {
-        u1[s] = be[s].x != 0.f || be[s].y != 0.f;
-        fs[s] = u1[s] ? be[s] : al[s];
-    }
-    const bool b2 = (d & 4) != 0, b1 = (d & 2) != 0, b0 = (d & 1) != 0;
-    const int chir = d >> 2, jj = d & 3;  // clover phase: chirality, first row
-
-    // ---- set-up (as k_ssor_warp): zero this CTA's slab of y, copy its chunk tables, FP16: scale ----
-    float4 *ys4 = reinterpret_cast<float4 *>(ys);
-    for (int i = threadIdx.x; i < a.slab_vol * L::ywords / 4; i += blockDim.x) ys4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = threadIdx.x; i <= nch; i += blockDim.x) cptr[i] = cptr_g[i] - tab0;
-    for (int i = threadIdx.x; i < ntab; i += blockDim.x) csite[i] = a.chunk_site[tab0 + i];
-    float inv_scale = 1.f, my_scale = 1.f;
-    if constexpr (HALF) {
-        float m = 0.f;
-        for (int i = threadIdx.x; i < a.slab_vol * 6; i += blockDim.x) {
-            const int sl = i / 6, q = i - 6 * sl;
-            const int off = a.own_off[rank * a.slab_vol + sl];
-            if (off < 0) continue;
-            const float4 v = a.f[(n0 + off) * 6 + q];
-            m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-        }
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (threadIdx.x == 0) yscale[0] = 0.f;
-        __syncthreads();
-        if (lane == 0) atomicMax(reinterpret_cast<int *>(yscale), __float_as_int(m));  // m >= 0
-        __syncthreads();
-        my_scale = yscale[0] > 0.f ? yscale[0] : 1.f;
-        inv_scale = 1.f / my_scale;
-        __syncthreads();
-        if (threadIdx.x == 0) yscale[0] = my_scale;
-    }
-    __syncthreads();
-    const int T = a.nsweep * 2 * nch;
-    int kiss = 0, tiss = 0;  // sweep position and ring slot of the next staging
-    // stage the records and sources of this warp's (up to 4) sites of the next timeline step
-    auto issue = [&](int t) {
-        if (t < T) {
-            const int ch = kiss < nch ? kiss : 2 * nch - 1 - kiss;
-            const int base = cptr[ch], cnt = cptr[ch + 1] - base;
-            float *stage = ring + (size_t)tiss * a.nslot * L::stage;
-            for (int s4 = warp * 4; s4 < cnt; s4 += nw * 4) {
-                const int ns = cnt - s4 < 4 ? cnt - s4 : 4;
-                for (int q = lane; q < ns * L::stage_chunks; q += 32) {
-                    const int i = q / L::stage_chunks, p = q - i * L::stage_chunks;
-                    const int2 e = csite[base + s4 + i];
-                    float *dst = stage + (s4 + i) * L::stage;
-                    if (p < L::chunks) cp_async16(dst + 4 * p, rec + (size_t)e.x * L::chunks + p);
-                    else cp_async16(dst + 4 * p, a.f + (n0 + e.y) * 6 + (p - L::chunks));
-                }
-            }
-            if (++kiss == 2 * nch) kiss = 0;
-            if (++tiss == kRing) tiss = 0;
-        }
-        cp_async_commit();
+        mine = slot < cnt;
+        return warp * 8 < cnt ? base + (mine ? slot : cnt - 1) : -1;
     };
-    // one SSOR site update by the 8 lanes of this group.  Every rounding step is the warp form's:
-    // the same per-direction products, the same butterfly tree over the directions (pairs
-    // differing in direction bit 2, then bit 1, then bit 0), the chiral components formed after
-    // the sum, the same clover row order; the two forms give identical bits.
-    auto update = [&](const float *sd) {
-        const int *sdi = reinterpret_cast<const int *>(sd);
-        // v: this direction's hop, [spin * 3 + colour][re, im]
-        float v[24];
+    auto next = [&](int k) { return k + 1 == 2 * nch ? 0 : k + 1; };
+    // the record, source and neighbour codes of the next update wait in registers: they are loaded while
+    // the CTA is between two steps, behind the arrival at the barrier
+    QuadRecord<HALF> w;
+    float2 fv[3];
+    int4 code = make_int4(0, 0, 0, 0), code1 = make_int4(0, 0, 0, 0);
+    bool mine0, mine1, mine2;
+    int k1 = next(0);
+    int p0 = position(0, mine0), p1 = position(k1, mine1);
+    auto load_source = [&](int off) {
 #pragma unroll
-        for (int i = 0; i < 24; i++) v[i] = 0.f;
-        const int code = sdi[L::nbr + d];
-        if (code >= 0) {
-            const int sl = code >> 24;
-            float sc = my_scale;
-            uint32_t ad = ys_u32 + 4u * (uint32_t)(code & 0xffffff);
-            if constexpr (CL) {
-                if (sl != rank) {
-                    ad = mapa_u32(ad, sl);
-                    if constexpr (HALF) sc = ld_cluster_f32(mapa_u32(scale_u32, sl));
+        for (int c = 0; c < 3; c++) fv[c] = __ldg(f2 + (size_t)off * 12 + c);
+    };
+    if (p0 >= 0) {
+        code = __ldg(a.quad + (size_t)p0 * 4 + j);
+        w.load(rec + (size_t)p0 * L::words);
+        load_source(code.w);
+    }
+    if (p1 >= 0) code1 = __ldg(a.quad + (size_t)p1 * 4 + j);
+
+    int flag = a.flags[k1];
+    for (int t = 0; t < T; t++) {
+        if (p0 >= 0) {
+            float v[24];  // this lane's hops, [spin][colour][re, im]
+            {
+                float2 q[12], h0[3], h1[3], g0[3], g1[3];
+                uint32_t ada = ys_u32 + 4u * (uint32_t)(code.x & 0xffffff), adb = ys_u32 + 4u * (uint32_t)(code.y & 0xffffff);
+                if constexpr (CL) {
+                    ada = mapa_u32(ada, code.x >> 24);
+                    adb = mapa_u32(adb, code.y >> 24);
+                }
+                ld_spinor_smem<HALF, CL>(ada, q);
+                float sca = 1.f, scb = 1.f;
+                if constexpr (HALF) {
+                    sca = yscale[code.x >> 24];
+                    scb = yscale[code.y >> 24];
+                }
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    h0[c] = cfma(za, q[9 + c], q[c]);
+                    h1[c] = cfma(zc, q[6 + c], q[3 + c]);
+                }
+                ld_spinor_smem<HALF, CL>(adb, q);
+                const bool tf = up && !bwd, tb = up && bwd;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const float2 qa = tf ? q[6 + c] : q[c], qb = tb ? q[c] : q[6 + c];
+                    const float2 qc = tf ? q[9 + c] : q[3 + c], qd = tb ? q[3 + c] : q[9 + c];
+                    g0[c] = cfma(zA, qb, qa);
+                    g1[c] = cfma(zC, qd, qc);
+                }
+#pragma unroll
+                for (int r = 0; r < 3; r++) {
+                    float2 w0 = make_float2(0.f, 0.f), w1 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        const float2 u = w.at(r * 3 + c);
+                        w0 = cfma(u, h0[c], w0);
+                        w1 = cfma(u, h1[c], w1);
+                    }
+                    if constexpr (HALF) { w0 = cscale(w0, sca); w1 = cscale(w1, sca); }
+                    const float2 e2 = cmul(f2a, w1), e3 = cmul(f3a, w0);
+                    v[2 * r] = w0.x; v[2 * r + 1] = w0.y;
+                    v[6 + 2 * r] = w1.x; v[6 + 2 * r + 1] = w1.y;
+                    v[12 + 2 * r] = e2.x; v[12 + 2 * r + 1] = e2.y;
+                    v[18 + 2 * r] = e3.x; v[18 + 2 * r + 1] = e3.y;
+                }
+#pragma unroll
+                for (int r = 0; r < 3; r++) {
+                    float2 w0 = make_float2(0.f, 0.f), w1 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        const float2 u = w.at(9 + r * 3 + c);
+                        w0 = cfma(u, g0[c], w0);
+                        w1 = cfma(u, g1[c], w1);
+                    }
+                    if constexpr (HALF) { w0 = cscale(w0, scb); w1 = cscale(w1, scb); }
+                    // one product of each sum is exact, so each is the rounded sum of the two hops
+                    v[2 * r] = fmaf(f0b, w0.x, v[2 * r]);
+                    v[2 * r + 1] = fmaf(f0b, w0.y, v[2 * r + 1]);
+                    v[6 + 2 * r] = fmaf(f0b, w1.x, v[6 + 2 * r]);
+                    v[6 + 2 * r + 1] = fmaf(f0b, w1.y, v[6 + 2 * r + 1]);
+                    const float2 e2 = cfma(f2b, w0, make_float2(v[12 + 2 * r], v[12 + 2 * r + 1]));
+                    const float2 e3 = cfma(f3b, w1, make_float2(v[18 + 2 * r], v[18 + 2 * r + 1]));
+                    v[12 + 2 * r] = e2.x; v[12 + 2 * r + 1] = e2.y;
+                    v[18 + 2 * r] = e3.x; v[18 + 2 * r + 1] = e3.y;
                 }
             }
-            auto nq = [&](int k) -> float2 {  // complex k = spin * 3 + colour of the neighbour spinor
-                if constexpr (CL) return ld_cl_c<HALF>(ad + 4u * (uint32_t)(k * L::cw));
-                else return ld_c<HALF>(ys + (code & 0xffffff) + k * L::cw);
-            };
-            float2 h0[3], h1[3];
+            // reduce-scatter over the four lanes: lane j ends with spin j of the sum
+            float u12[12], A[6];
 #pragma unroll
-            for (int cc = 0; cc < 3; cc++) {
-                h0[cc] = cfma(za, nq(pb * 3 + cc), nq(pa * 3 + cc));
-                h1[cc] = cfma(zc, nq(pd * 3 + cc), nq(pc * 3 + cc));
+            for (int i = 0; i < 12; i++) {
+                const float send = up ? v[i] : v[12 + i], keep = up ? v[12 + i] : v[i];
+                u12[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
             }
-            const float *W = sd + L::W + d * 9 * L::cw;
+#pragma unroll
+            for (int i = 0; i < 6; i++) {
+                const float send = bwd ? u12[i] : u12[6 + i], keep = bwd ? u12[6 + i] : u12[i];
+                A[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+            }
+            // chiral components: spins 0, 1 minus and plus spins 2, 3
+            float2 x[6];
+            {
+                float cv[6];
+#pragma unroll
+                for (int i = 0; i < 6; i++) {
+                    const float P = __shfl_xor_sync(0xffffffffu, A[i], 2);
+                    cv[i] = up ? P + A[i] : A[i] - P;
+                }
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    float2 o;
+                    o.x = __shfl_xor_sync(0xffffffffu, cv[2 * c], 1);
+                    o.y = __shfl_xor_sync(0xffffffffu, cv[2 * c + 1], 1);
+                    const float2 m = make_float2(cv[2 * c], cv[2 * c + 1]);
+                    x[c] = bwd ? o : m;
+                    x[3 + c] = bwd ? m : o;
+                }
+            }
+            float2 out[3];
 #pragma unroll
             for (int r = 0; r < 3; r++) {
-                float2 w0 = make_float2(0.f, 0.f), w1 = make_float2(0.f, 0.f);
+                float2 eta = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int cc = 0; cc < 3; cc++) {
-                    const float2 u = ld_c<HALF>(W + (r * 3 + cc) * L::cw);
-                    w0 = cfma(u, h0[cc], w0);
-                    w1 = cfma(u, h1[cc], w1);
-                }
-                if constexpr (HALF) { w0 = cscale(w0, sc); w1 = cscale(w1, sc); }
+                for (int m = 0; m < 6; m++) eta = cfma(w.at(18 + 6 * r + m), x[m], eta);
+                float2 Q;
+                Q.x = __shfl_xor_sync(0xffffffffu, eta.x, 2);
+                Q.y = __shfl_xor_sync(0xffffffffu, eta.y, 2);
+                out[r] = up ? csub(eta, Q) : cadd(eta, Q);
+            }
+            if (mine0) {
+                float *yp = ys + code.z + j * 3 * L::cw;
 #pragma unroll
-                for (int s = 0; s < 4; s++) {
-                    const float2 e = cmul(fs[s], u1[s] ? w1 : w0);  // exact: fs[s] is 0, +-1 or +-i
-                    v[2 * (s * 3 + r)] = e.x;
-                    v[2 * (s * 3 + r) + 1] = e.y;
+                for (int r = 0; r < 3; r++) {
+                    float2 yo = ld_c<HALF>(yp + r * L::cw), tt, yn;
+                    if constexpr (HALF) yo = cscale(yo, my_scale);
+                    tt.x = fmaf(a.kappa, out[r].x, fv[r].x);
+                    tt.y = fmaf(a.kappa, out[r].y, fv[r].y);
+                    yn.x = fmaf(a.omega, tt.x - yo.x, yo.x);
+                    yn.y = fmaf(a.omega, tt.y - yo.y, yo.y);
+                    if constexpr (HALF) yn = cscale(yn, inv_scale);
+                    st_c<HALF>(yp + r * L::cw, yn);
                 }
             }
         }
-        // reduce-scatter over the 8 directions: lane d ends with reals 3d .. 3d + 2 of the sum
-        float r12[12], r6[6], r3[3];
-#pragma unroll
-        for (int j = 0; j < 12; j++) {
-            const float send = b2 ? v[j] : v[12 + j], keep = b2 ? v[12 + j] : v[j];
-            r12[j] = keep + __shfl_xor_sync(gm, send, 4);
-        }
-#pragma unroll
-        for (int j = 0; j < 6; j++) {
-            const float send = b1 ? r12[j] : r12[6 + j], keep = b1 ? r12[6 + j] : r12[j];
-            r6[j] = keep + __shfl_xor_sync(gm, send, 2);
-        }
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const float send = b0 ? r6[j] : r6[3 + j], keep = b0 ? r6[3 + j] : r6[j];
-            r3[j] = keep + __shfl_xor_sync(gm, send, 1);
-        }
-        // all-gather: every lane gets the whole hop sum S
-        float g6[6], g12[12], S[24];
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const float o = __shfl_xor_sync(gm, r3[j], 1);
-            g6[j] = b0 ? o : r3[j];
-            g6[3 + j] = b0 ? r3[j] : o;
-        }
-#pragma unroll
-        for (int j = 0; j < 6; j++) {
-            const float o = __shfl_xor_sync(gm, g6[j], 2);
-            g12[j] = b1 ? o : g6[j];
-            g12[6 + j] = b1 ? g6[j] : o;
-        }
-#pragma unroll
-        for (int j = 0; j < 12; j++) {
-            const float o = __shfl_xor_sync(gm, g12[j], 4);
-            S[j] = b2 ? o : g12[j];
-            S[12 + j] = b2 ? g12[j] : o;
-        }
-        // chiral components of chirality chir: k = s * 3 + c (s = 0, 1), S_s -+ S_(s+2)
-        float x[12];
-#pragma unroll
-        for (int j = 0; j < 12; j++) x[j] = chir ? S[j] + S[12 + j] : S[j] - S[12 + j];
-        // rows jj and jj + 4 (the latter for jj < 2) of the chiral clover block chir
-        float2 eta[2];
-#pragma unroll
-        for (int t = 0; t < 2; t++) {
-            const int k = (t == 0 || jj < 2) ? jj + 4 * t : jj;
-            const float *row = sd + L::F + (36 * chir + 6 * k) * L::cw;
-            float2 e = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int m = 0; m < 6; m++) e = cfma(ld_c<HALF>(row + m * L::cw), make_float2(x[2 * m], x[2 * m + 1]), e);
-            eta[t] = e;
-        }
-        // the other chirality's rows (lane ^ 4); upper spins: eta0 + eta1, lower: eta1 - eta0
-#pragma unroll
-        for (int t = 0; t < 2; t++) {
-            float2 Q;
-            Q.x = __shfl_xor_sync(gm, eta[t].x, 4);
-            Q.y = __shfl_xor_sync(gm, eta[t].y, 4);
-            if (t == 0 || jj < 2) {
-                const int k = jj + 4 * t;
-                const float2 out = chir == 0 ? cadd(eta[t], Q) : csub(eta[t], Q);
-                const int idx = chir * 6 + k;  // spin * 3 + colour of the output
-                float *yp = ys + sdi[L::yoff] + idx * L::cw;
-                const float2 fv = *reinterpret_cast<const float2 *>(sd + L::words + idx * 2);
-                float2 yo = ld_c<HALF>(yp);
-                if constexpr (HALF) yo = cscale(yo, my_scale);
-                float2 tt;
-                tt.x = fmaf(a.kappa, out.x, fv.x);
-                tt.y = fmaf(a.kappa, out.y, fv.y);
-                float2 yn;
-                yn.x = fmaf(a.omega, tt.x - yo.x, yo.x);
-                yn.y = fmaf(a.omega, tt.y - yo.y, yo.y);
-                if constexpr (HALF) yn = cscale(yn, inv_scale);
-                st_c<HALF>(yp, yn);
-            }
-        }
-    };
-
-    issue(0);
-    issue(1);
-    if (CL) cg::this_cluster().sync();
-    else __syncthreads();
-    int k = 0, tring = 0;  // sweep position and ring slot of the current step
-    for (int t = 0; t < T; t++) {
-        issue(t + 2);
-        cp_async_wait<2>();
-        __syncwarp();
-        const int ch = k < nch ? k : 2 * nch - 1 - k;
-        const int base = cptr[ch], cnt = cptr[ch + 1] - base;
-        const float *stage = ring + (size_t)tring * a.nslot * L::stage;
-        for (int s4 = warp * 4; s4 < cnt; s4 += nw * 4)
-            if (s4 + grp < cnt) update(stage + (s4 + grp) * L::stage);
-        __syncwarp();  // this warp's ring slots may be restaged by the next issue
-        if (++k == 2 * nch) k = 0;
-        if (++tring == kRing) tring = 0;
         if (t + 1 < T) {
-            const unsigned char f = a.flags[k];
-            if (CL && f == 2) cg::this_cluster().sync();
-            else if (f == 1) __syncthreads();
+            if (CL && flag == 2) {
+                __syncwarp();
+                cg::this_cluster().barrier_arrive();
+            }
+            const int k2 = next(k1), nflag = a.flags[k2];
+            const int p2 = position(k2, mine2);
+            code = code1;
+            if (p1 >= 0) {
+                w.load(rec + (size_t)p1 * L::words);
+                load_source(code.w);
+            }
+            if (p2 >= 0) {
+                code1 = __ldg(a.quad + (size_t)p2 * 4 + j);
+                if constexpr (!CL) {  // without a cluster the records of many blocks stream from memory
+                    const float *pf = rec + (size_t)p2 * L::words - j * L::load_words;
+#pragma unroll
+                    for (int i = j * 32; i < L::words; i += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + i));
+                }
+            }
+            k1 = k2;
+            p0 = p1; p1 = p2;
+            mine0 = mine1; mine1 = mine2;
+            if (CL && flag == 2) cg::this_cluster().barrier_wait();
+            else if (flag == 1) __syncthreads();
+            flag = nflag;
         }
     }
-    cp_async_wait<0>();
+    // no CTA may leave its slab while a peer can still read it
     if (CL) cg::this_cluster().sync();
     else __syncthreads();
     for (int i = threadIdx.x; i < a.slab_vol * 6; i += blockDim.x) {
         const int sl = i / 6, q = i - 6 * sl;
         const int off = a.own_off[rank * a.slab_vol + sl];
         if (off < 0) continue;
-        const long n = n0 + off;
-        float4 v;
+        const float *yp = ys + (size_t)sl * a.ypitch + 2 * q * L::cw;
+        float2 lo = ld_c<HALF>(yp), hi = ld_c<HALF>(yp + L::cw);
         if constexpr (HALF) {
-            const float2 lo = cscale(ld_c<true>(ys + sl * 12 + 2 * q), my_scale);
-            const float2 hi = cscale(ld_c<true>(ys + sl * 12 + 2 * q + 1), my_scale);
-            v = make_float4(lo.x, lo.y, hi.x, hi.y);
-        } else {
-            v = ys4[i];
+            lo = cscale(lo, my_scale);
+            hi = cscale(hi, my_scale);
         }
-        a.y[n * 6 + q] = v;
+        a.y[(n0 + off) * 6 + q] = make_float4(lo.x, lo.y, hi.x, hi.y);
     }
 }
-
 
 // K3, thread form for the throughput regime (blocks that fit one CTA, many blocks per colour):
 // one CTA per block with the block spinor y in shared memory, and every site update of a level
@@ -1216,10 +982,8 @@ bool make_chunks(SapPlan &np, int C, int maxslots, bool check_smem = true) {
     size_t most_sites = 0;
     for (int r = 0; r < C; r++) most_sites = std::max(most_sites, lists[r].size());
     const int ywords = np.half ? Rec<true>::ywords : Rec<false>::ywords;
-    const int stage = np.half ? Rec<true>::stage : Rec<false>::stage;
-    np.smem_bytes = (size_t)np.slab_vol * ywords * 4 + (size_t)kRing * nslot * stage * sizeof(float) +
-                    sizeof(int) * ((nchunks + 1 + 3) & ~3) + sizeof(int2) * ((most_sites + 1) & ~1) +
-                    sizeof(float2) * 12 * nslot + 16;
+    np.smem_bytes = (size_t)np.slab_vol * ywords * 4 + (size_t)nslot * (np.half ? kSlotBytesHalf : kSlotBytes) +
+                    sizeof(int) * ((nchunks + 1 + 3) & ~3) + sizeof(int2) * ((most_sites + 1) & ~1) + 16;
     if (check_smem && np.smem_bytes > kSmemLimit) return false;
     np.h_chunk_ptr.clear();
     np.h_chunk_site.clear();
@@ -1300,7 +1064,54 @@ void make_flags(SapPlan &np) {
         if (!stabbed(v) && v.second > 0) np.h_flags[v.second % P] = 1;
 }
 
+// What k_ssor_quad runs: its instance, the timeline in as few steps as that instance allows (consecutive
+// chunks of a level together; the list of sites keeps its order), the barriers, made for these steps, the
+// neighbour codes (SsorArgs::quad) in the order of the list, and the shared memory.
+void make_run(SapPlan &np) {
+    {
+        const long ctas = (long)(np.nb[0] * np.nb[1]) * (np.nb[2] * np.nb[3]) / 2 * np.C;  // of one colour
+        np.form = np.C > 1 ? kFormCluster : ctas <= np.sms ? kFormAlone : kFormShared;
+        SapPlan run = np;
+        const int most[] = {kMaxRunShared, kMaxRunAlone, kMaxRun};
+        make_chunks(run, np.C, most[np.form], false);
+        make_flags(run);
+        np.nrun = run.nchunks;
+        np.nwarps = (run.nslot + 7) / 8;
+        np.h_run_ptr = run.h_chunk_ptr;
+        np.h_run_flags = run.h_flags;
+    }
+    const int plain = np.half ? Rec<true>::ywords : Rec<false>::ywords;
+    auto bytes = [&](int pitch) {
+        return sizeof(float) * ((size_t)(np.slab_vol + 1) * pitch + kMaxCluster + 4) + sizeof(int) * (np.nrun + 1);
+    };
+    // FP32: 28 words from spinor to spinor spread 16-byte accesses over all banks (24: over half of them)
+    np.ypitch = !np.half && bytes(28) <= kSmemLimit ? 28 : plain;
+    np.smem_bytes = bytes(np.ypitch);
+    np.h_quad.assign(16 * (size_t)np.vol, 0);
+    for (int k = 0; k < np.vol; k++) {
+        const int yl = np.h_chunk_site[k], own = np.h_own[yl];
+        int code[8];
+        int y = yl, stride = 1;
+        for (int m = 0; m < 4; m++) {
+            const int ym = y % np.b[m];
+            y /= np.b[m];
+            for (int back = 0; back < 2; back++) {
+                const bool leaves = back ? ym == 0 : ym + 1 == np.b[m];
+                const int o = leaves ? ((own & ~0xffffff) | np.slab_vol) : np.h_own[yl + (back ? -stride : stride)];
+                code[2 * m + back] = (o & ~0xffffff) | (o & 0xffffff) * np.ypitch;
+            }
+            stride *= np.b[m];
+        }
+        for (int j = 0; j < 4; j++) {
+            int *q = &np.h_quad[16 * (size_t)k + 4 * j];
+            q[0] = code[j]; q[1] = code[j + 4]; q[2] = (own & 0xffffff) * np.ypitch; q[3] = np.h_site_off[yl];
+        }
+    }
+}
+
 }  // namespace
+
+void sap_plan_flags(SapPlan &p) { make_flags(p); }
 
 bool sap_geometry_ok(const qcd_ctx *c, const int b[4], const int s[4]) { return geometry_ok(c, b, s); }
 
@@ -1393,7 +1204,6 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
                 tile_level_table(np);
                 np.nwarps = 0;
                 np.smem_bytes = tile_smem_bytes(np, 1);
-                make_flags(np);
                 return QCD_OK;
             }
         }
@@ -1443,7 +1253,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
         for (int C = 2; C <= 8; C *= 2)
             if (C > Cuse && (long)nblk1 * C <= sms) Cuse = C;
     if (!fit(Cuse)) return QCD_ERR_ARG;
-    make_flags(np);
+    make_run(np);
     return QCD_OK;
 }
 
@@ -1454,7 +1264,8 @@ size_t sap_table_bytes(const SapPlan &p) {
            up16(sizeof(int) * p.h_chunk_ptr.size()) + up16(sizeof(int2) * p.h_chunk_site.size()) +
            up16(sizeof(int) * p.h_site_off.size()) + up16(p.h_flags.size()) + up16(sizeof(int) * p.h_own.size()) +
            up16(sizeof(int) * p.h_own_off.size()) + up16(sizeof(int) * p.h_pos.size()) +
-           up16(sizeof(int4) * p.h_tile_pos.size()) +
+           up16(sizeof(int4) * p.h_tile_pos.size()) + up16(sizeof(int) * p.h_quad.size()) +
+           up16(sizeof(int) * p.h_run_ptr.size()) + up16(p.h_run_flags.size()) +
            (p.tile ? up16(sizeof(int) * p.h_tile_site.size()) + up16(sizeof(int4) * p.h_tile_item.size()) : 0);
 }
 
@@ -1485,11 +1296,15 @@ int sap_upload_tables(qcd_ctx *c, SapPlan &p, void *region) {
     p.d_own = (int *)put(p.h_own.data(), sizeof(int) * p.h_own.size());
     p.d_own_off = (int *)put(p.h_own_off.data(), sizeof(int) * p.h_own_off.size());
     p.d_pos = p.h_pos.empty() ? nullptr : (int *)put(p.h_pos.data(), sizeof(int) * p.h_pos.size());
+    p.d_run_ptr = p.h_quad.empty() ? nullptr : (int *)put(p.h_run_ptr.data(), sizeof(int) * p.h_run_ptr.size());
+    p.d_run_flags = p.h_quad.empty() ? nullptr : (unsigned char *)put(p.h_run_flags.data(), p.h_run_flags.size());
+    p.d_quad = p.h_quad.empty() ? nullptr : (int4 *)put(p.h_quad.data(), sizeof(int) * p.h_quad.size());
     p.d_tile_pos = p.tile ? (int4 *)put(p.h_tile_pos.data(), sizeof(int4) * p.h_tile_pos.size()) : nullptr;
     p.d_tile_site = p.tile ? (int *)put(p.h_tile_site.data(), sizeof(int) * p.h_tile_site.size()) : nullptr;
     p.d_tile_item = p.tile ? (int4 *)put(p.h_tile_item.data(), sizeof(int4) * p.h_tile_item.size()) : nullptr;
     if (!p.d_origin[0] || !p.d_origin[1] || !p.d_origin_site[0] || !p.d_origin_site[1] || !p.d_chunk_ptr ||
         !p.d_chunk_site || !p.d_site_off || !p.d_flags || !p.d_own || !p.d_own_off || (p.thread && !p.d_pos) ||
+        (!p.h_quad.empty() && (!p.d_quad || !p.d_run_ptr || !p.d_run_flags)) ||
         (p.tile && (!p.d_tile_pos || !p.d_tile_site || !p.d_tile_item)))
         return cuda_fail(c, cudaGetLastError(), "cudaMemcpyAsync(SAP tables)");
     // the host vectors may be released only once the copies have consumed them
@@ -1525,10 +1340,10 @@ int sap_build_records(qcd_ctx *c, SapPlan &p, float *rec) {
                                                                            p.d_origin[0], p.d_origin[1], p.nblk[0], total);
     } else if (p.half)
         k_sap_records<true><<<(unsigned)((total + 127) / 128), 128, 0, c->stream>>>(
-            rec, c->U32, c->F32, g, bg, p.d_own, p.d_origin[0], p.d_origin[1], p.nblk[0], total);
+            rec, c->U32, c->F32, g, bg, p.d_chunk_site, p.d_origin[0], p.d_origin[1], p.nblk[0], total);
     else
         k_sap_records<false><<<(unsigned)((total + 127) / 128), 128, 0, c->stream>>>(
-            rec, c->U32, c->F32, g, bg, p.d_own, p.d_origin[0], p.d_origin[1], p.nblk[0], total);
+            rec, c->U32, c->F32, g, bg, p.d_chunk_site, p.d_origin[0], p.d_origin[1], p.nblk[0], total);
     int rc = prof_end(c, QCD_K_OTHER, ev);
     if (rc) return rc;
     p.d_rec = rec;
@@ -1621,18 +1436,11 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     static std::atomic<unsigned long long> attr_done{0};
     static std::mutex attr_mu;
     if (int arc = once_per_device(attr_done, attr_mu, c->device, [&]() -> int {
-            const void *ks[] = {(const void *)k_ssor_warp<false, 16, false>, (const void *)k_ssor_warp<true, 16, false>,
-                                (const void *)k_ssor_warp<false, 32, false>, (const void *)k_ssor_warp<true, 32, false>,
-                                (const void *)k_ssor_warp<false, 16, true>, (const void *)k_ssor_warp<true, 16, true>,
-                                (const void *)k_ssor_warp<false, 32, true>, (const void *)k_ssor_warp<true, 32, true>};
+            const void *ks[] = {(const void *)k_ssor_quad<false, 0>, (const void *)k_ssor_quad<true, 0>,
+                                (const void *)k_ssor_quad<false, 1>, (const void *)k_ssor_quad<true, 1>,
+                                (const void *)k_ssor_quad<false, 2>, (const void *)k_ssor_quad<true, 2>};
             for (const void *k : ks) {
-                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
-                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            }
-            const void *ko[] = {(const void *)k_ssor_oct<false, false>, (const void *)k_ssor_oct<true, false>,
-                                (const void *)k_ssor_oct<false, true>, (const void *)k_ssor_oct<true, true>};
-            for (const void *k : ko) {
-                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
+                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemLimit));
                 QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             }
             QCD_CUDA(c, cudaFuncSetAttribute(k_ssor_soa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
@@ -1649,13 +1457,14 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     a.vol = p.vol;
     a.C = p.C;
     a.slab_vol = p.slab_vol;
-    a.nchunks = p.nchunks;
-    a.nslot = p.nslot;
-    a.chunk_ptr = p.d_chunk_ptr;
+    a.nchunks = p.thread ? p.nchunks : p.nrun;
+    a.ypitch = p.ypitch;
+    a.chunk_ptr = p.thread ? p.d_chunk_ptr : p.d_run_ptr;
+    a.quad = p.d_quad;
     a.chunk_site = p.d_chunk_site;
     a.site_off = p.d_site_off;
     a.own_off = p.d_own_off;
-    a.flags = p.d_flags;
+    a.flags = p.thread ? p.d_flags : p.d_run_flags;
     a.gate = gate;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1664,18 +1473,6 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.dynamicSmemBytes = p.smem_bytes;
-    // form of the block solve for this launch (the warp and octet forms give identical bits):
-    // the octet form issues about two thirds of the instructions per site update with a quarter
-    // of the warps, so it is taken where the grid keeps at least 16 of its warps resident per SM
-    // (the warp form then has 64 and is bound by instruction issue; measured on GB300)
-    const int w_oct = (p.nslot + 3) / 4;
-    auto octet = [&](int col) {
-        if (c->sap_form) return c->sap_form == 2;
-        const long ctas = (long)p.nblk[col] * p.C * nrhs;
-        long per_sm = std::min<long>((long)(kSmemPerSm / (p.smem_bytes + 1024)), 64 / w_oct);
-        per_sm = std::min<long>(std::min<long>(per_sm, 32), (ctas + p.sms - 1) / p.sms);
-        return per_sm * w_oct >= 16;
-    };
     cfg.stream = c->stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -1687,12 +1484,11 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
         for (int col = 0; col < 2; col++) {
             cudaEvent_t ev;
             a.rec = p.d_rec ? reinterpret_cast<const float4 *>(p.d_rec) +
-                                  (size_t)(col ? p.nblk[0] : 0) * p.vol * (p.half ? Rec<true>::chunks : Rec<false>::chunks)
+                                  (size_t)(col ? p.nblk[0] : 0) * p.vol * ((p.half ? Rec<true>::words : Rec<false>::words) / 4)
                             : nullptr;
             a.origin_site = p.d_origin_site[col];
             cfg.gridDim = dim3(p.nblk[col] * p.C, nrhs);
-            const bool oct = !p.thread && octet(col);
-            cfg.blockDim = dim3(32 * (oct ? w_oct : p.nwarps));
+            cfg.blockDim = dim3(32 * p.nwarps);
             prof_begin(c, QCD_K_SSOR, &ev);
             cudaError_t e;
             if (p.thread) {
@@ -1703,16 +1499,10 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
                 k_ssor_soa<<<dim3(p.nblk[col], nrhs), 32 * p.nwarps, p.smem_bytes, c->stream>>>(at);
                 e = cudaGetLastError();
             } else {
-                void (*kern)(SsorArgs);
-                if (oct)
-                    kern = p.C > 1 ? (p.half ? k_ssor_oct<true, true> : k_ssor_oct<false, true>)
-                                   : (p.half ? k_ssor_oct<true, false> : k_ssor_oct<false, false>);
-                else if (p.C > 1)
-                    kern = p.nwarps > 16 ? (p.half ? k_ssor_warp<true, 32, true> : k_ssor_warp<false, 32, true>)
-                                         : (p.half ? k_ssor_warp<true, 16, true> : k_ssor_warp<false, 16, true>);
-                else
-                    kern = p.nwarps > 16 ? (p.half ? k_ssor_warp<true, 32, false> : k_ssor_warp<false, 32, false>)
-                                         : (p.half ? k_ssor_warp<true, 16, false> : k_ssor_warp<false, 16, false>);
+                static constexpr void (*kKernel[2][3])(SsorArgs) = {
+                    {k_ssor_quad<false, 0>, k_ssor_quad<false, 1>, k_ssor_quad<false, 2>},
+                    {k_ssor_quad<true, 0>, k_ssor_quad<true, 1>, k_ssor_quad<true, 2>}};
+                void (*kern)(SsorArgs) = kKernel[p.half][p.form];
                 e = cudaLaunchKernelEx(&cfg, kern, a);
             }
             if (e != cudaSuccess) return cuda_fail(c, e, "launch of the SSOR block kernel");

@@ -479,6 +479,46 @@ def test_sap_lane_forms_identical(case):
     s.close()
 
 
+QUAD_EDGE_CASES = [
+    # dims, block, sub-block, storage, cluster width, right-hand sides: the ends of a step's warps and of the
+    # range of blocks.  A step takes 8 sites per warp, at most 64 (clusters), 96 (one CTA per SM) or 16 sites.
+    ((2, 2, 2, 2), (1, 1, 1, 1), (1, 1, 1, 1), q.QCD_F32, 1, 1),  # every hop leaves the block
+    ((2, 2, 4, 4), (1, 1, 2, 1), (1, 1, 1, 1), q.QCD_F16, 2, 2),  # a site per CTA, levels without a site in one
+    ((6, 6, 6, 12), (3, 3, 3, 6), (3, 3, 3, 6), q.QCD_F32, 16, 1),  # CTAs without a site in most levels
+    ((6, 6, 6, 12), (3, 3, 3, 6), (1, 1, 1, 2), q.QCD_F16, 3, 2),  # uneven shares
+    ((6, 10, 6, 10), (3, 5, 3, 5), (3, 1, 3, 5), q.QCD_F32, 7, 1),
+    ((12, 12, 12, 12), (6, 6, 6, 6), (2, 2, 2, 2), q.QCD_F16, 1, 1),  # a level of 486 sites: steps of at most 96
+    ((12, 12, 12, 12), (6, 6, 6, 6), (2, 2, 2, 2), q.QCD_F32, 8, 1),  # 61 sites in the widest step
+    ((16, 16, 8, 8), (8, 8, 4, 4), (2, 2, 2, 2), q.QCD_F16, 3, 1),  # 128 sites of 384: two steps of 64
+    ((16, 16, 16, 16), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 0, 2),
+    ((12, 12, 12, 24), (2, 2, 2, 2), (2, 2, 2, 2), q.QCD_F16, 0, 1),  # more blocks than SMs
+]
+
+
+@pytest.mark.parametrize("case", QUAD_EDGE_CASES, ids=lambda c: "%s-%s-%s-c%d-n%d" % (
+    "x".join(map(str, c[1])), "x".join(map(str, c[2])), "f16" if c[3] == q.QCD_F16 else "f32", c[4], c[5]))
+def test_sap_cluster_form_edges_vs_oracle(case):
+    """The four-lane site update at the ends of its range against the oracle (the tolerances of
+    the storage formats), with a source that is zero over half of the lattice: an FP16 slab's scale
+    may then be that of no source."""
+    dims, b, sb, storage, ctas, nrhs = case
+    kappa = 0.12
+    s, U, F = make_solver(dims, kappa, seed=1012)
+    v = qi.gaussian_spinor(dims, seed=2012, nrhs=nrhs)
+    v[:, : v.shape[1] // 2] = 0
+    prm = q.make_params(kappa, CSW, b, sb, omega=1.1, nsweep=2, nsap=2, sap_storage=storage)
+    q.qcd_set_sap_ctas(s.ctx, ctas)
+    vin = torch.from_numpy(v.astype(np.complex64)).cuda()
+    out = torch.empty_like(vin)
+    s.sap_precondition(out, vin, prm, nrhs=nrhs)
+    torch.cuda.synchronize()
+    tol = 1e-5 if storage == q.QCD_F32 else SAP_F16_TOL
+    for k in range(nrhs):
+        ref = oracle.sap(dims, U, F, kappa, b, sb, 1.1, 2, 2, v[k])
+        assert rel_norm(out[k].cpu().numpy().astype(np.complex128), ref) <= tol
+    s.close()
+
+
 EO_CASES = [
     # dims, block, MR steps, N_SAP
     ((4, 4, 4, 4), (2, 2, 2, 2), 3, 2),
