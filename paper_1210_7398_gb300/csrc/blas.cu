@@ -25,6 +25,7 @@ namespace {
 
 constexpr int RED_TPB = 256;
 constexpr int TPB = 256;
+constexpr long kOneLevelTiles = 6144;  // most tile partials that one block per right-hand side sums
 
 template <typename C> __device__ __forceinline__ double2 to_d(C a) { return make_double2((double)a.x, (double)a.y); }
 template <typename C> __device__ __forceinline__ C from_d(double2 a);
@@ -122,19 +123,6 @@ __global__ void __launch_bounds__(RED_TPB) k_reduce32(int kind, const float4 *__
         for (int k = 0; k < 3; k++) partial[((long)rhs * 3 + k) * gridDim.x + blockIdx.x] = v[k];
 }
 
-// out[rhs][3] = sum of the partials in index order
-__global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double *__restrict__ partial, int nblk,
-                                                          double *__restrict__ out) {
-    __shared__ double sh[3 * 32];
-    const int rhs = blockIdx.x;
-    double v[3] = {0, 0, 0};
-    for (int i = threadIdx.x; i < nblk; i += RED_TPB)
-        for (int k = 0; k < 3; k++) v[k] += partial[((long)rhs * 3 + k) * nblk + i];
-    block_sum3(v, sh);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; k++) out[rhs * 3 + k] = v[k];
-}
-
 // first level of a two-level sum: block b of right-hand side blockIdx.y sums its contiguous chunk
 // of the n partials [rhs][3][n] (thread-strided, then the fixed block tree) into [rhs][3][b]
 __global__ void __launch_bounds__(RED_TPB) k_sum_chunks(const double *__restrict__ part, long n,
@@ -159,13 +147,8 @@ __device__ __forceinline__ double2 ddiv(double2 a, double2 b) {
 __device__ __forceinline__ bool dfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 __device__ __forceinline__ double dabs(double2 a) { return sqrt(a.x * a.x + a.y * a.y); }
 
-// The scalar steps of BiCGStab for every right-hand side (one thread each).
-__global__ void k_scalars(int stage, BicgScalars *__restrict__ S, const double *__restrict__ red, int nrhs,
-                          double tol, const BicgScalars *__restrict__ gate) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nrhs) return;
-    BicgScalars &s = S[k];
-    const double *r = red + 3 * k;
+// The scalar steps of BiCGStab, for one right-hand side; gated: inactive whatever r says
+__device__ void scalar_step(int stage, BicgScalars &s, const double *r, double tol, bool gated) {
     switch (stage) {
         case SC_INIT:  // red = <rh, r>, |r|^2 with rh = r
             s.rho = make_double2(r[0], r[1]);
@@ -173,7 +156,7 @@ __global__ void k_scalars(int stage, BicgScalars *__restrict__ S, const double *
             s.rhn2 = r[2];
             s.q2 = r[2];
             s.rho0 = s.alpha = s.omega = make_double2(1.0, 0.0);
-            s.active = (s.q2 > 0.0 && isfinite(s.q2) && (!gate || gate[k].active)) ? 1 : 0;
+            s.active = (s.q2 > 0.0 && isfinite(s.q2) && !gated) ? 1 : 0;
             s.done = 0;
             s.breakdown = 0;
             s.iters = 0;
@@ -217,6 +200,29 @@ __global__ void k_scalars(int stage, BicgScalars *__restrict__ S, const double *
             if (!s.done) s.breakdown = 1;
             break;
     }
+}
+__global__ void k_scalars(int stage, BicgScalars *__restrict__ S, int nrhs, double tol) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < nrhs) scalar_step(stage, S[k], nullptr, tol, false);
+}
+
+// out[rhs][3] = sum of the partials in index order, and the scalar steps that follow from it
+__global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double *__restrict__ partial, long nblk,
+                                                          double *__restrict__ out, ScalarStep step) {
+    __shared__ double sh[3 * 32];
+    const int rhs = blockIdx.x;
+    double v[3] = {0, 0, 0};
+#pragma unroll 4
+    for (long i = threadIdx.x; i < nblk; i += RED_TPB)
+        for (int k = 0; k < 3; k++) v[k] += partial[((long)rhs * 3 + k) * nblk + i];
+    block_sum3(v, sh);
+    if (threadIdx.x != 0) return;
+    for (int k = 0; k < 3; k++) out[rhs * 3 + k] = v[k];
+    if (!step.S) return;
+    BicgScalars s = step.S[rhs];
+    scalar_step(step.stage, s, v, step.tol, step.gate && !step.gate[rhs].active);
+    if (step.beta) scalar_step(SC_BETA, s, v, step.tol, false);
+    step.S[rhs] = s;
 }
 
 // grid-stride element loop of one right-hand side: blockIdx.y = rhs, n elements each
@@ -344,25 +350,25 @@ static int reduce_nblk(long n) {
     return (int)(want < 1 ? 1 : (want > kRedMaxBlocks ? kRedMaxBlocks : want));
 }
 
-static int reduce_final(qcd_ctx *c, int nblk, int nrhs, double *out) {
+static int reduce_final(qcd_ctx *c, const double *partial, long nblk, int nrhs, double *out, const ScalarStep &step) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_BLAS, &ev);
-    k_reduce_final<<<nrhs, RED_TPB, 0, c->stream>>>(c->d_red, nblk, out);
+    k_reduce_final<<<nrhs, RED_TPB, 0, c->stream>>>(partial, nblk, out, step);
     return prof_end(c, QCD_K_BLAS, ev);
 }
 
 int reduce64(qcd_ctx *c, int kind, const double2 *a, const double2 *b, long n, int nrhs, double *out,
-             const BicgScalars *active) {
+             const BicgScalars *active, const ScalarStep &step) {
     const int nblk = reduce_nblk(n);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_BLAS, &ev);
     k_reduce64<<<dim3(nblk, nrhs), RED_TPB, 0, c->stream>>>(kind, a, b, n, c->d_red, active);
     int rc = prof_end(c, QCD_K_BLAS, ev);
     if (rc) return rc;
-    return reduce_final(c, nblk, nrhs, out);
+    return reduce_final(c, c->d_red, nblk, nrhs, out, step);
 }
 int reduce32(qcd_ctx *c, int kind, const float2 *a, const float2 *b, long n, int nrhs, double *out,
-             const BicgScalars *active) {
+             const BicgScalars *active, const ScalarStep &step) {
     const long n4 = n / 2;  // spinor fields hold 12 V complex numbers: an even count
     const int nblk = reduce_nblk(n4);
     cudaEvent_t ev;
@@ -371,24 +377,24 @@ int reduce32(qcd_ctx *c, int kind, const float2 *a, const float2 *b, long n, int
                                                             reinterpret_cast<const float4 *>(b), n4, c->d_red, active);
     int rc = prof_end(c, QCD_K_BLAS, ev);
     if (rc) return rc;
-    return reduce_final(c, nblk, nrhs, out);
+    return reduce_final(c, c->d_red, nblk, nrhs, out, step);
 }
-int reduce_partials(qcd_ctx *c, int nblk, int nrhs, double *out) { return reduce_final(c, nblk, nrhs, out); }
-
-int reduce_tiles(qcd_ctx *c, const double *part, long ntiles, int nrhs, double *out) {
+int reduce_tiles(qcd_ctx *c, const double *part, long ntiles, int nrhs, double *out, const ScalarStep &step) {
+    // one block sums a right-hand side's partials where there are few: a launch less (12^3x24 has 324)
+    if (ntiles <= kOneLevelTiles) return reduce_final(c, part, ntiles, nrhs, out, step);
     const int nblk = reduce_nblk(ntiles);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_BLAS, &ev);
     k_sum_chunks<<<dim3(nblk, nrhs), RED_TPB, 0, c->stream>>>(part, ntiles, c->d_red);
     int rc = prof_end(c, QCD_K_BLAS, ev);
     if (rc) return rc;
-    return reduce_final(c, nblk, nrhs, out);
+    return reduce_final(c, c->d_red, nblk, nrhs, out, step);
 }
 
-int scalars(qcd_ctx *c, int stage, BicgScalars *S, const double *red, int nrhs, double tol, const BicgScalars *gate) {
+int scalars(qcd_ctx *c, int stage, BicgScalars *S, int nrhs, double tol) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_BLAS, &ev);
-    k_scalars<<<(nrhs + 63) / 64, 64, 0, c->stream>>>(stage, S, red, nrhs, tol, gate);
+    k_scalars<<<(nrhs + 63) / 64, 64, 0, c->stream>>>(stage, S, nrhs, tol);
     return prof_end(c, QCD_K_BLAS, ev);
 }
 
@@ -431,7 +437,8 @@ int blas_xr_update32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const f
     QCD_BLAS_LAUNCH(k_xr_update<float4>, n / 2, nrhs, F4(x), F4(r), CF4(ph), CF4(sh), CF4(s), CF4(t), S)
 }
 int blas_xr_update_dot32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
-                         const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out) {
+                         const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out,
+                         const ScalarStep &step) {
     const long n4 = n / 2;
     const int nblk = reduce_nblk(n4);
     cudaEvent_t ev;
@@ -440,7 +447,7 @@ int blas_xr_update_dot32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, con
                                                                    CF4(rh), S, n4, c->d_red);
     int rc = prof_end(c, QCD_K_BLAS, ev);
     if (rc) return rc;
-    return reduce_final(c, nblk, nrhs, out);
+    return reduce_final(c, c->d_red, nblk, nrhs, out, step);
 }
 int blas_sub64(qcd_ctx *c, double2 *r, const double2 *b, const double2 *w, const int *mask, long n, int nrhs) {
     QCD_BLAS_LAUNCH(k_sub<double2>, n, nrhs, r, b, w, mask)

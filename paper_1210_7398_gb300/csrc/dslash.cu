@@ -303,7 +303,7 @@ int dslash32_prepare(qcd_ctx *c) { return ensure_u12(c, geo_of(c)); }
 // one), with FP32 accuracy.
 template <int MODE>
 static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, double *red,
-                         const BicgScalars *gate) {
+                         const BicgScalars *gate, const ScalarStep &step) {
     Geo g = geo_of(c);
     const unsigned nblk = (unsigned)((g.V + 127) / 128);
     double *part = MODE ? c->d_red_tiles : nullptr;
@@ -315,7 +315,7 @@ static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, co
         out, in, c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate);
     rc = prof_end(c, QCD_K_DSLASH32, ev);
     if (rc || !MODE) return rc;
-    return reduce_tiles(c, part, nblk, nrhs, red);
+    return reduce_tiles(c, part, nblk, nrhs, red, step);
 }
 
 int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
@@ -333,10 +333,10 @@ int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
 int dslash32_dot(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, int mode, double *red,
-                 const BicgScalars *gate) {
-    if (mode == 1) return dslash32_tile<1>(c, out, in, nrhs, other, red, gate);
-    if (mode == 2) return dslash32_tile<2>(c, out, in, nrhs, other, red, gate);
-    return dslash32_tile<0>(c, out, in, nrhs, nullptr, nullptr, gate);
+                 const BicgScalars *gate, const ScalarStep &step) {
+    if (mode == 1) return dslash32_tile<1>(c, out, in, nrhs, other, red, gate, step);
+    if (mode == 2) return dslash32_tile<2>(c, out, in, nrhs, other, red, gate, step);
+    return dslash32_tile<0>(c, out, in, nrhs, nullptr, nullptr, gate, step);
 }
 
 int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {

@@ -1065,7 +1065,7 @@ int learned_correct(qcd_ctx *c, float4 *out, const float4 *v, float4 *w1, float4
                     const BicgScalars *gate) {
     const long n4 = 6 * c->lat.V;
     int rc;
-    if ((rc = dslash32_dot(c, w1, out, nrhs, nullptr, 0, nullptr, gate))) return rc;
+    if ((rc = dslash32_dot(c, w1, out, nrhs, nullptr, 0, nullptr, gate, ScalarStep()))) return rc;
     for (int k = 0; k < nrhs; k++) {
         const BicgScalars *gk = gate ? gate + k : nullptr;
         cudaEvent_t ev;

@@ -234,6 +234,7 @@ int build_clover(qcd_ctx *c, double kappa, double csw);
 
 // operator D (dslash.cu)
 struct BicgScalars;
+struct ScalarStep;
 int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs);
 // makes the two-row link copy the inner solver's D reads (before any graph capture of it)
 int dslash32_prepare(qcd_ctx *c);
@@ -247,9 +248,10 @@ int dslash(qcd_ctx *c, void *out, const void *in, int prec, int nrhs);
 // FP32 D (two right-hand sides per thread when there are several) fused with the inner
 // products of the BiCGStab step that follows: mode 1: red[rhs] = <other, out>, |out|^2; mode 2:
 // <out, other>, |out|^2; mode 0: none.  Right-hand sides inactive in gate (may be null) are
-// skipped.  Every right-hand side's result is independent of the batch, bit for bit.
+// skipped.  Every right-hand side's result is independent of the batch, bit for bit.  step: what
+// the solver does with the inner products (modes 1 and 2).
 int dslash32_dot(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, int mode, double *red,
-                 const BicgScalars *gate);
+                 const BicgScalars *gate, const ScalarStep &step);
 
 // SSOR form for a call whose params carry sap_ctas (0: the context's qcd_set_sap_ctas setting);
 // rebuilds the SAP plan when it changes (api.cu)
@@ -333,19 +335,26 @@ struct BicgScalars {
 enum { SC_INIT = 0, SC_BETA = 1, SC_ALPHA = 2, SC_OMEGA = 3, SC_RHO = 4 };
 enum { RED_DOT = 0, RED_DOT_NORM = 1, RED_NORM = 2, RED_DOT_NORMA = 3 };
 constexpr int kRedMaxBlocks = 1216;  // 8 x 152 SMs
+// The step of BiCGStab (SC_*) that uses a reduction's result, taken by the kernel that ends the
+// reduction (S null: none).  SC_INIT: gate (may be null) deactivates right-hand sides that are
+// inactive in the outer solver.  beta: SC_BETA of the next iteration follows at once.
+struct ScalarStep {
+    BicgScalars *S = nullptr;
+    int stage = 0;
+    double tol = 0;
+    const BicgScalars *gate = nullptr;
+    bool beta = false;
+};
 // out[rhs][3] = Re, Im <a,b> and |b|^2 (DOT_NORM), |a|^2 (NORM, DOT_NORMA); gate: skip inactive rhs
 int reduce64(qcd_ctx *c, int kind, const double2 *a, const double2 *b, long n, int nrhs, double *out,
-             const BicgScalars *gate);
+             const BicgScalars *gate, const ScalarStep &step = ScalarStep());
 int reduce32(qcd_ctx *c, int kind, const float2 *a, const float2 *b, long n, int nrhs, double *out,
-             const BicgScalars *gate);
-// out[rhs][3] = the sums over nblk of the partials [rhs][3][nblk] in c->d_red, in index order
-int reduce_partials(qcd_ctx *c, int nblk, int nrhs, double *out);
-// the same for ntiles partials [rhs][3][ntiles] anywhere in device memory (two fixed levels:
-// contiguous chunks into c->d_red, then those in index order)
-int reduce_tiles(qcd_ctx *c, const double *part, long ntiles, int nrhs, double *out);
-// one scalar step of BiCGStab (SC_*) for every right-hand side; SC_INIT: gate (may be null)
-// deactivates right-hand sides that are inactive in the outer solver
-int scalars(qcd_ctx *c, int stage, BicgScalars *S, const double *red, int nrhs, double tol, const BicgScalars *gate);
+             const BicgScalars *gate, const ScalarStep &step = ScalarStep());
+// out[rhs][3] = the sums of ntiles partials [rhs][3][ntiles] in device memory (many: in two fixed
+// levels, contiguous chunks into c->d_red, then those in index order)
+int reduce_tiles(qcd_ctx *c, const double *part, long ntiles, int nrhs, double *out, const ScalarStep &step);
+// SC_BETA for every right-hand side
+int scalars(qcd_ctx *c, int stage, BicgScalars *S, int nrhs, double tol);
 int blas_zero(qcd_ctx *c, void *p, size_t bytes);
 int blas_copy(qcd_ctx *c, void *dst, const void *src, size_t bytes);
 // p = r + beta (p - om v)
@@ -361,7 +370,8 @@ int blas_xr_update32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const f
                      const float2 *t, const BicgScalars *S, long n, int nrhs);
 // the same, and out[rhs] = <rh, r>, |r|^2 of the new r (the reduction fused into the update)
 int blas_xr_update_dot32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
-                         const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out);
+                         const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out,
+                         const ScalarStep &step);
 // r = b - w where mask[rhs] (all when mask is null)
 int blas_sub64(qcd_ctx *c, double2 *r, const double2 *b, const double2 *w, const int *mask, long n, int nrhs);
 // rh = r, p = v = 0 where mask[rhs]

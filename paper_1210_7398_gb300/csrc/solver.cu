@@ -51,21 +51,19 @@ float2 *f2(float4 *a) { return reinterpret_cast<float2 *>(a); }
 int inner_iteration(qcd_ctx *c, const Ws &w, const qcd_params *p) {
     const long n = 12 * w.V;
     const int R = w.nrhs;
-    TRY(scalars(c, SC_BETA, w.Si, w.red, R, p->inner_tol, nullptr));
+    const ScalarStep alpha{w.Si, SC_ALPHA, p->inner_tol}, omega{w.Si, SC_OMEGA, p->inner_tol},
+        rho{w.Si, SC_RHO, p->inner_tol, nullptr, true};  // (beta for the next iteration)
     TRY(blas_p_update32(c, f2(w.ip), f2(w.ir), f2(w.iv), w.Si, n, R));
     TRY(sap_apply(c, w.ipt, w.ip, w.sapw, p->omega, p->nsweep, p->nsap, R, w.Si, p->block_solver));
     if (p->learned) TRY(learned_correct(c, w.ipt, w.ip, w.iv, reinterpret_cast<float4 *>(c->net.tmp), R, w.Si));
-    TRY(dslash32_dot(c, w.iv, w.ipt, R, w.irh, 1, w.red, w.Si));  // v = D p~; <rh, v>, |v|^2
-    TRY(scalars(c, SC_ALPHA, w.Si, w.red, R, p->inner_tol, nullptr));
+    TRY(dslash32_dot(c, w.iv, w.ipt, R, w.irh, 1, w.red, w.Si, alpha));  // v = D p~; <rh, v>, |v|^2
     TRY(blas_s_update32(c, f2(w.is), f2(w.ir), f2(w.iv), w.Si, n, R));
     TRY(sap_apply(c, w.ist, w.is, w.sapw, p->omega, p->nsweep, p->nsap, R, w.Si, p->block_solver));
     if (p->learned) TRY(learned_correct(c, w.ist, w.is, w.it, reinterpret_cast<float4 *>(c->net.tmp), R, w.Si));
-    TRY(dslash32_dot(c, w.it, w.ist, R, w.is, 2, w.red, w.Si));  // t = D s~; <t, s>, |t|^2
-    TRY(scalars(c, SC_OMEGA, w.Si, w.red, R, p->inner_tol, nullptr));
+    TRY(dslash32_dot(c, w.it, w.ist, R, w.is, 2, w.red, w.Si, omega));  // t = D s~; <t, s>, |t|^2
     // y += alpha p~ + omega s~, r = s - omega t; <rh, r>, |r|^2
     TRY(blas_xr_update_dot32(c, f2(w.y), f2(w.ir), f2(w.ipt), f2(w.ist), f2(w.is), f2(w.it), f2(w.irh), w.Si, n, R,
-                             w.red));
-    TRY(scalars(c, SC_RHO, w.Si, w.red, R, p->inner_tol, nullptr));
+                             w.red, rho));
     return QCD_OK;
 }
 
@@ -153,8 +151,8 @@ int inner_solve(qcd_ctx *c, const Ws &w, const qcd_params *p, cudaGraphExec_t *g
     TRY(blas_copy(c, w.irh, w.q, bytes));
     TRY(blas_zero(c, w.ip, bytes));
     TRY(blas_zero(c, w.iv, bytes));
-    TRY(reduce32(c, RED_DOT_NORM, f2(w.irh), f2(w.ir), n, R, w.red, nullptr));
-    TRY(scalars(c, SC_INIT, w.Si, w.red, R, p->inner_tol, w.So));
+    TRY(reduce32(c, RED_DOT_NORM, f2(w.irh), f2(w.ir), n, R, w.red, nullptr,
+                 {w.Si, SC_INIT, p->inner_tol, w.So, true}));
     *iters = 0;
     bool any = false;
     TRY(any_active(c, w, w.Si, w.hSi, &any, nullptr));
@@ -333,8 +331,7 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
     TRY(blas_copy(c, w.rh, w.r, b64));
     TRY(blas_zero(c, w.p, b64));
     TRY(blas_zero(c, w.v, b64));
-    TRY(reduce64(c, RED_DOT_NORM, w.rh, w.r, n, R, w.red, nullptr));
-    TRY(scalars(c, SC_INIT, w.So, w.red, R, p->tol, nullptr));
+    TRY(reduce64(c, RED_DOT_NORM, w.rh, w.r, n, R, w.red, nullptr, {w.So, SC_INIT, p->tol}));
     {
         // the outer tolerance is relative to |b|, not to the initial residual
         QCD_CUDA(c, cudaMemcpyAsync(w.hSo, w.So, sizeof(BicgScalars) * R, cudaMemcpyDeviceToHost, c->stream));
@@ -442,23 +439,20 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
                 if (w.hSo[k].active) w.hSo[k].rho = make_double2(0.0, 0.0);
             QCD_CUDA(c, cudaMemcpyAsync(w.So, w.hSo, sizeof(BicgScalars) * R, cudaMemcpyHostToDevice, c->stream));
         }
-        TRY(scalars(c, SC_BETA, w.So, w.red, R, p->tol, nullptr));
+        TRY(scalars(c, SC_BETA, w.So, R, p->tol));
         TRY(blas_p_update64(c, w.p, w.r, w.v, w.So, n, R));
         int its = 0;
         TRY(precondition(c, w, p, w.p, w.ph, gp, &its));
         inner += its;
         TRY(outer_D(c, w, p, w.v, w.ph));
-        TRY(reduce64(c, RED_DOT_NORM, w.rh, w.v, n, R, w.red, w.So));
-        TRY(scalars(c, SC_ALPHA, w.So, w.red, R, p->tol, nullptr));
+        TRY(reduce64(c, RED_DOT_NORM, w.rh, w.v, n, R, w.red, w.So, {w.So, SC_ALPHA, p->tol}));
         TRY(blas_s_update64(c, w.s, w.r, w.v, w.So, n, R));
         TRY(precondition(c, w, p, w.s, w.sh, gp, &its));
         inner += its;
         TRY(outer_D(c, w, p, w.t, w.sh));
-        TRY(reduce64(c, RED_DOT_NORMA, w.t, w.s, n, R, w.red, w.So));
-        TRY(scalars(c, SC_OMEGA, w.So, w.red, R, p->tol, nullptr));
+        TRY(reduce64(c, RED_DOT_NORMA, w.t, w.s, n, R, w.red, w.So, {w.So, SC_OMEGA, p->tol}));
         TRY(blas_xr_update64(c, w.x, w.r, w.ph, w.sh, w.s, w.t, w.So, n, R));
-        TRY(reduce64(c, RED_DOT_NORM, w.rh, w.r, n, R, w.red, w.So));
-        TRY(scalars(c, SC_RHO, w.So, w.red, R, p->tol, nullptr));
+        TRY(reduce64(c, RED_DOT_NORM, w.rh, w.r, n, R, w.red, w.So, {w.So, SC_RHO, p->tol}));
         outer++;
         // rhs that left the outer iteration (converged recursively or broke down) get their true residual checked
         bool dummy = false;

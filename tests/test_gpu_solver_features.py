@@ -48,6 +48,32 @@ def test_rhs_groups_give_the_batched_solutions_bit_for_bit():
     s.close()
 
 
+@pytest.mark.parametrize("lt,graphs", [(24, True), (32, True), (32, False)], ids=["6144", "8192", "8192-no-graph"])
+def test_solve_either_side_of_the_one_level_sum(lt, graphs):
+    """The inner products of the inner solver end in one kernel up to 6144 partials of 128 sites
+    each and in two beyond; both ends, with the loop on the device and without, reach the
+    tolerance, in about as many inner iterations (the same field, a third longer in t)."""
+    dims, kappa = (32, 32, 32, lt), 0.12
+    U = qi.gauge_field(dims, 0.3, seed=1013, device="cuda")
+    b = qi.gaussian_spinor_torch(dims, 2013, 2, "cuda")
+    b[1] = 0  # settled at once, inactive throughout
+    x = torch.zeros_like(b)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()  # (graphs need a stream of their own)
+    s = q.Solver(dims, stream=side.cuda_stream)
+    s.load_gauge(U)
+    s.build_clover(kappa, CSW)
+    q.qcd_set_graphs(s.ctx, graphs)
+    prm = q.make_params(kappa, CSW, (4, 4, 4, 4), (2, 2, 2, 2), nsweep=2, nsap=1, omega=1.4, tol=1e-10,
+                        sap_storage=q.QCD_F16, sap_ctas=-2)
+    st = s.solve(x, b, prm, nrhs=2)
+    torch.cuda.synchronize()
+    assert st["true_rel_res"] <= 1e-10
+    assert st["restarts"] == 0 and 4 <= st["inner_iters"] <= 80
+    assert torch.count_nonzero(x[1]) == 0
+    s.close()
+
+
 def test_tuning_cache_round_trip(tmp_path):
     dims, kappa = (8, 8, 8, 8), 0.12
     s, _ = make_solver(dims, kappa, seed=1012)
