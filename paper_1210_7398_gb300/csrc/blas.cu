@@ -209,6 +209,7 @@ __global__ void k_scalars(int stage, BicgScalars *__restrict__ S, int nrhs, doub
 // out[rhs][3] = sum of the partials in index order, and the scalar steps that follow from it
 __global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double *__restrict__ partial, long nblk,
                                                           double *__restrict__ out, ScalarStep step) {
+    chain_wait(partial);
     __shared__ double sh[3 * 32];
     const int rhs = blockIdx.x;
     double v[3] = {0, 0, 0};
@@ -353,7 +354,7 @@ static int reduce_nblk(long n) {
 static int reduce_final(qcd_ctx *c, const double *partial, long nblk, int nrhs, double *out, const ScalarStep &step) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_BLAS, &ev);
-    k_reduce_final<<<nrhs, RED_TPB, 0, c->stream>>>(partial, nblk, out, step);
+    launch_chained(c, k_reduce_final, nrhs, RED_TPB, 0, partial, nblk, out, step);
     return prof_end(c, QCD_K_BLAS, ev);
 }
 

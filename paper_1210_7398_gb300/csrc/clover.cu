@@ -250,6 +250,7 @@ int build_clover(qcd_ctx *c, double kappa, double csw) {
     prof_begin(c, QCD_K_OTHER, &ev);
     k_clover<<<(unsigned)((g.V + 63) / 64), 64, 0, c->stream>>>(c->F64, c->F32, c->U64, g, csw * kappa,
                                                                   c->d_status);
+    field_kernel(c);
     int rc = prof_end(c, QCD_K_OTHER, ev);
     if (rc) return rc;
     int h = 0;

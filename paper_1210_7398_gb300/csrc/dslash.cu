@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_kernel(SP *__restrict__ out,
                                                      const LK *__restrict__ U, const CL *__restrict__ F,
                                                      R kappa, Geo g, int nrhs) {
     using C = typename CT<R>::C;
+    chain_wait(in);
     // the right-hand side varies fastest over the (1-D) grid: the CTAs of one site block run
     // together and share its links and clover field through L2
     const long sblk = blockIdx.x / nrhs;
@@ -126,10 +127,10 @@ template <int MINB, int NR, typename R, typename SP, typename LK, typename CL, i
 __global__ void __launch_bounds__(128, MINB) dslash_kernel_nr(SP *__restrict__ out, const SP *__restrict__ in,
                                                      const LK *__restrict__ U, const CL *__restrict__ F,
                                                      R kappa, Geo g, int nrhs,
-                                                     const SP *__restrict__ other = nullptr,
-                                                     double *__restrict__ partial = nullptr,
-                                                     const BicgScalars *__restrict__ gate = nullptr) {
+                                                     const SP *__restrict__ other, double *__restrict__ partial,
+                                                     const BicgScalars *__restrict__ gate) {
     using C = typename CT<R>::C;
+    chain_wait(in, other, gate);
     // the right-hand-side tile varies fastest over the (1-D) grid: the CTAs of one site block
     // run together and share its links and clover field through L2
     const int ntile = (nrhs + NR - 1) / NR;
@@ -275,8 +276,8 @@ int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs) {
     dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH64, &ev);
-    dslash_kernel<3, double, double2, double2, double2><<<grid, 128, 0, c->stream>>>(out, in, c->U64, c->F64,
-                                                                                     c->kappa, g, nrhs);
+    launch_chained(c, dslash_kernel<3, double, double2, double2, double2>, grid, 128, 0, out, in, c->U64, c->F64,
+                   c->kappa, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
 }
 
@@ -289,6 +290,7 @@ static int ensure_u12(qcd_ctx *c, const Geo &g) {
     }
     if (c->u12_version != c->field_version) {
         k_links_to_rows<<<(unsigned)((g.V + 255) / 256), 256, 0, c->stream>>>(c->U12, c->U32, g.V);
+        field_kernel(c);
         QCD_CUDA(c, cudaGetLastError());
         c->u12_version = c->field_version;
     }
@@ -311,8 +313,8 @@ static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, co
     if (rc) return rc;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
-    dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE><<<dim3(nblk * nrhs), 128, 0, c->stream>>>(
-        out, in, c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate);
+    launch_chained(c, dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE>, dim3(nblk * nrhs), 128, 0, out, in,
+                   c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate);
     rc = prof_end(c, QCD_K_DSLASH32, ev);
     if (rc || !MODE) return rc;
     return reduce_tiles(c, part, nblk, nrhs, red, step);
@@ -323,12 +325,12 @@ int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<5, float, float4, float2, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
-            out, in, c->U32, c->F32, (float)c->kappa, g, 1);
+        launch_chained(c, dslash_kernel<5, float, float4, float2, float4>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
+                       out, in, c->U32, c->F32, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * ((nrhs + 1) / 2)));
-        dslash_kernel_nr<4, 2, float, float4, float2, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U32, c->F32,
-                                                                                 (float)c->kappa, g, nrhs);
+        launch_chained(c, dslash_kernel_nr<4, 2, float, float4, float2, float4>, grid, 128, 0, out, in, c->U32, c->F32,
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
@@ -348,18 +350,19 @@ int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     }
     if (c->half_version != c->field_version) {
         k_fields_to_half<<<(unsigned)((g.V + 255) / 256), 256, 0, c->stream>>>(c->U16, c->F16, c->U32, c->F32, g.V);
+        field_kernel(c);
         QCD_CUDA(c, cudaGetLastError());
         c->half_version = c->field_version;
     }
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<4, float, float4, __half2, uint2><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
-            out, in, c->U16, c->F16, (float)c->kappa, g, 1);
+        launch_chained(c, dslash_kernel<4, float, float4, __half2, uint2>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
+                       out, in, c->U16, c->F16, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
-        dslash_kernel_nr<4, 1, float, float4, __half2, uint2><<<grid, 128, 0, c->stream>>>(out, in, c->U16, c->F16,
-                                                                                     (float)c->kappa, g, nrhs);
+        launch_chained(c, dslash_kernel_nr<4, 1, float, float4, __half2, uint2>, grid, 128, 0, out, in, c->U16, c->F16,
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
@@ -370,12 +373,12 @@ int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
     if (nrhs == 1) {
-        dslash_kernel<4, float, float4, float4, float4><<<dim3((unsigned)((g.V + 127) / 128), 1), 128, 0, c->stream>>>(
-            out, in, c->U12, c->F32, (float)c->kappa, g, 1);
+        launch_chained(c, dslash_kernel<4, float, float4, float4, float4>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
+                       out, in, c->U12, c->F32, (float)c->kappa, g, 1);
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
-        dslash_kernel_nr<4, 1, float, float4, float4, float4><<<grid, 128, 0, c->stream>>>(out, in, c->U12, c->F32,
-                                                                                     (float)c->kappa, g, nrhs);
+        launch_chained(c, dslash_kernel_nr<4, 1, float, float4, float4, float4>, grid, 128, 0, out, in, c->U12, c->F32,
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }

@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(128, MINB) dslash_x2_kernel(double2 *__restric
                                                           const float4 *__restrict__ Ux2,
                                                           const float4 *__restrict__ Fx2, float kh, float kl,
                                                           Geo g, int nrhs) {
+    chain_wait(in);
     // the right-hand side fastest over the grid: a site block's links and clover are shared
     // through L2 by all right-hand sides (measured as fast as the right-hand side slowest, which
     // keeps one sweep's neighbour slices in L2, at 24^3x48 and 48^3x96)
@@ -310,6 +311,7 @@ int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) {
     }
     if (c->x2_version != c->field_version) {
         k_fields_to_x2<<<(unsigned)((g.V + 255) / 256), 256, 0, c->stream>>>(c->Ux2, c->Fx2, c->U64, c->F64, g.V);
+        field_kernel(c);
         QCD_CUDA(c, cudaGetLastError());
         c->x2_version = c->field_version;
     }
@@ -320,8 +322,8 @@ int dslash_x2(qcd_ctx *c, double2 *out, const float4 *in, int nrhs) {
     // four CTAs of 128 threads per SM (128 registers, some spilled): the instruction fetch that the
     // long unrolled body stalls on is hidden by more warps.  24^3x48, 4 right-hand sides: 1332 / 1241 /
     // 1199 / 2131 us with 2 / 3 / 4 / 5
-    dslash_x2_kernel<4><<<dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, c->stream>>>(out, in, c->Ux2, c->Fx2,
-                                                                                           kh, kl, g, nrhs);
+    launch_chained(c, dslash_x2_kernel<4>, dim3((unsigned)((g.V + 127) / 128 * nrhs)), 128, 0, out, in, c->Ux2, c->Fx2, kh,
+                   kl, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
 }
 

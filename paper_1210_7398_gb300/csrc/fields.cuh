@@ -52,14 +52,24 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(
 
 // ---- loads / stores in the internal layouts ---------------------------------
 
+// Waits until the kernels before this one in the stream have ended and what they wrote is visible
+// (launch_chained; at once in a kernel launched otherwise).  The pointers come back unknown to the
+// compiler, so that no load through them moves up or takes the read-only path.
+__device__ __forceinline__ void chain_wait() { cudaGridDependencySynchronize(); }
+template <typename T, typename... P> __device__ __forceinline__ void chain_wait(T &p, P &...more) {
+    chain_wait(more...);
+    asm volatile("" : "+l"(p)::"memory");
+}
+
 // Spinors lie site by site, [rhs][V][12] complex (the caller's layout): one site's 96 (FP32) or 192
 // (FP64) bytes are read and written as 32-byte vectors, whole sectors for any set of sites a warp
-// takes, in half the instructions of 16-byte accesses.  Every spinor base is 32-byte aligned.
+// takes, in half the instructions of 16-byte accesses.  Every spinor base is 32-byte aligned.  load_spinor
+// is for data the kernel does not write, from a pointer that chain_wait has returned.
 __device__ __forceinline__ void load_spinor(const float4 *__restrict__ p, long n, float2 s[12]) {
     const float4 *q = p + 6 * n;
 #pragma unroll
     for (int k = 0; k < 3; k++)
-        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        asm("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
             : "=f"(s[4 * k].x), "=f"(s[4 * k].y), "=f"(s[4 * k + 1].x), "=f"(s[4 * k + 1].y), "=f"(s[4 * k + 2].x),
               "=f"(s[4 * k + 2].y), "=f"(s[4 * k + 3].x), "=f"(s[4 * k + 3].y)
             : "l"(q + 2 * k));
@@ -68,7 +78,7 @@ __device__ __forceinline__ void load_spinor(const double2 *__restrict__ p, long 
     const double2 *q = p + 12 * n;
 #pragma unroll
     for (int k = 0; k < 6; k++)
-        asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
+        asm("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
             : "=d"(s[2 * k].x), "=d"(s[2 * k].y), "=d"(s[2 * k + 1].x), "=d"(s[2 * k + 1].y)
             : "l"(q + 2 * k));
 }

@@ -58,6 +58,7 @@ int links_to_internal(qcd_ctx *c, const double2 *canon) {
     cudaEvent_t ev;
     prof_begin(c, QCD_K_OTHER, &ev);
     k_links<<<(unsigned)((c->lat.V + TPB - 1) / TPB), TPB, 0, c->stream>>>(c->U64, c->U32, canon, c->lat.V);
+    field_kernel(c);
     return prof_end(c, QCD_K_OTHER, ev);
 }
 

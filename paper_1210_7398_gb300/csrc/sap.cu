@@ -264,6 +264,7 @@ struct SsorArgs {
 // or an octet of lanes where many CTAs shared an SM).
 template <bool HALF, int FORM>
 __global__ void __launch_bounds__(quad_threads(HALF, FORM), FORM == kFormShared && HALF ? 8 : 0) k_ssor_quad(SsorArgs a) {
+    chain_wait();
     constexpr bool CL = FORM == kFormCluster;
     using L = Rec<HALF>;
     extern __shared__ __align__(16) float sm[];
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(quad_threads(HALF, FORM), FORM == kFormShared 
     int p0 = position(0, mine0), p1 = position(k1, mine1);
     auto load_source = [&](int off) {
 #pragma unroll
-        for (int c = 0; c < 3; c++) fv[c] = __ldg(f2 + (size_t)off * 12 + c);
+        for (int c = 0; c < 3; c++) fv[c] = f2[(size_t)off * 12 + c];
     };
     if (p0 >= 0) {
         code = __ldg(a.quad + (size_t)p0 * 4 + j);
@@ -683,6 +684,7 @@ __global__ void __launch_bounds__(128) k_sap_hop(float4 *__restrict__ r, float4 
                                                  const float4 *__restrict__ F, float kappa, Geo g, BlockGeo bg,
                                                  int colour, int upd_in, int upd_cross,
                                                  const BicgScalars *__restrict__ gate) {
+    chain_wait(r, x, y, gate);
     const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= g.V) return;
     if (gate && !gate[blockIdx.y].active) return;
@@ -1330,6 +1332,7 @@ int sap_build_records(qcd_ctx *c, SapPlan &p, float *rec) {
     const long total = (long)(p.nblk[0] + p.nblk[1]) * p.vol;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_OTHER, &ev);
+    field_kernel(c);
     if (p.tile) {
         int trc = tile_build_records(c, p, rec);
         if (trc) return trc;
@@ -1414,8 +1417,8 @@ int sap_apply_eo(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, float
             if ((rc = prof_end(c, QCD_K_SSOR, ev))) return rc;
             const int last = (j == nsap - 1);
             prof_begin(c, QCD_K_SAPHOP, &ev);
-            k_sap_hop<<<dim3((unsigned)((V + 127) / 128), nrhs), 128, 0, c->stream>>>(
-                r, x, y, c->U32, c->F32, (float)c->kappa, g, bg, col, !last, !(last && col == 1), gate);
+            launch_chained(c, k_sap_hop, dim3((unsigned)((V + 127) / 128), nrhs), 128, 0, r, x, y, c->U32, c->F32,
+                           (float)c->kappa, g, bg, col, !last, !(last && col == 1), gate);
             if ((rc = prof_end(c, QCD_K_SAPHOP, ev))) return rc;
         }
     }
@@ -1467,7 +1470,9 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     a.flags = p.thread ? p.d_flags : p.d_run_flags;
     a.gate = gate;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];  // (the second as in launch_chained)
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = p.C;
     attr[0].val.clusterDim.y = 1;
@@ -1475,7 +1480,6 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     cfg.dynamicSmemBytes = p.smem_bytes;
     cfg.stream = c->stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
     int rc;
     if (p.tile) return tile_sap_apply(c, p, x, v, r, y, omega, nsweep, nsap, nrhs, gate);
     if ((rc = blas_copy(c, r, v, sizeof(float4) * 6 * V * nrhs))) return rc;
@@ -1503,14 +1507,16 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
                     {k_ssor_quad<false, 0>, k_ssor_quad<false, 1>, k_ssor_quad<false, 2>},
                     {k_ssor_quad<true, 0>, k_ssor_quad<true, 1>, k_ssor_quad<true, 2>}};
                 void (*kern)(SsorArgs) = kKernel[p.half][p.form];
+                cfg.numAttrs = c->fields_fresh ? 1 : 2;
+                c->fields_fresh = false;
                 e = cudaLaunchKernelEx(&cfg, kern, a);
             }
             if (e != cudaSuccess) return cuda_fail(c, e, "launch of the SSOR block kernel");
             if ((rc = prof_end(c, QCD_K_SSOR, ev))) return rc;
             const int last = (j == nsap - 1);
             prof_begin(c, QCD_K_SAPHOP, &ev);
-            k_sap_hop<<<dim3((unsigned)((V + 127) / 128), nrhs), 128, 0, c->stream>>>(
-                r, x, y, c->U32, c->F32, (float)c->kappa, g, bg, col, !last, !(last && col == 1), gate);
+            launch_chained(c, k_sap_hop, dim3((unsigned)((V + 127) / 128), nrhs), 128, 0, r, x, y, c->U32, c->F32,
+                           (float)c->kappa, g, bg, col, !last, !(last && col == 1), gate);
             if ((rc = prof_end(c, QCD_K_SAPHOP, ev))) return rc;
         }
     }

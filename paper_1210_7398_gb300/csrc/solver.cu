@@ -91,8 +91,9 @@ bool capturable(qcd_ctx *c) {
 
 // the condition of the inner loop's graph: another iteration while any right-hand side is
 // active and fewer than max_inner have run (the counter starts at 0 with each launch)
-__global__ void k_inner_continue(cudaGraphConditionalHandle h, const BicgScalars *__restrict__ S, int nrhs,
-                                 int *__restrict__ iter, int max_inner) {
+__global__ void k_inner_continue(cudaGraphConditionalHandle h, const BicgScalars *S, int nrhs, int *iter,
+                                 int max_inner) {
+    cudaGridDependencySynchronize();  // (launch_chained)
     if (threadIdx.x != 0) return;
     int any = 0;
     for (int k = 0; k < nrhs; k++) any |= S[k].active;
@@ -125,7 +126,7 @@ cudaError_t build_loop_graph(qcd_ctx *c, const Ws &w, const qcd_params *p, cudaG
             const long l0 = c->total_launches;
             *rc = inner_iteration(c, w, p);
             if (!*rc) {
-                k_inner_continue<<<1, 32, 0, c->stream>>>(h, w.Si, w.nrhs, c->d_loop, p->max_inner);
+                launch_chained(c, k_inner_continue, 1, 32, 0, h, w.Si, w.nrhs, c->d_loop, p->max_inner);
                 c->total_launches++;
             }
             c->graph_launches = c->total_launches - l0;

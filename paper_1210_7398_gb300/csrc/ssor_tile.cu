@@ -419,6 +419,7 @@ __device__ __forceinline__ void load_y_other(const TileArgs &a, int rhs, long mm
 // keeps what it needs of them in its own tensor-memory columns.  ALL: every item has a slot there.
 template <bool HALF, int R, bool ALL>
 __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(TileArgs a) {
+    chain_wait();
     using L = TileRec<HALF>;
     extern __shared__ __align__(16) float sm[];
     __shared__ float scale_s[R];
@@ -1256,7 +1257,7 @@ int tile_sap_apply(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
             a.other_base = col ? 0 : p.nblk[0];
             cudaEvent_t ev;
             prof_begin(c, QCD_K_SSOR, &ev);
-            k<<<dim3(p.nblk[col], (nrhs + R - 1) / R), T, smem, c->stream>>>(a);
+            launch_chained(c, k, dim3(p.nblk[col], (nrhs + R - 1) / R), T, smem, a);
             int rc = prof_end(c, QCD_K_SSOR, ev);
             if (rc) return rc;
         }

@@ -242,3 +242,84 @@ def test_smem_peak_hook():
     t = q.qcd_bench_smem_peak(s.ctx, 64)
     assert 5000.0 < t < 100000.0, t  # GB300: 152 SMs x 128 B per cycle x about 2 GHz is about 40 TB/s
     s.close()
+
+
+CHAINS = [
+    # dims, right-hand sides, precision of D or SAP block, sub-block, storage, cluster width
+    ((4, 4, 4, 4), 1, "f32", None), ((8, 6, 10, 14), 3, "f32", None), ((4, 4, 4, 4), 2, "f64", None),
+    ((8, 8, 8, 16), 1, "f16", None), ((8, 8, 8, 8), 3, "su3", None), ((8, 8, 8, 8), 2, "x2", None),
+    ((8, 8, 8, 16), 2, "sap", ((4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F16, -2)),
+    ((8, 8, 8, 8), 1, "sap", ((4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 2)),
+    ((8, 8, 8, 8), 1, "sap", ((4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, -1)),
+]
+
+
+@pytest.mark.parametrize("case", CHAINS, ids=lambda c: "%s-%s-%d%s" % (
+    "x".join(map(str, c[0])), c[2], c[1], "" if c[3] is None else "-c%d" % c[3][3]))
+def test_calls_in_a_row_equal_calls_apart(case):
+    """Kernels may be set up while their predecessor in the stream runs.  Calls that each read what
+    the one before wrote, a call right after the fields were made again, torch kernels in between, and
+    the same calls captured in a graph give bit for bit what the calls give when the device is idle
+    before each."""
+    dims, nrhs, kind, sap = case
+    U = [torch.from_numpy(qi.gauge_field(dims, 0.3, seed=s)).cuda() for s in (1014, 1015)]
+    dt = torch.complex128 if kind == "f64" else torch.complex64
+    v = torch.from_numpy(qi.gaussian_spinor(dims, seed=2014, nrhs=nrhs)).to(dt).cuda()
+    bufs = [torch.empty_like(v) for _ in range(2)]
+    wide = torch.empty_like(v, dtype=torch.complex128)
+    prec = {"f32": q.QCD_F32, "f64": q.QCD_F64, "f16": q.QCD_F16, "su3": q.QCD_F32_SU3, "x2": q.QCD_F32X2}.get(kind)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    s = q.Solver(dims, stream=side.cuda_stream)
+    if sap:
+        q.qcd_set_sap_ctas(s.ctx, sap[3])
+        prm = q.make_params(0.12, CSW, sap[0], sap[1], omega=1.1, nsweep=2, nsap=2, sap_storage=sap[2])
+
+    def calls(apart):
+        def settle():
+            if apart:
+                torch.cuda.synchronize()
+        src = v
+        for k in range(6):
+            dst = bufs[k % 2]
+            settle()
+            if sap:
+                s.sap_precondition(dst, src, prm, nrhs=nrhs)
+            elif kind == "x2":
+                s.apply_D(wide, src, prec, nrhs)
+                settle()
+                dst.copy_(wide)
+            else:
+                s.apply_D(dst, src, prec, nrhs)
+            src = dst
+            if k == 3:
+                settle()
+                bufs[1].mul_(0.5)
+        settle()
+        return bufs[1]
+
+    def fields(k):
+        s.load_gauge(U[k])
+        s.build_clover(0.12, CSW)
+
+    with torch.cuda.stream(side):
+        want = []
+        for k in (0, 1):
+            fields(k)
+            want.append(calls(True).clone())
+            torch.cuda.synchronize()
+        for k in (0, 1):
+            fields(k)
+            got = calls(False).clone()
+            torch.cuda.synchronize()
+            assert torch.equal(got, want[k]), k
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            calls(False)
+        for _ in range(3):
+            bufs[1].zero_()
+            graph.replay()
+            got = bufs[1].clone()
+            torch.cuda.synchronize()
+            assert torch.equal(got, want[1])
+    s.close()
