@@ -1,14 +1,14 @@
-// K1: the operator D = 1 - kappa F H of Eq. (2) on the whole lattice, in FP64,
-// FP32, and FP32 with FP16 storage of links and clover; one thread per site and
-// one or two right-hand sides.
+// K1: the operator D = 1 - kappa F H of Eq. (2) on the whole lattice, in FP64
+// (dslash64_kernel), FP32, and FP32 with FP16 storage of links and clover; one thread
+// per site and one or two right-hand sides.
 //
 // Each thread gathers its 8 neighbour spinors, projects each to a half-spinor
 // (the rank-2 projector 1 -/+ gamma_mu), multiplies by the link, reconstructs
 // and accumulates; then applies the chiral-block clover term and forms
-// in - kappa F (H in).  Loads are 16-byte (FP32 spinors, clover) or 8/16-byte
-// (links) per plane, coalesced across the warp; neighbours of consecutive
-// threads are consecutive, so neighbour re-reads hit L1/L2 and the HBM traffic
-// stays close to one read of each field (768 B/site in FP32).
+// in - kappa F (H in).  Spinors are read site by site as 32-byte vectors, links (8 or
+// 16 bytes) and clover (16 bytes) plane by plane, coalesced across the warp; neighbours
+// of consecutive threads are consecutive, so neighbour re-reads hit L1/L2 and the HBM
+// traffic stays close to one read of each field (768 B/site in FP32).
 #include <algorithm>
 
 #include "fields.cuh"
@@ -55,17 +55,18 @@ __device__ __forceinline__ void load_link(const float4 *__restrict__ U, long V, 
     u[8] = cross(u[0], u[4], u[1], u[3]);
 }
 
-// MINB: resident blocks per SM requested from the register allocator.  The FP32
-// kernel is bound by memory latency, so it trades registers for occupancy
-// (7 blocks of 128 threads); the FP64 kernel is bound by GB300's FP64 rate and
-// keeps its registers.  NR: right-hand sides per thread; each link and the
+// MINB: resident blocks per SM requested from the register allocator.  One right-hand side in
+// FP32 is bound by HBM (48^3x96: 1.40 ms, 5.8 TB/s of algorithmic bytes, 5 blocks; 2.04 ms from
+// plane-by-plane spinors), several by latency and L1 requests (24^3x48, 12: 672 us, 1200 before; L2 at
+// 55%, HBM at 45%, issue at 42%; staging spinors through shared memory, two lanes per site and links site by
+// site were all slower, 811 to 1170 us).  NR: right-hand sides per thread; each link and the
 // clover field are loaded once and applied to all of them, so the field bytes
 // per right-hand side drop from 576 to 576 / NR (FP32).  Over the grid the
 // right-hand side (tile) index varies fastest, so the CTAs of one site block run
 // close together and the field bytes come from HBM about once for all of them.
 // With FP32 fields two right-hand sides per thread (4 blocks of 128 threads) are
-// faster than one (7 blocks, the fields then read once per right-hand side from
-// L2); with FP16 or two-row fields one per thread is, so those launch NR = 1.
+// faster than one, three or four (672 us against 730 for three and 812 for four); with
+// FP16 or two-row fields one per thread is, so those launch NR = 1.
 template <int MINB, typename R, typename SP, typename LK, typename CL>
 __global__ void __launch_bounds__(128, MINB) dslash_kernel(SP *__restrict__ out, const SP *__restrict__ in,
                                                      const LK *__restrict__ U, const CL *__restrict__ F,
@@ -238,6 +239,139 @@ __device__ __forceinline__ void dslash_site(SP *__restrict__ out, const SP *__re
     }
 }
 
+// ---- FP64 -----------------------------------------------------------------------------------------
+// w = U h (U^dag h) for both spin rows of a half-spinor, added to the w it is given (SUB: subtracted)
+template <bool DAG, bool SUB> __device__ __forceinline__ void mul64(const double2 u[9], const double2 h[6], double2 w[6]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            double2 v = DAG ? u[b * 3 + a] : u[a * 3 + b];
+            if (SUB) v = make_double2(-v.x, -v.y);
+            w[a] = DAG ? cfmac(v, h[b], w[a]) : cfma(v, h[b], w[a]);
+            w[3 + a] = DAG ? cfmac(v, h[3 + b], w[3 + a]) : cfma(v, h[3 + b], w[3 + a]);
+        }
+}
+// a + s b
+__device__ __forceinline__ double2 axpy64(double s, double2 b, double2 a) {
+    return make_double2(fma(s, b.x, a.x), fma(s, b.y, a.y));
+}
+// y = H x for the packed chiral block b of F/2 at site n, the large diagonal last
+__device__ __forceinline__ void herm6_64(const double2 *__restrict__ F, long V, long n, int b, const double2 x[6],
+                                         double2 y[6]) {
+    double f[36];
+#pragma unroll
+    for (int k = 0; k < 18; k++) {
+        const double2 v = __ldg(F + (18 * b + k) * V + n);
+        f[2 * k] = v.x;
+        f[2 * k + 1] = v.y;
+    }
+    int k = 6;
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        y[i] = make_double2(0, 0);
+#pragma unroll
+        for (int j = 0; j < i; j++) {
+            const double2 a = make_double2(f[k], f[k + 1]);
+            k += 2;
+            y[i] = cfma(a, x[j], y[i]);
+            y[j] = cfmac(a, x[i], y[j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; i++) y[i] = axpy64(f[i], x[i], y[i]);
+}
+// D in FP64.  Bound by the FP64 pipe (2 operations per clock and SM, which it reaches), so the order is the
+// one with few operations, 1,092 a site (1,200 in the plain order):
+//  - t first, the colour products starting the sums (the projector's factor 2 and the boundary sign
+//    multiply them when the next hop is added);
+//  - along x, y, z the backward product is subtracted from the forward one as it is formed, D = w+ - w-, which is
+//    what the lower spins need, and the upper spins add 2 w+ - D: 36 operations instead of 48 for the two
+//    reconstructions.
+// Together these round a little more (the error against 80-bit arithmetic, of random sites with unitary links
+// and a clover term of 0.5 +- 0.03, rises by 3%); the clover's diagonal, its largest entries, added last
+// rounds less, and the error ends 15% below that of the plain order (0.94e-16 against 1.12e-16).  Applying the
+// second chiral block on top of the first one's result would save 12 more, but raises it by 12%.
+// 24^3x48: 1337 -> 1257 us (1497 at first).
+__global__ void __launch_bounds__(128, 3) dslash64_kernel(double2 *__restrict__ out, const double2 *__restrict__ in,
+                                                          const double2 *__restrict__ U, const double2 *__restrict__ F,
+                                                          double kappa, Geo g, int nrhs) {
+    chain_wait(in);
+    // the right-hand side varies fastest over the (1-D) grid: the CTAs of one site block run
+    // together and share its links and clover field through L2
+    const long sblk = blockIdx.x / nrhs;
+    const int rhs = (int)(blockIdx.x - sblk * nrhs);
+    const long n = sblk * blockDim.x + threadIdx.x;
+    if (n >= g.V) return;
+    const double2 *src = in + (long)rhs * 12 * g.V;
+    int x[4];
+    site_coords(g, n, x);
+    double2 up[6], lo[6], psi[12], u[9];  // the hop sum's upper and lower two spins
+#pragma unroll
+    for (int k = 0; k < 6; k++) up[k] = lo[k] = make_double2(0, 0);
+    {
+        const long m = nbr_fwd<3>(g, n, x);
+        load_spinor(src, m, psi);
+        load_link(U, g.V, n, 3, u);
+        mul64<false, false>(u, psi + 6, lo);
+    }
+    {
+        const long m = nbr_bwd<3>(g, n, x);
+        load_spinor(src, m, psi);
+        load_link(U, g.V, m, 3, u);
+        mul64<true, false>(u, psi, up);
+    }
+    const double sf = x[3] == g.L[3] - 1 ? 2.0 * g.bc_t : 2.0, sb = x[3] == 0 ? 2.0 * g.bc_t : 2.0;
+#define QCD_PAIR(MU)                                                                                  \
+    {                                                                                                 \
+        double2 h[6], w[6], d[6];                                                                     \
+        const long mf = nbr_fwd<MU>(g, n, x), mb = nbr_bwd<MU>(g, n, x);                              \
+        load_spinor(src, mf, psi);                                                                    \
+        load_link(U, g.V, n, MU, u);                                                                  \
+        hop_project<MU, true>(psi, 1.0, h);                                                           \
+        _Pragma("unroll") for (int k = 0; k < 6; k++) w[k] = make_double2(0, 0);                      \
+        mul64<false, false>(u, h, w);                                                                 \
+        load_spinor(src, mb, psi);                                                                    \
+        load_link(U, g.V, mb, MU, u);                                                                 \
+        hop_project<MU, false>(psi, 1.0, h);                                                          \
+        _Pragma("unroll") for (int k = 0; k < 6; k++) d[k] = w[k];                                    \
+        mul64<true, true>(u, h, d);                                                                   \
+        _Pragma("unroll") for (int k = 0; k < 6; k++) {                                               \
+            /* lower spins: spin 2 from row 1 (x, y) or 0 (z), spin 3 from the other */               \
+            const double2 dk = d[MU == 2 ? k : k < 3 ? k + 3 : k - 3];                                \
+            const double2 p = MU == 0 ? cmulmi(dk)                                                    \
+                            : MU == 1 ? (k < 3 ? make_double2(-dk.x, -dk.y) : dk)                     \
+                                      : (k < 3 ? cmulmi(dk) : cmuli(dk));                             \
+            if (MU == 0) {                                                                            \
+                up[k] = axpy64(sb, up[k], axpy64(2.0, w[k], make_double2(-d[k].x, -d[k].y)));         \
+                lo[k] = axpy64(sf, lo[k], p);                                                         \
+            } else {                                                                                  \
+                up[k] = axpy64(2.0, w[k], csub(up[k], d[k]));                                         \
+                lo[k] = cadd(lo[k], p);                                                               \
+            }                                                                                         \
+        }                                                                                             \
+    }
+    QCD_PAIR(0)
+    QCD_PAIR(1)
+    QCD_PAIR(2)
+#undef QCD_PAIR
+    // F: e0 = H_0 (up - lo), e1 = H_1 (up + lo); upper spins e0 + e1, lower e1 - e0
+    double2 c[6], e0[6], e1[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++) c[k] = csub(up[k], lo[k]);
+    herm6_64(F, g.V, n, 0, c, e0);
+#pragma unroll
+    for (int k = 0; k < 6; k++) c[k] = cadd(up[k], lo[k]);
+    herm6_64(F, g.V, n, 1, c, e1);
+    load_spinor(src, n, psi);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        psi[k] = axpy64(-kappa, cadd(e0[k], e1[k]), psi[k]);
+        psi[6 + k] = axpy64(-kappa, csub(e1[k], e0[k]), psi[6 + k]);
+    }
+    store_spinor(out + (long)rhs * 12 * g.V, n, psi);
+}
+
 namespace {
 // first two rows of every FP32 link
 __global__ void k_links_to_rows(float4 *__restrict__ U12, const float2 *__restrict__ U32, long V) {
@@ -276,8 +410,7 @@ int dslash64(qcd_ctx *c, double2 *out, const double2 *in, int nrhs) {
     dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH64, &ev);
-    launch_chained(c, dslash_kernel<3, double, double2, double2, double2>, grid, 128, 0, out, in, c->U64, c->F64,
-                   c->kappa, g, nrhs);
+    launch_chained(c, dslash64_kernel, grid, 128, 0, out, in, c->U64, c->F64, c->kappa, g, nrhs);
     return prof_end(c, QCD_K_DSLASH64, ev);
 }
 
@@ -300,9 +433,8 @@ static int ensure_u12(qcd_ctx *c, const Geo &g) {
 int dslash32_prepare(qcd_ctx *c) { return ensure_u12(c, geo_of(c)); }
 
 // The inner solver's D: FP32 with the links in the two-row form (the third row rebuilt in
-// registers), one right-hand side per thread.  At 48^3x96 with 4 right-hand sides it takes 3.54 ms
-// against 4.13 ms with full FP32 links and two right-hand sides per thread (1.17 against 1.37 ms for
-// one), with FP32 accuracy.
+// registers), one right-hand side per thread, with FP32 accuracy.  At 24^3x48 with 12 right-hand sides
+// and the fused inner products it takes 0.71 ms.
 template <int MODE>
 static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, double *red,
                          const BicgScalars *gate, const ScalarStep &step) {

@@ -46,8 +46,6 @@ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 caddi(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.y, b.x)); }
 __device__ __forceinline__ float2 csubi(float2 a, float2 b) { return __fadd2_rn(a, make_float2(b.y, -b.x)); }
-// y + s a
-__device__ __forceinline__ double2 caxpy(double s, double2 a, double2 y) { return make_double2(fma(s, a.x, y.x), fma(s, a.y, y.y)); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 
 // ---- loads / stores in the internal layouts ---------------------------------
@@ -182,11 +180,7 @@ __device__ __forceinline__ void clover_mul(const R f[72], const C v[12], C out[1
 // to acc (Dirac representation, gamma_k = [[0,-i s_k],[i s_k,0]], gamma_4 =
 // diag(1,1,-1,-1)); the projector has rank 2, so the colour multiply acts on
 // the two-component half-spinor h only.  sgn is the boundary sign of a hop
-// across the t edge (only MU = 3 can carry one).  Along t the half-spinor is twice two of psi's
-// spins; in FP64, where every operation counts (24 of 1,200 a site: D on 24^3x48 1376 -> 1340 us), the
-// factor and the sign join the sum over the hops instead.  FP32 keeps them in the half-spinor: the other
-// way there measured 1.5% slower (684 against 674 us, 12 right-hand sides).
-
+// across the t edge (only MU = 3 can carry one).  
 // the half-spinor h[spin row * 3 + colour] of (1 -/+ gamma_mu) psi
 template <int MU, bool FWD, typename C>
 __device__ __forceinline__ void hop_project(const C psi[12], decltype(C::x) sgn, C h[6]) {
@@ -204,12 +198,8 @@ __device__ __forceinline__ void hop_project(const C psi[12], decltype(C::x) sgn,
             h0 = FWD ? caddi(p0, p2) : csubi(p0, p2);
             h1 = FWD ? csubi(p1, p3) : caddi(p1, p3);
         } else {
-            h0 = FWD ? p2 : p0;
-            h1 = FWD ? p3 : p1;
-            if constexpr (sizeof(sgn) == 4) {
-                h0 = cscale(h0, 2 * sgn);
-                h1 = cscale(h1, 2 * sgn);
-            }
+            h0 = FWD ? cscale(p2, 2 * sgn) : cscale(p0, 2 * sgn);
+            h1 = FWD ? cscale(p3, 2 * sgn) : cscale(p1, 2 * sgn);
         }
         h[c] = h0;
         h[3 + c] = h1;
@@ -219,19 +209,13 @@ __device__ __forceinline__ void hop_project(const C psi[12], decltype(C::x) sgn,
 // adds the transported half-spinor w (both spin rows) to acc, reconstructing the other two
 // spin components of (1 -/+ gamma_mu)
 template <int MU, bool FWD, typename C>
-__device__ __forceinline__ void hop_reconstruct(const C w[6], decltype(C::x) sgn, C acc[12]) {
+__device__ __forceinline__ void hop_reconstruct(const C w[6], C acc[12]) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         const C w0 = w[a], w1 = w[3 + a];
         if (MU == 3) {
-            constexpr int k = FWD ? 6 : 0;
-            if constexpr (sizeof(sgn) == 4) {
-                acc[k + a] = cadd(acc[k + a], w0);
-                acc[k + 3 + a] = cadd(acc[k + 3 + a], w1);
-            } else {
-                acc[k + a] = caxpy(2 * sgn, w0, acc[k + a]);
-                acc[k + 3 + a] = caxpy(2 * sgn, w1, acc[k + 3 + a]);
-            }
+            if (FWD) { acc[6 + a] = cadd(acc[6 + a], w0); acc[9 + a] = cadd(acc[9 + a], w1); }
+            else     { acc[a] = cadd(acc[a], w0);         acc[3 + a] = cadd(acc[3 + a], w1); }
             continue;
         }
         acc[a] = cadd(acc[a], w0);
@@ -271,7 +255,7 @@ __device__ __forceinline__ void hop_term(const C psi[12], const C u[9], decltype
         w[a] = w0;
         w[3 + a] = w1;
     }
-    hop_reconstruct<MU, FWD>(w, sgn, acc);
+    hop_reconstruct<MU, FWD>(w, acc);
 }
 
 // The same hop with the transport matrix given as it acts: W = U_mu(n) forward and
