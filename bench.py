@@ -46,7 +46,7 @@ D_BYTES_PER_SITE = {"f32": 768, "f64": 1536, "f16": 480, "su3": 672,  # in + out
 L2_BYTES = 126 << 20
 # DRAM bytes (read + write) per unit of work of a kernel, from one ncu capture of the kernel
 # source identified by its SHA-256 prefix; reported only while the source is unchanged
-NCU_TRAFFIC = {"ssor": {"sha": "2d5f2563905eaedb", "nsap": 1, "nsweep": 2, "per_launch": [629.6, 703.0],
+NCU_TRAFFIC = {"ssor": {"sha": "1b19ad956fd07538", "nsap": 1, "nsweep": 2, "per_launch": [290.7, 319.7],
                          "capture": "ncu, k_sap_tile<FP16, 4> on 24^3x48 (4^4 / 2^4 blocks, 4 right-hand sides, "
                                     "2 sweeps, 1 cycle): DRAM bytes per (site, right-hand side) of the colour of "
                                     "each launch of one application, averaged and scaled to this launch"}}
@@ -825,14 +825,16 @@ def run_gpu_on_stream(args, q, qi, torch, stream, rank, world, local):
                 "units_per_launch": units,
                 "model": "average tile SAP launch (one colour, %d right-hand sides): V/2 x nrhs x (2 nsweep + "
                          "(nsap - 1) / nsap) site updates x 1896 flop (Table 1; the residual's in-block operator "
-                         "only where a later cycle reads it), time from a profiled pass of one group of the "
-                         "chosen solve" % g}
+                         "only where a later cycle reads it; the kernel keeps the hop sum over the neighbours "
+                         "not updated since and forms the other half, about 1236 flop an update), time from a "
+                         "profiled pass of one group of the chosen solve" % g}
         if dom == "ssor":
             sb = sap_smem_bytes_per_launch(V, g, chosen_p.nsweep, chosen_p.nsap, chosen_p.sap_storage == q.QCD_F16)
             roof["smem"] = {"achieved": sb / (avg_ms * 1e-3) / 1e9, "peak": smem_gbs, "unit": "GB/s",
                             "frac": sb / (avg_ms * 1e-3) / 1e9 / smem_gbs,
                             "peak_source": "measured: conflict-free 16-byte shared loads (qcd_bench_smem_peak)",
-                            "model": "per (site, right-hand side): 2 nsweep x 11 spinors (8 neighbours, y, f read, "
+                            "model": "an upper bound, all 8 neighbours counted where the kernel reads the half "
+                                     "updated since: per (site, right-hand side): 2 nsweep x 11 spinors (8 neighbours, y, f read, "
                                      "y written), 1 for x += y, 9 for the kept residual, the source write and the "
                                      "y copy-out, 48 B each in FP16 storage, averaged over an application"}
         src = "paper_1210_7398_gb300/csrc/ssor_tile.cu"

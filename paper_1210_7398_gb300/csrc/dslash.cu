@@ -56,8 +56,9 @@ __device__ __forceinline__ void load_link(const float4 *__restrict__ U, long V, 
 }
 
 // MINB: resident blocks per SM requested from the register allocator.  One right-hand side in
-// FP32 is bound by HBM (48^3x96: 1.40 ms, 5.8 TB/s of algorithmic bytes, 5 blocks; 2.04 ms from
-// plane-by-plane spinors), several by latency and L1 requests (24^3x48, 12: 672 us, 1200 before; L2 at
+// FP32 is bound by HBM (48^3x96: 1.40 ms, 5.8 TB/s of algorithmic bytes, 5 blocks; 2.04 ms with the
+// conversions to and from planes that the caller's layout does without), several by latency and L1
+// requests (24^3x48, 12: 672 us, 1200 with the conversions; L2 at
 // 55%, HBM at 45%, issue at 42%; staging spinors through shared memory, two lanes per site and links site by
 // site were all slower, 811 to 1170 us).  NR: right-hand sides per thread; each link and the
 // clover field are loaded once and applied to all of them, so the field bytes

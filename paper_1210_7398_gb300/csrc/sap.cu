@@ -550,8 +550,8 @@ __global__ void __launch_bounds__(quad_threads(HALF, FORM), FORM == kFormShared 
 // in K1), with a CTA barrier between levels.  The links and clover of each block are stored per
 // block in level order and structure-of-arrays form ([block][element][level position]), so the
 // threads of a level read consecutive addresses: the loads are coalesced and every byte is
-// used.  A site update costs about 1,200 thread instructions against the warp form's ~400
-// warp instructions.  The level order is the warp form's, so the same values are read.
+// used.  A site update costs about 1,200 thread instructions.  The level order is the cluster
+// form's, so the same values are read.
 constexpr int kTsY = 28;  // padded words of one site's spinor in shared memory
 constexpr int kTsMaxThreads = 256;
 constexpr int kSoaLinks = 72;   // float2 per site: 8 hop links (U_mu(n) forward, U_mu(n - mu) backward)
