@@ -1195,6 +1195,13 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
         for (int m = 0; m < 4; m++) { y[m] = r % b[m]; r /= b[m]; }
         np.h_site_off[yl] = y[0] + c->lat.L[0] * (y[1] + c->lat.L[1] * (y[2] + c->lat.L[2] * y[3]));
     }
+    int sms = c->sms_override;
+    if (sms < 1 &&
+        (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms < 1)) {
+        cudaGetLastError();
+        sms = 1;
+    }
+    np.sms = sms;
     // the right-hand-side tiled thread form on request (min_ctas == -2), the block spinor of
     // one right-hand side in one CTA
     if (min_ctas == -2) {
@@ -1230,13 +1237,6 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
     // CTAs per block: C <= 16 whose shared memory fits.  With min_ctas >= 1 the smallest such
     // C >= min_ctas; with min_ctas = 0 the largest one that keeps the blocks of one colour (one
     // CTA cluster each) within the SM count, and at least the smallest that fits
-    int sms = c->sms_override;
-    if (sms < 1 &&
-        (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms < 1)) {
-        cudaGetLastError();
-        sms = 1;
-    }
-    np.sms = sms;
     const int nblk1 = np.nb[0] * np.nb[1] * np.nb[2] * np.nb[3] / 2;
     // up to 32 sites (warps) per step and CTA where one colour's blocks leave SMs idle and the
     // staging ring fits (fewer dependent steps), else 16 (more registers per thread; several

@@ -1152,6 +1152,25 @@ int tile_threads(const SapPlan &p, int R) {
 // warp items (16 (site, right-hand side) pairs) of level l
 int tile_level_items(const SapPlan &p, int l, int R) { return ((p.h_step_ptr[l + 1] - p.h_step_ptr[l]) * R + 15) / 16; }
 
+// Relative time of an application with R right-hand sides per CTA: the share of the SMs' warps that its warp
+// items take, each costing more the more sites (16 / R) its record loads cover, and the rounds of items that a
+// CTA's warps take level by level.  The weights fit measured applications; us with the R that the most
+// right-hand sides would give -> with the least cost (R in parentheses): 24^3x48, 4^4 blocks, FP16, 3 right-hand
+// sides 1026 (2) -> 892 (4), 5 1704 (4) -> 1501 (2); 16^3x32, 2^4 blocks, FP16, 3 599 (2) -> 367 (4), 5 705 (4)
+// -> 523 (8); 8^3x16, 4^4 blocks, FP16, 2 85 (2) -> 65 (1), 8 141 (4) -> 66 (1).
+float tile_cost(const SapPlan &p, int R, int nrhs) {
+    const int nw = tile_threads(p, R) / 32;
+    int items = 0, rounds = 0;
+    for (int l = 0; l < p.nsteps; l++) {
+        const int n = tile_level_items(p, l, R);
+        items += n;
+        rounds += (n + nw - 1) / nw;
+    }
+    const float ctas = (float)std::max(p.nblk[0], p.nblk[1]) * (float)((nrhs + R - 1) / R);
+    const float filled = ctas * (float)items * (1.f + 1.12f / (float)R) / ((float)std::max(1, p.sms) * 16.f);
+    return filled + 0.73f * (float)rounds;
+}
+
 // Tensor memory of a CTA: a slot of 12 FP32 columns per warp item, the items dealt to the warps in turn;
 // warps four apart share a lane quarter.  As many slots as fit the columns that leave the CTAs resident
 // that the other resources allow; if not all do, one more slot is the place where an uncached item holds
@@ -1193,12 +1212,20 @@ void tile_level_table(SapPlan &p) {
 }
 
 int tile_choose(const SapPlan &p, int nrhs, int *R, int *threads, size_t *smem) {
-    // the most right-hand sides per CTA (up to 8) that still let kTileMinBlocks CTAs share an
-    // SM (the registers allow that many of 256 threads); one per CTA up to the whole shared
-    // memory otherwise
+    // The right-hand sides per CTA, of those that let kTileMinBlocks CTAs share an SM (the registers
+    // allow that many of 256 threads): the most that nrhs fills, unless tile_cost finds another at least
+    // 5% cheaper.
     const size_t share = kTileSmemPerSm / kTileMinBlocks - 1024;
     int r = 1;
     while (r * 2 <= kTileMaxRhs && r * 2 <= nrhs && tile_smem_bytes(p, r * 2) <= share) r *= 2;
+    float least = 0.95f * tile_cost(p, r, nrhs);
+    for (int q = 1; q <= kTileMaxRhs && q < 2 * nrhs && (q == 1 || tile_smem_bytes(p, q) <= share); q *= 2) {
+        const float cost = tile_cost(p, q, nrhs);
+        if (cost < least) {
+            least = cost;
+            r = q;
+        }
+    }
     if (tile_smem_bytes(p, r) > kTileSmemLimit) return QCD_ERR_ARG;
     *R = r;
     *threads = tile_threads(p, r);

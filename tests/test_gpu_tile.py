@@ -193,3 +193,32 @@ def test_tile_solve_true_residual_under_oracle(st):
         r = b[k] - oracle.apply_D(dims, U, F, kappa, x[k])
         assert np.linalg.norm(r) / np.linalg.norm(b[k]) <= 1e-10, (k, st_)
     s.close()
+
+
+@pytest.mark.parametrize("case", [
+    # dims, block, sub-block, storage, right-hand sides: tiles of 4 with an idle slot, of 8 with three, of 2 with
+    # one (a grid that fills the GPU), of 1 and 2 (one that does not)
+    ((16, 16, 16, 16), (2, 2, 2, 2), (1, 1, 1, 1), q.QCD_F16, 3),
+    ((16, 16, 16, 16), (2, 2, 2, 2), (1, 1, 1, 1), q.QCD_F32, 5),
+    ((16, 16, 16, 32), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 5),
+    ((8, 8, 8, 16), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F16, 7),
+    ((8, 8, 8, 8), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 12),
+], ids=lambda c: "%s-%s-%s-n%d" % ("x".join(map(str, c[0])), "x".join(map(str, c[1])),
+                                   "f16" if c[3] == q.QCD_F16 else "f32", c[4]))
+def test_tile_width_does_not_change_results(case):
+    """However many right-hand sides a CTA takes, and with idle ones in its last tile, each result is
+    that of the right-hand side alone, bit for bit."""
+    dims, b, sb, storage, nrhs = case
+    s = q.Solver(dims)
+    s.load_gauge(qi.gauge_field(dims, 0.3, seed=1016, device="cuda"))
+    s.build_clover(0.12, 1.6)
+    v = qi.gaussian_spinor_torch(dims, 2016, nrhs, "cuda").to(torch.complex64).contiguous()
+    prm = q.make_params(0.12, 1.6, b, sb, omega=1.2, nsweep=2, nsap=2, sap_storage=storage)
+    q.qcd_set_sap_ctas(s.ctx, -2)
+    out, one = torch.empty_like(v), torch.empty_like(v[:1])
+    s.sap_precondition(out, v, prm, nrhs=nrhs)
+    for k in range(nrhs):
+        s.sap_precondition(one, v[k:k + 1].contiguous(), prm)
+        torch.cuda.synchronize()
+        assert torch.equal(one[0], out[k]), k
+    s.close()
