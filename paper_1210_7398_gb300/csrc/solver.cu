@@ -320,7 +320,11 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
     bool x0_zero = true;
     for (int k = 0; k < R; k++) {
         bn2[k] = h[3 * k + 2];
-        x0_zero = x0_zero && h[3 * (R + k) + 2] == 0.0;
+        if (h[3 * (R + k) + 2] == 0.0) continue;
+        if (bn2[k] == 0)  // solved by x = 0, whatever the initial guess
+            QCD_CUDA(c, cudaMemsetAsync(w.x + (size_t)k * n, 0, sizeof(double2) * n, c->stream));
+        else
+            x0_zero = false;
     }
     // r = b - D x (r = b when every initial guess is zero); rh = r; p = v = 0
     if (x0_zero) {
@@ -362,7 +366,7 @@ int solve(qcd_ctx *c, double2 *x, const double2 *b, const qcd_params *p, int nrh
                 relres[k] = !std::isfinite(bn2[k]) ? INFINITY : bn2[k] > 0 ? std::sqrt(h[3 * k + 2] / bn2[k]) : 0.0;
         return QCD_OK;
     };
-    // rhs with b = 0 are solved by x = 0; rhs whose initial residual is small enough are done;
+    // rhs with b = 0 are solved (x = 0, inactive: r = 0); rhs whose initial residual is small enough are done;
     // rhs holding a non-finite value are settled (not converged) at once
     {
         bool any = false;

@@ -74,6 +74,27 @@ def test_solve_either_side_of_the_one_level_sum(lt, graphs):
     s.close()
 
 
+@pytest.mark.parametrize("others,guess", [(0, 1.0), (2, 1.0), (2, float("nan"))], ids=["alone", "beside", "beside-nan"])
+def test_zero_source_is_solved_by_zero(others, guess):
+    """b = 0 with an initial guess that is not 0: x = 0, alone and beside other right-hand sides, whose
+    solutions are those without it, bit for bit."""
+    dims, kappa = (8, 8, 8, 8), 0.12
+    s, _ = make_solver(dims, kappa, seed=1017)
+    prm = q.make_params(kappa, CSW, (4, 4, 4, 4), (2, 2, 2, 2), nsweep=2, nsap=1, omega=1.4, tol=1e-10)
+    b = qi.gaussian_spinor_torch(dims, 2017, others + 1, "cuda")
+    b[others] = 0
+    x = torch.zeros_like(b)
+    x[others] = guess
+    st = s.solve(x, b, prm, nrhs=others + 1)
+    assert torch.count_nonzero(x[others]) == 0
+    assert st["true_rel_res"] <= 1e-10
+    if others:
+        one = torch.zeros_like(b[:others])
+        s.solve(one, b[:others].contiguous(), prm, nrhs=others)
+        assert torch.equal(one, x[:others])
+    s.close()
+
+
 def test_tuning_cache_round_trip(tmp_path):
     dims, kappa = (8, 8, 8, 8), 0.12
     s, _ = make_solver(dims, kappa, seed=1012)
