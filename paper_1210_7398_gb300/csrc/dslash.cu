@@ -118,26 +118,40 @@ __device__ __forceinline__ void dslash_site(SP *__restrict__ out, const SP *__re
                                             const Geo &g, long n, int r0, const bool act[NR],
                                             const SP *__restrict__ other, float part[NR][3]);
 
+// The order in which the site blocks (128 sites) are taken: chunk by chunk of a t-slice, each through all of
+// t, so that what a chunk shares with the next slice is still in L2.
+struct BlockOrder {
+    int row = 0, chunk = 0;  // blocks per t-slice, per chunk (0: in order)
+};
+__device__ __forceinline__ int block_of(const BlockOrder &o, int q, int nblk) {
+    const int rows = nblk / o.row;
+    if (q >= rows * o.row) return q;  // past the whole slices
+    const int c = q / (o.chunk * rows), first = c * o.chunk, w = min(o.chunk, o.row - first);
+    q -= first * rows;
+    return q / w * o.row + first + q % w;
+}
+
 // The same with NR right-hand sides per thread (each link and the clover field loaded once for
 // all of them).  MODE fuses the inner products the BiCGStab step after D needs into the
 // epilogue: 1: <other, out> and |out|^2, 2: <out, other> and |out|^2, 0: none; each CTA (128
 // consecutive sites) sums its sites per right-hand side by a fixed tree (a butterfly within each
-// warp, then the four warps in order) into partial[rhs][3][blockIdx.x], so a right-hand side's
-// inner products do not depend on which others share its threads.  partial[rhs][3][site block].  Right-hand sides inactive
+// warp, then the four warps in order) into partial[rhs][3][site block], so a right-hand side's
+// inner products do not depend on which others share its threads.  Right-hand sides inactive
 // in gate (may be null) are skipped, their partials zero.
-template <int MINB, int NR, typename R, typename SP, typename LK, typename CL, int MODE = 0>
+template <int MINB, int NR, typename R, typename SP, typename LK, typename CL, int MODE = 0, bool CHUNKED = false>
 __global__ void __launch_bounds__(128, MINB) dslash_kernel_nr(SP *__restrict__ out, const SP *__restrict__ in,
                                                      const LK *__restrict__ U, const CL *__restrict__ F,
                                                      R kappa, Geo g, int nrhs,
                                                      const SP *__restrict__ other, double *__restrict__ partial,
-                                                     const BicgScalars *__restrict__ gate) {
+                                                     const BicgScalars *__restrict__ gate, BlockOrder order) {
     using C = typename CT<R>::C;
     chain_wait(in, other, gate);
     // the right-hand-side tile varies fastest over the (1-D) grid: the CTAs of one site block
     // run together and share its links and clover field through L2
     const int ntile = (nrhs + NR - 1) / NR;
-    const long sblk = blockIdx.x / ntile;
+    long sblk = blockIdx.x / ntile;
     const int r0 = (int)(blockIdx.x - sblk * ntile) * NR;
+    if constexpr (CHUNKED) sblk = block_of(order, (int)sblk, gridDim.x / ntile);
     const long n = sblk * blockDim.x + threadIdx.x;
     float part[NR][3];
 #pragma unroll
@@ -433,9 +447,30 @@ static int ensure_u12(qcd_ctx *c, const Geo &g) {
 
 int dslash32_prepare(qcd_ctx *c) { return ensure_u12(c, geo_of(c)); }
 
+// Where the fields and vectors of one t-slice exceed the 126 MB of L2 its blocks are taken in chunks of 32 MB,
+// else in order.  us per launch of dslash32_tile, in order -> chunks of 16 / 32 / 48 / 64 MB: 48^3x96, 4 right-hand
+// sides (212 MB a slice) 4575 -> 4411 / 4373 / 4432 / 4563, 1 (117 MB) 1451 -> 1374 / 1346 / 1345 / 1350; 40^3x80, 4
+// (123 MB) 2248 -> 2150 / 2132 / 2160 / 2217; 32^3x64, 12 (138 MB) 2510 -> 2464 / 2453 / 2488 / 2594; but 40^3x80, 1
+// (68 MB) 629 -> 666 / 652 / 654 / 657, 32^3x64, 4 (63 MB) 849 -> 864 / 856 / 874 / 880, 24^3x48, 12 (58 MB) 700 -> 718
+// / 714 / 731 / 725.
+static BlockOrder block_order(const Geo &g, int nrhs) {
+    const long slice = (long)g.L[0] * g.L[1] * g.L[2], site = 288L * nrhs + 768;  // bytes: in, other, out; links, clover
+    BlockOrder o;
+    if (slice * site > 96L << 20) {
+        o.row = (int)std::max(1L, slice / 128);
+        o.chunk = (int)std::max(1L, (32L << 20) / (128 * site));
+    }
+    return o;
+}
+
 // The inner solver's D: FP32 with the links in the two-row form (the third row rebuilt in
-// registers), one right-hand side per thread, with FP32 accuracy.  At 24^3x48 with 12 right-hand sides
-// and the fused inner products it takes 0.71 ms.
+// registers), one right-hand side per thread, with FP32 accuracy.  A lane's spinor lies 96 bytes from its neighbour
+// lane's, so a 32-byte load of a warp touches 24 lines where a plane of the earlier layout took 4, and the kernel
+// is slower than it was on planes: 24^3x48 with 12 right-hand sides 700 us against 620, 48^3x96 with 4 4373
+// against 3873, with 1 1346 against 1332.  us with 3 / 4 / 5 / 6 / 7 blocks per SM: 24^3x48 with 12 810 / 700 / 730 /
+// 711 / 723, 48^3x96 with 4 (in order) 5196 / 4572 / 4802 / 4749 / 4794; two right-hand sides per thread with 3 / 4
+// blocks 834 / 815 and 5519 / 5457; full links 813 and 5047, two per thread 834 and 5394; two or four right-hand sides in
+// the lanes of a warp 723 to 878 and 4654 to 5261.
 template <int MODE>
 static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, const float4 *other, double *red,
                          const BicgScalars *gate, const ScalarStep &step) {
@@ -446,8 +481,11 @@ static int dslash32_tile(qcd_ctx *c, float4 *out, const float4 *in, int nrhs, co
     if (rc) return rc;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
-    launch_chained(c, dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE>, dim3(nblk * nrhs), 128, 0, out, in,
-                   c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate);
+    const BlockOrder order = block_order(g, nrhs);
+    auto kernel = order.chunk ? dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE, true>
+                              : dslash_kernel_nr<4, 1, float, float4, float4, float4, MODE>;
+    launch_chained(c, kernel, dim3(nblk * nrhs), 128, 0, out, in, c->U12, c->F32, (float)c->kappa, g, nrhs, other, part, gate,
+                   order);
     rc = prof_end(c, QCD_K_DSLASH32, ev);
     if (rc || !MODE) return rc;
     return reduce_tiles(c, part, nblk, nrhs, red, step);
@@ -463,7 +501,7 @@ int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * ((nrhs + 1) / 2)));
         launch_chained(c, dslash_kernel_nr<4, 2, float, float4, float2, float4>, grid, 128, 0, out, in, c->U32, c->F32,
-                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr, BlockOrder());
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
@@ -495,7 +533,7 @@ int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
         launch_chained(c, dslash_kernel_nr<4, 1, float, float4, __half2, uint2>, grid, 128, 0, out, in, c->U16, c->F16,
-                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr, BlockOrder());
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }
@@ -511,7 +549,7 @@ int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     } else {
         dim3 grid((unsigned)((g.V + 127) / 128 * nrhs));
         launch_chained(c, dslash_kernel_nr<4, 1, float, float4, float4, float4>, grid, 128, 0, out, in, c->U12, c->F32,
-                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr);
+                       (float)c->kappa, g, nrhs, nullptr, nullptr, nullptr, BlockOrder());
     }
     return prof_end(c, QCD_K_DSLASH32, ev);
 }

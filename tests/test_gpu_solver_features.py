@@ -74,6 +74,28 @@ def test_solve_either_side_of_the_one_level_sum(lt, graphs):
     s.close()
 
 
+@pytest.mark.parametrize("dims,block,sub", [((30, 36, 30, 4), (5, 6, 5, 2), (5, 2, 5, 1)),  # 253.1 blocks of 128 sites a slice
+                                            ((32, 32, 32, 2), (4, 4, 4, 1), (2, 2, 2, 1))])  # 256
+def test_chunked_block_order_does_not_change_results(dims, block, sub):
+    """With 12 right-hand sides a t-slice exceeds L2, and the inner solver's D takes its site blocks chunk by
+    chunk (62 of them, the last chunk narrower, a block past the whole slices); alone it takes them in
+    order.  The solutions are the same, bit for bit."""
+    kappa = 0.12
+    s = q.Solver(dims)
+    s.load_gauge(qi.gauge_field(dims, 0.3, seed=1018, device="cuda"))
+    s.build_clover(kappa, CSW)
+    prm = q.make_params(kappa, CSW, block, sub, nsweep=2, nsap=1, omega=1.4, tol=1e-10, sap_storage=q.QCD_F16, sap_ctas=-2)
+    b = qi.gaussian_spinor_torch(dims, 2018, 12, "cuda")
+    x, one = torch.zeros_like(b), torch.zeros_like(b[:1])
+    st = s.solve(x, b, prm, nrhs=12)
+    assert st["true_rel_res"] <= 1e-10
+    for k in (0, 11):
+        one.zero_()
+        s.solve(one, b[k:k + 1].contiguous(), prm)
+        assert torch.equal(one[0], x[k])
+    s.close()
+
+
 @pytest.mark.parametrize("others,guess", [(0, 1.0), (2, 1.0), (2, float("nan"))], ids=["alone", "beside", "beside-nan"])
 def test_zero_source_is_solved_by_zero(others, guess):
     """b = 0 with an initial guess that is not 0: x = 0, alone and beside other right-hand sides, whose
