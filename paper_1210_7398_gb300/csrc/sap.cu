@@ -1254,7 +1254,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
     int Cuse = Cfit;
     if (min_ctas <= 0)
         for (int C = 2; C <= 8; C *= 2)
-            if (C > Cuse && (long)nblk1 * C <= sms) Cuse = C;
+            if (C > Cuse && C <= np.vol && (long)nblk1 * C <= sms) Cuse = C;  // (a site per CTA at least)
     if (!fit(Cuse)) return QCD_ERR_ARG;
     make_run(np);
     return QCD_OK;

@@ -483,6 +483,8 @@ QUAD_EDGE_CASES = [
     # dims, block, sub-block, storage, cluster width, right-hand sides: the ends of a step's warps and of the
     # range of blocks.  A step takes 8 sites per warp, at most 64 (clusters), 96 (one CTA per SM) or 16 sites.
     ((2, 2, 2, 2), (1, 1, 1, 1), (1, 1, 1, 1), q.QCD_F32, 1, 1),  # every hop leaves the block
+    ((2, 2, 2, 2), (1, 1, 1, 1), (1, 1, 1, 1), q.QCD_F32, 0, 1),  # the automatic width: a CTA per site at most
+    ((2, 4, 2, 2), (1, 2, 1, 1), (1, 1, 1, 1), q.QCD_F16, 0, 2),
     ((2, 2, 4, 4), (1, 1, 2, 1), (1, 1, 1, 1), q.QCD_F16, 2, 2),  # a site per CTA, levels without a site in one
     ((6, 6, 6, 12), (3, 3, 3, 6), (3, 3, 3, 6), q.QCD_F32, 16, 1),  # CTAs without a site in most levels
     ((6, 6, 6, 12), (3, 3, 3, 6), (1, 1, 1, 2), q.QCD_F16, 3, 2),  # uneven shares

@@ -160,6 +160,16 @@ def test_automatic_width_on_gb300():
     assert t["ctas"] >= 1  # the thread form does not fit a 2592-site block: the warp form stands in
 
 
+@pytest.mark.parametrize("half", [False, True], ids=["f32", "f16"])
+@pytest.mark.parametrize("block,ctas", [((1, 1, 1, 1), 1), ((1, 2, 1, 1), 2), ((1, 1, 3, 1), 2), ((2, 1, 2, 1), 4), ((1, 5, 1, 1), 4)])
+def test_automatic_width_of_small_blocks(block, ctas, half):
+    """A block of few sites takes no more CTAs than it has sites, however many SMs are free."""
+    dims = tuple(2 * b for b in block)
+    t = q.qcd_sap_plan_tables(dims, block, (1, 1, 1, 1), half=half, sms=152)
+    assert t["ctas"] == ctas
+    check_schedule(block, (1, 1, 1, 1), t)
+
+
 def test_rejected_geometry():
     with pytest.raises(q.QcdError):
         q.qcd_sap_plan_tables((12, 12, 12, 24), (4, 4, 4, 4), (2, 2, 2, 2))  # 3 blocks along x
