@@ -417,7 +417,8 @@ __device__ __forceinline__ void load_y_other(const TileArgs &a, int rhs, long mm
 // A warp item is 16 (site, right-hand side) pairs of one level, two lanes each; the items of a level are
 // dealt to the warps in turn, the same in every pass, so a lane meets the same sites throughout and
 // keeps what it needs of them in its own tensor-memory columns.  ALL: every item has a slot there.
-template <bool HALF, int R, bool ALL>
+// FLAT (FP32): the prologue takes the block in one go (tile_flat).
+template <bool HALF, int R, bool ALL, bool FLAT = false>
 __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(TileArgs a) {
     chain_wait();
     using L = TileRec<HALF>;
@@ -514,14 +515,15 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
     float *const yh = ys + y_me + half_w, *const fh = fs + y_me + half_w;  // the lane's half in slot 0
 
     // ---- prologue: f = r (or v) + kappa F H_{cc'} y_{c'} on the block's sites ----
-    // FP16: f waits in tensor memory (in r without a slot) until the scale is known; r holds it where
-    // the epilogue needs it
+    // FP16: f waits in tensor memory (in r without a slot) until the scale is known, with the lanes that will
+    // take its sites; r holds it where the epilogue needs it.  FP32: r holds it, and a block of narrow levels is
+    // taken in one go (tile_flat)
     constexpr bool f_tm = HALF && ALL;
     const bool f_r = !f_tm || a.store_r;
     const float4 *src = a.first ? a.v + roff : rr;
     float m = 0.f;  // largest |component| of f seen by this thread (FP16 scale)
-    for (int l = 0; l <= top; l++) {
-        const int4 lv = __ldg(a.levels + l);
+    for (int l = 0; l <= (FLAT ? 0 : top); l++) {
+        const int4 lv = FLAT ? make_int4(0, a.vol * R, 0, 0) : __ldg(a.levels + l);
         int slot = lv.w + (warp < lv.z);
         for (int j = warp < lv.z ? warp - lv.z + nwarp : warp - lv.z; j * 16 < lv.y; j += nwarp, slot++) {
             if (!warp_active) continue;
@@ -579,7 +581,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
                 }
                 if (f_r) st_half(rr + 6 * (long)pt.x, f);
                 if constexpr (!HALF)
-                    if (l == 0) first_update(yh + (pt.y & 0xffff) * a.stride, f);
+                    if (FLAT ? pos < __ldg(a.levels).y / R : l == 0) first_update(yh + (pt.y & 0xffff) * a.stride, f);
             }
             __syncwarp();
             if (f_tm) tmem_st12(tm + 12 * slot, f);
@@ -1117,24 +1119,25 @@ int tile_build_records(qcd_ctx *c, const SapPlan &p, void *rec) {
 
 namespace {
 using TileKernel = void (*)(TileArgs);
-template <bool HALF, bool ALL> TileKernel tile_kernel(int R) {
+template <bool HALF, bool ALL, bool FLAT = false> TileKernel tile_kernel(int R) {
     switch (R) {
-        case 1: return k_sap_tile<HALF, 1, ALL>;
-        case 2: return k_sap_tile<HALF, 2, ALL>;
-        case 4: return k_sap_tile<HALF, 4, ALL>;
-        default: return k_sap_tile<HALF, 8, ALL>;
+        case 1: return k_sap_tile<HALF, 1, ALL, FLAT>;
+        case 2: return k_sap_tile<HALF, 2, ALL, FLAT>;
+        case 4: return k_sap_tile<HALF, 4, ALL, FLAT>;
+        default: return k_sap_tile<HALF, 8, ALL, FLAT>;
     }
 }
-TileKernel tile_kernel(bool half, bool all, int R) {
-    return half ? (all ? tile_kernel<true, true>(R) : tile_kernel<true, false>(R))
-                : (all ? tile_kernel<false, true>(R) : tile_kernel<false, false>(R));
+TileKernel tile_kernel(bool half, bool all, bool flat, int R) {
+    if (half) return all ? tile_kernel<true, true>(R) : tile_kernel<true, false>(R);
+    if (!all) return tile_kernel<false, false>(R);
+    return flat ? tile_kernel<false, true, true>(R) : tile_kernel<false, true>(R);
 }
 }  // namespace
 
 int tile_set_attributes(qcd_ctx *c) {
     for (int R = 1; R <= kTileMaxRhs; R *= 2)
-        for (int k = 0; k < 4; k++)
-            QCD_CUDA(c, cudaFuncSetAttribute((const void *)tile_kernel(k & 1, k >> 1, R),
+        for (int k = 0; k < 8; k++)
+            QCD_CUDA(c, cudaFuncSetAttribute((const void *)tile_kernel(k & 1, k >> 1 & 1, k >> 2, R),
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemLimit));
     return QCD_OK;
 }
@@ -1170,6 +1173,15 @@ float tile_cost(const SapPlan &p, int R, int nrhs) {
     const float filled = ctas * (float)items * (1.f + 1.12f / (float)R) / ((float)std::max(1, p.sms) * 16.f);
     return filled + 0.73f * (float)rounds;
 }
+
+// Whether the FP32 prologue takes the block's sites in one go instead of level by level: where no level has
+// more than 24 (site, right-hand side) pairs, one and a half warp items (and all hop sums have a slot).  The levels'
+// rounds then wait for memory one after the other for a few sites each.  us, level by level -> in one go: 2^4
+// blocks (levels of 1, 4, 6, 4, 1 sites), 2 cycles, 16^3x32: one right-hand side 680 -> 596, two 721 -> 655, four 873 ->
+// 839; 48^3x96: one 49262 -> 42981, four 63112 -> 60113; 2^3x4 blocks, 16^3x32: one 423 -> 381, two 497 -> 478, four (48
+// pairs) 734 -> 734.  Where levels fill their items the sites better stay with the lanes that sweep them: 3^3x6
+// blocks, 12^2x18x12, four (level of 52 to 156 pairs) 965 -> 987; 4^3x8, 32^3x64, four 10924 -> 11138.
+bool tile_flat(const SapPlan &p, int R) { return p.max_step * R <= 24; }
 
 // Tensor memory of a CTA: a slot of 12 FP32 columns per warp item, the items dealt to the warps in turn;
 // warps four apart share a lane quarter.  As many slots as fit the columns that leave the CTAs resident
@@ -1268,7 +1280,7 @@ int tile_sap_apply(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
         a.b[m] = p.b[m];
         a.nb[m] = p.nb[m];
     }
-    const TileKernel k = tile_kernel(p.half, all, R);
+    const TileKernel k = tile_kernel(p.half, all, tile_flat(p, R), R);
     const size_t rec_words = (size_t)p.vol * ((p.half ? kTileRecordBytesHalf : kTileRecordBytes) / 16);
     for (int j = 0; j < nsap; j++)
         for (int col = 0; col < 2; col++) {

@@ -84,6 +84,8 @@ EDGE_CASES = [
     ((6, 4, 6, 10), (3, 2, 3, 5), (3, 2, 3, 5), 1.1, 1, 1),
     ((6, 10, 2, 14), (3, 5, 1, 7), (1, 5, 1, 7), 0.9, 3, 2),
     ((12, 4, 4, 8), (6, 2, 2, 4), (2, 2, 1, 2), 1.3, 2, 1),
+    ((4, 4, 4, 4), (2, 2, 2, 2), (1, 1, 1, 1), 1.2, 2, 3),  # narrow levels: FP32 takes the prologue in one go
+    ((4, 4, 4, 8), (2, 2, 2, 4), (1, 1, 1, 2), 1.2, 1, 2),
 ]
 
 
@@ -203,6 +205,8 @@ def test_tile_solve_true_residual_under_oracle(st):
     ((16, 16, 16, 32), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 5),
     ((8, 8, 8, 16), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F16, 7),
     ((8, 8, 8, 8), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 12),
+    # levels of 12 pairs alone (the FP32 prologue in one go), of 48 for four (level by level)
+    ((16, 16, 16, 32), (2, 2, 2, 4), (1, 1, 1, 2), q.QCD_F32, 4),
 ], ids=lambda c: "%s-%s-%s-n%d" % ("x".join(map(str, c[0])), "x".join(map(str, c[1])),
                                    "f16" if c[3] == q.QCD_F16 else "f32", c[4]))
 def test_tile_width_does_not_change_results(case):
