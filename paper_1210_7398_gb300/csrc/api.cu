@@ -138,6 +138,12 @@ int ensure_io(qcd_ctx *c, size_t bytes) {
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 bool aligned32(const void *p) { return ((uintptr_t)p & 31) == 0; }
+// a caller's spinors to or from a copy of the library's
+int stage(qcd_ctx *c, void *dst, const void *src, size_t bytes, bool on_device) {
+    if (on_device) return copy_spinors(c, dst, src, bytes);
+    QCD_CUDA(c, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->stream));
+    return QCD_OK;
+}
 bool overlap(const void *a, size_t na, const void *b, size_t nb) {
     return (const char *)a < (const char *)b + nb && (const char *)b < (const char *)a + na;
 }
@@ -313,9 +319,9 @@ int qcd_apply_D(qcd_ctx *c, void *out, const void *in, int prec, int nrhs) {
     char *io = (char *)c->d_io;
     const void *din = cp_in ? io : in;
     void *dout = cp_out ? io + (cp_in ? bytes : 0) : out;
-    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(io, in, bytes, cudaMemcpyDefault, c->stream));
+    if (cp_in && (rc = stage(c, io, in, bytes, dev_in))) return rc;
     if ((rc = dslash(c, dout, din, prec, nrhs))) return rc;
-    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, dout, obytes, cudaMemcpyDefault, c->stream));
+    if (cp_out && (rc = stage(c, out, dout, obytes, dev_out))) return rc;
     if (!dev_in || !dev_out) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     return QCD_OK;
 }
@@ -341,9 +347,9 @@ int qcd_sap_precondition(qcd_ctx *c, float *out, const float *in, const qcd_para
     char *end = (char *)c->d_io + nw * bytes;
     const float4 *v = cp_in ? (const float4 *)end : (const float4 *)in;
     float4 *x = cp_out ? (float4 *)(end + (cp_in ? bytes : 0)) : (float4 *)out;
-    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(end, in, bytes, cudaMemcpyDefault, c->stream));
+    if (cp_in && (rc = stage(c, end, in, bytes, dev_in))) return rc;
     if ((rc = sap_apply(c, x, v, work, p->omega, p->nsweep, p->nsap, nrhs, nullptr, p->block_solver))) return rc;
-    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, x, bytes, cudaMemcpyDefault, c->stream));
+    if (cp_out && (rc = stage(c, out, x, bytes, dev_out))) return rc;
     if (!dev_in || !dev_out) QCD_CUDA(c, cudaStreamSynchronize(c->stream));
     return QCD_OK;
 }

@@ -150,11 +150,10 @@ extern "C" int qcd_sap_precondition_noalloc(qcd_ctx *c, float *out, const float 
     const size_t bytes = sizeof(float4) * 6 * (size_t)c->lat.V;
     const bool cp_in = ((uintptr_t)in & 31) || ((const char *)in < (char *)out + bytes && (char *)out < (const char *)in + bytes);
     const bool cp_out = ((uintptr_t)out & 31) != 0;
-    if (cp_in) QCD_CUDA(c, cudaMemcpyAsync(v, in, bytes, cudaMemcpyDeviceToDevice, c->stream));
+    if (cp_in && (rc = copy_spinors(c, v, in, bytes))) return rc;
     float4 *dst = cp_out ? x : reinterpret_cast<float4 *>(out);
     if ((rc = sap_apply_plan(c, plan, dst, cp_in ? v : reinterpret_cast<const float4 *>(in), work, p->omega, p->nsweep,
                              p->nsap)))
         return rc;
-    if (cp_out) QCD_CUDA(c, cudaMemcpyAsync(out, x, bytes, cudaMemcpyDeviceToDevice, c->stream));
-    return QCD_OK;
+    return cp_out ? copy_spinors(c, out, x, bytes) : QCD_OK;
 }

@@ -229,6 +229,8 @@ void dev_free(qcd_ctx *c, void *p);
 int spinor64_to_32(qcd_ctx *c, float4 *dst, const double2 *src, int nrhs);
 int spinor32_to_64(qcd_ctx *c, double2 *dst, const float4 *src, int nrhs);
 int links_to_internal(qcd_ctx *c, const double2 *canon);
+// copies device spinors that do not overlap, both on 16-byte boundaries
+int copy_spinors(qcd_ctx *c, void *dst, const void *src, size_t bytes);
 
 // clover (clover.cu)
 int build_clover(qcd_ctx *c, double kappa, double csw);

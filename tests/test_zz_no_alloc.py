@@ -82,6 +82,24 @@ def test_noalloc_kernel_forms_and_no_device_allocation(ctas):
     s.close()
 
 
+def test_noalloc_alignment_and_overlap():
+    """Spinors on a 16- but not a 32-byte boundary, and in place: copies in the fixed array, the same bits."""
+    dims, kappa = (4, 6, 4, 8), 0.12
+    s = solver(dims, kappa, seed=1003)
+    prm = q.make_params(kappa, CSW, (2, 3, 2, 4), (1, 3, 1, 2), omega=1.1, nsweep=2, nsap=2)
+    v = torch.from_numpy(qi.gaussian_spinor(dims, seed=3004)[0].astype(np.complex64)).cuda()
+    out, inplace = torch.empty_like(v), v.clone()
+    off = [torch.zeros(v.numel() + 2, dtype=v.dtype, device="cuda")[2:].view(v.shape) for _ in range(2)]
+    assert all(t.data_ptr() % 32 == 16 for t in off)
+    off[0].copy_(v)
+    q.qcd_sap_precondition_noalloc(s.ctx, out, v, prm)
+    q.qcd_sap_precondition_noalloc(s.ctx, off[1], off[0], prm)
+    q.qcd_sap_precondition_noalloc(s.ctx, inplace, inplace, prm)
+    torch.cuda.synchronize()
+    assert torch.equal(off[1], out) and torch.equal(inplace, out)
+    s.close()
+
+
 def test_noalloc_rejects_lattices_above_its_limit():
     dims = (16, 16, 16, 16)  # 65,536 sites > 41,472
     s = solver(dims, 0.12, seed=7)
