@@ -258,7 +258,7 @@ int qcd_set_graphs(qcd_ctx *ctx, int on);
  * right-hand sides of a block in one CTA.  min_ctas >= 1: the cluster form with
  * the smallest such C >= min_ctas.  0 (default): the cluster form with the
  * largest C in {1, 2, 4, 8} for which one colour's clusters still fit the SM
- * count (at least the smallest C that fits).  -1: the thread form where it fits,
+ * count, and at least the smallest power of two that fits.  -1: the thread form where it fits,
  * -2: the tile form where it fits, else as 0.  More CTAs per block spread a
  * level's sites over more SMs at the price of more cluster barriers. */
 int qcd_set_sap_ctas(qcd_ctx *ctx, int min_ctas);

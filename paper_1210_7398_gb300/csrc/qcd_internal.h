@@ -35,10 +35,10 @@ struct Lattice {
 
 // SAP geometry: block decomposition (Eq. (3)) plus the ll-order schedule of
 // the SSOR passes, grouped into dependency levels (steps) whose sites are
-// pairwise non-adjacent.  For the SSOR kernel each block is dealt over C CTAs
+// pairwise non-adjacent.  For the cluster form each block is dealt over C CTAs
 // (a thread-block cluster when C > 1), each CTA owning an equal share of every
 // level, and each level into chunks of at most nslot sites per CTA; the chunks
-// form the kernel's timeline (forward pass, then the reversed backward pass).
+// are the kernel's steps (forward pass, then the reversed backward pass).
 // flags[p] (p < 2*nchunks) asks for a CTA (1) or cluster (2) barrier before
 // timeline step p of every sweep.
 struct SapPlan {
@@ -59,14 +59,12 @@ struct SapPlan {
     size_t smem_bytes = 0;
     std::vector<int> h_chunk_ptr;   // [C][nchunks + 1], offsets into h_chunk_site
     std::vector<int> h_chunk_site;  // block-local site indices, CTA-major
-    std::vector<unsigned char> h_flags;  // [2 * nchunks], thread form
+    std::vector<unsigned char> h_flags;  // [2 * nchunks] barrier before a step (tile form: made for diagnostics only)
     std::vector<int> h_site_off;    // [vol] global index offset of a block-local site from its block origin
     std::vector<int> h_own;         // [vol] (owning CTA << 24) | index in that CTA's slab of y
     std::vector<int> h_own_off;     // [C][slab_vol] global offset of each owned site, -1 past the last
     std::vector<int> h_quad;        // cluster form: [vol][4 lanes][4] neighbour codes in the order of h_chunk_site
-    std::vector<int> h_run_ptr;     // cluster form: [C][nrun + 1] steps of the kernel, offsets into h_chunk_site
-    std::vector<unsigned char> h_run_flags;  // cluster form: [2 * nrun] barrier before a step
-    int nrun = 0, form = 0;  // steps; which instance of the kernel
+    int form = 0;                   // cluster form: which instance of the kernel
     int ypitch = 0;                 // cluster form: words from spinor to spinor in a CTA's slab
     std::vector<int> h_pos;         // thread form: [vol] level position of each block-local site
     std::vector<int> h_origin_site[2];  // [nblk[c]] global index of each block origin
@@ -74,11 +72,8 @@ struct SapPlan {
     int2 *d_chunk_site = nullptr;   // (block-local site, global offset from the block origin)
     unsigned char *d_flags = nullptr;
     int *d_site_off = nullptr;
-    int *d_own = nullptr;
     int *d_own_off = nullptr;
     int4 *d_quad = nullptr;
-    int *d_run_ptr = nullptr;
-    unsigned char *d_run_flags = nullptr;
     int *d_pos = nullptr;
     int *d_origin_site[2] = {nullptr, nullptr};
     std::vector<int4> h_tile_pos;   // tile form: [2][vol][2] per pass, level position and lane of a pair
@@ -88,7 +83,7 @@ struct SapPlan {
     std::vector<int4> h_tile_item;  // tile form: [4][nsteps] the levels' positions and warps, R = 1, 2, 4, 8
     int4 *d_tile_item = nullptr;
     int tile_zslots = 1;            // tile form: zero slots after the vol site slots
-    float *d_rec = nullptr;         // per-site records (links, clover, neighbour codes), V x 912 bytes
+    float *d_rec = nullptr;         // per-site records (links, clover) of the form's layout
     long rec_version = -1;          // field version the records were built from
 };
 

@@ -74,9 +74,8 @@ __device__ __forceinline__ void masked_hops(const float4 *src, const float2 *__r
 
 namespace cg = cooperative_groups;
 
-constexpr int kMaxSlots = 32;      // most sites of one CTA in one chunk of the plan
-// Most sites of one CTA in one step of the kernel (consecutive chunks of a level run together): clusters;
-// one CTA per block and per SM; one CTA per block, several per SM.  Sites beyond the warps of a step start
+// Most sites of one CTA in one step of the kernel: clusters; one CTA per block and per SM; one CTA per block,
+// several per SM.  Sites beyond the warps of a step start
 // another step without a barrier, but wait for their records then.  Measured, 6^3x12 blocks: 24^3x48 FP16,
 // C = 1: 24 sites 6190 us, 48 4122, 64 3342, 96 2919; 12^3x24 FP32, C = 8 (52 sites in the widest level):
 // 24 sites 1633 us, 32 1487, 64 1258, and 8^4 blocks FP16: 32 sites 297 us, 48 273, 64 250, 96 327.  Where
@@ -86,9 +85,8 @@ constexpr int kMaxRunAlone = 96;
 constexpr int kMaxRunShared = 16;
 constexpr int kMaxCluster = 16;    // CTAs per SAP block (clusters above 8 need the non-portable size)
 constexpr size_t kSmemLimit = 200 * 1024;
-// shared memory a plan sets aside per site of a chunk, beside the slab, when it chooses the CTAs per block
-constexpr size_t kSlotBytes = 3984, kSlotBytesHalf = 2256;
-constexpr size_t kCtaSmemLimit = 227 * 1024;  // dynamic shared memory of one CTA (GB300)
+// most bytes of spinors per CTA of the cluster form where 16 CTAs allow it
+constexpr size_t kSlabLimit = 128 * 1024, kSlabLimitHalf = 140 * 1024;
 
 // Per-site record of the SSOR kernel (k_ssor_quad), in 4-byte words: what its four lanes read, 36 complex
 // numbers each (2 words in FP32 storage, 1 word, a half2, in FP16).  Lane j has W_d of directions j and
@@ -948,10 +946,8 @@ void assign_owners(SapPlan &np, int C) {
 }
 
 // Deals the block over C CTAs (assign_owners) and cuts every step (level) of each CTA into
-// chunks of at most maxslots sites, of equal size.  Returns false if the shared memory of a
-// CTA (its slab of y plus the staging ring) would exceed kSmemLimit.
-bool make_chunks(SapPlan &np, int C, int maxslots, bool check_smem = true) {
-    if (C > np.vol) return false;
+// chunks of at most maxslots sites, of equal size: the steps that the kernel runs.
+void make_chunks(SapPlan &np, int C, int maxslots) {
     np.C = C;
     assign_owners(np, C);
     std::vector<std::vector<int>> per(C);
@@ -980,13 +976,6 @@ bool make_chunks(SapPlan &np, int C, int maxslots, bool check_smem = true) {
     }
     np.nchunks = nchunks;
     np.nslot = nslot;
-    np.nwarps = nslot;
-    size_t most_sites = 0;
-    for (int r = 0; r < C; r++) most_sites = std::max(most_sites, lists[r].size());
-    const int ywords = np.half ? Rec<true>::ywords : Rec<false>::ywords;
-    np.smem_bytes = (size_t)np.slab_vol * ywords * 4 + (size_t)nslot * (np.half ? kSlotBytesHalf : kSlotBytes) +
-                    sizeof(int) * ((nchunks + 1 + 3) & ~3) + sizeof(int2) * ((most_sites + 1) & ~1) + 16;
-    if (check_smem && np.smem_bytes > kSmemLimit) return false;
     np.h_chunk_ptr.clear();
     np.h_chunk_site.clear();
     for (int r = 0; r < C; r++) {
@@ -994,7 +983,6 @@ bool make_chunks(SapPlan &np, int C, int maxslots, bool check_smem = true) {
         for (int v : ptr[r]) np.h_chunk_ptr.push_back(off + v);
         np.h_chunk_site.insert(np.h_chunk_site.end(), lists[r].begin(), lists[r].end());
     }
-    return true;
 }
 
 // Barriers of the timeline.  A site reads its in-block neighbours (those owned
@@ -1066,29 +1054,27 @@ void make_flags(SapPlan &np) {
         if (!stabbed(v) && v.second > 0) np.h_flags[v.second % P] = 1;
 }
 
-// What k_ssor_quad runs: its instance, the timeline in as few steps as that instance allows (consecutive
-// chunks of a level together; the list of sites keeps its order), the barriers, made for these steps, the
-// neighbour codes (SsorArgs::quad) in the order of the list, and the shared memory.
-void make_run(SapPlan &np) {
-    {
-        const long ctas = (long)(np.nb[0] * np.nb[1]) * (np.nb[2] * np.nb[3]) / 2 * np.C;  // of one colour
-        np.form = np.C > 1 ? kFormCluster : ctas <= np.sms ? kFormAlone : kFormShared;
-        SapPlan run = np;
-        const int most[] = {kMaxRunShared, kMaxRunAlone, kMaxRun};
-        make_chunks(run, np.C, most[np.form], false);
-        make_flags(run);
-        np.nrun = run.nchunks;
-        np.nwarps = (run.nslot + 7) / 8;
-        np.h_run_ptr = run.h_chunk_ptr;
-        np.h_run_flags = run.h_flags;
-    }
+// The cluster form with C CTAs per block: the instance of k_ssor_quad, its steps and its shared memory.
+// False where the block has fewer sites, a CTA's spinors exceed slab_limit or its shared memory kSmemLimit.
+bool make_quad_plan(SapPlan &np, int C, size_t slab_limit) {
+    if (C > np.vol) return false;
+    const long ctas = (long)(np.nb[0] * np.nb[1]) * (np.nb[2] * np.nb[3]) / 2 * C;  // of one colour
+    np.form = C > 1 ? kFormCluster : ctas <= np.sms ? kFormAlone : kFormShared;
+    const int most[] = {kMaxRunShared, kMaxRunAlone, kMaxRun};
+    make_chunks(np, C, most[np.form]);
+    np.nwarps = (np.nslot + 7) / 8;
     const int plain = np.half ? Rec<true>::ywords : Rec<false>::ywords;
     auto bytes = [&](int pitch) {
-        return sizeof(float) * ((size_t)(np.slab_vol + 1) * pitch + kMaxCluster + 4) + sizeof(int) * (np.nrun + 1);
+        return sizeof(float) * ((size_t)(np.slab_vol + 1) * pitch + kMaxCluster + 4) + sizeof(int) * (np.nchunks + 1);
     };
     // FP32: 28 words from spinor to spinor spread 16-byte accesses over all banks (24: over half of them)
     np.ypitch = !np.half && bytes(28) <= kSmemLimit ? 28 : plain;
     np.smem_bytes = bytes(np.ypitch);
+    return sizeof(float) * plain * (size_t)np.slab_vol <= slab_limit && np.smem_bytes <= kSmemLimit;
+}
+
+// the neighbour codes (SsorArgs::quad) of the cluster form, in the order of the chunks' list of sites
+void make_codes(SapPlan &np) {
     np.h_quad.assign(16 * (size_t)np.vol, 0);
     for (int k = 0; k < np.vol; k++) {
         const int yl = np.h_chunk_site[k], own = np.h_own[yl];
@@ -1205,7 +1191,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
     // the right-hand-side tiled thread form on request (min_ctas == -2), the block spinor of
     // one right-hand side in one CTA
     if (min_ctas == -2) {
-        make_chunks(np, 1, 1 << 20, false);  // one chunk per level, in level order (diagnostics)
+        make_chunks(np, 1, 1 << 20);  // one chunk per level, in level order (diagnostics)
         if (np.vol + kTileZeroSlotsHalf < (1 << 16)) {  // slots are 16-bit
             tile_make_positions(np);
             if (tile_positions_valid(np) && tile_smem_bytes(np, 1) <= kTileSmemLimit) {
@@ -1221,7 +1207,7 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
     }
     // the thread form on request (min_ctas = -1), FP32 storage, the block spinor in one CTA
     if (min_ctas == -1 && !half) {
-        make_chunks(np, 1, 1 << 20, false);  // one chunk per level, in level order
+        make_chunks(np, 1, 1 << 20);  // one chunk per level, in level order
         const size_t smem = (size_t)np.vol * kTsY * 4 + sizeof(int) * ((np.nchunks + 1 + 3) & ~3) +
                             sizeof(int2) * ((np.vol + 1) & ~1);
         if (smem <= kSmemLimit) {
@@ -1234,29 +1220,27 @@ int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &np,
             return QCD_OK;
         }
     }
-    // CTAs per block: C <= 16 whose shared memory fits.  With min_ctas >= 1 the smallest such
-    // C >= min_ctas; with min_ctas = 0 the largest one that keeps the blocks of one colour (one
-    // CTA cluster each) within the SM count, and at least the smallest that fits
+    // CTAs per block.  With min_ctas >= 1 the smallest C >= min_ctas whose spinors keep to the slab limit; with
+    // min_ctas = 0 the smallest such power of two, and then as many (up to 8, the portable cluster size) as keep
+    // one colour's clusters within the SM count.  A block too large for that takes 16 CTAs.
+    // Few CTAs with large slabs leave an SM few warps, and a C that is no power of two breaks the dealing of
+    // whole sub-blocks to CTAs (two sweeps, one cycle, one right-hand side, us): 32^3x64, 8^4 blocks, FP32: C = 2
+    // (192 KB) 2881, 3 3913, 4 (96 KB) 3021, 5 5264, 8 3856; FP16: 1 (192 KB) 6541, 2 (96 KB) 2005, 3 2408, 4 2024;
+    // 48^3x32, 8^2x12x4, FP32: 2 (144 KB) 4459, 3 7221, 4 4780; 24^3x48, 6^3x8, FP32: 1 (162 KB) 2002, 2 999, 3 1613,
+    // 4 843; 12^4, FP16: 5 1663, 6 1356, 8 (122 KB) 1742, 10 1485, 16 1178, FP32: 10 (194 KB) 2652, 16 (122 KB) 1468.
+    // Filling the SMs, 12^3x24, 6^3x12 blocks, 3^3x6 sub-blocks, 4 sweeps and cycles: C = 4 1798 us, 8 1159, 12
+    // 1545, 16 1201; natural order 3921, 3161, 2882, 3013; 16^3x32, 8^4 blocks, FP16: 300, 241, 217, 252.
     const int nblk1 = np.nb[0] * np.nb[1] * np.nb[2] * np.nb[3] / 2;
-    // up to 32 sites (warps) per step and CTA where one colour's blocks leave SMs idle and the
-    // staging ring fits (fewer dependent steps), else 16 (more registers per thread; several
-    // blocks share an SM when many blocks fill the GPU)
-    const bool few = (long)nblk1 < sms;
-    auto fit = [&](int C) { return (few && make_chunks(np, C, kMaxSlots)) || make_chunks(np, C, 16); };
-    int Cfit = 0;
-    for (int C = std::max(1, min_ctas); C <= kMaxCluster && !Cfit; C++)
-        if (fit(C)) Cfit = C;
-    if (!Cfit) return QCD_ERR_ARG;
-    // automatic width: the largest power of two up to 8 (the portable cluster size) that keeps one
-    // colour's clusters within the SM count.  12^3x24, 6^3x12 blocks, 3^3x6 sub-blocks, 4 sweeps and
-    // cycles: C = 4 1798 us, 8 1159, 12 1545, 16 1201; natural order 3921, 3161, 2882, 3013; 16^3x32, 8^4
-    // blocks, FP16: 300, 241, 217, 252
-    int Cuse = Cfit;
+    int Cuse = 0;
+    for (int C = std::max(1, min_ctas); C <= kMaxCluster && !Cuse; C += min_ctas >= 1 ? 1 : C)
+        if (make_quad_plan(np, C, half ? kSlabLimitHalf : kSlabLimit)) Cuse = C;
+    if (!Cuse) Cuse = kMaxCluster;
     if (min_ctas <= 0)
         for (int C = 2; C <= 8; C *= 2)
             if (C > Cuse && C <= np.vol && (long)nblk1 * C <= sms) Cuse = C;  // (a site per CTA at least)
-    if (!fit(Cuse)) return QCD_ERR_ARG;
-    make_run(np);
+    if (!make_quad_plan(np, Cuse, kSmemLimit)) return QCD_ERR_ARG;
+    make_flags(np);
+    make_codes(np);
     return QCD_OK;
 }
 
@@ -1265,10 +1249,8 @@ size_t sap_table_bytes(const SapPlan &p) {
     return up16(sizeof(int) * p.h_origin[0].size()) + up16(sizeof(int) * p.h_origin[1].size()) +
            up16(sizeof(int) * p.h_origin_site[0].size()) + up16(sizeof(int) * p.h_origin_site[1].size()) +
            up16(sizeof(int) * p.h_chunk_ptr.size()) + up16(sizeof(int2) * p.h_chunk_site.size()) +
-           up16(sizeof(int) * p.h_site_off.size()) + up16(p.h_flags.size()) + up16(sizeof(int) * p.h_own.size()) +
-           up16(sizeof(int) * p.h_own_off.size()) + up16(sizeof(int) * p.h_pos.size()) +
+           up16(sizeof(int) * p.h_site_off.size()) + up16(p.h_flags.size()) + up16(sizeof(int) * p.h_own_off.size()) + up16(sizeof(int) * p.h_pos.size()) +
            up16(sizeof(int4) * p.h_tile_pos.size()) + up16(sizeof(int) * p.h_quad.size()) +
-           up16(sizeof(int) * p.h_run_ptr.size()) + up16(p.h_run_flags.size()) +
            (p.tile ? up16(sizeof(int) * p.h_tile_site.size()) + up16(sizeof(int4) * p.h_tile_item.size()) : 0);
 }
 
@@ -1296,18 +1278,15 @@ int sap_upload_tables(qcd_ctx *c, SapPlan &p, void *region) {
     p.d_chunk_site = (int2 *)put(cs.data(), sizeof(int2) * cs.size());
     p.d_site_off = (int *)put(p.h_site_off.data(), sizeof(int) * p.h_site_off.size());
     p.d_flags = (unsigned char *)put(p.h_flags.data(), p.h_flags.size());
-    p.d_own = (int *)put(p.h_own.data(), sizeof(int) * p.h_own.size());
     p.d_own_off = (int *)put(p.h_own_off.data(), sizeof(int) * p.h_own_off.size());
     p.d_pos = p.h_pos.empty() ? nullptr : (int *)put(p.h_pos.data(), sizeof(int) * p.h_pos.size());
-    p.d_run_ptr = p.h_quad.empty() ? nullptr : (int *)put(p.h_run_ptr.data(), sizeof(int) * p.h_run_ptr.size());
-    p.d_run_flags = p.h_quad.empty() ? nullptr : (unsigned char *)put(p.h_run_flags.data(), p.h_run_flags.size());
     p.d_quad = p.h_quad.empty() ? nullptr : (int4 *)put(p.h_quad.data(), sizeof(int) * p.h_quad.size());
     p.d_tile_pos = p.tile ? (int4 *)put(p.h_tile_pos.data(), sizeof(int4) * p.h_tile_pos.size()) : nullptr;
     p.d_tile_site = p.tile ? (int *)put(p.h_tile_site.data(), sizeof(int) * p.h_tile_site.size()) : nullptr;
     p.d_tile_item = p.tile ? (int4 *)put(p.h_tile_item.data(), sizeof(int4) * p.h_tile_item.size()) : nullptr;
     if (!p.d_origin[0] || !p.d_origin[1] || !p.d_origin_site[0] || !p.d_origin_site[1] || !p.d_chunk_ptr ||
-        !p.d_chunk_site || !p.d_site_off || !p.d_flags || !p.d_own || !p.d_own_off || (p.thread && !p.d_pos) ||
-        (!p.h_quad.empty() && (!p.d_quad || !p.d_run_ptr || !p.d_run_flags)) ||
+        !p.d_chunk_site || !p.d_site_off || !p.d_flags || !p.d_own_off || (p.thread && !p.d_pos) ||
+        (!p.h_quad.empty() && !p.d_quad) ||
         (p.tile && (!p.d_tile_pos || !p.d_tile_site || !p.d_tile_item)))
         return cuda_fail(c, cudaGetLastError(), "cudaMemcpyAsync(SAP tables)");
     // the host vectors may be released only once the copies have consumed them
@@ -1444,7 +1423,7 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
                                 (const void *)k_ssor_quad<false, 1>, (const void *)k_ssor_quad<true, 1>,
                                 (const void *)k_ssor_quad<false, 2>, (const void *)k_ssor_quad<true, 2>};
             for (const void *k : ks) {
-                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemLimit));
+                QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
                 QCD_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             }
             QCD_CUDA(c, cudaFuncSetAttribute(k_ssor_soa, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit));
@@ -1461,14 +1440,14 @@ int sap_apply_plan(qcd_ctx *c, const SapPlan &p, float4 *x, const float4 *v, flo
     a.vol = p.vol;
     a.C = p.C;
     a.slab_vol = p.slab_vol;
-    a.nchunks = p.thread ? p.nchunks : p.nrun;
+    a.nchunks = p.nchunks;
     a.ypitch = p.ypitch;
-    a.chunk_ptr = p.thread ? p.d_chunk_ptr : p.d_run_ptr;
+    a.chunk_ptr = p.d_chunk_ptr;
     a.quad = p.d_quad;
     a.chunk_site = p.d_chunk_site;
     a.site_off = p.d_site_off;
     a.own_off = p.d_own_off;
-    a.flags = p.thread ? p.d_flags : p.d_run_flags;
+    a.flags = p.d_flags;
     a.gate = gate;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];  // (the second as in launch_chained)

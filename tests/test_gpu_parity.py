@@ -494,6 +494,7 @@ QUAD_EDGE_CASES = [
     ((16, 16, 8, 8), (8, 8, 4, 4), (2, 2, 2, 2), q.QCD_F16, 3, 1),  # 128 sites of 384: two steps of 64
     ((16, 16, 16, 16), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 0, 2),
     ((12, 12, 12, 24), (2, 2, 2, 2), (2, 2, 2, 2), q.QCD_F16, 0, 1),  # more blocks than SMs
+    ((24, 24, 24, 28), (12, 12, 12, 14), (6, 6, 6, 7), q.QCD_F32, 0, 1),  # 16 CTAs of 1512 sites, 169 KB each
 ]
 
 

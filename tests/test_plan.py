@@ -153,11 +153,38 @@ def test_automatic_width_on_gb300():
     """The widths the kernels run with on 152 SMs: 8 CTAs per 6^3 x 12 block on 12^3 x 24 (8
     blocks per colour), one per block where the blocks of one colour fill the GPU."""
     t = q.qcd_sap_plan_tables((12, 12, 12, 24), (6, 6, 6, 12), (3, 3, 3, 6), sms=152)
-    assert (t["ctas"], t["levels"], t["nslot"]) == (8, 12, 26)
+    assert (t["ctas"], t["levels"], t["nslot"]) == (8, 12, 52)  # (52 sites of the widest level, one step)
     t = q.qcd_sap_plan_tables((24, 24, 24, 48), (4, 4, 4, 4), (2, 2, 2, 2), sms=152)
     assert t["ctas"] == 1
     t = q.qcd_sap_plan_tables((12, 12, 12, 24), (6, 6, 6, 12), (3, 3, 3, 6), sap_ctas=-1, sms=152)
     assert t["ctas"] >= 1  # the thread form does not fit a 2592-site block: the warp form stands in
+
+
+@pytest.mark.parametrize("dims,block,half,auto,least", [
+    # at the slab limits: 128 KB of FP32 spinors (1365 sites), 140 KB of FP16 ones (2986)
+    ((48, 48, 48, 48), (6, 6, 6, 6), False, 1, 1),
+    ((48, 48, 48, 48), (6, 6, 6, 8), False, 2, 2),
+    ((48, 48, 48, 32), (8, 8, 12, 4), False, 4, 3),
+    ((48, 48, 48, 32), (8, 8, 12, 4), True, 2, 2),
+    ((32, 32, 32, 64), (8, 8, 8, 16), False, 8, 7),
+    ((48, 48, 48, 48), (12, 12, 12, 12), False, 16, 16),
+    ((48, 48, 48, 48), (12, 12, 12, 12), True, 8, 7),
+    ((24, 24, 24, 32), (12, 12, 12, 16), False, 16, 16),  # beyond it with 16 CTAs, in 200 KB each
+])
+def test_width_of_large_blocks(dims, block, half, auto, least):
+    """Where the blocks fill the SMs: the automatic width is a power of two, a fixed one the least that
+    holds the block, up to 16 CTAs of 200 KB."""
+    sub = tuple(b // 2 for b in block)
+    t = q.qcd_sap_plan_tables(dims, block, sub, half=half, sms=152)
+    assert t["ctas"] == auto and t["smem_bytes"] <= 200 * 1024
+    check_schedule(block, sub, t)
+    t = q.qcd_sap_plan_tables(dims, block, sub, sap_ctas=1, half=half, sms=152)
+    assert t["ctas"] == least and t["smem_bytes"] <= 200 * 1024
+
+
+def test_block_beyond_a_cluster_is_rejected():
+    with pytest.raises(q.QcdError):  # 41,472 sites: 249 KB of FP32 spinors in each of 16 CTAs
+        q.qcd_sap_plan_tables((24, 24, 24, 48), (12, 12, 12, 24), (6, 6, 6, 12), sms=152)
 
 
 @pytest.mark.parametrize("half", [False, True], ids=["f32", "f16"])
