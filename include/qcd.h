@@ -276,14 +276,12 @@ int qcd_set_sap_form(qcd_ctx *ctx, int form);
  * block has a dependency level (a site's level is one more than the highest
  * level of its in-block neighbours earlier in the ll order); each CTA of the
  * block's cluster owns some sites of every level; each level is cut into
- * chunks (timeline steps of the forward pass; the backward pass runs them in
- * reverse, step 2 nchunks - 1 - c for chunk c; the cluster form runs consecutive
- * chunks of a level as one step, with the flags of the same rule for its steps),
- * and a barrier flag before a
+ * chunks (the kernel's steps in the forward pass; the backward pass runs them in
+ * reverse, step 2 nchunks - 1 - c for chunk c), and a barrier flag before a
  * step orders the steps that exchange data (1: CTA barrier, 2: cluster
- * barrier).  meta[8] receives: sites per block, levels, CTAs per block (C),
+ * barrier; the tile form has a barrier before every level and ignores the flags).  meta[8] receives: sites per block, levels, CTAs per block (C),
  * chunks, most sites of one CTA in one chunk, most sites one CTA owns,
- * thread form (0/1), shared memory bytes per CTA.  The arrays, each NULL or
+ * form (0 cluster, 1 thread, 2 tile), shared memory bytes per CTA.  The arrays, each NULL or
  * sized as stated, receive per block-local site (lexicographic, x fastest;
  * meta[0] entries): its level, its owning CTA, its offset in that CTA's slab
  * of the block spinor, its chunk; and flags[2 * meta[3]] per timeline step.
@@ -292,6 +290,16 @@ int qcd_set_sap_form(qcd_ctx *ctx, int form);
 int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half,
                         int sms, int meta[8], int *level, int *owner, int *slot, int *chunk,
                         unsigned char *flags);
+
+/* Diagnostic as qcd_sap_plan_tables: where the cluster form's kernel finds the spinors of a block.
+ * *pitch (may be NULL) receives the 4-byte words from one spinor to the next in a CTA's slab,
+ * codes (NULL or 10 entries per site of the block, in the block-local order above) for each site
+ * the neighbours in directions d = 2 mu + (backward) as (owning CTA << 24) | word in that CTA's
+ * slab (the zero spinor behind the slab where the hop leaves the block), the word of the site's own
+ * spinor, and the site's global index relative to the block origin.  QCD_ERR_ARG as there, and where
+ * another form would run. */
+int qcd_sap_plan_codes(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half,
+                       int sms, int *pitch, int *codes);
 
 /* Autotuner (no counterpart in the paper, which fixes 6^4 blocks with 3^4
  * sub-blocks).  Starting from *base (kappa, csw, tol, inner_tol, bc_t, limits),

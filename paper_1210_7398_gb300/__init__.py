@@ -26,7 +26,7 @@ KERNEL_CLASSES = ("dslash32", "dslash64", "ssor", "saphop", "blas", "other", "le
 EXPORTS = ("qcd_create", "qcd_destroy", "qcd_last_error", "qcd_set_boundary", "qcd_load_gauge",
            "qcd_build_clover", "qcd_apply_D", "qcd_sap_precondition", "qcd_solve", "qcd_set_profiling",
            "qcd_kernel_stats", "qcd_launch_count", "qcd_bench_dslash", "qcd_sap_precondition_noalloc",
-           "qcd_set_sap_ctas", "qcd_set_sap_form", "qcd_sap_plan_tables", "qcd_set_graphs", "qcd_autotune", "qcd_learned_weight_count",
+           "qcd_set_sap_ctas", "qcd_set_sap_form", "qcd_sap_plan_tables", "qcd_sap_plan_codes", "qcd_set_graphs", "qcd_autotune", "qcd_learned_weight_count",
            "qcd_learned_set_weights", "qcd_learned_get_weights", "qcd_learned_apply", "qcd_learned_loss_grad",
            "qcd_learned_train", "qcd_learned_evaluate", "qcd_solve_multi", "qcd_set_tune_cache", "qcd_bench_fp32_peak", "qcd_bench_smem_peak",
            "qcd_debug_inject_breakdown", "qcd_learned_save", "qcd_learned_load", "qcd_debug_tc_skip_commit")
@@ -96,6 +96,7 @@ def load_library(path: str = LIB_PATH):
         "qcd_set_sap_ctas": (I, [P, I]),
         "qcd_set_sap_form": (I, [P, I]),
         "qcd_sap_plan_tables": (I, [P, P, P, I, I, I, P, P, P, P, P, P]),
+        "qcd_sap_plan_codes": (I, [P, P, P, I, I, I, ctypes.POINTER(I), P]),
         "qcd_set_graphs": (I, [P, I]),
         "qcd_learned_weight_count": (ctypes.c_long, []),
         "qcd_learned_set_weights": (I, [P, P, ctypes.c_long]),
@@ -250,6 +251,19 @@ def qcd_sap_plan_tables(dims, block, subblock, sap_ctas: int = 0, half: bool = F
     out = {k: int(meta[i]) for i, k in enumerate(names)}
     out.update(level=arrs[0], owner=arrs[1], slot=arrs[2], chunk=arrs[3], flags=flags)
     return out
+
+
+def qcd_sap_plan_codes(dims, block, subblock, sap_ctas: int = 0, half: bool = False, sms: int = 152):
+    """(pitch, codes [vol][10]): where the cluster form finds a site's eight neighbours, itself and its
+    lattice site (host only, no GPU)."""
+    iv = lambda v: (ctypes.c_int * 4)(*[int(x) for x in v])
+    pitch = ctypes.c_int()
+    codes = np.empty((int(np.prod(block)), 10), dtype=np.int32)
+    rc = load_library().qcd_sap_plan_codes(iv(dims), iv(block), iv(subblock), int(sap_ctas), int(bool(half)), int(sms),
+                                           ctypes.byref(pitch), codes.ctypes.data_as(ctypes.c_void_p))
+    if rc != QCD_OK:
+        raise QcdError(rc, "qcd_sap_plan_codes: geometry rejected, or not the cluster form")
+    return pitch.value, codes
 
 
 def qcd_set_sap_form(ctx, form: int):

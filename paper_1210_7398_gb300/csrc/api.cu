@@ -502,10 +502,11 @@ int qcd_set_sap_form(qcd_ctx *c, int form) {
     return QCD_OK;  // the cluster form has one form
 }
 
-int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half, int sms,
-                        int meta[8], int *level, int *owner, int *slot, int *chunk, unsigned char *flags) {
-    if (!dims || !block || !subblock || !meta || sap_ctas < -2 || sap_ctas > 16 || sms < 1) return QCD_ERR_ARG;
-    qcd_ctx c;  // host-side planning only: no device, stream or allocation is touched
+// host-side planning only: no device, stream or allocation is touched
+static int plan_of(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half, int sms,
+                   SapPlan &p) {
+    if (!dims || !block || !subblock || sap_ctas < -2 || sap_ctas > 16 || sms < 1) return QCD_ERR_ARG;
+    qcd_ctx c;
     c.lat.V = 1;
     for (int m = 0; m < 4; m++) {
         if (dims[m] < 2) return QCD_ERR_ARG;
@@ -513,9 +514,33 @@ int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subbloc
         c.lat.V *= dims[m];
     }
     c.sms_override = sms;
+    return sap_plan_host(&c, block, subblock, p, sap_ctas, half != 0) == QCD_OK ? QCD_OK : QCD_ERR_ARG;
+}
+
+int qcd_sap_plan_codes(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half, int sms,
+                       int *pitch, int *codes) {
     SapPlan p;
-    if (sap_plan_host(&c, block, subblock, p, sap_ctas, half != 0) != QCD_OK) return QCD_ERR_ARG;
-    sap_plan_flags(p);
+    if (plan_of(dims, block, subblock, sap_ctas, half, sms, p) != QCD_OK || p.h_quad.empty()) return QCD_ERR_ARG;
+    if (pitch) *pitch = p.ypitch;
+    for (int k = 0; codes && k < p.vol; k++) {
+        const int *q = &p.h_quad[16 * (size_t)k];  // four lanes: directions j and j + 4, own word, offset
+        int *o = codes + 10 * (size_t)p.h_chunk_site[k];
+        for (int j = 0; j < 4; j++) {
+            o[j] = q[4 * j];
+            o[j + 4] = q[4 * j + 1];
+            if (q[4 * j + 2] != q[2] || q[4 * j + 3] != q[3]) return QCD_ERR_ARG;  // the lanes share these
+        }
+        o[8] = q[2];
+        o[9] = q[3];
+    }
+    return QCD_OK;
+}
+
+int qcd_sap_plan_tables(const int dims[4], const int block[4], const int subblock[4], int sap_ctas, int half, int sms,
+                        int meta[8], int *level, int *owner, int *slot, int *chunk, unsigned char *flags) {
+    SapPlan p;
+    if (!meta || plan_of(dims, block, subblock, sap_ctas, half, sms, p) != QCD_OK) return QCD_ERR_ARG;
+    if (p.tile) sap_plan_flags(p);
     const int vals[8] = {p.vol, p.nsteps, p.C, p.nchunks, p.nslot, p.slab_vol, p.tile ? 2 : p.thread ? 1 : 0,
                          (int)p.smem_bytes};
     for (int k = 0; k < 8; k++) meta[k] = vals[k];

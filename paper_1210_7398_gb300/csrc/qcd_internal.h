@@ -259,7 +259,7 @@ void use_sap_ctas(qcd_ctx *c, int sap_ctas);
 // block decomposition valid for the lattice (L % block == 0, L / block even and >= 2,
 // block % subblock == 0)
 bool sap_geometry_ok(const qcd_ctx *c, const int b[4], const int s[4]);
-// the barrier flags of the plan's chunks (sap_plan_host makes those its kernel runs with)
+// the barrier flags of a tile plan's chunks (diagnostics; sap_plan_host makes those that a kernel runs with)
 void sap_plan_flags(SapPlan &plan);
 // host part of a plan (tables in h_*; device pointers left null); QCD_ERR_ARG on bad geometry
 int sap_plan_host(const qcd_ctx *c, const int b[4], const int s[4], SapPlan &plan, int min_ctas = 1,

@@ -1,4 +1,5 @@
-"""Host-side pins of the SSOR block kernel's schedule (qcd_sap_plan_tables; no GPU needed).
+"""Host-side pins of the SSOR block kernel's schedule (qcd_sap_plan_tables, qcd_sap_plan_codes; no GPU
+needed).
 
 The schedule is checked against facts derived here, independently of the planner: the ll
 order from the oracle (Sec. 3), the block's nearest-neighbour relation from coordinates, and
@@ -7,10 +8,14 @@ the data each site update reads (its in-block neighbours) and writes (itself).
 * levels: every in-block neighbour that comes earlier in the ll order sits on a lower level
   and every later one on a higher level (so a level-by-level sweep reads what the sequential
   sweep reads), and levels are as low as that allows (longest-chain levels);
-* chunks: each chunk holds one level, chunks follow the level order, no CTA has more than
-  nslot sites in a chunk;
+* chunks (the steps that the kernel runs): each chunk holds one level, chunks follow the level
+  order, no CTA has more than nslot sites in a chunk, and (cluster form) nslot keeps to the kernel's
+  64 sites in clusters, 96 with one CTA per block and SM, 16 with several CTAs per SM;
 * ownership: every site has one owner and one slab offset, offsets are unique per CTA and
-  below the slab size, and (warp form) every level is dealt evenly over the CTAs;
+  below the slab size, and (cluster form) every level is dealt evenly over the CTAs;
+* neighbour codes (cluster form): each names the neighbour's owner and place in that CTA's slab, or
+  the zero spinor behind the reader's own slab where the hop leaves the block, and all lie within the
+  shared memory;
 * barriers: over three consecutive sweeps of the timeline (forward chunk c at step c,
   backward at 2 nchunks - 1 - c, periodic flags, the set-up barrier before step 0), every
   read of a neighbour's value is separated from the neighbour's previous and next write by
@@ -149,6 +154,59 @@ def test_ssor_schedule_is_consistent(geom, ctas, half):
     check_schedule(b, s, t)
 
 
+def check_codes(dims, b, s, t, ctas, half):
+    """The cluster form's neighbour codes against the owner and slot tables, and its step limits."""
+    pitch, codes = q.qcd_sap_plan_codes(dims, b, s, sap_ctas=ctas, half=half, sms=152)
+    vol, slab = t["vol"], t["slab_vol"]
+    assert pitch >= (12 if half else 24) and pitch % 4 == 0  # a spinor's words, 16-byte accesses
+    assert (slab + 1) * pitch * 4 <= t["smem_bytes"] <= 200 * 1024
+    blocks = int(np.prod(dims)) // vol // 2
+    assert t["nslot"] <= (64 if t["ctas"] > 1 else 96 if blocks <= 152 else 16)
+    y = np.array(np.unravel_index(np.arange(vol), b, order="F")).T
+    own = t["owner"].astype(np.int64)
+    stride = 1
+    for m in range(4):
+        for back in range(2):
+            leaves = y[:, m] == 0 if back else y[:, m] + 1 == b[m]
+            nb = np.where(leaves, 0, np.arange(vol) + (-stride if back else stride))
+            want = np.where(leaves, own << 24 | slab * pitch, own[nb] << 24 | t["slot"][nb].astype(np.int64) * pitch)
+            assert np.array_equal(codes[:, 2 * m + back], want)
+        stride *= b[m]
+    assert np.array_equal(codes[:, 8], t["slot"] * pitch)
+    assert np.array_equal(codes[:, 9], np.ravel_multi_index(tuple(y.T), dims, order="F"))
+
+
+@pytest.mark.parametrize("half", [False, True], ids=["f32", "f16"])
+@pytest.mark.parametrize("ctas", [0, 1, 2, 3, 8, 16])
+@pytest.mark.parametrize("geom", GEOMS, ids=lambda g: "x".join(map(str, g[1])) + "/" + "x".join(map(str, g[2])))
+def test_neighbour_codes(geom, ctas, half):
+    dims, b, s = geom
+    try:
+        t = q.qcd_sap_plan_tables(dims, b, s, sap_ctas=ctas, half=half, sms=152)
+    except q.QcdError:
+        assert ctas != 0
+        return
+    check_codes(dims, b, s, t, ctas, half)
+
+
+def test_neighbour_codes_only_of_the_cluster_form():
+    g = ((8, 8, 8, 8), (4, 4, 4, 4), (2, 2, 2, 2))
+    for ctas in (-1, -2):
+        assert q.qcd_sap_plan_tables(*g, sap_ctas=ctas)["thread"]
+        with pytest.raises(q.QcdError):
+            q.qcd_sap_plan_codes(*g, sap_ctas=ctas)
+
+
+def test_schedule_check_sees_a_missing_barrier():
+    """check_schedule fails on a table whose cluster barriers are CTA barriers, and on one with none."""
+    g = ((12, 12, 12, 24), (6, 6, 6, 12), (3, 3, 3, 6))
+    t = q.qcd_sap_plan_tables(*g, sms=152)
+    check_schedule(g[1], g[2], t)
+    for flags in (np.minimum(t["flags"], 1), 0 * t["flags"]):
+        with pytest.raises(AssertionError, match="without a barrier"):
+            check_schedule(g[1], g[2], dict(t, flags=flags))
+
+
 def test_automatic_width_on_gb300():
     """The widths the kernels run with on 152 SMs: 8 CTAs per 6^3 x 12 block on 12^3 x 24 (8
     blocks per colour), one per block where the blocks of one colour fill the GPU."""
@@ -157,7 +215,7 @@ def test_automatic_width_on_gb300():
     t = q.qcd_sap_plan_tables((24, 24, 24, 48), (4, 4, 4, 4), (2, 2, 2, 2), sms=152)
     assert t["ctas"] == 1
     t = q.qcd_sap_plan_tables((12, 12, 12, 24), (6, 6, 6, 12), (3, 3, 3, 6), sap_ctas=-1, sms=152)
-    assert t["ctas"] >= 1  # the thread form does not fit a 2592-site block: the warp form stands in
+    assert t["ctas"] >= 1  # the thread form does not fit a 2592-site block: the cluster form stands in
 
 
 @pytest.mark.parametrize("dims,block,half,auto,least", [
@@ -228,6 +286,8 @@ def test_ssor_schedule_random_shapes(geom, ctas, half):
         assert ctas not in (0, -1, -2)
         return
     check_schedule(b, s, t)
+    if t["thread"] == 0:
+        check_codes(dims, b, s, t, ctas, half)
 
 
 @pytest.mark.parametrize("C", [2, 4, 8, 16])
