@@ -453,10 +453,9 @@ FORM_CASES = [
 
 @pytest.mark.parametrize("case", FORM_CASES, ids=lambda c: "%s-%s-c%d-n%d" % (
     "x".join(map(str, c[1])), "f16" if c[3] == q.QCD_F16 else "f32", c[4], c[5]))
-def test_sap_lane_forms_identical(case):
-    """The 32-lane and the 8-lane site updates of the SSOR kernel perform the same
-    rounding steps in the same order: their SAP outputs are equal bit for bit (and the
-    automatic choice, per launch, equals both)."""
+def test_sap_cluster_form_repeats_and_batches(case):
+    """The cluster form against the oracle; a repeated call, the calls after each qcd_set_sap_form value (kept
+    without effect) and each right-hand side alone give the same bits."""
     dims, b, sb, storage, ctas, nrhs = case
     kappa = 0.12
     s, U, F = make_solver(dims, kappa, seed=1008)
@@ -464,18 +463,22 @@ def test_sap_lane_forms_identical(case):
     prm = q.make_params(kappa, CSW, b, sb, omega=1.1, nsweep=2, nsap=2, sap_storage=storage)
     q.qcd_set_sap_ctas(s.ctx, ctas)
     vin = torch.from_numpy(v.astype(np.complex64)).cuda()
-    outs = []
+    out, again, one = torch.empty_like(vin), torch.empty_like(vin), torch.empty_like(vin[:1])
+    s.sap_precondition(out, vin, prm, nrhs=nrhs)
     for form in (1, 2, 0):
         q.qcd_set_sap_form(s.ctx, form)
-        out = torch.empty_like(vin)
-        s.sap_precondition(out, vin, prm, nrhs=nrhs)
+        s.sap_precondition(again, vin, prm, nrhs=nrhs)
         torch.cuda.synchronize()
-        outs.append(out)
-    assert torch.equal(outs[0], outs[1])
-    assert torch.equal(outs[0], outs[2])
-    ref = oracle.sap(dims, U, F, kappa, b, sb, 1.1, 2, 2, v[0])
+        assert torch.equal(again, out)
+    with pytest.raises(q.QcdError):
+        q.qcd_set_sap_form(s.ctx, 3)
     tol = 1e-5 if storage == q.QCD_F32 else SAP_F16_TOL
-    assert rel_norm(outs[1][0].cpu().numpy().astype(np.complex128), ref) <= tol
+    for k in range(nrhs):
+        s.sap_precondition(one, vin[k:k + 1].contiguous(), prm)
+        torch.cuda.synchronize()
+        assert torch.equal(one[0], out[k])
+        ref = oracle.sap(dims, U, F, kappa, b, sb, 1.1, 2, 2, v[k])
+        assert rel_norm(out[k].cpu().numpy().astype(np.complex128), ref) <= tol
     s.close()
 
 
