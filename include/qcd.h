@@ -103,8 +103,8 @@ typedef struct {
                            qcd_learned_evaluate found it slower than plain SAP, in
                            which case plain SAP is used (the fallback).  2: always use
                            the learned correction                                     */
-    int sap_ctas;       /* SSOR kernel form, as qcd_set_sap_ctas (-1..16); 0 = context
-                           setting; results do not depend on it                       */
+    int sap_ctas;       /* SSOR kernel form, as qcd_set_sap_ctas (-2..16); 0 = context
+                           setting; results do not depend on it beyond rounding       */
     int block_solver;   /* SAP block inverse A_BB.  0: ll-ordered SSOR (Sec. 3; uses
                            subblock, omega, nsweep).  1: the even-odd alternative
                            Sec. 3 compares it with: nsweep minimal-residual steps on
@@ -220,7 +220,9 @@ int qcd_sap_precondition_noalloc(qcd_ctx *ctx, float *out, const float *in, cons
  * right-hand sides (complex128 [nrhs][V][4][3]), all advancing together
  * (batched kernels, per right-hand side scalars on the device; a converged
  * right-hand side drops out).  x holds the initial guess
- * on entry (zero it for x0 = 0) and the solution on return.  Synchronises.
+ * on entry (zero it for x0 = 0) and the solution on return (0 where b = 0).  A device x on
+ * a 32-byte boundary is iterated in place: after an error (QCD_ERR_CUDA, QCD_ERR_OOM,
+ * QCD_ERR_TIMEOUT) it holds the iterate reached, as after QCD_ERR_NOCONV.  Synchronises.
  * st may be NULL.  Returns QCD_OK when every right-hand side reached the
  * true relative residual p->tol. */
 int qcd_solve(qcd_ctx *ctx, double *x, const double *b, const qcd_params *p, int nrhs,
@@ -247,8 +249,9 @@ int qcd_solve_multi(int n, qcd_ctx *const *ctxs, double *const *x, const double 
  * host reading the active flags after each).  Results do not depend on it. */
 int qcd_set_graphs(qcd_ctx *ctx, int on);
 
-/* Tuning knob of the SAP block kernel; results do not depend on it.  The
- * block solve has three forms.  The cluster form runs four lanes per site
+/* Tuning knob of the SAP block kernel; results do not depend on it beyond rounding
+ * (the forms add a site's hops in different orders, and FP16 storage has one scale
+ * per CTA or block).  The block solve has three forms.  The cluster form runs four lanes per site
  * update over a cluster of C CTAs per block (C <= 16, each CTA owning an equal
  * share of every dependency level of the sweep and keeping its sites' spinors
  * in its shared memory, which must fit).  The thread form (FP32 storage, blocks

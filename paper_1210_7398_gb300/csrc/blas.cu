@@ -25,12 +25,12 @@ namespace {
 
 constexpr int RED_TPB = 256;
 constexpr int TPB = 256;
-constexpr long kOneLevelTiles = 6144;  // most tile partials that one block per right-hand side sums
+// Most tile partials that one block per right-hand side sums, in one launch instead of two.  Solves, us, two levels ->
+// one: 324 partials (12^3x24) 5112 -> 4959, 1024 7443 -> 7228 (four right-hand sides 18321 -> 18097), 2592 16080 ->
+// 15976, 5184 26050 -> 26056 (twelve 202133 -> 202097), 6144 30452 -> 30492 (238226 -> 238297), 8192 38266 -> 38398,
+// 16384 72432 -> 72991.
+constexpr long kOneLevelTiles = 6144;
 
-template <typename C> __device__ __forceinline__ double2 to_d(C a) { return make_double2((double)a.x, (double)a.y); }
-template <typename C> __device__ __forceinline__ C from_d(double2 a);
-template <> __device__ __forceinline__ double2 from_d<double2>(double2 a) { return a; }
-template <> __device__ __forceinline__ float2 from_d<float2>(double2 a) { return make_float2((float)a.x, (float)a.y); }
 
 // block-wide sum of 3 doubles in a fixed order (butterfly within each warp, then the warp sums
 // in warp order); result valid in thread 0.  sh: at least 3 * (RED_TPB / 32) doubles
@@ -244,7 +244,6 @@ template <typename A, typename E> __device__ __forceinline__ E v_msub(A a, E x, 
     a.y = -a.y;
     return v_madd(a, x, y);
 }
-__device__ __forceinline__ float4 v_sub(float4 x, float4 y) { return make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w); }
 __device__ __forceinline__ double2 v_sub(double2 x, double2 y) { return make_double2(x.x - y.x, x.y - y.y); }
 template <typename E> struct Scal { using T = double2; };
 template <> struct Scal<float4> { using T = float2; };
@@ -432,10 +431,6 @@ int blas_s_update32(qcd_ctx *c, float2 *s, const float2 *r, const float2 *v, con
 int blas_xr_update64(qcd_ctx *c, double2 *x, double2 *r, const double2 *ph, const double2 *sh, const double2 *s,
                      const double2 *t, const BicgScalars *S, long n, int nrhs) {
     QCD_BLAS_LAUNCH(k_xr_update<double2>, n, nrhs, x, r, ph, sh, s, t, S)
-}
-int blas_xr_update32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
-                     const float2 *t, const BicgScalars *S, long n, int nrhs) {
-    QCD_BLAS_LAUNCH(k_xr_update<float4>, n / 2, nrhs, F4(x), F4(r), CF4(ph), CF4(sh), CF4(s), CF4(t), S)
 }
 int blas_xr_update_dot32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
                          const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out,

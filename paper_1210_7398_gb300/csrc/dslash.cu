@@ -55,12 +55,12 @@ __device__ __forceinline__ void load_link(const float4 *__restrict__ U, long V, 
     u[8] = cross(u[0], u[4], u[1], u[3]);
 }
 
-// MINB: resident blocks per SM requested from the register allocator.  One right-hand side in
-// FP32 is bound by HBM (48^3x96: 1.40 ms, 5.8 TB/s of algorithmic bytes, 5 blocks; 2.04 ms with the
-// conversions to and from planes that the caller's layout does without), several by latency and L1
-// requests (24^3x48, 12: 672 us, 1200 with the conversions; L2 at
-// 55%, HBM at 45%, issue at 42%; staging spinors through shared memory, two lanes per site and links site by
-// site were all slower, 811 to 1170 us).  NR: right-hand sides per thread; each link and the
+// MINB: resident blocks per SM requested from the register allocator (each launch says what 3 to 7
+// take).  One right-hand side in FP32 is bound by HBM (48^3x96: 1.40 ms, 5.8 TB/s of algorithmic bytes;
+// 2.04 ms with the conversions to and from planes that the caller's layout does without), several by
+// latency and L1 requests (24^3x48, 12: 675 us, 1200 with the conversions; L2 at 55%, HBM at 45%, issue
+// at 42%; staging spinors through shared memory, two lanes per site and links site by site were all
+// slower, 811 to 1170 us).  NR: right-hand sides per thread; each link and the
 // clover field are loaded once and applied to all of them, so the field bytes
 // per right-hand side drop from 576 to 576 / NR (FP32).  Over the grid the
 // right-hand side (tile) index varies fastest, so the CTAs of one site block run
@@ -297,7 +297,7 @@ __device__ __forceinline__ void herm6_64(const double2 *__restrict__ F, long V, 
     for (int i = 0; i < 6; i++) y[i] = axpy64(f[i], x[i], y[i]);
 }
 // D in FP64.  Bound by the FP64 pipe (2 operations per clock and SM, which it reaches), so the order is the
-// one with few operations, 1,092 a site (1,200 in the plain order):
+// one with few operations, 1,092 a site (1,176 in the plain order):
 //  - t first, the colour products starting the sums (the projector's factor 2 and the boundary sign
 //    multiply them when the next hop is added);
 //  - along x, y, z the backward product is subtracted from the forward one as it is formed, D = w+ - w-, which is
@@ -495,6 +495,9 @@ int dslash32(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     Geo g = geo_of(c);
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
+    // us with 3 / 4 / 5 / 6 / 7 blocks per SM: one right-hand side on 8^3x16 3.76 / 3.81 / 3.87 / 4.30 / 5.64, 24^3x48 86.6 /
+    // 80.3 / 81.9 / 85.9 / 97.5, 48^3x96 1481 / 1434 / 1392 / 1429 / 1584; two per thread: four on 8^3x16 7.02 / 7.26 /
+    // 9.83 / 11.2 / 12.3, 48^3x96 4824 / 4407 / 6099 / 7033 / 8238, twelve on 24^3x48 777 / 682 / 1067 / 1280 / 1520
     if (nrhs == 1) {
         launch_chained(c, dslash_kernel<5, float, float4, float2, float4>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
                        out, in, c->U32, c->F32, (float)c->kappa, g, 1);
@@ -527,6 +530,10 @@ int dslash16(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     }
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
+    // us with 3 / 4 / 5 / 6 / 7 blocks per SM: one right-hand side on 8^3x16 3.66 / 3.68 / 3.82 / 3.89 / 4.13, 24^3x48 68.6 /
+    // 62.0 / 63.8 / 62.9 / 63.4, 48^3x96 1079 / 977 / 990 / 959 / 965; four on 8^3x16 4.53 / 4.69 / 4.89 / 5.02 / 5.20,
+    // 24^3x48 230 / 208 / 212 / 204 / 207, 48^3x96 4041 / 3841 / 3949 / 3720 / 3867; twelve on 24^3x48 668 / 610 / 619 /
+    // 586 / 594
     if (nrhs == 1) {
         launch_chained(c, dslash_kernel<4, float, float4, __half2, uint2>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
                        out, in, c->U16, c->F16, (float)c->kappa, g, 1);
@@ -543,6 +550,9 @@ int dslash12(qcd_ctx *c, float4 *out, const float4 *in, int nrhs) {
     if (int rc = ensure_u12(c, g)) return rc;
     cudaEvent_t ev;
     prof_begin(c, QCD_K_DSLASH32, &ev);
+    // us with 3 / 4 / 5 / 6 / 7 blocks per SM: one right-hand side on 8^3x16 3.63 / 3.66 / 3.81 / 4.02 / 4.20, 24^3x48 76.9 /
+    // 71.7 / 74.4 / 73.7 / 74.9, 48^3x96 1298 / 1184 / 1238 / 1192 / 1197; four on 24^3x48 241 / 213 / 222 / 223 / 224,
+    // 48^3x96 4327 / 3900 / 4220 / 4118 / 4179; twelve on 24^3x48 710 / 623 / 657 / 655 / 656
     if (nrhs == 1) {
         launch_chained(c, dslash_kernel<4, float, float4, float4, float4>, dim3((unsigned)((g.V + 127) / 128)), 128, 0,
                        out, in, c->U12, c->F32, (float)c->kappa, g, 1);

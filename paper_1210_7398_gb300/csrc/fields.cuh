@@ -180,7 +180,7 @@ __device__ __forceinline__ void clover_mul(const R f[72], const C v[12], C out[1
 // to acc (Dirac representation, gamma_k = [[0,-i s_k],[i s_k,0]], gamma_4 =
 // diag(1,1,-1,-1)); the projector has rank 2, so the colour multiply acts on
 // the two-component half-spinor h only.  sgn is the boundary sign of a hop
-// across the t edge (only MU = 3 can carry one).  
+// across the t edge (only MU = 3 can carry one).
 // the half-spinor h[spin row * 3 + colour] of (1 -/+ gamma_mu) psi
 template <int MU, bool FWD, typename C>
 __device__ __forceinline__ void hop_project(const C psi[12], decltype(C::x) sgn, C h[6]) {
@@ -258,8 +258,6 @@ __device__ __forceinline__ void hop_term(const C psi[12], const C u[9], decltype
     hop_reconstruct<MU, FWD>(w, acc);
 }
 
-// The same hop with the transport matrix given as it acts: W = U_mu(n) forward and
-// W = U_mu(n-mu)^dag backward, both as W h (row-major W[a][b]); sgn as above.
 // third row of a special unitary 3x3 matrix from its first two: row2 = conj(row0 x row1)
 // (Table 1's reconstruction of a link from 12 reals)
 template <typename C> __device__ __forceinline__ void su3_third_row(C W[9]);

@@ -10,8 +10,8 @@
 // allocates the gauge and clover fields) once at set-up, and afterwards call
 // this entry point, which only launches kernels and copies.
 //
-// Its scratch memory (the internal-layout input and output spinors, the two
-// SAP work spinors, the per-site SSOR records and the ll-schedule tables) lives in one file-scope
+// Its scratch memory (copies of an input and output that need one, the two SAP work
+// spinors, the per-site SSOR records and the ll-schedule tables) lives in one file-scope
 // __device__ array of fixed size, so the library reserves it on every GPU
 // that loads the library, until the process exits.  In host code the array's
 // name is only a host-side stand-in for the symbol; the device address is
@@ -20,8 +20,8 @@
 //
 // The array keeps what the last call built: the schedule tables and per-site records of one
 // context's fields, geometry and kernel form (per device).  A call that matches them only
-// converts the input, launches the SAP kernels and converts the output, all asynchronously on
-// the context stream; a call with another context, changed fields, geometry or form first plans
+// launches the SAP kernels on the caller's spinors (on copies of those off a 32-byte boundary or
+// overlapping), asynchronously on the context stream; a call with another context, changed fields, geometry or form first plans
 // on the host, uploads the tables and rebuilds the records, which synchronises the stream.
 #include <algorithm>
 #include <cstring>

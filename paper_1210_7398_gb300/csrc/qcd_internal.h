@@ -364,8 +364,6 @@ int blas_s_update32(qcd_ctx *c, float2 *s, const float2 *r, const float2 *v, con
 // x += alpha ph + om sh;  r = s - om t
 int blas_xr_update64(qcd_ctx *c, double2 *x, double2 *r, const double2 *ph, const double2 *sh, const double2 *s,
                      const double2 *t, const BicgScalars *S, long n, int nrhs);
-int blas_xr_update32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
-                     const float2 *t, const BicgScalars *S, long n, int nrhs);
 // the same, and out[rhs] = <rh, r>, |r|^2 of the new r (the reduction fused into the update)
 int blas_xr_update_dot32(qcd_ctx *c, float2 *x, float2 *r, const float2 *ph, const float2 *sh, const float2 *s,
                          const float2 *t, const float2 *rh, const BicgScalars *S, long n, int nrhs, double *out,

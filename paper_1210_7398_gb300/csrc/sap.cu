@@ -257,8 +257,8 @@ struct SsorArgs {
 // never the chain's longest part) and issue a quarter more per site; a warp per update, with its records
 // staged in shared memory, was bound by instruction issue (about 450 per site, 100 here).  Loads wait for
 // the arrival at the barrier: issued before it, they delay its release (1313 us instead of 1192).
-// 12^3x24, 6^3x12 blocks, 3^3x6 sub-blocks, FP32, 4 sweeps, 4 cycles: 2010 -> 1192 us; 24^3x48, FP16, 2
-// sweeps, 4 right-hand sides: 6^3x12 blocks 6098 -> 2749, 4^4 blocks 3619 -> 1880 (before: a warp per update,
+// 12^3x24, 6^3x12 blocks, 3^3x6 sub-blocks, FP32, 4 sweeps, 4 cycles: 2010 -> 1169 us; 24^3x48, FP16, 2
+// sweeps, 4 right-hand sides: 6^3x12 blocks 6098 -> 2708, 4^4 blocks 3619 -> 1873 (before: a warp per update,
 // or an octet of lanes where many CTAs shared an SM).
 template <bool HALF, int FORM>
 __global__ void __launch_bounds__(quad_threads(HALF, FORM), FORM == kFormShared && HALF ? 8 : 0) k_ssor_quad(SsorArgs a) {
