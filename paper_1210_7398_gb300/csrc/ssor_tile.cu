@@ -417,7 +417,7 @@ __device__ __forceinline__ void load_y_other(const TileArgs &a, int rhs, long mm
 // A warp item is 16 (site, right-hand side) pairs of one level, two lanes each; the items of a level are
 // dealt to the warps in turn, the same in every pass, so a lane meets the same sites throughout and
 // keeps what it needs of them in its own tensor-memory columns.  ALL: every item has a slot there.
-// FLAT (FP32): the prologue takes the block in one go (tile_flat).
+// FLAT: the prologue and the epilogue take the block in one go, not level by level (tile_flat).
 template <bool HALF, int R, bool ALL, bool FLAT = false>
 __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(TileArgs a) {
     chain_wait();
@@ -515,9 +515,8 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
     float *const yh = ys + y_me + half_w, *const fh = fs + y_me + half_w;  // the lane's half in slot 0
 
     // ---- prologue: f = r (or v) + kappa F H_{cc'} y_{c'} on the block's sites ----
-    // FP16: f waits in tensor memory (in r without a slot) until the scale is known, with the lanes that will
-    // take its sites; r holds it where the epilogue needs it.  FP32: r holds it, and a block of narrow levels is
-    // taken in one go (tile_flat)
+    // FP16: f waits in tensor memory (in r without a slot) until the scale is known; r holds it where the
+    // epilogue needs it.  FP32: r holds it
     constexpr bool f_tm = HALF && ALL;
     const bool f_r = !f_tm || a.store_r;
     const float4 *src = a.first ? a.v + roff : rr;
@@ -599,15 +598,16 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
         my_scale = scale_s[r_me] > 0.f ? scale_s[r_me] : 1.f;
         inv_scale = 1.f / my_scale;
         // the source of the sweeps into shared memory, in the right-hand side's units, by the lanes
-        // that will read it
-        for (int l = 0; l <= top; l++) {
-            const int4 lv = __ldg(a.levels + l);
+        // that hold it
+        for (int l = 0; l <= (FLAT ? 0 : top); l++) {
+            const int4 lv = FLAT ? make_int4(0, a.vol * R, 0, 0) : __ldg(a.levels + l);
             int slot = lv.w + (warp < lv.z);
             for (int j = warp < lv.z ? warp - lv.z + nwarp : warp - lv.z; j * 16 < lv.y; j += nwarp, slot++) {
                 if (!warp_active) continue;
                 const int i = j * 16 + pair;
                 const bool mine = i < lv.y && me_active;
-                const int4 pt = __ldg(a.pos + 2 * (lv.x + (i < lv.y ? i : 0) / R) + h);
+                const int pos = lv.x + (i < lv.y ? i : 0) / R;
+                const int4 pt = __ldg(a.pos + 2 * pos + h);
                 float2 f[6];
                 if constexpr (f_tm) tmem_ld12(tm + 12 * slot, f);
                 else if (mine) ld_half(rr + 6 * (long)pt.x, f);
@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
 #pragma unroll
                     for (int k = 0; k < 6; k++) f[k] = h2f(f2h(cscale(f[k], inv_scale)));
                     st_y6<true>(fh + (pt.y & 0xffff) * a.stride, f);
-                    if (l == 0) first_update(yh + (pt.y & 0xffff) * a.stride, f);
+                    if (FLAT ? pos < __ldg(a.levels).y / R : l == 0) first_update(yh + (pt.y & 0xffff) * a.stride, f);
                 }
                 __syncwarp();
             }
@@ -669,8 +669,8 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
         const bool more = sw + 1 < a.nsweep;
         const int rep = !ep && (fwd ? l == top : l == 0 && more) ? 2 : 1;
         // (the last level has no later neighbours, the first no earlier ones)
-        const bool other = (ep || !fwd || sw > 0) && l != (fwd ? top : 0), keep = !ep && (fwd || more || a.store_r);
-        const int4 lv = __ldg(a.levels + l);
+        const bool other = (ep || !fwd || sw > 0) && l != (fwd ? top : 0), keep = !ep && (fwd || more || (!FLAT && a.store_r));
+        const int4 lv = FLAT && ep ? make_int4(0, a.vol * R, 0, 0) : __ldg(a.levels + l);
         const int4 *posp = a.pos + (fwd ? 0 : 2 * a.vol) + h;
         int j = warp < lv.z ? warp - lv.z + nwarp : warp - lv.z, slot = lv.w + (warp < lv.z);
         // what does not depend on the other warps is loaded before the barrier
@@ -697,11 +697,12 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
             bool add = other && cached;  // the other side's sum is in tensor memory
             float2 c[6], fa[6];  // fa: F H_BB y (FP16: in the units of the right-hand side's scale)
             bool done = false;
-            if constexpr (!ALL) {
-                if (other && !cached) {  // no slot: sum the other side too, and set it aside
+            if constexpr (!ALL || FLAT) {
+                // no slot, or the epilogue in one go: sum the other side too, and set it aside
+                if (FLAT ? ep : other && !cached) {
                     const int4 po = __ldg(a.pos + (fwd ? 2 * a.vol : 0) + h + 2 * pos);
                     const unsigned no = __reduce_or_sync(0xffffffffu, (unsigned)po.y >> 16 & 15u);
-                    if (no) {
+                    if (FLAT || no) {
                         add = done = true;
 #pragma unroll 1
                         for (int side = 0; side < 2; side++) {
@@ -770,6 +771,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, kTileMinBlocks) k_sap_tile(Ti
             if (have) fetch();
         }
         // the next step
+        if (FLAT && ep) break;
         if (ep || (fwd && l < top)) {
             l++;
         } else if (fwd) {
@@ -1128,9 +1130,9 @@ template <bool HALF, bool ALL, bool FLAT = false> TileKernel tile_kernel(int R) 
     }
 }
 TileKernel tile_kernel(bool half, bool all, bool flat, int R) {
-    if (half) return all ? tile_kernel<true, true>(R) : tile_kernel<true, false>(R);
-    if (!all) return tile_kernel<false, false>(R);
-    return flat ? tile_kernel<false, true, true>(R) : tile_kernel<false, true>(R);
+    if (!all) return half ? tile_kernel<true, false>(R) : tile_kernel<false, false>(R);
+    if (flat) return half ? tile_kernel<true, true, true>(R) : tile_kernel<false, true, true>(R);
+    return half ? tile_kernel<true, true>(R) : tile_kernel<false, true>(R);
 }
 }  // namespace
 
@@ -1174,14 +1176,15 @@ float tile_cost(const SapPlan &p, int R, int nrhs) {
     return filled + 0.73f * (float)rounds;
 }
 
-// Whether the FP32 prologue takes the block's sites in one go instead of level by level: where no level has
-// more than 24 (site, right-hand side) pairs, one and a half warp items (and all hop sums have a slot).  The levels'
-// rounds then wait for memory one after the other for a few sites each.  us, level by level -> in one go: 2^4
-// blocks (levels of 1, 4, 6, 4, 1 sites), 2 cycles, 16^3x32: one right-hand side 680 -> 596, two 721 -> 655, four 873 ->
-// 839; 48^3x96: one 49262 -> 42981, four 63112 -> 60113; 2^3x4 blocks, 16^3x32: one 423 -> 381, two 497 -> 478, four (48
-// pairs) 734 -> 734.  Where levels fill their items the sites better stay with the lanes that sweep them: 3^3x6
-// blocks, 12^2x18x12, four (level of 52 to 156 pairs) 965 -> 987; 4^3x8, 32^3x64, four 10924 -> 11138.
-bool tile_flat(const SapPlan &p, int R) { return p.max_step * R <= 24; }
+// Whether the prologue and the epilogue take the block's sites in one go instead of level by level: where no
+// level has more than 24 (FP16: 12) (site, right-hand side) pairs (and all hop sums have a slot).  The levels' rounds
+// would wait for memory one after the other for a few sites each; the epilogue forms all eight hops for it.
+// us, level by level -> in one go, one sweep and three cycles (four and two): 2^4 blocks (levels of 1, 4, 6, 4, 1
+// sites) on 32^3x64, FP16, one right-hand side 13787 -> 10387 (16851 -> 14779), two 13712 -> 11123 (16680 -> 15481), four
+// (24 pairs) 16103 -> 15928 (19915 -> 19926); FP32 10693 -> 8606 (15716 -> 14300), 11485 -> 9442 (16528 -> 15360), 14180 ->
+// 13531 (19885 -> 19294); 2^3x4 blocks, FP16, one 6960 -> 5472 (8559 -> 7811), two (24) 8129 -> 8116 (10074 -> 10155);
+// FP32, two 7559 -> 7150 (10654 -> 10241), four (48) 12111 -> 12502 (16199 -> 16212).
+bool tile_flat(const SapPlan &p, int R) { return p.max_step * R <= (p.half ? 12 : 24); }
 
 // Tensor memory of a CTA: a slot of 12 FP32 columns per warp item, the items dealt to the warps in turn;
 // warps four apart share a lane quarter.  As many slots as fit the columns that leave the CTAs resident

@@ -205,8 +205,15 @@ def test_tile_solve_true_residual_under_oracle(st):
     ((16, 16, 16, 32), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 5),
     ((8, 8, 8, 16), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F16, 7),
     ((8, 8, 8, 8), (4, 4, 4, 4), (2, 2, 2, 2), q.QCD_F32, 12),
-    # levels of 12 pairs alone (the FP32 prologue in one go), of 48 for four (level by level)
+    # levels of 12 pairs alone (prologue and epilogue in one go), of 48 for four (level by level); FP16: 12, then 24
     ((16, 16, 16, 32), (2, 2, 2, 4), (1, 1, 1, 2), q.QCD_F32, 4),
+    ((16, 16, 16, 32), (2, 2, 2, 4), (1, 1, 1, 2), q.QCD_F16, 2),
+    # in one go, a warp item of the last level's sites alone
+    ((16, 8, 8, 8), (4, 1, 1, 1), (2, 1, 1, 1), q.QCD_F32, 8),
+    # 96 threads alone, with some sums formed anew without them; 128 and 256 threads
+    ((12, 12, 12, 32), (3, 3, 3, 4), (1, 1, 1, 2), q.QCD_F16, 2),
+    ((16, 16, 16, 32), (4, 2, 4, 4), (2, 1, 2, 2), q.QCD_F32, 2),
+    ((8, 8, 8, 16), (4, 2, 4, 4), (2, 1, 2, 2), q.QCD_F32, 2),
 ], ids=lambda c: "%s-%s-%s-n%d" % ("x".join(map(str, c[0])), "x".join(map(str, c[1])),
                                    "f16" if c[3] == q.QCD_F16 else "f32", c[4]))
 def test_tile_width_does_not_change_results(case):
