@@ -41,6 +41,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "fields.cuh"
 #include "qcd_internal.h"
@@ -1146,16 +1147,41 @@ int tile_set_attributes(qcd_ctx *c) {
 
 namespace {
 
-// threads of a CTA with R right-hand sides: two per (site, right-hand side) of the largest level, up to
-// kTileMaxThreads, and at least two warps, which share a small block's prologue (8^3x16, 2^4 blocks, one
-// right-hand side: 92 us per application with one warp, 62 with two, 66 with three; on 24^3x48 1480,
-// 1408, 1944)
-int tile_threads(const SapPlan &p, int R) {
-    const int t = ((p.max_step * R * 2 + 31) / 32) * 32;
-    return std::max(64, std::min(t, kTileMaxThreads));
-}
 // warp items (16 (site, right-hand side) pairs) of level l
 int tile_level_items(const SapPlan &p, int l, int R) { return ((p.h_step_ptr[l + 1] - p.h_step_ptr[l]) * R + 15) / 16; }
+// CTAs of T threads that an SM holds: by registers (128 a thread) and shared memory
+long tile_fit(size_t smem, int T) { return std::min<long>(kTileSmemPerSm / (smem + 1024), std::min(512 / T, 16)); }
+
+// Threads of a CTA with R right-hand sides: two per (site, right-hand side) of the largest level, up to
+// kTileMaxThreads, and at least two warps, which share a small block's prologue (8^3x16, 2^4 blocks, one
+// right-hand side: 92 us per application with one warp, 62 with two, 66 with three; on 24^3x48 1480,
+// 1408, 1944).
+//  - Two CTAs of 192 or 224 threads leave registers of an SM unused: 256 instead, or 128 where the SMs then take the
+//    levels in fewer rounds (its waves times the rounds of a wave).  us with 128 / 192 / 256, FP32, two sweeps of the SAP cycle: 4x2x4^2 blocks, two right-hand
+//    sides, 32^3x64 5806 / 7415 / 6836, 16^3x32 439 / 554 / 514, 8^3x16 233 / 191 / 174; 4^4, one, 32^3x64 3512 / 4157 /
+//    3782, 16^3x32 357 / 312 / 287; 3^3x6 in natural order, four (224), 30^3x60 14108 / 12619 / 12127.
+//  - FP16 blocks of narrow levels whose sums do not fit the tensor memory of eight CTAs of 64 threads (which
+//    reach half of its lanes): 96, unless the grid then takes more waves than that loses CTAs.  us with 64 / 96: 3^3x4
+//    blocks, 30^3x64 4631 / 4242, 18^3x32 (864 CTAs a colour) 559 / 598; 3^3x6 in natural order 30^3x60 4726 / 4423,
+//    18^3x36 855 / 735 (FP32 5089 / 5496 and 947 / 806: left).
+int tile_threads(const SapPlan &p, int R) {
+    const int t = std::max(64, std::min(((p.max_step * R * 2 + 31) / 32) * 32, kTileMaxThreads));
+    const double ctas = std::max(p.nblk[0], p.nblk[1]), sms = std::max(1, p.sms);
+    if (t == 192 || t == 224) {
+        auto time = [&](int T) {
+            int rounds = 0;
+            for (int l = 0; l < p.nsteps; l++) rounds += (tile_level_items(p, l, R) + T / 32 - 1) / (T / 32);
+            return std::ceil(ctas / (sms * std::max<long>(1, tile_fit(tile_smem_bytes(p, R), T)))) * rounds;
+        };
+        return time(128) < 0.85 * time(256) ? 128 : 256;
+    }
+    if (t == 64 && p.half) {
+        int items = 0;
+        for (int l = 0; l < p.nsteps; l++) items += tile_level_items(p, l, R);
+        if ((items + 1) / 2 * 12 > 64 && std::ceil(ctas / (sms * 5)) <= 1.7 * std::ceil(ctas / (sms * 8))) return 96;
+    }
+    return t;
+}
 
 // Relative time of an application with R right-hand sides per CTA: the share of the SMs' warps that its warp
 // items take, each costing more the more sites (16 / R) its record loads cover, and the rounds of items that a
@@ -1195,9 +1221,9 @@ bool tile_tmem(const SapPlan &p, int R, int T, size_t smem, long grid, TileArgs 
     int items = 0;
     for (int l = 0; l < p.nsteps; l++) items += tile_level_items(p, l, R);
     const int nw = T / 32, share = (nw + 3) / 4, need = (items + nw - 1) / nw;
-    // CTAs an SM will hold: by registers (128 a thread), shared memory and what the grid offers
-    const long sms = std::max(1, p.sms), fit = std::min<long>(kTileSmemPerSm / (smem + 1024), std::min(512 / T, 16));
-    const int ctas = (int)std::max<long>(1, std::min(fit, (grid + sms - 1) / sms));
+    // CTAs an SM will hold: what it can and what the grid offers
+    const long sms = std::max(1, p.sms);
+    const int ctas = (int)std::max<long>(1, std::min(tile_fit(smem, T), (grid + sms - 1) / sms));
     int most = 32;  // columns per CTA
     while (most * 2 <= 512 && most * 2 * ctas <= 512) most *= 2;
     // up to a third of the CTAs is given up for keeping more sums, where the grid's waves grow by no more than
